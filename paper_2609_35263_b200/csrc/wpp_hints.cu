@@ -27,67 +27,131 @@ __host__ __device__ inline uint64_t chain_step(uint64_t parent, uint64_t digest,
     return mix64(parent ^ mix64(digest + extra) ^ salt_term);
 }
 
-// One warp per token block: lanes add the terms of their tokens, a shuffle tree adds the lanes.  What is left
-// where the block's hash will go is mix64(digest + extraKeys): everything of the chain step that does not depend
-// on the parent hash is done here, in parallel.
+// Digests.  A warp takes kBlocks consecutive blocks: 16 or 8 token loads are in flight together, and the request the
+// blocks start in is found once, by a search whose every step is one load of 32 offsets (a bisection by one lane per
+// block was eight dependent loads in front of every block).  Every warp has one job, so that the hardware's own
+// scheduling of CTAs covers one warp's search with another's arithmetic.  What is left where a block's hash will go is
+// c ^ c >> 30 with c = mix64(digest + extraKeys) ^ salt term: everything of the chain step that does not depend on the
+// parent hash.  Bound by the arithmetic of the terms (two 64-bit products per token).
+template <int kBlocks>
 __global__ void __launch_bounds__(256) wpp_block_digest_kernel(const int32_t* __restrict__ tokens,
                                                                 const int64_t* __restrict__ token_offsets,
                                                                 const int64_t* __restrict__ block_offsets,
-                                                                int num_requests, int block_size,
+                                                                int num_requests, int block_size, uint64_t salt_term,
                                                                 const uint64_t* __restrict__ extra,
                                                                 uint64_t* __restrict__ out, int64_t total_blocks) {
     const int lane = threadIdx.x & 31;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t blk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; blk < total_blocks; blk += warps) {
-        int lo = 0, hi = num_requests;              // largest i with block_offsets[i] <= blk
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (block_offsets[mid] <= blk) lo = mid; else hi = mid;
-        }
-        const int32_t* src = tokens + token_offsets[lo] + (blk - block_offsets[lo]) * block_size;
-        uint64_t d = 0;
-        for (int k = lane; k < block_size; k += 32) d += token_term(src[k], (uint32_t)k);
+    const int64_t first = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kBlocks;
+    if (first >= total_blocks) return;
+    int lo = 0, hi = num_requests;              // largest i with block_offsets[i] <= first
+    while (hi - lo > 1) {
+        const int width = (hi - lo + 31) / 32, i = lo + lane * width;
+        const unsigned le = __ballot_sync(0xffffffffu, i < hi && block_offsets[i] <= first) | 1u;
+        const int last = 31 - __clz((int)le);
+        hi = min(hi, lo + (last + 1) * width);
+        lo += last * width;
+    }
+    // lane j < kBlocks: where block first + j starts
+    const int cnt = (int)min((int64_t)kBlocks, total_blocks - first);
+    int64_t start = 0;
+    if (lane < cnt) {
+        int r = lo;
+        while (r + 1 < num_requests && block_offsets[r + 1] <= first + lane) ++r;
+        start = token_offsets[r] + (first + lane - block_offsets[r]) * block_size;
+    }
+    const int32_t* src[kBlocks];
+    uint64_t d[kBlocks];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        if (lane == 0) out[blk] = mix64(d + (extra ? extra[blk] : 0ull));
+    for (int j = 0; j < kBlocks; ++j) {
+        src[j] = tokens + __shfl_sync(0xffffffffu, start, j);
+        d[j] = 0;
+    }
+    constexpr int kU = kBlocks == 1 ? 8 : 2;
+    for (int k0 = 0; k0 < block_size; k0 += 32 * kU) {
+        int32_t t[kBlocks][kU];
+#pragma unroll
+        for (int j = 0; j < kBlocks; ++j)
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int k = k0 + 32 * u + lane;
+                t[j][u] = (j < cnt && k < block_size) ? __ldg(src[j] + k) : 0;
+            }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int k = k0 + 32 * u + lane;
+            if (k0 + 32 * u >= block_size) break;
+#pragma unroll
+            for (int j = 0; j < kBlocks; ++j) d[j] += k < block_size ? token_term(t[j][u], (uint32_t)k) : 0ull;
+        }
+    }
+    uint64_t mine = 0;
+#pragma unroll
+    for (int j = 0; j < kBlocks; ++j) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d[j] += __shfl_xor_sync(0xffffffffu, d[j], o);
+        if (lane == j) mine = d[j];
+    }
+    if (lane < cnt) {
+        const uint64_t c = mix64(mine + (extra ? extra[first + lane] : 0ull)) ^ salt_term;
+        out[first + lane] = c ^ (c >> 30);
     }
 }
 
-// One thread per request walks its blocks in order: H_i = mix64(H_{i-1} xor m_i xor salt term).  The chain is
-// sequential by definition; the loads are not, so eight of them are in flight ahead of it.
-__global__ void wpp_hash_chain_kernel(const int64_t* __restrict__ block_offsets, int num_requests, uint64_t salt_term,
-                                      uint64_t* __restrict__ hashes) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= num_requests) return;
-    uint64_t h = 0;
-    const int64_t end = block_offsets[i + 1];
-    int64_t b = block_offsets[i];
-    if (b + 8 <= end) {
-        uint64_t cur[8], nxt[8];
+// The chain H_i = mix64(H_{i-1} ^ mix64(digest_i + extraKeys_i) ^ salt term) is sequential by definition: one lane of a
+// warp walks a request's blocks, and what bounds it is the step's own dependent arithmetic (79 clocks, measured alone).
+// With z the value before mix64's last shift, h = z ^ z >> 31, the next step starts from
+//     h ^ c ^ (h ^ c) >> 30  =  z ^ z >> 30 ^ z >> 31 ^ z >> 61 ^ (c ^ c >> 30),
+// whose shifts are independent of one another and whose last term the digests left ready: two dependent operations
+// between the multiplications instead of four.  The warp moves kStage blocks at a time through shared memory - the next
+// stage's loads are in flight while this one is chained, the finished hashes leave as coalesced stores - so that the
+// walk never waits on global memory; inside a stage eight terms are read before and eight hashes written after the
+// eight steps between them (a load that may alias the store before it would put shared-memory latency into every step).
+constexpr int kStage = 128, kPerLane = kStage / 32;
+__global__ void __launch_bounds__(32) wpp_hash_chain_kernel(const int64_t* __restrict__ block_offsets,
+                                                            uint64_t* __restrict__ hashes) {
+    __shared__ uint64_t buf[kStage];
+    const int lane = threadIdx.x;
+    const int64_t b0 = block_offsets[blockIdx.x], n = block_offsets[blockIdx.x + 1] - b0;
+    uint64_t* h = hashes + b0;
+    uint64_t nxt[kPerLane];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) cur[k] = hashes[b + k];
-        for (; b + 8 <= end; b += 8) {
-            const bool more = b + 16 <= end;
-            if (more) {                         // the next eight are requested before this eight is chained
+    for (int u = 0; u < kPerLane; ++u) nxt[u] = u * 32 + lane < n ? h[u * 32 + lane] : 0ull;
+    uint64_t z = 0;
+    for (int64_t first = 0; first < n; first += kStage) {
 #pragma unroll
-                for (int k = 0; k < 8; ++k) nxt[k] = hashes[b + 8 + k];
-            }
+        for (int u = 0; u < kPerLane; ++u) buf[u * 32 + lane] = nxt[u];
+        __syncwarp();
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                h = mix64(h ^ cur[k] ^ salt_term);
-                cur[k] = h;
-            }
+        for (int u = 0; u < kPerLane; ++u) {
+            const int64_t i = first + kStage + u * 32 + lane;
+            nxt[u] = i < n ? h[i] : 0ull;
+        }
+        if (lane == 0) {
+            const int cnt = (int)min((int64_t)kStage, n - first);
+#pragma unroll 1
+            for (int i = 0; i < cnt; i += 8) {          // (steps past the last block compute on zeros nobody reads)
+                uint64_t c[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) hashes[b + k] = cur[k];
-            if (more) {
+                for (int j = 0; j < 8; ++j) c[j] = buf[i + j];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) cur[k] = nxt[k];
+                for (int j = 0; j < 8; ++j) {
+                    uint64_t x = (z ^ (z >> 30)) ^ ((z >> 31) ^ (z >> 61)) ^ c[j];
+                    x *= 0xBF58476D1CE4E5B9ull;
+                    x ^= x >> 27;
+                    z = x * 0x94D049BB133111EBull;
+                    c[j] = z ^ (z >> 31);
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) buf[i + j] = c[j];
             }
         }
-    }
-    for (; b < end; ++b) {
-        h = mix64(h ^ hashes[b] ^ salt_term);
-        hashes[b] = h;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < kPerLane; ++u) {
+            const int64_t i = first + u * 32 + lane;
+            if (i < n) h[i] = buf[u * 32 + lane];
+        }
+        __syncwarp();
     }
 }
 
@@ -122,12 +186,18 @@ extern "C" int wpp_hash_blocks(const wpp_ctx* ctx, const int32_t* tokens, const 
     if (!tokens || !token_offsets || !block_offsets || !hashes_out) return WPP_ERR_INVALID_ARG;
     if (int rc = wpp_ctx_check_device(ctx)) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    int64_t blocks = (total_blocks * 32 + 255) / 256;
-    if (blocks > 148 * 16) blocks = 148 * 16;
-    wpp_block_digest_kernel<<<(unsigned)blocks, 256, 0, st>>>(tokens, token_offsets, block_offsets, num_requests,
-                                                              block_size, extra, hashes_out, total_blocks);
-    wpp_hash_chain_kernel<<<(unsigned)((num_requests + 31) / 32), 32, 0, st>>>(
-        block_offsets, num_requests, salt * 0x9E3779B97F4A7C15ull, hashes_out);
+    const uint64_t salt_term = salt * 0x9E3779B97F4A7C15ull;
+    // eight blocks per warp once that still gives every SM 32 warps; one below, where a warp's latency is all that counts
+    const bool wide = total_blocks >= 8ll * 32 * 148;
+    const int64_t ctas = (total_blocks + (wide ? 63 : 7)) / (wide ? 64 : 8);
+    if (ctas > 0x7fffffffll) return WPP_ERR_INVALID_ARG;
+    if (wide)
+        wpp_block_digest_kernel<8><<<(unsigned)ctas, 256, 0, st>>>(tokens, token_offsets, block_offsets, num_requests,
+                                                                   block_size, salt_term, extra, hashes_out, total_blocks);
+    else
+        wpp_block_digest_kernel<1><<<(unsigned)ctas, 256, 0, st>>>(tokens, token_offsets, block_offsets, num_requests,
+                                                                   block_size, salt_term, extra, hashes_out, total_blocks);
+    wpp_hash_chain_kernel<<<(unsigned)num_requests, 32, 0, st>>>(block_offsets, hashes_out);
     return cudaGetLastError() == cudaSuccess ? WPP_OK : WPP_ERR_CUDA;
 }
 
