@@ -396,8 +396,10 @@ typedef struct {
     int32_t num_slots;      /* slots of state_pool, each H * d_k * d_v floats */
     int32_t snap_interval;  /* > 0: snapshot whenever the tokens folded into S reach a multiple of it; 0: none */
     int32_t max_snaps;      /* row length of snap_slots (0 when snap_interval is 0) */
-    int32_t layout;         /* 0: the library chooses (the chunk-parallel form when a large enough workspace is given
-                             * and the wave has at least 64 tokens per request on average, else 1 or 2);
+    int32_t layout;         /* 0: the library chooses (when a large enough workspace is given and the wave has at least
+                             * 64 tokens per request on average, the chunk-parallel form or the same arithmetic in
+                             * groups of 16 positions with the state in registers, whichever is estimated to be faster
+                             * for these sizes; else 1 or 2);
                              * 1: token by token, one CTA per (request, head); 2: token by token, four CTAs per
                              * (request, head) of 32 columns each; 3: chunk-parallel on the tensor cores */
     int64_t total_tokens;   /* T = row_offsets[R] */
@@ -425,7 +427,7 @@ typedef struct {
  * A request with an empty chunk copies state_in to state_out.  Returns WPP_ERR_INVALID_ARG for null or misaligned
  * pointers or negative sizes, WPP_ERR_UNSUPPORTED for d_k, d_v other than 128, WPP_ERR_WORKSPACE_TOO_SMALL when
  * layout 3 is asked for without enough workspace, WPP_ERR_CUDA for a launch failure.  The chunk-parallel form
- * enqueues three kernels (block offsets, per-block preparation, the chain over the blocks), the others one. */
+ * of layout 3 enqueues three kernels (block offsets, per-block preparation, the chain over the blocks), the others one. */
 int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const void* q, const void* k, const void* v,
                   const float* alpha, const float* beta, const int64_t* row_offsets, const int32_t* prefix_lens,
                   float* state_pool, const int32_t* state_in, const int32_t* state_out, const int32_t* snap_slots,

@@ -25,7 +25,7 @@ struct MapKey {
     const void* base;
     uint64_t dims[4], strides[3];
     uint32_t box[4];
-    int rank;
+    int rank, swizzle;
 };
 struct MapEntry {
     MapKey key;
@@ -215,16 +215,17 @@ extern "C" int wpp_selftest_bounded_wait(const wpp_ctx* ctx, int64_t limit_cycle
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// bf16 tensor map with 128-byte swizzle; dims/strides innermost first, strides in bytes for dims 1..rank-1.
+// bf16 tensor map, with 128-byte swizzle unless told otherwise; dims/strides innermost first, strides in bytes for dims 1..rank-1.
 // Looked up in the context's cache first (six maps per attention call; encoding them costs more than a small
 // wave's kernel).
 static int make_map(const wpp_ctx* cctx, CUtensorMap* m, const void* base, int rank, const uint64_t* dims,
-                    const uint64_t* strides_bytes, const uint32_t* box) {
+                    const uint64_t* strides_bytes, const uint32_t* box, bool swizzle = true) {
     wpp_ctx* ctx = const_cast<wpp_ctx*>(cctx);
     MapKey key;
     memset(&key, 0, sizeof(key));
     key.base = base;
     key.rank = rank;
+    key.swizzle = swizzle;
     for (int i = 0; i < rank; ++i) { key.dims[i] = dims[i]; key.box[i] = box[i]; }
     for (int i = 0; i < rank - 1; ++i) key.strides[i] = strides_bytes[i];
     std::lock_guard<std::mutex> guard(*ctx->map_lock);
@@ -245,7 +246,7 @@ static int make_map(const wpp_ctx* cctx, CUtensorMap* m, const void* base, int r
     for (int i = 0; i < rank; ++i) { gd[i] = dims[i]; bx[i] = box[i]; es[i] = 1; }
     for (int i = 0; i < rank - 1; ++i) gs[i] = strides_bytes[i];
     CUresult r = ctx->encode_tiled(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), gd,
-                                   gs, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                   gs, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cuda_fail(ctx, (int)r);
     MapEntry& en = ctx->maps[victim];
@@ -416,7 +417,7 @@ extern "C" int wpp_prefill_attention_varlen_static(const wpp_ctx* ctx, const wpp
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// Recurrent-state layer.  Workspace of the chunk-parallel form: block offsets, then per (block, head) the cut mask,
+// Recurrent-state layer.  Workspace of the chunk-parallel form's two passes: block offsets, then per (block, head) the cut mask,
 // the decay products at sub-block ends and the ten operand arrays the preparation kernel leaves for the chain kernel.
 struct KdaWorkspace {
     int64_t max_blocks, n_bh;
@@ -447,6 +448,30 @@ extern "C" size_t wpp_kda_workspace_bytes(const wpp_kda_desc* desc) {
     return kda_workspace(desc).bytes;
 }
 
+// Which chunk-parallel kernel: 0 = blocks of 64 tokens in two passes (preparation for all blocks in parallel, then the
+// chain), 1..3 = groups of 16 tokens with the state in registers (wpp_kda_group.cu), in CTAs of 128, 64 or 32 columns.
+// The two-pass form reads and writes 144 KB of operands per block but its chain is the fastest per token; the group form
+// has nothing in front of its chain and moves nothing but inputs and outputs.  The estimates below are microseconds for
+// C tokens per request, measured on 148 SMs (us; group with 128 / 64 / 32 columns | two passes):
+//     requests x heads x tokens    8x32x2048  677 / 801 / 1224 | 733     1x32x512    91 /  75 /   51 |   62
+//                                  4x32x256    51 /  58 /  105 |  75     1x8x2048   336 / 276 /  178 |  142
+//                                  4x32x4096  670 / 801 / 1374 | 722     2x32x8192 1328 / 1103 / 1369 | 913
+//                                  8x32x64     34 /  36 /   67 |  50     64x32x256  659 / 740 / 1409 | 782
+// Error against the fp32 token-by-token form, rms of the states over their rms: 6.0e-6 (two passes: 4.9e-6); outputs equal.
+static int kda_chunk_form(const wpp_kda_desc* d, int sms) {
+    const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
+    auto rounds = [&](double ctas) { return ceil(ctas / sms); };
+    const double prep = n * C * 0.9e-3 * 148 / sms, chain = rounds(n) * C * 0.0525, operands = n * C * 0.49e-3;
+    const double t[4] = {35 + prep + (chain > operands ? chain : operands),
+                         rounds(n) * C * 0.165,                                                       // one CTA per SM
+                         2 * n <= sms ? C * 0.135 : rounds(n) * C * 0.195,                            // two per SM
+                         rounds(4 * n) * C * 0.084};
+    int best = 0;
+    for (int i = 1; i < 4; ++i)
+        if (t[i] < t[best]) best = i;
+    return best;
+}
+
 extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const void* q, const void* k, const void* v,
                              const float* alpha, const float* beta, const int64_t* row_offsets,
                              const int32_t* prefix_lens, float* state_pool, const int32_t* state_in,
@@ -473,6 +498,10 @@ extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const
         if (!workspace || workspace_bytes < w.bytes) return WPP_ERR_WORKSPACE_TOO_SMALL;
         if ((reinterpret_cast<uintptr_t>(workspace) & 255) != 0) return WPP_ERR_INVALID_ARG;
         if (w.n_bh * 64 > 0x7fffffffll || desc->total_tokens > 0x7fffffffll) return WPP_ERR_UNSUPPORTED;
+    }
+    // (layout 3 is always the two passes: their result does not depend on how long the rest of the chunk is)
+    const int form = tensor_form && desc->layout == 0 ? kda_chunk_form(desc, ctx->sm_count) : 0;
+    if (tensor_form && form == 0) {
         char* ws = static_cast<char*>(workspace);
         wpp::KdaTcParams p;
         memset(&p, 0, sizeof(p));
@@ -561,7 +590,27 @@ extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const
     p.num_slots = desc->num_slots;
     p.snap_interval = desc->snap_interval;
     p.max_snaps = desc->max_snaps;
-    int e = wpp_launch_kda(&p, ctx->sm_count, desc->layout, cuda_stream);
+    int e;
+    if (tensor_form) {
+        CUtensorMap maps[4];
+        memset(maps, 0, sizeof(maps));
+        int rc;
+        if (desc->total_tokens > 0) {
+            // boxes of the 16 rows of a group: whole rows of q, k and alpha (fp32 as a bf16 map with twice the elements:
+            // the copies move bytes), 64-column swizzled halves of v
+            const uint64_t H = (uint64_t)desc->num_heads, T = (uint64_t)desc->total_tokens;
+            const uint64_t dims[3] = {128, H, T}, dims_a[3] = {256, H, T};
+            const uint64_t strides[2] = {256, 256 * H}, strides_a[2] = {512, 512 * H};
+            const uint32_t box[3] = {128, 1, 16}, box_v[3] = {64, 1, 16}, box_a[3] = {256, 1, 16};
+            if ((rc = make_map(ctx, &maps[0], q, 3, dims, strides, box, false)) != WPP_OK) return rc;
+            if ((rc = make_map(ctx, &maps[1], k, 3, dims, strides, box, false)) != WPP_OK) return rc;
+            if ((rc = make_map(ctx, &maps[2], v, 3, dims, strides, box_v)) != WPP_OK) return rc;
+            if ((rc = make_map(ctx, &maps[3], alpha, 3, dims_a, strides_a, box_a, false)) != WPP_OK) return rc;
+        }
+        e = wpp_launch_kda_group(&p, maps, form, cuda_stream);
+    } else {
+        e = wpp_launch_kda(&p, ctx->sm_count, desc->layout, cuda_stream);
+    }
     if (e != 0) return cuda_fail(ctx, e);
     const_cast<wpp_ctx*>(ctx)->launches += 1;
     return WPP_OK;

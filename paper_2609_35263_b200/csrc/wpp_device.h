@@ -104,6 +104,8 @@ int wpp_launch_attention_small(int head_dim, const CUtensorMap* tq, const CUtens
                                const wpp::AttnParams* p, int num_ctas, void* stream);
 int wpp_launch_append(const wpp::AppendParams* p, int num_sms, void* stream);
 int wpp_launch_combine(const wpp::CombineParams* p, int num_combine, void* stream);
+// maps: q, k, v, alpha; form: 1, 2, 3 = CTAs of 128, 64, 32 columns of the state
+int wpp_launch_kda_group(const wpp::KdaParams* p, const CUtensorMap* maps, int form, void* stream);
 int wpp_launch_kda(const wpp::KdaParams* p, int num_sms, int layout, void* stream);
 int wpp_launch_selftest_wait(long long limit_cycles, int32_t* status, long long* waited_cycles, void* stream);
 }

@@ -14,10 +14,13 @@
 // producer warps of the same CTA leave them a group ahead.  Nothing crosses HBM but the inputs, the outputs and the
 // states.
 //
-// Why not the tensor cores' asynchronous form, whose rate is four times higher: with the state in tensor memory every
-// step is a chain of hand-overs between the issuing thread, the tensor pipe and the warps that scale, split and store
-// (measured: 6.5 K clocks per 64 tokens and chain for the chain alone, 14.5 K clocks of an SM per 64 tokens for the
-// operands, which crossed HBM twice).  Here a group's chain stays inside a warp.
+// Why mma.sync beside the tensor cores' asynchronous form (wpp_kda_tc.cu), whose rate is eight times higher: with the
+// state in tensor memory a step is a chain of hand-overs between the issuing thread, the tensor pipe and the warps that
+// scale, split and store, and its operands need a pass of their own in front (14.5 K clocks of an SM per 64 tokens, 144 KB
+// written and read back).  Here a group's chain stays inside a warp: 22 K clocks of an SM per 64 tokens in all, no second
+// pass.  8 x 2,048 tokens, 32 heads: 733 -> 677 us; 8 x 64: 50 -> 34 us; 1 x 512: 62 -> 51 us (the choice: kda_chunk_form).
+// What bounds a group now (clocks, 5.6 K): the products 3.5 K of which the MMA pipe is busy 2.6 K, U 0.6 K, hand-over and
+// outputs 1.5 K; the producers are idle half the time.
 //
 // Precision.  Every operand is split into two bf16 terms, x = hi + lo (16 significant bits), and every product is three
 // MMAs, hi hi + hi lo + lo hi (the dropped lo lo is 2^-17 relative), accumulated in fp32.
@@ -791,17 +794,16 @@ static int launch(const Maps& maps, const KdaParams& p, cudaStream_t st) {
 }  // namespace wpp
 
 // maps: q, k, v, alpha with boxes of 16 rows (v: 64 columns, 128-byte swizzle; the others whole rows, no swizzle)
-extern "C" int wpp_launch_kda_group(const wpp::KdaParams* p, const CUtensorMap* maps, int num_sms, void* stream) {
+// form 1: CTAs of 128 columns (eight column warps, two producer warpgroups, one CTA per SM): the operands of a group are
+//         made once per chain; for waves with enough (request, head) pairs to fill the SMs.
+// form 2: 64 columns (four column warps, one producer warpgroup, two CTAs per SM).
+// form 3: 32 columns, the channels halved between paired warps: the shortest chain per group, for a few long chains.
+extern "C" int wpp_launch_kda_group(const wpp::KdaParams* p, const CUtensorMap* maps, int form, void* stream) {
     using namespace wpp::kdag;
     Maps m;
     m.q = maps[0]; m.k = maps[1]; m.v = maps[2]; m.alpha = maps[3];
     cudaStream_t st = (cudaStream_t)stream;
-    const long long chains = (long long)p->num_heads * p->num_requests;
-    int variant = 4 * chains <= num_sms ? 3 : (chains <= num_sms ? 2 : 1);
-#ifdef WPP_KDA_VARIANT
-    variant = WPP_KDA_VARIANT;
-#endif
-    if (variant == 3) return launch<32, 1, 2, 2, 1>(m, *p, st);
-    if (variant == 2) return launch<64, 1, 1, 1, 2>(m, *p, st);
+    if (form == 3) return launch<32, 1, 2, 2, 1>(m, *p, st);
+    if (form == 2) return launch<64, 1, 1, 1, 2>(m, *p, st);
     return launch<128, 1, 1, 2, 1>(m, *p, st);
 }

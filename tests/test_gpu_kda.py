@@ -268,3 +268,25 @@ def test_random_waves_in_the_chunk_parallel_form(seed):
     assert status == 0 and np.isfinite(got_o).all() and np.isfinite(got_pool).all()
     _close_out(got_o, ref_o, "outputs")
     _close_state(got_pool, ref_pool, "state pool")
+
+
+@pytest.mark.parametrize("H_", [1, 7, 9, 17])        # 5 requests: CTAs of 32 columns (up to 37 chains), of 64 (up to 74), of 128
+@pytest.mark.parametrize("interval,decays", [(0, False), (7, True), (64, False), (1000, True)])
+def test_groups_of_sixteen_positions_match_the_oracle(H_, interval, decays):
+    """The library's choice for short chunks, groups of 16 positions with the state in registers: chunk lengths and
+    prefixes around the group size, an empty chunk, snapshots inside groups, decays that have to end a group or go to
+    the state directly.  Operands have 16 significant bits as in the chunk-parallel form: the same tolerances."""
+    lens, prefix = [0, 1, 17, 130, 333], [5, 16, 31, 0, 4097]
+    w = W.kda_workload("groups", 70 + H_, lens, H_, prefix, resume=[True, False, True, False, True], snap_interval=interval)
+    t = w.tensors()
+    if decays:
+        rng = np.random.default_rng(H_)
+        a = t["alpha"].numpy()
+        for val, count in ((0.0, 6), (1e-9, 6), (1e-30, 4), (0.2, 200)):
+            a[rng.integers(0, a.shape[0], count), rng.integers(0, H_, count), rng.integers(0, 128, count)] = val
+    got_o, got_pool, status = _gpu(w, t)
+    assert status == 0
+    heads = [0, H_ - 1]
+    ref_o, ref_pool = _oracle(w, t, heads=heads)
+    _close_out(got_o[:, heads], ref_o, "outputs")
+    _close_state(got_pool[:, heads], ref_pool, "state pool")
