@@ -387,7 +387,9 @@ extern "C" int wpp_prefill_attention_varlen(const wpp_ctx* ctx, const wpp_batch_
         c.o_head_stride = d.o_head_stride;
         c.num_q_heads = d.num_q_heads;
         c.head_dim = d.head_dim;
-        c.tile_m = hd->tile_m;
+        c.max_rows = hd->max_combine_rows;
+        c.off_q_offsets = hd->off_q_offsets;
+        c.off_combine = hd->off_combine;
         e = wpp_launch_combine(&c, hd->num_combine, cuda_stream);
         if (e != 0) return cuda_fail(ctx, e);
         const_cast<wpp_ctx*>(ctx)->launches += 1;

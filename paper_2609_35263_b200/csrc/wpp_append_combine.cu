@@ -52,39 +52,67 @@ __global__ void __launch_bounds__(256) wpp_append_kernel(const AppendParams p) {
     }
 }
 
-// One block per split half tile; one warp per row, lanes across head_dim.  Partials are merged in increasing split
-// order with weights exp2(lse_s - max lse), so the result does not depend on scheduling.
-__global__ void __launch_bounds__(256) wpp_combine_kernel(const CombineParams p) {
+// Combine: one warp per row of a split half tile, eight rows per block, grid (half tiles, row groups).  Partials are merged
+// in increasing split order with weights exp2(lse_s - max lse), so the result does not depend on scheduling.  The pass is
+// a read of the partials; what bounds it is how many of them are in flight.  A lane takes the weight of one part (parts
+// beyond 32 in further rounds) and then four (head_dim 64: two) columns of every part, eight parts' loads at a time.  One
+// block per half tile whose warps walked the rows, a part's scalar loads after the other's, took 23 us for the 272 half
+// tiles x 64 rows x 2 parts of 32 x 64 new tokens over 32,768 cached ones.
+constexpr int kCombineRows = 8, kCombineBatch = 8;
+template <int D>
+__global__ void __launch_bounds__(32 * kCombineRows) wpp_combine_kernel(const CombineParams p) {
+    constexpr int kV = D / 32;
     const char* plan = static_cast<const char*>(p.plan);
-    const WppPlanHeader* hd = reinterpret_cast<const WppPlanHeader*>(plan);
-    const int32_t* q_offsets = reinterpret_cast<const int32_t*>(plan + hd->off_q_offsets);
-    const WppCombine cu = reinterpret_cast<const WppCombine*>(plan + hd->off_combine)[blockIdx.x];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int D = p.head_dim;
-    for (int r = warp; r < cu.rows; r += 8) {
-        float m = -INFINITY;
-        for (int s = 0; s < cu.num_splits; ++s)
-            m = fmaxf(m, p.ws_lse[((int64_t)(cu.slot0 + s) * 2 + cu.half) * 128 + cu.lane0 + r]);
-        const int64_t tok = (int64_t)q_offsets[cu.request] + cu.row0 + r;
-        __nv_bfloat16* dst = p.out + tok * p.o_token_stride + (int64_t)cu.head * p.o_head_stride;
-        float wsum = 0.f;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        if (m > -INFINITY) {
-            for (int s = 0; s < cu.num_splits; ++s) {
-                const int64_t row = ((int64_t)(cu.slot0 + s) * 2 + cu.half) * 128 + cu.lane0 + r;
-                const float l = p.ws_lse[row];
-                if (l == -INFINITY) continue;       // that part saw no key of this row; its O row is not defined
-                const float w = exp2f(l - m);
-                wsum += w;
-                for (int e = lane, k = 0; e < D; e += 32, ++k) acc[k] += w * p.ws_o[row * D + e];
+    const WppCombine cu = reinterpret_cast<const WppCombine*>(plan + p.off_combine)[blockIdx.x];
+    const int lane = threadIdx.x & 31, r = blockIdx.y * kCombineRows + (threadIdx.x >> 5);
+    if (r >= cu.rows) return;
+    const int64_t tok = (int64_t)reinterpret_cast<const int32_t*>(plan + p.off_q_offsets)[cu.request] + cu.row0 + r;
+    const int64_t row = ((int64_t)cu.slot0 * 2 + cu.half) * 128 + cu.lane0 + r;      // + 256 per part
+    float m = -INFINITY, wsum = 0.f;
+    for (int s = lane; s < cu.num_splits; s += 32) m = fmaxf(m, p.ws_lse[row + s * 256]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    float acc[kV];
+#pragma unroll
+    for (int k = 0; k < kV; ++k) acc[k] = 0.f;
+    if (m > -INFINITY) {
+        for (int s0 = 0; s0 < cu.num_splits; s0 += 32) {
+            const int cnt = min(32, cu.num_splits - s0);
+            // a part that saw no key of this row has lse -inf: weight zero, its O row is not defined and not used
+            const float w_mine = lane < cnt ? exp2f(p.ws_lse[row + (s0 + lane) * 256] - m) : 0.f;
+            for (int b0 = 0; b0 < cnt; b0 += kCombineBatch) {
+                float x[kCombineBatch][kV], w[kCombineBatch];
+#pragma unroll
+                for (int u = 0; u < kCombineBatch; ++u) {
+                    w[u] = __shfl_sync(0xffffffffu, w_mine, (b0 + u) & 31);
+                    const bool use = b0 + u < cnt && w[u] > 0.f;
+                    const float* src = p.ws_o + (row + (int64_t)(s0 + b0 + u) * 256) * D + lane * kV;
+                    if constexpr (kV == 4) {
+                        const float4 v = use ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        x[u][0] = v.x; x[u][1] = v.y; x[u][2] = v.z; x[u][3] = v.w;
+                    } else {
+                        const float2 v = use ? *reinterpret_cast<const float2*>(src) : make_float2(0.f, 0.f);
+                        x[u][0] = v.x; x[u][1] = v.y;
+                    }
+                    if (!use) w[u] = 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < kCombineBatch; ++u) {
+                    wsum += w[u];
+#pragma unroll
+                    for (int k = 0; k < kV; ++k) acc[k] += w[u] * x[u][k];
+                }
             }
         }
-        const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
-        for (int e = lane, k = 0; e < D; e += 32, ++k) dst[e] = __float2bfloat16_rn(acc[k] * inv);
-        if (p.lse && lane == 0)
-            p.lse[tok * p.num_q_heads + cu.head] =
-                wsum > 0.f ? (m + log2f(wsum)) * 0.6931471805599453f : -INFINITY;
     }
+    const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
+    __nv_bfloat16* dst = p.out + tok * p.o_token_stride + (int64_t)cu.head * p.o_head_stride + lane * kV;
+    if constexpr (kV == 4)
+        *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv));
+    else
+        *reinterpret_cast<uint32_t*>(dst) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
+    if (p.lse && lane == 0)
+        p.lse[tok * p.num_q_heads + cu.head] = wsum > 0.f ? (m + log2f(wsum)) * 0.6931471805599453f : -INFINITY;
 }
 
 // Self-test of the bounded wait every kernel of the library relies on: one warp waits, with a short limit, on
@@ -129,6 +157,8 @@ extern "C" int wpp_launch_append(const wpp::AppendParams* p, int num_sms, void* 
 
 extern "C" int wpp_launch_combine(const wpp::CombineParams* p, int num_combine, void* stream) {
     if (num_combine == 0) return 0;
-    wpp::wpp_combine_kernel<<<(unsigned)num_combine, 256, 0, (cudaStream_t)stream>>>(*p);
+    const dim3 grid((unsigned)num_combine, (unsigned)((p->max_rows + wpp::kCombineRows - 1) / wpp::kCombineRows));
+    if (p->head_dim == 128) wpp::wpp_combine_kernel<128><<<grid, 32 * wpp::kCombineRows, 0, (cudaStream_t)stream>>>(*p);
+    else wpp::wpp_combine_kernel<64><<<grid, 32 * wpp::kCombineRows, 0, (cudaStream_t)stream>>>(*p);
     return (int)cudaGetLastError();
 }

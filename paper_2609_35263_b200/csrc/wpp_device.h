@@ -48,7 +48,9 @@ struct CombineParams {
     __nv_bfloat16* out;
     float* lse;
     int64_t o_token_stride, o_head_stride;
-    int32_t num_q_heads, head_dim, tile_m;
+    int32_t num_q_heads, head_dim;
+    int32_t max_rows;                // most rows of a combine record
+    uint32_t off_q_offsets, off_combine;
 };
 
 struct KdaParams {

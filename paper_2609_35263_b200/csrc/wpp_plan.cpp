@@ -373,6 +373,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     hd.num_units = (int32_t)n_units;
     hd.num_combine = (int32_t)combines.size();
     hd.num_split_slots = slots;
+    for (const WppCombine& c : combines) hd.max_combine_rows = std::max(hd.max_combine_rows, c.rows);
     hd.tile_m = TM;
     hd.tile_n = WPP_TILE_N;
     hd.head_dim = d.head_dim;

@@ -4,7 +4,7 @@
 #include <stdint.h>
 
 #define WPP_PLAN_MAGIC 0x31505057u /* "WPP1" */
-#define WPP_PLAN_VERSION 7u
+#define WPP_PLAN_VERSION 8u
 #define WPP_TILE_N 128             /* keys per step */
 #define WPP_WS_HEADER_BYTES 256
 #define WPP_HALF_M 128             /* query rows per tensor-core tile (one TMEM lane per row) */
@@ -24,7 +24,8 @@ struct WppPlanHeader {
     uint32_t off_combine;           // WppCombine [num_combine]
     int32_t shape;                  // 1: two-half CTAs, one per SM; 2: single-half CTAs, two per SM (work item = half a unit)
     int32_t nonempty_halves;
-    uint32_t pad[6];
+    int32_t max_combine_rows;       // most rows of a combine record (sizes the combine pass's grid)
+    uint32_t pad[5];
 };
 
 // One work tile = two 128-row "halves" that share one K/V stream (same request, same KV head).  Each half

@@ -382,3 +382,13 @@ def test_cfg2_sampled_rows():
     got_lse = res["lse"][rows, heads].double().cpu().numpy()
     assert np.abs(got_lse - ref_lse).max() < 2e-2
     assert not torch.isnan(res["out"].float()).any()
+
+
+@pytest.mark.parametrize("d,Hq", [(128, 4), (64, 8)])
+@pytest.mark.parametrize("splits", [8, 9, 33, 64])
+def test_combine_of_many_parts(d, Hq, splits):
+    """The combine pass takes parts eight at a time and their weights 32 at a time: part counts around both, rows that do
+    not fill a block of eight, parts above a row's diagonal, packed heads and a whole 128-row half."""
+    w = W.custom_workload([8300, 37], [13, 129], Hq, 2, d, 64, seed=51, spare_pages=4)
+    res, _ = _full_parity(w, opts=wpp.PlanOpts(256, 0, splits, 0))
+    assert res["plan"].info.num_split_tiles > splits // 2
