@@ -274,13 +274,15 @@ def wpp_validate_batch(desc: BatchDesc, block_tables, prefix_lens, chunk_lens) -
     return int(load_library().wpp_validate_batch(ctypes.byref(desc), bt.ctypes.data, P.ctypes.data, C.ctypes.data))
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+# Addresses and streams go to the library as plain integers (the argument types convert them): an object per argument
+# and a torch.cuda.Stream per call were a third of the host time of a small wave.
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(ctx: Context, stream) -> int:
+    """The raw stream of `stream`, or of the current stream of the context's device (which must be the current device)."""
+    return torch._C._cuda_getCurrentRawStream(ctx.device) if stream is None else stream.cuda_stream
 
 
 def wpp_kv_append(ctx: Context, desc: BatchDesc, k_new, v_new, k_cache, v_cache, block_tables, prefix_lens,
@@ -288,8 +290,8 @@ def wpp_kv_append(ctx: Context, desc: BatchDesc, k_new, v_new, k_cache, v_cache,
     """Queue the KV append of one wave on `stream` (device tensors; int32 metadata on the device)."""
     st = load_library().wpp_kv_append(ctx.handle, ctypes.byref(desc), _ptr(k_new), _ptr(v_new), _ptr(k_cache),
                                       _ptr(v_cache), _ptr(block_tables), _ptr(prefix_lens), _ptr(chunk_lens),
-                                      ctypes.c_void_p(plan.host.data_ptr()), _ptr(plan.dev), _ptr(status),
-                                      _stream(stream))
+                                      plan.host.data_ptr(), _ptr(plan.dev), _ptr(status),
+                                      _stream(ctx, stream))
     _check(st, "wpp_kv_append")
 
 
@@ -300,8 +302,8 @@ def wpp_prefill_attention_varlen(ctx: Context, desc: BatchDesc, q, out, lse, k_c
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     st = load_library().wpp_prefill_attention_varlen(
         ctx.handle, ctypes.byref(desc), _ptr(q), _ptr(out), _ptr(lse), _ptr(k_cache), _ptr(v_cache),
-        _ptr(block_tables), _ptr(prefix_lens), _ptr(chunk_lens), ctypes.c_void_p(plan.host.data_ptr()),
-        _ptr(plan.dev), _ptr(workspace), ws_bytes, _ptr(status), _stream(stream))
+        _ptr(block_tables), _ptr(prefix_lens), _ptr(chunk_lens), plan.host.data_ptr(),
+        _ptr(plan.dev), _ptr(workspace), ws_bytes, _ptr(status), _stream(ctx, stream))
     _check(st, "wpp_prefill_attention_varlen")
 
 
@@ -322,15 +324,15 @@ def wpp_prefill_attention_varlen_static(ctx: Context, desc: BatchDesc, q, out, l
     stream capture."""
     st = load_library().wpp_prefill_attention_varlen_static(
         ctx.handle, ctypes.byref(desc), _ptr(q), _ptr(out), _ptr(lse), _ptr(k_cache), _ptr(v_cache),
-        _ptr(block_tables), _ptr(prefix_lens), _ptr(chunk_lens), ctypes.c_void_p(plan.host.data_ptr()),
-        _ptr(plan.dev), _ptr(status), _stream(stream))
+        _ptr(block_tables), _ptr(prefix_lens), _ptr(chunk_lens), plan.host.data_ptr(),
+        _ptr(plan.dev), _ptr(status), _stream(ctx, stream))
     _check(st, "wpp_prefill_attention_varlen_static")
 
 
 def wpp_selftest_bounded_wait(ctx: Context, limit_cycles: int, status, waited_cycles=None, stream=None) -> None:
     """Launch the bounded-wait self-test: a warp waits at most `limit_cycles` on a barrier nothing arrives on."""
     st = load_library().wpp_selftest_bounded_wait(ctx.handle, int(limit_cycles), _ptr(status), _ptr(waited_cycles),
-                                                  _stream(stream))
+                                                  _stream(ctx, stream))
     _check(st, "wpp_selftest_bounded_wait")
 
 
@@ -373,7 +375,7 @@ def wpp_hash_blocks(ctx: Context, tokens, token_offsets, block_offsets, block_si
         out = torch.empty(total, dtype=torch.int64, device=tokens.device)
     st = load_library().wpp_hash_blocks(ctx.handle, _ptr(tokens), _ptr(token_offsets), _ptr(block_offsets), max(R, 0),
                                         int(block_size), ctypes.c_uint64(int(salt) & (2 ** 64 - 1)), _ptr(extra_keys),
-                                        _ptr(out), total, _stream(stream))
+                                        _ptr(out), total, _stream(ctx, stream))
     _check(st, "wpp_hash_blocks")
     return out
 
@@ -478,6 +480,6 @@ def wpp_kda_chunk(ctx: Context, q, k, v, alpha, beta, row_offsets, state_pool, s
     st = load_library().wpp_kda_chunk(ctx.handle, ctypes.byref(desc), _ptr(q), _ptr(k), _ptr(v), _ptr(alpha), _ptr(beta),
                                       _ptr(row_offsets), _ptr(prefix_lens), _ptr(state_pool), _ptr(state_in),
                                       _ptr(state_out), _ptr(snap_slots), _ptr(out), _ptr(workspace), ws_bytes,
-                                      _ptr(status), _stream(stream))
+                                      _ptr(status), _stream(ctx, stream))
     _check(st, "wpp_kda_chunk")
     return out
