@@ -115,7 +115,7 @@ typedef struct {
                                  of a tile against 128-key steps (long tiles: the two halves and the tensor pipe overlap
                                  inside the CTA); 2: two small CTAs per SM, each working on one half against 64-key
                                  steps (short tiles: one CTA's tile start and end hide under the other's steps);
-                                 0: the library decides from the mean number of key steps per half */
+                                 0: the library decides, by estimated time */
 } wpp_plan_opts;
 
 typedef struct {
@@ -193,8 +193,10 @@ int wpp_kv_append(const wpp_ctx* ctx, const wpp_batch_desc* desc, const void* k_
  *                   at the same time need a workspace each.
  * A request whose prefix_lens[i] or chunk_lens[i] on the device differ from the plan's sets *status_dev =
  * WPP_ERR_PLAN_MISMATCH; its tiles are skipped (its output rows are not computed; rows of split tiles read as zero).
- * Enqueues a 256-byte memset and one persistent kernel (the shape the plan names), plus one combine kernel iff the
- * plan has split tiles.
+ * Enqueues one persistent kernel (the shape the plan names), a 256-byte memset in front of it when the tiles are taken
+ * from the counter (the small shape deals few or equally long tiles out instead), and one combine kernel iff the
+ * plan has split tiles.  The kernels may be set up on the GPU while the kernel before them in the stream still runs;
+ * they wait for its end before they touch memory.
  * Results are bit-reproducible for a given plan, whichever CTA takes which tile (no atomics on outputs; partials
  * are merged in a fixed order). */
 int wpp_prefill_attention_varlen(const wpp_ctx* ctx, const wpp_batch_desc* desc, const void* q, void* out,

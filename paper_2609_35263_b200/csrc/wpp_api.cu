@@ -366,11 +366,23 @@ extern "C" int wpp_prefill_attention_varlen(const wpp_ctx* ctx, const wpp_batch_
     const double scale = d.sm_scale > 0.f ? (double)d.sm_scale : 1.0 / sqrt((double)d.head_dim);
     p.scale_log2 = (float)(scale * 1.4426950408889634);
 
-    // the counter the CTAs take their tiles from starts at zero (a memset node on the caller's stream)
-    int e = (int)cudaMemsetAsync(workspace, 0, WPP_WS_HEADER_BYTES, (cudaStream_t)cuda_stream);
-    if (e != 0) return cuda_fail(ctx, e);
+    p.off_q_offsets = hd->off_q_offsets;
+    p.off_prefix = hd->off_prefix;
+    p.off_units = hd->off_units;
+    p.num_units = hd->num_units;
+    // The counter the CTAs take their tiles from starts at zero (a memset node on the caller's stream).  The small shape
+    // needs none when its items are dealt out: then nothing stands between it and the kernel before it.
+    int e = 0;
+    p.item_shift = hd->nonempty_halves > hd->num_units ? 1 : 0;
+    const int64_t items = (int64_t)hd->num_units << p.item_shift;
+    if (hd->shape == 2 && hd->deal_items) {
+        p.tile_counter = nullptr;
+    } else {
+        e = (int)cudaMemsetAsync(workspace, 0, WPP_WS_HEADER_BYTES, (cudaStream_t)cuda_stream);
+        if (e != 0) return cuda_fail(ctx, e);
+    }
     p.stats = ctx->stats_dev;
-    e = hd->shape == 2 ? wpp_launch_attention_small(d.head_dim, tq, &tk, &tv, &p, hd->num_ctas, cuda_stream)
+    e = hd->shape == 2 ? wpp_launch_attention_small(d.head_dim, tq, &tk, &tv, &p, (int)(items < hd->num_ctas ? items : hd->num_ctas), cuda_stream)
                        : wpp_launch_attention(d.head_dim, tq, &tk, &tv, &p, hd->num_ctas, choose_late_rescale(ctx),
                                               cuda_stream);
     if (e != 0) return cuda_fail(ctx, e);

@@ -15,6 +15,7 @@ namespace wpp {
 // nothing of it is written and the status word becomes WPP_ERR_PLAN_MISMATCH (Section 4.6: a position mismatch
 // fails execution instead of writing against the wrong cache state).
 __global__ void __launch_bounds__(256) wpp_append_kernel(const AppendParams p) {
+    grid_launch_dependents();
     const char* plan = static_cast<const char*>(p.plan);
     const WppPlanHeader* hd = reinterpret_cast<const WppPlanHeader*>(plan);
     const int32_t* q_offsets = reinterpret_cast<const int32_t*>(plan + hd->off_q_offsets);
@@ -62,6 +63,7 @@ constexpr int kCombineRows = 8, kCombineBatch = 8;
 template <int D>
 __global__ void __launch_bounds__(32 * kCombineRows) wpp_combine_kernel(const CombineParams p) {
     constexpr int kV = D / 32;
+    grid_dependency_wait();           // (launched while the attention kernel may still be running)
     const char* plan = static_cast<const char*>(p.plan);
     const WppCombine cu = reinterpret_cast<const WppCombine*>(plan + p.off_combine)[blockIdx.x];
     const int lane = threadIdx.x & 31, r = blockIdx.y * kCombineRows + (threadIdx.x >> 5);
@@ -158,7 +160,14 @@ extern "C" int wpp_launch_append(const wpp::AppendParams* p, int num_sms, void* 
 extern "C" int wpp_launch_combine(const wpp::CombineParams* p, int num_combine, void* stream) {
     if (num_combine == 0) return 0;
     const dim3 grid((unsigned)num_combine, (unsigned)((p->max_rows + wpp::kCombineRows - 1) / wpp::kCombineRows));
-    if (p->head_dim == 128) wpp::wpp_combine_kernel<128><<<grid, 32 * wpp::kCombineRows, 0, (cudaStream_t)stream>>>(*p);
-    else wpp::wpp_combine_kernel<64><<<grid, 32 * wpp::kCombineRows, 0, (cudaStream_t)stream>>>(*p);
-    return (int)cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(32 * wpp::kCombineRows);
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute overlap;
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &overlap;
+    cfg.numAttrs = 1;
+    return (int)cudaLaunchKernelEx(&cfg, p->head_dim == 128 ? wpp::wpp_combine_kernel<128> : wpp::wpp_combine_kernel<64>, *p);
 }

@@ -177,13 +177,13 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_launch_dependents();
 
     const char* plan = static_cast<const char*>(p.plan);
-    const WppPlanHeader* hd = reinterpret_cast<const WppPlanHeader*>(plan);
-    const int32_t* q_offsets = reinterpret_cast<const int32_t*>(plan + hd->off_q_offsets);
-    const int32_t* plan_prefix = reinterpret_cast<const int32_t*>(plan + hd->off_prefix);
-    const WppUnit* units = reinterpret_cast<const WppUnit*>(plan + hd->off_units);
-    const int num_units = hd->num_units;
+    const int32_t* q_offsets = reinterpret_cast<const int32_t*>(plan + p.off_q_offsets);
+    const int32_t* plan_prefix = reinterpret_cast<const int32_t*>(plan + p.off_prefix);
+    const WppUnit* units = reinterpret_cast<const WppUnit*>(plan + p.off_units);
+    const int num_units = p.num_units;
     // next tile index for a consuming role: -1 = no more tiles, -2 = the wait was abandoned
     Ring tile_ring = {0, 0};
     auto next_tile = [&]() -> int {
@@ -206,12 +206,15 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             // Tiles are requested in the order the issuers first touch them: K(0), K(1), V(0), K(2), V(1), ...
             Ring ring_k = {0, 0}, ring_v = {0, 0};
             uint32_t q_phase = 0;
-            bool dead = false;
+            bool dead = false, first = true;
             while (!dead) {
-                // take the next tile of the planner's order and tell the other roles
-                int u = 0;
-                if (lane == 0) u = (int)atomicAdd(p.tile_counter, 1u);
-                u = __shfl_sync(0xffffffffu, u, 0);
+                // take the next tile of the planner's order (the first one is this CTA's own) and tell the other roles
+                int u = (int)blockIdx.x;
+                if (!first) {
+                    if (lane == 0) u = (int)(gridDim.x + atomicAdd(p.tile_counter, 1u));
+                    u = __shfl_sync(0xffffffffu, u, 0);
+                }
+                first = false;
                 if (u >= num_units) u = -1;
                 {
                     const bool ok = mbar_wait(bTileEmpty + 8 * tile_ring.stage, tile_ring.phase ^ 1u, abort_flag);

@@ -18,11 +18,15 @@ struct AttnParams {
     float* ws_o;                     // split partials: [slots][2][128][d]
     float* ws_lse;                   // [slots][2][128], log2 units
     int32_t* status;                 // sticky device status word or null
-    uint32_t* tile_counter;          // zeroed before the launch: index of the next tile nobody has taken yet
+    uint32_t* tile_counter;          // zeroed before the launch: how many tiles have been taken beyond the first one per CTA;
+                                     // or null: round k of the CTAs takes tiles k gridDim .., rotated by k
     unsigned long long* stats;       // or null: [0] += key steps of the softmax warps, [1] += those that rescaled O
     int64_t o_token_stride, o_head_stride;
     int32_t num_q_heads, group, page_size, max_blocks, num_pages;
     float scale_log2;                // sm_scale * log2(e)
+    uint32_t off_q_offsets, off_prefix, off_units;   // of the plan's arrays (as in its header: one dependent read less)
+    int32_t num_units;
+    int32_t item_shift;              // small shape: 1 if an item is half a unit, 0 if no unit has a second half
 };
 
 struct AppendParams {

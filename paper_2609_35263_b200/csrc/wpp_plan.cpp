@@ -83,6 +83,36 @@ static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 constexpr int kTailSplitMaxRounds = 16, kTailSplitMaxParts = 4, kTailSplitMinSteps = 8, kTailSplitMinGainPct = 10;
 constexpr int64_t kTileFixedCost = 3, kPartExtraCost = 2, kCombineCost = 20;
 
+// Estimated microseconds of a wave on either kernel shape: tiles (or halves) handed out in order to the CTA free first,
+// each with a start and end and a time per 128-key step.  Constants from waves timed on 148 SMs, attention call in us, SM-wide |
+// small (requests x new tokens over cached ones, 64/8 heads of 128):
+//     1 x 64            20 |   7        32 x 64           45 |  21        32 x 256       117 | 105
+//     1 x 64 / 2048     34 |  22        32 x 64 / 256     61 |  43        32 x 512       306 | 290
+//     1 x 512           26 |  17        32 x 64 / 1024    96 | 108        32 x 1024      845 | 930
+//     1 x 2048         106 | 147        32 x 1 / 1024     58 |  37        4 x 1024       107 | 126
+//     8 x 256           41 |  31        32 x 64 / 4096   280 | 407        8 x 512 / 4096 523 | 730
+struct StepCount {
+    int64_t sum = 0;
+    int32_t longest = 0, shortest = 0x7fffffff;
+    void add(int32_t n) {
+        sum += n;
+        longest = std::max(longest, n);
+        shortest = std::min(shortest, n);
+    }
+};
+static double wave_us(const StepCount& s, int64_t n, int64_t slots, double fixed, double per_step) {
+    const double longest = fixed + per_step * s.longest;
+    if (n <= slots) return longest;
+    const double mean = fixed + per_step * (double)s.sum / (double)n;
+    return std::max(longest, mean * ((double)n / (double)slots + (n % slots ? 0.5 : 0.0)));    // a partly filled last round
+}
+static double wide_shape_us(const StepCount& units, int64_t n_units, int64_t nonempty_halves, int max_ctas) {
+    return 10.0 + wave_us(units, n_units, max_ctas, 5.0, nonempty_halves > n_units ? 1.9 : 1.55);
+}
+static double small_shape_us(const StepCount& halves, int64_t n_items, int max_ctas) {
+    return 0.5 + wave_us(halves, n_items, 2 * (int64_t)max_ctas, 3.3, 3.0);
+}
+
 static int resolve_opts(const wpp_ctx* ctx, const wpp_plan_opts* in, wpp_plan_opts* o) {
     wpp_plan_opts z = {0, 0, 0, 0, 0, 0};
     *o = in ? *in : z;
@@ -313,6 +343,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     std::vector<WppCombine> combines;
     int32_t slots = 0;
     int64_t n_units = 0, key_steps = 0, n_split_units = 0, nonempty_halves = 0;
+    StepCount unit_steps, half_steps;
     for (int64_t k = 0; k < n_base; ++k) {
         const RowBlock& t = rbs[(size_t)tiles[(size_t)k].rb];
         const int32_t h = tiles[(size_t)k].head;
@@ -328,10 +359,19 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
         u.head[0] = h; u.head[1] = h + t.head_b;
         u.pack = t.pack;
         nonempty_halves += (int64_t)parts * ((t.rows[0] > 0) + (t.rows[1] > 0));
+        auto count_steps = [&](int32_t a, int32_t b) {
+            int32_t n[2];
+            for (int hf = 0; hf < 2; ++hf) {
+                n[hf] = std::max(0, std::min(b, t.end[hf]) - a);
+                if (t.rows[hf] > 0) half_steps.add(n[hf]);
+            }
+            unit_steps.add(std::max(n[0], n[1]));
+        };
         if (parts == 1) {
             u.kv_begin = 0; u.kv_end = t.steps; u.split_slot = -1; u.cost = t.cost();
             us[n_units++] = u;
             key_steps += u.cost;
+            count_steps(0, t.steps);
         } else {
             for (int hf = 0; hf < 2; ++hf)
                 for (int kk = 0; kk < t.pack && t.rows[hf] > 0; ++kk)
@@ -344,6 +384,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
                 u.cost = cost_of(t, u.kv_begin, u.kv_end);
                 us[n_units++] = u;
                 key_steps += u.cost;
+                count_steps(u.kv_begin, u.kv_end);
                 ++n_split_units;
             }
             slots += parts;
@@ -351,9 +392,11 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     }
     if (n_units > 0x3fffffff) return WPP_ERR_INVALID_ARG;
     // ---- kernel shape: short tiles (few key steps per half) go to the small CTAs, two per SM, where the start and end of
-    //      one tile hide under the other CTA's steps; long tiles to the SM-wide CTA whose two halves overlap each other
+    //      one tile hide under the other CTA's steps; long tiles to the SM-wide CTA whose two halves overlap each other.
+    //      The choice is by estimated time (see small_shape_us).
     int shape = o.shape;
-    if (shape == 0) shape = (key_steps <= WPP_SMALL_SHAPE_MAX_STEPS * nonempty_halves) ? 2 : 1;
+    const int64_t n_items = nonempty_halves > n_units ? 2 * n_units : n_units;       // of the small shape
+    if (shape == 0) shape = small_shape_us(half_steps, n_items, o.max_ctas) <= wide_shape_us(unit_steps, n_units, nonempty_halves, o.max_ctas) ? 2 : 1;
     const int num_ctas = shape == 2 ? (int)std::max<int64_t>(1, std::min<int64_t>(2 * (int64_t)o.max_ctas, 2 * n_units))
                                     : (int)std::max<int64_t>(1, std::min<int64_t>(o.max_ctas, n_units));
     off += sizeof(WppUnit) * (size_t)n_units;
@@ -378,6 +421,10 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     hd.tile_n = WPP_TILE_N;
     hd.head_dim = d.head_dim;
     hd.shape = shape;
+    // The small shape's items are dealt out without a counter when they are few, or equally long: that saves the memset and
+    // the round trips to the counter, and the kernel can be set up while the one before it runs.
+    hd.deal_items = n_items <= 4 * (int64_t)num_ctas ||
+                    (n_items <= 16 * (int64_t)num_ctas && half_steps.longest <= 2 * std::max(1, half_steps.shortest));
     hd.nonempty_halves = (int32_t)std::min<int64_t>(nonempty_halves, 0x7fffffff);
     hd.total_new_tokens = T;
     hd.key_steps = key_steps;

@@ -25,7 +25,8 @@ struct WppPlanHeader {
     int32_t shape;                  // 1: two-half CTAs, one per SM; 2: single-half CTAs, two per SM (work item = half a unit)
     int32_t nonempty_halves;
     int32_t max_combine_rows;       // most rows of a combine record (sizes the combine pass's grid)
-    uint32_t pad[5];
+    int32_t deal_items;             // small shape: its items are dealt out to the CTAs, without the workspace's counter
+    uint32_t pad[4];
 };
 
 // One work tile = two 128-row "halves" that share one K/V stream (same request, same KV head).  Each half

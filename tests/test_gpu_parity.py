@@ -392,3 +392,13 @@ def test_combine_of_many_parts(d, Hq, splits):
     w = W.custom_workload([8300, 37], [13, 129], Hq, 2, d, 64, seed=51, spare_pages=4)
     res, _ = _full_parity(w, opts=wpp.PlanOpts(256, 0, splits, 0))
     assert res["plan"].info.num_split_tiles > splits // 2
+
+
+@pytest.mark.parametrize("ctas", [1, 3, 148])
+@pytest.mark.parametrize("C,Hq", [([64] * 9, 8), ([128, 128, 128], 3), ([1, 130, 64, 17], 8)])
+def test_small_shape_items_dealt_out_or_counted(C, Hq, ctas):
+    """The small shape's items are dealt out to the CTAs (few or equally long ones: one round, several rotated rounds) or
+    taken from the counter (unequal ones on few CTAs), as halves of units or, when no unit has a second half, as units."""
+    w = W.custom_workload([40 * i for i in range(len(C))], C, Hq, 1, 128, 64, seed=61, spare_pages=4)
+    for tile_m in (128, 256):
+        _full_parity(w, opts=wpp.PlanOpts(tile_m, 0, 1, ctas, 0, 2))
