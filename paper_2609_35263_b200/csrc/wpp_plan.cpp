@@ -107,10 +107,22 @@ static double wave_us(const StepCount& s, int64_t n, int64_t slots, double fixed
     return std::max(longest, mean * ((double)n / (double)slots + (n % slots ? 0.5 : 0.0)));    // a partly filled last round
 }
 static double wide_shape_us(const StepCount& units, int64_t n_units, int64_t nonempty_halves, int max_ctas) {
-    return 10.0 + wave_us(units, n_units, max_ctas, 5.0, nonempty_halves > n_units ? 1.9 : 1.55);
+    return 10.0 + wave_us(units, n_units, max_ctas, 5.0, nonempty_halves > n_units ? 1.9 : 1.4);
 }
 static double small_shape_us(const StepCount& halves, int64_t n_items, int max_ctas) {
     return 0.5 + wave_us(halves, n_items, 2 * (int64_t)max_ctas, 3.3, 3.0);
+}
+
+// Few tiles are cut along the keys so that the CTAs have work: the part length, the tile height and the kernel shape are
+// those with the smallest estimated time.  Measured, attention call in us, every CTA given a part whatever that costs | now:
+// 1 x 64 new tokens over 16,384 cached ones 86 | 56, 1 x 256 over 8,192 107 | 80, 8 x 64 over 8,192 (32 heads) 109 | 87.
+constexpr int32_t kMinPartSteps = 2;
+constexpr double kCombineUs = 6.0, kPartUs = 0.04;
+constexpr uint64_t kSplitScratchBytes = 16u << 20;      // what the built-in scratch array holds
+static int32_t parts_of(int32_t steps, int32_t part_eighths) {      // part length in eighths of a key step
+    if (part_eighths == 0) return 1;
+    const uint32_t parts = (8u * (uint32_t)steps + (uint32_t)part_eighths - 1u) / (uint32_t)part_eighths;
+    return std::max(1, std::min((int32_t)parts, steps / kMinPartSteps));
 }
 
 static int resolve_opts(const wpp_ctx* ctx, const wpp_plan_opts* in, wpp_plan_opts* o) {
@@ -131,7 +143,7 @@ static int resolve_opts(const wpp_ctx* ctx, const wpp_plan_opts* in, wpp_plan_op
 static size_t plan_bytes_bound(const wpp_batch_desc* d, const wpp_plan_opts* o, int64_t T) {
     const int64_t q_tiles = T / WPP_HALF_M + d->num_requests;   // worst case: the planner falls back to 128-row tiles
     const int64_t base = q_tiles * d->num_q_heads;
-    // automatic cuts add at most max_ctas parts (few tiles) or kTailSplitMaxParts per tile of one round (tail)
+    // automatic cuts make at most four rounds of max_ctas parts (few tiles), or kTailSplitMaxParts per tile of one round (tail)
     const int64_t units = o->force_kv_splits >= 2 ? base * o->force_kv_splits : base + kTailSplitMaxParts * (int64_t)o->max_ctas;
     size_t n = sizeof(WppPlanHeader);
     n += 2 * align_up(sizeof(int32_t) * (size_t)(d->num_requests + 1), 16);   // row offsets, prefix copy
@@ -234,8 +246,73 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     };
     int TM = o.tile_m;
     int64_t n_base = build_rows(TM);
-    if (auto_tile_m && TM == 256 && n_base < o.max_ctas) {   // few tiles: prefer more, smaller ones
-        TM = 128;
+    int32_t part_eighths = 0;      // length of a tile's parts in eighths of a key step (0: whole tiles)
+    int few_shape = 0;             // the kernel shape these parts were chosen for
+    if (o.force_kv_splits == 0 && n_base > 0 && n_base < o.max_ctas) {
+        const int tms[2] = {128, 256};
+        double best = 0.0;
+        int best_tm = TM;
+        uint64_t slots_cap = kSplitScratchBytes / ((uint64_t)2 * WPP_HALF_M * (d.head_dim + 1) * sizeof(float));
+        if (slots_cap > 0) --slots_cap;                                    // (the workspace's header)
+        // (or within what cutting the 128-row tiles so that there are at least max_ctas parts takes, if that is more)
+        if (auto_tile_m) n_base = build_rows(128);
+        uint64_t even_parts = 0;
+        for (const RowBlock& rb : rbs) {
+            const int32_t parts = std::min((int32_t)((o.max_ctas + n_base - 1) / n_base), rb.steps / kMinPartSteps);
+            if (n_base < o.max_ctas && parts > 1) even_parts += (uint64_t)parts * (uint64_t)(Hq / rb.per_tile);
+        }
+        slots_cap = std::max(slots_cap, even_parts);
+        for (int ti = 0; ti < 2; ++ti) {
+            if (!auto_tile_m && tms[ti] != TM) continue;
+            if (build_rows(tms[ti]) == 0) continue;
+            // tiles cut into parts of `ps` eighths of a key step: items of either shape and their steps
+            struct Count { int64_t units, halves, cut; StepCount unit, half; };
+            auto count = [&](int32_t ps, bool steps_too) {
+                Count c = {0, 0, 0, StepCount(), StepCount()};
+                for (const RowBlock& rb : rbs) {
+                    const int32_t parts = parts_of(rb.steps, ps);
+                    const int64_t times = Hq / rb.per_tile;
+                    c.units += parts * times;
+                    c.halves += parts * times * (rb.rows[1] > 0 ? 2 : 1);
+                    c.cut += parts > 1 ? parts * times : 0;
+                    if (!steps_too) continue;
+                    const int32_t part = (rb.steps + parts - 1) / parts;
+                    c.unit.sum += times * std::max(rb.end[0], rb.end[1]);
+                    c.half.sum += times * ((int64_t)rb.end[0] + rb.end[1]);
+                    c.unit.longest = std::max(c.unit.longest, part);
+                    c.half.longest = std::max(c.half.longest, part);
+                }
+                return c;
+            };
+            int32_t longest = 0;
+            for (const RowBlock& rb : rbs) longest = std::max(longest, rb.steps);
+            for (int shape = 2; shape >= 1; --shape) {
+                if (o.shape != 0 && o.shape != shape) continue;
+                for (int rounds = 0; rounds <= 2; ++rounds) {
+                    // the shortest parts that make at most `rounds` rounds of items (0: whole tiles)
+                    int32_t ps = 0;
+                    if (rounds > 0) {
+                        const int64_t slots = (int64_t)rounds * o.max_ctas * (shape == 2 ? 2 : 1);
+                        int32_t lo = 8 * kMinPartSteps, hi = 8 * longest;
+                        if (hi < lo) continue;
+                        while (lo < hi) {
+                            const int32_t mid = lo + (hi - lo) / 2;
+                            const Count c = count(mid, false);
+                            const int64_t items = shape == 2 ? (c.halves > c.units ? 2 * c.units : c.units) : c.units;
+                            if (items <= slots && (uint64_t)c.cut <= slots_cap) hi = mid; else lo = mid + 1;
+                        }
+                        ps = lo;
+                    }
+                    const Count c = count(ps, true);
+                    if (c.cut > 0 && (uint64_t)c.cut > slots_cap) continue;
+                    double us = shape == 2 ? small_shape_us(c.half, c.halves > c.units ? 2 * c.units : c.units, o.max_ctas)
+                                           : wide_shape_us(c.unit, c.units, c.halves, o.max_ctas);
+                    if (c.cut > 0) us += kCombineUs + kPartUs * (double)c.cut;
+                    if (few_shape == 0 || us < best) { best = us; best_tm = tms[ti]; part_eighths = ps; few_shape = shape; }
+                }
+            }
+        }
+        TM = best_tm;
         n_base = build_rows(TM);
     }
     if (n_base > 0x3fffffff) return WPP_ERR_INVALID_ARG;
@@ -275,12 +352,9 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     }
 
     // ---- split decision: into how many key ranges each tile is cut (1 = not at all)
-    int32_t few_want = 0;          // fewer tiles than CTAs: every tile is cut so that all CTAs have work (>= 2 steps per part)
     int64_t tail = 0;              // tiles of a partly filled last round ...
     int32_t tail_parts = 1;        // ... and the number of key ranges each of them is cut into
-    if (o.force_kv_splits == 0 && n_base > 0 && n_base < o.max_ctas) {
-        few_want = (int32_t)((o.max_ctas + n_base - 1) / n_base);
-    } else if (o.force_kv_splits == 0 && n_base % o.max_ctas != 0 && n_base < kTailSplitMaxRounds * (int64_t)o.max_ctas) {
+    if (o.force_kv_splits == 0 && few_shape == 0 && n_base % o.max_ctas != 0 && n_base < kTailSplitMaxRounds * (int64_t)o.max_ctas) {
         // A few rounds of long tiles: the last, partly filled round leaves CTAs idle for a whole tile.  Cutting the
         // tiles of that round into p key ranges each fills it.  The candidates are compared on a model of the run
         // (tiles handed out in order to the CTA that is free first; a tile costs its key steps plus a fixed start
@@ -349,7 +423,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
         const int32_t h = tiles[(size_t)k].head;
         int32_t parts = 1;
         if (o.force_kv_splits >= 2) parts = std::max(1, std::min(o.force_kv_splits, t.steps));
-        else if (few_want > 1) parts = std::max(1, std::min(few_want, t.steps / 2));
+        else if (few_shape != 0) parts = parts_of(t.steps, part_eighths);
         else if (k >= n_base - tail) parts = tail_parts;
         if (n_units + parts > unit_cap) return WPP_ERR_PLAN_MISMATCH;
         WppUnit u;
@@ -396,7 +470,8 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     //      The choice is by estimated time (see small_shape_us).
     int shape = o.shape;
     const int64_t n_items = nonempty_halves > n_units ? 2 * n_units : n_units;       // of the small shape
-    if (shape == 0) shape = small_shape_us(half_steps, n_items, o.max_ctas) <= wide_shape_us(unit_steps, n_units, nonempty_halves, o.max_ctas) ? 2 : 1;
+    if (shape == 0 && few_shape != 0) shape = few_shape;
+    else if (shape == 0) shape = small_shape_us(half_steps, n_items, o.max_ctas) <= wide_shape_us(unit_steps, n_units, nonempty_halves, o.max_ctas) ? 2 : 1;
     const int num_ctas = shape == 2 ? (int)std::max<int64_t>(1, std::min<int64_t>(2 * (int64_t)o.max_ctas, 2 * n_units))
                                     : (int)std::max<int64_t>(1, std::min<int64_t>(o.max_ctas, n_units));
     off += sizeof(WppUnit) * (size_t)n_units;
