@@ -106,6 +106,12 @@ __global__ void __launch_bounds__(256) wpp_block_digest_kernel(const int32_t* __
 // stage's loads are in flight while this one is chained, the finished hashes leave as coalesced stores - so that the
 // walk never waits on global memory; inside a stage eight terms are read before and eight hashes written after the
 // eight steps between them (a load that may alias the store before it would put shared-memory latency into every step).
+__device__ __forceinline__ uint64_t chain_product(uint64_t z, uint64_t c) {
+    uint64_t x = (z ^ (z >> 30)) ^ ((z >> 31) ^ (z >> 61)) ^ c;
+    x *= 0xBF58476D1CE4E5B9ull;
+    x ^= x >> 27;
+    return x * 0x94D049BB133111EBull;
+}
 constexpr int kStage = 128, kPerLane = kStage / 32;
 __global__ void __launch_bounds__(32) wpp_hash_chain_kernel(const int64_t* __restrict__ block_offsets,
                                                             uint64_t* __restrict__ hashes) {
@@ -135,10 +141,7 @@ __global__ void __launch_bounds__(32) wpp_hash_chain_kernel(const int64_t* __res
                 for (int j = 0; j < 8; ++j) c[j] = buf[i + j];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    uint64_t x = (z ^ (z >> 30)) ^ ((z >> 31) ^ (z >> 61)) ^ c[j];
-                    x *= 0xBF58476D1CE4E5B9ull;
-                    x ^= x >> 27;
-                    z = x * 0x94D049BB133111EBull;
+                    z = chain_product(z, c[j]);
                     c[j] = z ^ (z >> 31);
                 }
 #pragma unroll
@@ -152,6 +155,94 @@ __global__ void __launch_bounds__(32) wpp_hash_chain_kernel(const int64_t* __res
             if (i < n) h[i] = buf[u * 32 + lane];
         }
         __syncwarp();
+    }
+}
+
+// Digests and chain of long prompts in one kernel, a CTA per request: twelve warps work on the digests of the next stage of
+// 96 blocks while one lane chains the current ones out of shared memory, so that only the first stage's digests stand in
+// front of the chain.  The chain's warp is the only one of its scheduler (warps 7, 11 and 15 leave at once): beside digest
+// warps its dependent steps waited for issue slots (170 us instead of 144 for 64 requests x 3,125 blocks of 64 tokens).
+constexpr int kFusedWarps = 12, kFusedStage = 8 * kFusedWarps, kFusedThreads = 512;
+__global__ void __launch_bounds__(kFusedThreads, 1) wpp_hash_fused_kernel(const int32_t* __restrict__ tokens,
+                                                                          const int64_t* __restrict__ token_offsets,
+                                                                          const int64_t* __restrict__ block_offsets,
+                                                                          int block_size, uint64_t salt_term,
+                                                                          const uint64_t* __restrict__ extra,
+                                                                          uint64_t* __restrict__ out) {
+    __shared__ uint64_t s_m[2][kFusedStage], s_h[2][kFusedStage];
+    const int req = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp > 3 && (warp & 3) == 3) return;
+    const int dw = warp - (warp >> 2);                 // digest warps 0..11 (the chain's warp is 3)
+    auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(32 * (kFusedWarps + 1)) : "memory"); };
+    const int64_t b0 = block_offsets[req], n = block_offsets[req + 1] - b0;
+    const int32_t* src = tokens + token_offsets[req];
+    const int n_stages = (int)((n + kFusedStage - 1) / kFusedStage);
+    auto digest = [&](int s) {
+        const int64_t first = (int64_t)s * kFusedStage + dw * 8;
+        uint64_t d[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) d[j] = 0;
+        for (int k0 = 0; k0 < block_size; k0 += 64) {
+            int32_t t[8][2];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int k = k0 + 32 * u + lane;
+                    t[j][u] = (k < block_size && first + j < n) ? __ldg(src + (first + j) * block_size + k) : 0;
+                }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int k = k0 + 32 * u + lane;
+                if (k0 + 32 * u >= block_size) break;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) d[j] += k < block_size ? token_term(t[j][u], (uint32_t)k) : 0ull;
+            }
+        }
+        uint64_t mine = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) d[j] += __shfl_xor_sync(0xffffffffu, d[j], o);
+            if (lane == j) mine = d[j];
+        }
+        if (lane < 8) {                     // (entries past the request's last block are never used)
+            const uint64_t c = mix64(mine + ((extra && first + lane < n) ? extra[b0 + first + lane] : 0ull)) ^ salt_term;
+            s_m[s & 1][dw * 8 + lane] = c ^ (c >> 30);
+        }
+    };
+    if (warp != 3 && n_stages > 0) digest(0);
+    sync();
+    uint64_t z = 0;
+    for (int s = 0; s <= n_stages; ++s) {
+        if (warp == 3) {
+            if (lane == 0 && s < n_stages) {
+                const uint64_t* m = s_m[s & 1];
+                uint64_t* h = s_h[s & 1];
+                const int cnt = (int)min((int64_t)kFusedStage, n - (int64_t)s * kFusedStage);
+#pragma unroll 1
+                for (int i = 0; i < cnt; i += 8) {
+                    uint64_t c[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) c[j] = m[i + j];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        z = chain_product(z, c[j]);
+                        c[j] = z ^ (z >> 31);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) h[i + j] = c[j];
+                }
+            }
+            __syncwarp();
+        } else {
+            if (s > 0) {
+                const int64_t i = (int64_t)(s - 1) * kFusedStage + dw * 8 + lane;
+                if (lane < 8 && i < n) out[b0 + i] = s_h[(s - 1) & 1][dw * 8 + lane];
+            }
+            if (s + 1 < n_stages) digest(s + 1);
+        }
+        sync();
     }
 }
 
@@ -187,6 +278,14 @@ extern "C" int wpp_hash_blocks(const wpp_ctx* ctx, const int32_t* tokens, const 
     if (int rc = wpp_ctx_check_device(ctx)) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const uint64_t salt_term = salt * 0x9E3779B97F4A7C15ull;
+    // One kernel when every request can have an SM and its twelve warps keep up with the chain (blocks of up to 64 tokens:
+    // an SM makes a block's digest in less than a chain step).  us, one kernel | two: 64 requests x 3,125 blocks of 64
+    // 144 | 172, 64 x 100 11 | 15, 148 x 3,125 156 | 222; blocks of 128: 1 x 1,500 90 | 72, 64 x 3,125 269 | 199.
+    if (num_requests <= 148 && block_size <= 64) {
+        wpp_hash_fused_kernel<<<(unsigned)num_requests, kFusedThreads, 0, st>>>(tokens, token_offsets, block_offsets, block_size,
+                                                                               salt_term, extra, hashes_out);
+        return cudaGetLastError() == cudaSuccess ? WPP_OK : WPP_ERR_CUDA;
+    }
     // eight blocks per warp once that still gives every SM 32 warps; one below, where a warp's latency is all that counts
     const bool wide = total_blocks >= 8ll * 32 * 148;
     const int64_t ctas = (total_blocks + (wide ? 63 : 7)) / (wide ? 64 : 8);

@@ -138,17 +138,19 @@ def test_gpu_hashes_match_the_oracle(B):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("B,many", [(1, False), (33, False), (65, False), (130, False), (2, True), (300, False)])
+@pytest.mark.parametrize("B,many", [(1, False), (33, False), (64, False), (65, False), (130, False), (2, True), (300, False)])
 def test_gpu_hashes_at_the_edges_of_the_kernels(B, many):
-    """The digests take one or eight blocks per warp, across requests, the chain stages of 128 blocks: request lengths
-    around both, more requests than one search step tells apart, enough blocks for the wide form (`many`), and block
-    sizes that are no multiple of a warp; hashes are whole numbers, so they must be equal."""
+    """The digests take one or eight blocks per warp, across requests, the chain stages of 128 blocks, the one-kernel form
+    (blocks of up to 64 tokens, up to 148 requests) stages of 96: request lengths around them, more requests than one
+    search step tells apart, enough blocks and requests for the wide form (`many`), and block sizes that are no multiple
+    of a warp; hashes are whole numbers, so they must be equal."""
     rng = np.random.default_rng(B)
     reqs = [rng.integers(-5, 1 << 31, n * B + extra).astype(np.int32)
-            for n, extra in ((127, 0), (128, B // 2), (129, 0), (1, 0), (0, B - 1), (8, 0), (9, 0), (256, 0), (257, 0))]
+            for n, extra in ((127, 0), (128, B // 2), (129, 0), (1, 0), (0, B - 1), (8, 0), (9, 0), (256, 0), (257, 0),
+                             (95, 0), (96, 0), (97, B // 2), (192, 0), (193, 0))]
     reqs += [rng.integers(0, 1 << 31, int(n)).astype(np.int32) for n in rng.integers(0, 3 * B, 70)]
     if many:
-        reqs += [rng.integers(0, 1 << 31, 38000 * B).astype(np.int32)] + reqs[:40]
+        reqs += [rng.integers(0, 1 << 31, 38000 * B).astype(np.int32)] + reqs[:80]
     tok_off = np.concatenate([[0], np.cumsum([len(t) for t in reqs])]).astype(np.int64)
     blk_off = np.concatenate([[0], np.cumsum([len(t) // B for t in reqs])]).astype(np.int64)
     out = wpp.wpp_hash_blocks(wpp.Context(0), torch.from_numpy(np.concatenate(reqs)).cuda(), torch.from_numpy(tok_off).cuda(),
