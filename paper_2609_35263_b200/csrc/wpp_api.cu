@@ -467,17 +467,17 @@ extern "C" size_t wpp_kda_workspace_bytes(const wpp_kda_desc* desc) {
 // The two-pass form reads and writes 144 KB of operands per block but its chain is the fastest per token; the group form
 // has nothing in front of its chain and moves nothing but inputs and outputs.  The estimates below are microseconds for
 // C tokens per request, measured on 148 SMs (us; group with 128 / 64 / 32 columns | two passes):
-//     requests x heads x tokens    8x32x2048  677 / 801 / 1224 | 733     1x32x512    91 /  75 /   51 |   62
+//     requests x heads x tokens    8x32x2048  640 / 801 / 1224 | 733     1x32x512    91 /  75 /   51 |   62
 //                                  4x32x256    51 /  58 /  105 |  75     1x8x2048   336 / 276 /  178 |  142
-//                                  4x32x4096  670 / 801 / 1374 | 722     2x32x8192 1328 / 1103 / 1369 | 913
-//                                  8x32x64     34 /  36 /   67 |  50     64x32x256  659 / 740 / 1409 | 782
+//                                  4x32x4096  635 / 801 / 1374 | 722     2x32x8192 1328 / 1103 / 1369 | 913
+//                                  8x32x64     34 /  36 /   67 |  50     64x32x256  630 / 740 / 1409 | 782
 // Error against the fp32 token-by-token form, rms of the states over their rms: 6.0e-6 (two passes: 4.9e-6); outputs equal.
 static int kda_chunk_form(const wpp_kda_desc* d, int sms) {
     const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
     auto rounds = [&](double ctas) { return ceil(ctas / sms); };
     const double prep = n * C * 0.9e-3 * 148 / sms, chain = rounds(n) * C * 0.0525, operands = n * C * 0.49e-3;
     const double t[4] = {35 + prep + (chain > operands ? chain : operands),
-                         rounds(n) * C * 0.165,                                                       // one CTA per SM
+                         rounds(n) * C * 0.157,                                                       // one CTA per SM
                          2 * n <= sms ? C * 0.135 : rounds(n) * C * 0.195,                            // two per SM
                          rounds(4 * n) * C * 0.084};
     int best = 0;

@@ -17,10 +17,12 @@
 // Why mma.sync beside the tensor cores' asynchronous form (wpp_kda_tc.cu), whose rate is eight times higher: with the
 // state in tensor memory a step is a chain of hand-overs between the issuing thread, the tensor pipe and the warps that
 // scale, split and store, and its operands need a pass of their own in front (14.5 K clocks of an SM per 64 tokens, 144 KB
-// written and read back).  Here a group's chain stays inside a warp: 22 K clocks of an SM per 64 tokens in all, no second
-// pass.  8 x 2,048 tokens, 32 heads: 733 -> 677 us; 8 x 64: 50 -> 34 us; 1 x 512: 62 -> 51 us (the choice: kda_chunk_form).
-// What bounds a group now (clocks, 5.6 K): the products 3.5 K of which the MMA pipe is busy 2.6 K, U 0.6 K, hand-over and
-// outputs 1.5 K; the producers are idle half the time.
+// written and read back).  Here a group's chain stays inside a warp: 21 K clocks of an SM per 64 tokens in all, no second
+// pass.  8 x 2,048 tokens, 32 heads: 733 -> 640 us; 8 x 64: 50 -> 33 us; 1 x 512: 62 -> 51 us (the choice: kda_chunk_form).
+// What bounds a group now (clocks, 5.3 K): the products 3.4 K of which the MMA pipe is busy 2.6 K, U 0.4 K, hand-over and
+// outputs 1.2 K; the producers are idle half the time.  Also tried: four column warps of 32 columns with 216 registers
+// (809 us: one warp per scheduler waits), one producer warpgroup (660), a thirteenth warp for T and the copies (711: four
+// warps in a quarter of the SM leave 128 registers each).
 //
 // Precision.  Every operand is split into two bf16 terms, x = hi + lo (16 significant bits), and every product is three
 // MMAs, hi hi + hi lo + lo hi (the dropped lo lo is 2^-17 relative), accumulated in fp32.
@@ -44,6 +46,11 @@ constexpr int kL = 16;                 // tokens per group
 constexpr int kD = 128;                // d_k = d_v
 constexpr float kMinGamma = 9.094947e-13f;       // 2^-40: smallest decay product a group may contain
 constexpr float kSafeGamma = 9.5367432e-7f;      // 2^-20: two halves above it need no closer look
+// registers per thread of the 128-column CTAs (eight column warps, eight producer warps, launched with 128 each): the
+// column warps keep more operands in flight (8 x 2,048 tokens x 32 heads: 128 / 128 660 us, 144 / 112 656, 152 / 104 640,
+// 160 / 96 652)
+constexpr int kRegsColumn = 152, kRegsProducer = 104;
+static_assert(kRegsColumn + kRegsProducer <= 256, "the launch's registers");
 
 // hi/lo split of two fp32 values into two packed bf16 pairs (element 0 in the low half)
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
@@ -159,7 +166,7 @@ struct Smem {
     static constexpr int kNumBars = kP * (2 * kStages + kRaw);
     static constexpr int kOffMisc = kOffBars + 8 * kNumBars;
     static constexpr int kBytes = kOffMisc + 16 + 1024;
-    static_assert(kBytes <= (kP > 1 ? 232448 : 115712), "one CTA per SM, or two");
+    static_assert(kBytes <= 232448, "more shared memory than a CTA can have");
 };
 
 // kSlice value columns per CTA; a column warp owns kMT x 16 of them, or kKS warps share 16 of them and half the channels
@@ -173,6 +180,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
     constexpr int kVH = kSlice == kD ? 2 : 1;
     using SM = Smem<kP, kVH, kNC, kKS>;
     using Stage = StageT<kVH>;
+    static_assert(kMinCtas * (SM::kBytes + 1024) <= 233472, "shared memory of an SM");
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
@@ -227,6 +235,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
 
     if (warp >= kNC) {
         // ================================================================ producers
+        if constexpr (kNC == 8) setmaxnreg_dec<kRegsProducer>();
         const int w = (warp - kNC) >> 2;                     // which producer warpgroup: blocks w, w + kP, ...
         const int bar_id = 1 + 2 * w;                      // named barriers: 1 + 2w all four warps, 2 + 2w two of them
         const int ptid = tid & 127, pw = warp & 3;
@@ -266,16 +275,17 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
             request_v(w, 0);
         }
         float beta_next = (pw == 3 && lane < kL) ? beta_of(w) : 0.f;
+        constexpr int kAhead = kMinCtas == 2 ? 4 : 8;          // k-steps of the producers' products whose operands are loaded together
 
         int stage = 0, raw = 0;
         uint32_t ph_stage = 0, ph_raw = 0;
         bool dead = false;
-        for (int b = w; b < n_blocks && !dead; b += kP) {
+        for (int b = w; b < n_blocks; b += kP) {
             const int t_lo = max(0, P - (first_block + b) * kL), t_hi = min(kL, P + C - (first_block + b) * kL);
             // this thread's channel pair and first token: alpha (fp32), k and q (bf16)
             const uint32_t r_alpha = base + SM::kOffRaw + (w * SM::kRaw + raw) * SM::kRawBytes + SM::kRawAlpha + half * 8 * kD * 4 + cp * 8;
             const uint32_t r_kq = base + SM::kOffRaw + (w * SM::kRaw + raw) * SM::kRawBytes + SM::kRawK + half * 8 * kD * 2 + cp * 4;
-            dead = !mbar_wait(bRaw(w, raw), ph_raw, abort_flag);
+            dead |= !mbar_wait(bRaw(w, raw), ph_raw, abort_flag);
             const uint32_t s_beta = s_betas + (b / kP & 1) * kL * 4;       // (the previous block's may still be in use)
             if (pw == 3 && lane < kL) {
                 sts1f(s_beta + lane * 4, beta_next);
@@ -295,7 +305,6 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                 int pre = 0;
                 const int e_max = e;
                 const uint32_t st = base + stage_off(w, stage);
-                dead |= !mbar_wait(bEmpty(w, stage), ph_stage ^ 1u, abort_flag);
 
                 // ---- decay products of this thread's two channels and eight tokens, from the group's first token on
                 float2 g[8];
@@ -338,7 +347,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                     if (bad >= e) break;
                     if (bad == a) pre = 1; else e = bad;
                 }
-                if (dead) break;
+                if (dead) break;                           // (everybody: the barrier above has told)
                 if (e < e_max) snap_here = false;
                 if (snap_here && p.snap_slots) {
                     const int n = ((first_block + b) * kL + e) / p.snap_interval - P / p.snap_interval - 1;
@@ -397,15 +406,21 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                     const uint32_t row_b = st + Stage::kKhH + l16 * Stage::kTile + (nt * 8 + ln7) * 256 + ((l8 ^ ln7) << 4);
                     float x0[4] = {0.f, 0.f, 0.f, 0.f}, x1[4] = {0.f, 0.f, 0.f, 0.f}, x2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
-                        uint32_t ah[4], al[4], bb[4];
-                        const int x = (kk & 3) << 5, y = (kk >> 2) * 128;
-                        ldsm4(ah, (row_a ^ x) + y);
-                        ldsm4(al, (row_a ^ x) + y + Stage::kTile);
-                        ldsm4(bb, (row_b ^ x) + y);
-                        mma16(x0, ah, bb[0], bb[1]);
-                        mma16(x1, ah, bb[2], bb[3]);
-                        mma16(x2, al, bb[0], bb[1]);
+                    for (int k0 = 0; k0 < 8; k0 += kAhead) {
+                        uint32_t ah[kAhead][4], al[kAhead][4], bb[kAhead][4];
+#pragma unroll
+                        for (int u = 0; u < kAhead; ++u) {
+                            const int x = ((k0 + u) & 3) << 5, y = ((k0 + u) >> 2) * 128;
+                            ldsm4(ah[u], (row_a ^ x) + y);
+                            ldsm4(bb[u], (row_b ^ x) + y);
+                            ldsm4(al[u], (row_a ^ x) + y + Stage::kTile);
+                        }
+#pragma unroll
+                        for (int u = 0; u < kAhead; ++u) {
+                            mma16(x0, ah[u], bb[u][0], bb[u][1]);
+                            mma16(x1, ah[u], bb[u][2], bb[u][3]);
+                            mma16(x2, al[u], bb[u][0], bb[u][1]);
+                        }
                     }
                     const int s = nt * 8 + 2 * (lane & 3);
                     float x[4];
@@ -430,32 +445,43 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                         }
                     }
                 }
-                // ---- T = (I + A)^-1 diag(beta), a column per lane, columns of the identity pushed through I + A
+                // ---- T = (I + A)^-1 diag(beta): columns of the identity pushed through I + A; lane c has rows 0..7 of column c,
+                //      lane c + 16 its rows 8..15 (it gets the upper rows' values, as they become final, by shuffles)
                 if (pw == 0) {
-                    const int c = lane & 15;
-                    float x[16];
+                    const int c = lane & 15, r0 = (lane >> 4) * 8;
+                    float x[8];
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) x[r] = (r == c) ? 1.f : 0.f;
+                    for (int r = 0; r < 8; ++r) x[r] = (r0 + r == c) ? 1.f : 0.f;
 #pragma unroll
-                    for (int q = 0; q < 15; ++q) {
+                    for (int q = 0; q < 8; ++q) {
+                        const float xq = __shfl_sync(0xffffffffu, x[q], c);
+                        const float4 a0 = lds4f(s_at + (q * 20 + r0) * 4), a1 = lds4f(s_at + (q * 20 + r0 + 4) * 4);
+                        // (entries at or above the diagonal are zero: rows that are final already do not change)
+                        x[0] = fmaf(-a0.x, xq, x[0]); x[1] = fmaf(-a0.y, xq, x[1]);
+                        x[2] = fmaf(-a0.z, xq, x[2]); x[3] = fmaf(-a0.w, xq, x[3]);
+                        x[4] = fmaf(-a1.x, xq, x[4]); x[5] = fmaf(-a1.y, xq, x[5]);
+                        x[6] = fmaf(-a1.z, xq, x[6]); x[7] = fmaf(-a1.w, xq, x[7]);
+                    }
 #pragma unroll
-                        for (int r4 = (q + 1) / 4 * 4; r4 < 16; r4 += 4) {
-                            const float4 av = lds4f(s_at + (q * 20 + r4) * 4);
-                            x[r4] = fmaf(-av.x, x[q], x[r4]);            // (entries at or above the diagonal are zero)
-                            x[r4 + 1] = fmaf(-av.y, x[q], x[r4 + 1]);
-                            x[r4 + 2] = fmaf(-av.z, x[q], x[r4 + 2]);
-                            x[r4 + 3] = fmaf(-av.w, x[q], x[r4 + 3]);
-                        }
+                    for (int q = 8; q < 15; ++q) {
+                        // rows 8..15: the lower half warp's own (the upper one multiplies by zeros it reads itself)
+                        const float xq = r0 ? x[q - 8] : 0.f;
+                        const float4 a0 = lds4f(s_at + (q * 20 + 8) * 4), a1 = lds4f(s_at + (q * 20 + 12) * 4);
+                        x[0] = fmaf(-a0.x, xq, x[0]); x[1] = fmaf(-a0.y, xq, x[1]);
+                        x[2] = fmaf(-a0.z, xq, x[2]); x[3] = fmaf(-a0.w, xq, x[3]);
+                        x[4] = fmaf(-a1.x, xq, x[4]); x[5] = fmaf(-a1.y, xq, x[5]);
+                        x[6] = fmaf(-a1.z, xq, x[6]); x[7] = fmaf(-a1.w, xq, x[7]);
                     }
                     const float bt = (c >= a && c < e) ? lds1f(s_beta + c * 4) : 0.f;
-                    const uint32_t dst = st + (lane >= 16 ? Stage::kTL : Stage::kTH) + (c & 7) * 2;
+                    const uint32_t dst = st + Stage::kTH + r0 * 32 + (c & 7) * 2;
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) {
+                    for (int r = 0; r < 8; ++r) {
                         const float v = x[r] * bt;
                         const __nv_bfloat16 hi = __float2bfloat16_rn(v);
                         const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-                        const unsigned short bits = lane >= 16 ? __bfloat16_as_ushort(lo) : __bfloat16_as_ushort(hi);
-                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(dst + sq_off(r, c >> 3)), "h"(bits));
+                        const uint32_t at = dst + sq_off(r, c >> 3);             // (the swizzle of row r0 + r is that of row r)
+                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(at), "h"(__bfloat16_as_ushort(hi)));
+                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(at + Stage::kTL - Stage::kTH), "h"(__bfloat16_as_ushort(lo)));
                     }
                 }
                 __syncwarp();
@@ -464,14 +490,20 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                 if (pw == 3) {
                     const int next = e < t_hi ? b : b + kP;
                     if (e == t_hi && b + SM::kRaw * kP < n_blocks) request_raw(b + SM::kRaw * kP, raw);    // the raw tile is spent
-                    if (next < n_blocks && __all_sync(0xffffffffu, mbar_wait(bEmpty(w, stage), ph_stage ^ 1u, abort_flag))) request_v(next, stage);
+                    // (the only wait for a free stage: the others learn of it by the barrier behind the decay products)
+                    if (next < n_blocks) {
+                        if (__all_sync(0xffffffffu, mbar_wait(bEmpty(w, stage), ph_stage ^ 1u, abort_flag))) request_v(next, stage);
+                        else dead = true;
+                    }
                 }
                 a = e;
             }
+            if (a < t_hi) break;                               // given up: everybody is here
             if (++raw == SM::kRaw) { raw = 0; ph_raw ^= 1u; }
         }
     } else {
         // ================================================================ the state's columns
+        if constexpr (kNC == 8) setmaxnreg_inc<kRegsColumn>();
         constexpr int kNT = 16 / kKS;                      // 8-channel tiles per warp
         const int m0 = (kKS == 1 ? warp : (warp >> 1)) * kMT * 16;          // first column inside the slice
         const int kq = kKS == 1 ? 0 : (warp & 1);
