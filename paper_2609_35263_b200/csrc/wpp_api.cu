@@ -462,6 +462,43 @@ extern "C" size_t wpp_kda_workspace_bytes(const wpp_kda_desc* desc) {
     return kda_workspace(desc).bytes;
 }
 
+// Microseconds of the two passes over C tokens per request, measured on 148 SMs: preparation of a token of a chain on all SMs,
+// a token of a chain that has an SM to itself, and what a token's operands take at the memory's rate.
+constexpr double kPrepUs = 0.9e-3, kChainUs = 0.0525, kOperandsUs = 0.49e-3, kSegmentUs = 12.0;
+
+// Segments of the two-pass form.  Few long chains leave most SMs idle: the chunk is cut so that a segment's preparation runs
+// beside the chain of the segment before.  Each segment is longer than the one before by what the chain takes longer per
+// block than the preparation on the SMs left, so that only the first segment's preparation is waited for.  Returns the
+// number of segments with the smallest estimated time, which comes back in *us, and where they begin, in blocks.
+// 1 x 16,384 tokens x 32 heads: in one piece 1340 us, 4 equal segments 1060, 8 equal ones 1068.
+constexpr int kMaxSegments = 6;
+static int kda_segments(const wpp_kda_desc* d, int sms, double* us, int32_t* begin) {
+    const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
+    const double prep = n * C * kPrepUs * 148 / sms, operands = n * C * kOperandsUs, chain = ceil(n / sms) * C * kChainUs;
+    const int64_t blocks = d->total_tokens / d->num_requests / 64 + 1;
+    int best = 1;
+    double best_us = prep + (chain > operands ? chain : operands);
+    const double growth = 2 * n <= sms ? chain / (prep * sms / (sms - n)) : 0.0;
+    double best_first = 1.0;
+    for (int s = 2; growth > 1.05 && s <= kMaxSegments; ++s) {
+        const double g = growth < 4.0 ? growth : 4.0, first = (g - 1.0) / (pow(g, s) - 1.0);
+        if (first * (double)blocks < 4.0) break;
+        const double t = prep * first + chain + kSegmentUs * (s - 1);
+        if (t < best_us) { best = s; best_us = t; best_first = first; }
+    }
+    if (us) *us = best_us;
+    if (begin) {
+        const double g = growth < 4.0 ? growth : 4.0;
+        double at = 0.0, len = best_first;
+        for (int s = 0; s < best; ++s) {
+            begin[s] = (int32_t)(at * (double)blocks);
+            at += len;
+            len *= g;
+        }
+    }
+    return best;
+}
+
 // Which chunk-parallel kernel: 0 = blocks of 64 tokens in two passes (preparation for all blocks in parallel, then the
 // chain), 1..3 = groups of 16 tokens with the state in registers (wpp_kda_group.cu), in CTAs of 128, 64 or 32 columns.
 // The two-pass form reads and writes 144 KB of operands per block but its chain is the fastest per token; the group form
@@ -475,8 +512,9 @@ extern "C" size_t wpp_kda_workspace_bytes(const wpp_kda_desc* desc) {
 static int kda_chunk_form(const wpp_kda_desc* d, int sms) {
     const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
     auto rounds = [&](double ctas) { return ceil(ctas / sms); };
-    const double prep = n * C * 0.9e-3 * 148 / sms, chain = rounds(n) * C * 0.0525, operands = n * C * 0.49e-3;
-    const double t[4] = {35 + prep + (chain > operands ? chain : operands),
+    double two_passes = 0.0;
+    kda_segments(d, sms, &two_passes, nullptr);
+    const double t[4] = {35 + two_passes,
                          rounds(n) * C * 0.157,                                                       // one CTA per SM
                          2 * n <= sms ? C * 0.135 : rounds(n) * C * 0.195,                            // two per SM
                          rounds(4 * n) * C * 0.084};
@@ -579,9 +617,13 @@ extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const
             const uint64_t strides[2] = {512, 512 * H};
             if ((rc = make_map(ctx, &maps[12], alpha, 3, dims, strides, box)) != WPP_OK) return rc;
         }
-        int e = wpp_launch_kda_tc(&p, maps, desc->total_tokens > 0 ? (int)w.max_blocks : 0, ctx->sm_count, cuda_stream);
+        // few long chains leave most SMs to the next segment's preparation
+        int32_t seg_begin[kMaxSegments] = {0};
+        const int segments = kda_segments(desc, ctx->sm_count, nullptr, seg_begin);
+        int e = wpp_launch_kda_tc(&p, maps, desc->total_tokens > 0 ? (int)w.max_blocks : 0, ctx->sm_count, segments, seg_begin,
+                                  cuda_stream);
         if (e != 0) return cuda_fail(ctx, e);
-        const_cast<wpp_ctx*>(ctx)->launches += 3;
+        const_cast<wpp_ctx*>(ctx)->launches += 1 + 2 * segments;
         return WPP_OK;
     }
     wpp::KdaParams p;

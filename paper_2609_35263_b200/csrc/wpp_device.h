@@ -91,6 +91,8 @@ struct KdaTcParams {
     __nv_bfloat16* out;
     int32_t* status;
     int32_t num_requests, num_heads, num_slots, snap_interval, max_snaps;
+    int32_t seg_lo, seg_hi;         // blocks [seg_lo, seg_hi) of every request belong to this launch
+    int32_t beside;                 // preparation: launched beside the chain of the segment before
     int32_t* blk_off;               // [R+1] exclusive scan of the requests' block counts
     unsigned long long* ws_mask;    // [bh] bit t: token t of the block starts a sub-block
     float* ws_e;                    // [bh][64][128] decay product at a sub-block's last token (other rows unused)
@@ -103,7 +105,8 @@ struct KdaTcParams {
 
 extern "C" {
 // maps: 0..5 the operand arrays W0, Qt, Kb (hi, lo each), 6..7 M (hi, lo), 8 U0, 9..12 q, k, v, alpha
-int wpp_launch_kda_tc(const wpp::KdaTcParams* p, const CUtensorMap* maps, int max_blocks, int num_sms, void* stream);
+int wpp_launch_kda_tc(const wpp::KdaTcParams* params, const CUtensorMap* maps, int max_blocks, int num_sms, int segments,
+                      const int32_t* seg_begin, void* stream);
 int wpp_launch_attention(int head_dim, const CUtensorMap* tq, const CUtensorMap* tk, const CUtensorMap* tv,
                          const wpp::AttnParams* p, int num_ctas, int late_rescale, void* stream);
 int wpp_launch_attention_small(int head_dim, const CUtensorMap* tq, const CUtensorMap* tk, const CUtensorMap* tv,

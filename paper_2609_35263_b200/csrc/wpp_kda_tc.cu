@@ -175,7 +175,12 @@ struct PrepMaps {
     CUtensorMap q, k, v, alpha;                            // inputs (loads): (channel, head, row)
 };
 
-// The (block, head) item `item` of the wave: its request's geometry and the block's place in it.
+// Blocks of request i that belong to the launch's segment.
+__device__ __forceinline__ int seg_blocks(const KdaTcParams& p, int i) {
+    const int n = p.blk_off[i + 1] - p.blk_off[i];
+    return max(0, min(n, p.seg_hi) - p.seg_lo);
+}
+// The (block, head) item `item` of the launch: its request's geometry and the block's place in it.
 struct PrepItem {
     int gb, head, blk, t_lo, t_hi;
     int64_t row_t0;
@@ -185,10 +190,21 @@ __device__ __forceinline__ PrepItem prep_item(const KdaTcParams& p, int item) {
     const int H = p.num_heads, R = p.num_requests;
     it.gb = item / H;
     it.head = item - it.gb * H;
-    int lo_r = 0, hi_r = R;                 // request: largest i with blk_off[i] <= gb (empty requests share offsets)
-    while (hi_r - lo_r > 1) {
-        const int mid = (lo_r + hi_r) >> 1;
-        if (p.blk_off[mid] <= it.gb) lo_r = mid; else hi_r = mid;
+    int lo_r = 0;
+    if (p.seg_hi != 0x7fffffff || p.seg_lo != 0) {
+        // the blocks of a segment, request by request (few requests: the segments are for waves of few chains)
+        for (;; ++lo_r) {
+            const int c = seg_blocks(p, lo_r);
+            if (it.gb < c) break;
+            it.gb -= c;
+        }
+        it.gb += p.blk_off[lo_r] + p.seg_lo;
+    } else {
+        int hi_r = R;                       // request: largest i with blk_off[i] <= gb (empty requests share offsets)
+        while (hi_r - lo_r > 1) {
+            const int mid = (lo_r + hi_r) >> 1;
+            if (p.blk_off[mid] <= it.gb) lo_r = mid; else hi_r = mid;
+        }
     }
     const ReqBlocks g = req_blocks(p, lo_r);
     it.blk = g.first_block + (it.gb - p.blk_off[lo_r]);
@@ -227,8 +243,16 @@ kda_tc_prep_kernel(const __grid_constant__ PrepMaps maps, const KdaTcParams p) {
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int H = p.num_heads;
-    const int n_items = p.blk_off[p.num_requests] * H;
-    if ((int)blockIdx.x >= n_items) return;
+    int n_items = p.blk_off[p.num_requests] * H;
+    if (p.seg_hi != 0x7fffffff || p.seg_lo != 0) {
+        n_items = 0;
+        for (int i = 0; i < p.num_requests; ++i) n_items += seg_blocks(p, i);
+        n_items *= H;
+    }
+    if ((int)blockIdx.x >= n_items) {
+        if (p.beside) grid_dependency_wait();
+        return;
+    }
     const size_t tile_elems = (size_t)kL * kD;
 
     // alpha into the slots and the raw keys and queries into the Kt tiles of the item `it`
@@ -800,6 +824,8 @@ kda_tc_prep_kernel(const __grid_constant__ PrepMaps maps, const KdaTcParams p) {
         tmem_dealloc(tmem, 256);
     }
     if (!ok && tid == 0 && p.status) atomicCAS(p.status, 0, WPP_ERR_TIMEOUT);
+    // beside a chain: this kernel ends after that one, so that the kernel after it has both behind it
+    if (p.beside) grid_dependency_wait();
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -874,6 +900,9 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int head = blockIdx.x, req = blockIdx.y, H = p.num_heads;
     const ReqBlocks g = req_blocks(p, req);
+    grid_launch_dependents();              // (the next segment's preparation, on the SMs this kernel leaves free)
+    const int b_lo = min(p.seg_lo, g.n_blocks), b_hi = min(p.seg_hi, g.n_blocks);
+    if (p.seg_lo > 0 && b_lo >= b_hi) return;
 
     // slot ids: anything outside [-1, num_slots) is reported and treated as -1
     int slot_in = p.state_in[req], slot_out = p.state_out[req];
@@ -921,7 +950,7 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
         // the first product, U0 by the row threads, Kb after the state product, M after the second output product),
         // and each is requested again for the next block the moment it is free.
         uint32_t ph_e = 0;
-        for (int b = 0; b < g.n_blocks; ++b) {
+        for (int b = b_lo; b < b_hi; ++b) {
             const size_t bh = (size_t)(gb0 + b) * H + head;
             const int row = (int)(bh * kL);
             bool okw = __all_sync(0xffffffffu, mbar_wait(bWQEmpty, ph_e ^ 1u, abort_flag));
@@ -959,10 +988,11 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
         Ring step = {0, 0};
         bool dead = false;
         const int interval = p.snap_interval;
-        int64_t next_snap = interval > 0 ? ((int64_t)g.P / interval + 1) * interval : -1;
-        int n_snap = 0;
-        for (int b = 0; b <= g.n_blocks && !dead; ++b) {
-            if (b == g.n_blocks) {      // terminal record
+        const int pos0 = b_lo > 0 ? (g.first_block + b_lo) * kL : g.P;         // tokens folded into S before this launch
+        int64_t next_snap = interval > 0 ? ((int64_t)pos0 / interval + 1) * interval : -1;
+        int n_snap = interval > 0 ? pos0 / interval - g.P / interval : 0;
+        for (int b = b_lo; b <= b_hi && !dead; ++b) {
+            if (b == b_hi) {            // terminal record
                 const bool okw = mbar_wait(bStepEmpty(step.stage), step.phase ^ 1u, abort_flag);
                 if (!__all_sync(0xffffffffu, okw)) break;
                 if (lane == 0) {
@@ -1078,9 +1108,13 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
         const int r = tid & 127;
         const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         const int cbase = wg * 64;                     // this warpgroup's channels (columns of S^T)
+        // where this warpgroup's half of the state waits between two segments, before block b
+        auto between = [&](int b) { return p.ws_u0 + ((size_t)(gb0 + b - 2 + wg) * H + head) * (size_t)kL * kD + r; };
         // initial state: S[c][r] for this warpgroup's c
         {
+            // (of a later segment: channels [0, 64) and [64, 128) lie where U0 of the last two blocks before it was)
             const float* src = slot_in >= 0 ? p.state_pool + ((size_t)slot_in * H + head) * head_floats + r : nullptr;
+            if (b_lo > 0) src = between(b_lo) - (size_t)cbase * kD;
 #pragma unroll 1
             for (int c0 = cbase; c0 < cbase + 64; c0 += 32) {
                 float x[32];
@@ -1090,8 +1124,7 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
             }
             tmem_wait_st();
         }
-        auto store_state = [&](int slot) {
-            float* dst = p.state_pool + ((size_t)slot * H + head) * head_floats + r;
+        auto store_state_at = [&](float* dst) {
 #pragma unroll 1
             for (int c0 = cbase; c0 < cbase + 64; c0 += 32) {
                 float x[32];
@@ -1101,6 +1134,7 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
                 for (int i = 0; i < 32; ++i) dst[(size_t)(c0 + i) * kD] = x[i];
             }
         };
+        auto store_state = [&](int slot) { store_state_at(p.state_pool + ((size_t)slot * H + head) * head_floats + r); };
         // outputs of a finished step (second warpgroup): rows [a, b) of the block, from result region `n`.  A thread
         // holds one value column of all 64 tokens; the tile is turned round in shared memory so that global memory
         // sees 16-byte stores of whole rows.
@@ -1234,12 +1268,17 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
             }
         }
         if (!dead && wg == 1 && prev_a >= 0) dead = !write_outputs(prev_a, prev_b, prev_row, n - 1);
-        if (!dead && slot_out >= 0) {
+        if (!dead && (slot_out >= 0 || b_hi < g.n_blocks)) {
             bool oks = true;
             if (s_pending) oks = mbar_wait(bSReady, ph_s, abort_flag);
             if (__all_sync(0xffffffffu, oks)) {
                 tc_fence_after();
-                store_state(slot_out);
+                if (b_hi == g.n_blocks) {
+                    store_state(slot_out);
+                } else {
+                    // (U0 of those blocks is in shared memory: this thread has waited for it)
+                    store_state_at(between(b_hi) - (size_t)cbase * kD);
+                }
             }
         }
     }
@@ -1262,8 +1301,10 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
 }  // namespace kdatc
 }  // namespace wpp
 
-extern "C" int wpp_launch_kda_tc(const wpp::KdaTcParams* p, const CUtensorMap* maps, int max_blocks, int num_sms,
-                                 void* stream) {
+// segments > 1: segment s has the blocks from seg_begin[s] to seg_begin[s + 1] of every request (the last one the rest), and the
+// preparation of a segment runs beside the chain of the one before, on the SMs that chain leaves free.
+extern "C" int wpp_launch_kda_tc(const wpp::KdaTcParams* params, const CUtensorMap* maps, int max_blocks, int num_sms,
+                                 int segments, const int32_t* seg_begin, void* stream) {
     using namespace wpp::kdatc;
     static bool attr_set[64] = {};
     int dev = 0;
@@ -1276,17 +1317,35 @@ extern "C" int wpp_launch_kda_tc(const wpp::KdaTcParams* p, const CUtensorMap* m
         attr_set[dev] = true;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    kda_tc_setup_kernel<<<1, 1024, 0, st>>>(*p);
-    if (max_blocks > 0) {
-        PrepMaps pm;
-        pm.w0_h = maps[0]; pm.w0_l = maps[1]; pm.qt_h = maps[2]; pm.qt_l = maps[3]; pm.m_h = maps[6]; pm.m_l = maps[7];
-        pm.u0 = maps[8]; pm.q = maps[9]; pm.k = maps[10]; pm.v = maps[11]; pm.alpha = maps[12];
-        const long long items = (long long)max_blocks * p->num_heads;
-        const unsigned grid_a = (unsigned)(items < 2ll * num_sms ? items : 2ll * num_sms);
-        kda_tc_prep_kernel<<<grid_a, kPrepThreads, PrepSmem::kBytes, st>>>(pm, *p);
+    wpp::KdaTcParams p = *params;
+    kda_tc_setup_kernel<<<1, 1024, 0, st>>>(p);
+    PrepMaps pm;
+    pm.w0_h = maps[0]; pm.w0_l = maps[1]; pm.qt_h = maps[2]; pm.qt_l = maps[3]; pm.m_h = maps[6]; pm.m_l = maps[7];
+    pm.u0 = maps[8]; pm.q = maps[9]; pm.k = maps[10]; pm.v = maps[11]; pm.alpha = maps[12];
+    const dim3 grid_b((unsigned)p.num_heads, (unsigned)p.num_requests);
+    const long long chains = (long long)p.num_heads * p.num_requests;
+    for (int s = 0; s < segments; ++s) {
+        p.seg_lo = seg_begin[s];
+        p.seg_hi = s + 1 < segments ? seg_begin[s + 1] : 0x7fffffff;
+        p.beside = s > 0;
+        if (max_blocks > 0) {
+            const long long items = (long long)max_blocks * p.num_heads;
+            const long long ctas = 2ll * (s > 0 ? num_sms - chains : num_sms);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(items < ctas ? items : ctas));
+            cfg.blockDim = dim3(kPrepThreads);
+            cfg.dynamicSmemBytes = PrepSmem::kBytes;
+            cfg.stream = st;
+            cudaLaunchAttribute beside;
+            beside.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            beside.val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = &beside;
+            cfg.numAttrs = s > 0 ? 1 : 0;
+            cudaError_t e = cudaLaunchKernelEx(&cfg, kda_tc_prep_kernel, pm, p);
+            if (e != cudaSuccess) return (int)e;
+        }
+        kda_tc_chain_kernel<<<grid_b, 352, ChainSmem::kBytes, st>>>(maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], maps[6],
+                                                                   maps[7], p);
     }
-    dim3 grid_b((unsigned)p->num_heads, (unsigned)p->num_requests);
-    kda_tc_chain_kernel<<<grid_b, 352, ChainSmem::kBytes, st>>>(maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], maps[6],
-                                                               maps[7], *p);
     return (int)cudaGetLastError();
 }

@@ -290,3 +290,32 @@ def test_groups_of_sixteen_positions_match_the_oracle(H_, interval, decays):
     ref_o, ref_pool = _oracle(w, t, heads=heads)
     _close_out(got_o[:, heads], ref_o, "outputs")
     _close_state(got_pool[:, heads], ref_pool, "state pool")
+
+
+@pytest.mark.parametrize("lens,prefix,interval", [([5000], [70], 0), ([9000], [0], 192), ([14000, 10, 0], [63, 5, 64], 1000),
+                                                  ([4500, 4200], [0, 129], 64)])
+def test_long_chunks_in_segments_match_the_oracle(lens, prefix, interval):
+    """Few long chains run the chunk-parallel form in segments, the preparation of one beside the chain of the one before,
+    the state handed from chain to chain: requests of unequal length (some end in the first segment), snapshots on and
+    off the cuts.  The arithmetic is that of one piece: the same tolerances, and the same bits as two resumed calls cut
+    at a multiple of 64 positions."""
+    w = W.kda_workload("segments", 91, lens, 2, prefix, snap_interval=interval)
+    t = w.tensors()
+    ref_o, ref_pool = _oracle(w, t)
+    got_o, got_pool, status = _gpu(w, t, layout=3)
+    assert status == 0
+    _close_out(got_o, ref_o, "outputs")
+    _close_state(got_pool, ref_pool, "state pool")
+    if len(lens) == 1 and interval == 0:
+        cut = 64 * 20 - prefix[0] % 64
+        pool, parts = t["state_pool"].clone(), []
+        for sl, s_in, pre in ((slice(0, cut), w.state_in, prefix[0]), (slice(cut, lens[0]), w.state_out, prefix[0] + cut)):
+            wp = W.kda_workload("part", 91, [sl.stop - sl.start], 2, [pre])
+            wp.num_slots = w.num_slots
+            o, new_pool, status = _gpu(wp, {k: (v[sl].contiguous() if k != "state_pool" else pool) for k, v in t.items()},
+                                       state_in=s_in, state_out=w.state_out, layout=3)
+            assert status == 0
+            parts.append(o)
+            pool = torch.from_numpy(new_pool).float()
+        assert np.array_equal(np.concatenate(parts), got_o)
+        assert np.array_equal(pool.double().numpy(), got_pool)
