@@ -344,7 +344,7 @@ extern "C" int wpp_prefill_attention_varlen(const wpp_ctx* ctx, const wpp_batch_
         if ((rc = make_map(ctx, &tv, v_cache, 4, dims, strides, box)) != WPP_OK) return rc;
     }
 
-    wpp::AttnParams p;
+    wpp::SmallAttnParams p;
     memset(&p, 0, sizeof(p));
     p.plan = plan_dev;
     p.block_tables = block_tables;

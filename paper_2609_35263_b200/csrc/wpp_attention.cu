@@ -180,10 +180,11 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     grid_launch_dependents();
 
     const char* plan = static_cast<const char*>(p.plan);
-    const int32_t* q_offsets = reinterpret_cast<const int32_t*>(plan + p.off_q_offsets);
-    const int32_t* plan_prefix = reinterpret_cast<const int32_t*>(plan + p.off_prefix);
-    const WppUnit* units = reinterpret_cast<const WppUnit*>(plan + p.off_units);
-    const int num_units = p.num_units;
+    const WppPlanHeader* hd = reinterpret_cast<const WppPlanHeader*>(plan);
+    const int32_t* q_offsets = reinterpret_cast<const int32_t*>(plan + hd->off_q_offsets);
+    const int32_t* plan_prefix = reinterpret_cast<const int32_t*>(plan + hd->off_prefix);
+    const WppUnit* units = reinterpret_cast<const WppUnit*>(plan + hd->off_units);
+    const int num_units = hd->num_units;
     // next tile index for a consuming role: -1 = no more tiles, -2 = the wait was abandoned
     Ring tile_ring = {0, 0};
     auto next_tile = [&]() -> int {

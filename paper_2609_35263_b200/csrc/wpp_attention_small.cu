@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 wpp_attn_small_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_q64,
                       const __grid_constant__ CUtensorMap tm_q32, const __grid_constant__ CUtensorMap tm_q16,
                       const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                      const AttnParams p) {
+                      const SmallAttnParams p) {
     using C = Cfg<D>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -542,7 +542,7 @@ wpp_attn_small_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 }
 
 template <int D>
-static cudaError_t launch(const CUtensorMap* tq, const CUtensorMap& tk, const CUtensorMap& tv, const AttnParams& p,
+static cudaError_t launch(const CUtensorMap* tq, const CUtensorMap& tk, const CUtensorMap& tv, const SmallAttnParams& p,
                           int num_ctas, cudaStream_t stream) {
     static bool attr_set[64] = {};
     int dev = 0;
@@ -571,7 +571,7 @@ static cudaError_t launch(const CUtensorMap* tq, const CUtensorMap& tk, const CU
 
 // tq: four maps of q with boxes of 128, 64, 32 and 16 rows; tk, tv: maps whose boxes have min(page_size, 64) rows
 extern "C" int wpp_launch_attention_small(int head_dim, const CUtensorMap* tq, const CUtensorMap* tk, const CUtensorMap* tv,
-                                          const wpp::AttnParams* p, int num_ctas, void* stream) {
+                                          const wpp::SmallAttnParams* p, int num_ctas, void* stream) {
     if (head_dim == 128) return (int)wpp::small::launch<128>(tq, *tk, *tv, *p, num_ctas, (cudaStream_t)stream);
     if (head_dim == 64) return (int)wpp::small::launch<64>(tq, *tk, *tv, *p, num_ctas, (cudaStream_t)stream);
     return (int)cudaErrorInvalidValue;

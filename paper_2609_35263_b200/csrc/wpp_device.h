@@ -19,14 +19,19 @@ struct AttnParams {
     float* ws_lse;                   // [slots][2][128], log2 units
     int32_t* status;                 // sticky device status word or null
     uint32_t* tile_counter;          // zeroed before the launch: how many tiles have been taken beyond the first one per CTA;
-                                     // or null: round k of the CTAs takes tiles k gridDim .., rotated by k
+                                     // or null (small shape): round k of the CTAs takes tiles k gridDim .., rotated by k
     unsigned long long* stats;       // or null: [0] += key steps of the softmax warps, [1] += those that rescaled O
     int64_t o_token_stride, o_head_stride;
     int32_t num_q_heads, group, page_size, max_blocks, num_pages;
     float scale_log2;                // sm_scale * log2(e)
+};
+
+// The small shape's parameters (apart from AttnParams: with more members there the SM-wide kernel, at its register limit,
+// spills twice as much).
+struct SmallAttnParams : AttnParams {
     uint32_t off_q_offsets, off_prefix, off_units;   // of the plan's arrays (as in its header: one dependent read less)
     int32_t num_units;
-    int32_t item_shift;              // small shape: 1 if an item is half a unit, 0 if no unit has a second half
+    int32_t item_shift;              // 1 if an item is half a unit, 0 if no unit has a second half
 };
 
 struct AppendParams {
@@ -110,7 +115,7 @@ int wpp_launch_kda_tc(const wpp::KdaTcParams* params, const CUtensorMap* maps, i
 int wpp_launch_attention(int head_dim, const CUtensorMap* tq, const CUtensorMap* tk, const CUtensorMap* tv,
                          const wpp::AttnParams* p, int num_ctas, int late_rescale, void* stream);
 int wpp_launch_attention_small(int head_dim, const CUtensorMap* tq, const CUtensorMap* tk, const CUtensorMap* tv,
-                               const wpp::AttnParams* p, int num_ctas, void* stream);
+                               const wpp::SmallAttnParams* p, int num_ctas, void* stream);
 int wpp_launch_append(const wpp::AppendParams* p, int num_sms, void* stream);
 int wpp_launch_combine(const wpp::CombineParams* p, int num_combine, void* stream);
 // maps: q, k, v, alpha; form: 1, 2, 3 = CTAs of 128, 64, 32 columns of the state
