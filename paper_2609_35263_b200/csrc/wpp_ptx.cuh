@@ -87,6 +87,45 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 // The kernel after may be set up on the SMs from here on (it waits for this one's end before it touches memory).
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// ------------------------------------------------------------------ taking over CTAs of this grid that have not started
+// Asks for one: 16 bytes arrive at `response`, counted on `bar`.  Not to be asked again after a refusal.  One thread.
+__device__ __forceinline__ void launch_cancel_request(uint32_t response, uint32_t bar) {
+    mbar_arrive_expect_tx(bar, 16);
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+                     response),
+                 "r"(bar)
+                 : "memory");
+}
+// False: none is left (or none is to be taken).  True: the CTA (bx, by, 0) will not be started, its work is the caller's.
+__device__ __forceinline__ bool launch_cancel_result(uint32_t response, int& bx, int& by) {
+    uint32_t ok, x, y;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 h;\n\t.reg .b32 z, w;\n\t"
+        "ld.shared.b128 h, [%3];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+        "mov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, %2, z, w}, h;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok), "=r"(x), "=r"(y)
+        : "r"(response)
+        : "memory");
+    bx = (int)x, by = (int)y;
+    return ok != 0;
+}
+
+// ------------------------------------------------------------------ bulk copy of contiguous bytes (16-byte aligned, multiple of 16)
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+                 "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
+__device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+
 // ------------------------------------------------------------------ TMA tile loads (no cluster broadcast)
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* m) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");

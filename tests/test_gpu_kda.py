@@ -177,6 +177,23 @@ def test_in_place_slots_and_pure_decay(layout):
     _close_out(got_o, ref, "o = S0^T q")
 
 
+@pytest.mark.parametrize("layout,requests,heads", [(1, 23, 29), (1, 149, 1), (2, 23, 8)])
+def test_more_items_than_sms_are_taken_over_one_after_the_other(layout, requests, heads):
+    """The token-by-token forms' CTAs go on with items that no CTA has started: lengths on both sides of a stage of 16 tokens and
+    of the 8 left when the next item is asked for, empty chunks, requests from the zero state and without a final state."""
+    rng = np.random.default_rng(requests)
+    lens = [int(n) for n in rng.choice([0, 1, 7, 8, 9, 15, 16, 17, 23, 24, 25, 31, 32, 33, 40], requests)]
+    w = W.kda_workload("items", 5, lens, heads, [int(n) for n in rng.integers(0, 40, requests)], snap_interval=13)
+    t = w.tensors()
+    w.state_in[rng.random(requests) < 0.2] = -1
+    w.state_out[rng.random(requests) < 0.2] = -1
+    ref_o, ref_pool = _oracle(w, t)
+    got_o, got_pool, status = _gpu(w, t, layout=layout)
+    assert status == 0
+    _close_out(got_o, ref_o, "outputs")
+    _close_state(got_pool, ref_pool, "state pool")
+
+
 def test_bad_slot_ids_are_reported_and_skipped():
     w = W.kda_workload("bad", 2, [20, 20, 20], 1, [4, 4, 4])
     t = w.tensors()
