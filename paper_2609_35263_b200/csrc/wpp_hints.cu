@@ -98,19 +98,42 @@ __global__ void __launch_bounds__(256) wpp_block_digest_kernel(const int32_t* __
 }
 
 // The chain H_i = mix64(H_{i-1} ^ mix64(digest_i + extraKeys_i) ^ salt term) is sequential by definition: one lane of a
-// warp walks a request's blocks, and what bounds it is the step's own dependent arithmetic (79 clocks, measured alone).
+// warp walks a request's blocks, and what bounds it is the step's own dependent arithmetic.
 // With z the value before mix64's last shift, h = z ^ z >> 31, the next step starts from
 //     h ^ c ^ (h ^ c) >> 30  =  z ^ z >> 30 ^ z >> 31 ^ z >> 61 ^ (c ^ c >> 30),
 // whose shifts are independent of one another and whose last term the digests left ready: two dependent operations
-// between the multiplications instead of four.  The warp moves kStage blocks at a time through shared memory - the next
+// between the multiplications instead of four.  The step works on 32-bit halves, because a 64-bit product's low half is
+// there long before its high half: all of a shift that comes from the low half is folded in while the high half is on its
+// way, and the high half is the sum of three products that do not wait for one another.  64 requests x 3,125 blocks, the
+// fused kernel with its tokens in L2: 64-bit operations 143 us, halves with wide products 129, this order 125.
+// The warp moves kStage blocks at a time through shared memory - the next
 // stage's loads are in flight while this one is chained, the finished hashes leave as coalesced stores - so that the
 // walk never waits on global memory; inside a stage eight terms are read before and eight hashes written after the
 // eight steps between them (a load that may alias the store before it would put shared-memory latency into every step).
+__device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+}
+__device__ __forceinline__ uint32_t mul_hi(uint32_t a, uint32_t b) {     // (apart from the low half: a wide product is later)
+    uint32_t r;
+    asm("mul.hi.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ uint32_t mul_lo(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("mul.lo.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
 __device__ __forceinline__ uint64_t chain_product(uint64_t z, uint64_t c) {
-    uint64_t x = (z ^ (z >> 30)) ^ ((z >> 31) ^ (z >> 61)) ^ c;
-    x *= 0xBF58476D1CE4E5B9ull;
-    x ^= x >> 27;
-    return x * 0x94D049BB133111EBull;
+    constexpr uint32_t k1l = 0x1CE4E5B9u, k1h = 0xBF58476Du, k2l = 0x133111EBu, k2h = 0x94D049BBu;
+    const uint32_t l = (uint32_t)z, h = (uint32_t)(z >> 32), cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
+    const uint32_t early = xor3(l, cl, l >> 30) ^ (l >> 31);
+    const uint32_t xl = xor3(h << 2, h << 1, h >> 29) ^ early, xh = xor3(h ^ ch, h >> 30, h >> 31);
+    const uint32_t pl = mul_lo(xl, k1l), ph = mul_hi(xl, k1l) + mul_lo(xl, k1h) + mul_lo(xh, k1l);
+    const uint32_t yl = xor3(pl, pl >> 27, ph << 5), yh = ph ^ (ph >> 27);
+    const uint32_t ql = mul_lo(yl, k2l), qh = mul_hi(yl, k2l) + mul_lo(yl, k2h) + mul_lo(yh, k2l);
+    return ((uint64_t)qh << 32) | ql;
 }
 constexpr int kStage = 128, kPerLane = kStage / 32;
 __global__ void __launch_bounds__(32) wpp_hash_chain_kernel(const int64_t* __restrict__ block_offsets,
@@ -162,6 +185,9 @@ __global__ void __launch_bounds__(32) wpp_hash_chain_kernel(const int64_t* __res
 // 96 blocks while one lane chains the current ones out of shared memory, so that only the first stage's digests stand in
 // front of the chain.  The chain's warp is the only one of its scheduler (warps 7, 11 and 15 leave at once): beside digest
 // warps its dependent steps waited for issue slots (170 us instead of 144 for 64 requests x 3,125 blocks of 64 tokens).
+// The tokens of a stage are requested a stage ahead (requested with their use, a stage of tokens that come from HBM took
+// longer than its chain: 154 us however short the chain's step), the chain's next eight terms eight steps ahead (137 us
+// without, 129 with).
 constexpr int kFusedWarps = 12, kFusedStage = 8 * kFusedWarps, kFusedThreads = 512;
 __global__ void __launch_bounds__(kFusedThreads, 1) wpp_hash_fused_kernel(const int32_t* __restrict__ tokens,
                                                                           const int64_t* __restrict__ token_offsets,
@@ -177,28 +203,30 @@ __global__ void __launch_bounds__(kFusedThreads, 1) wpp_hash_fused_kernel(const 
     const int64_t b0 = block_offsets[req], n = block_offsets[req + 1] - b0;
     const int32_t* src = tokens + token_offsets[req];
     const int n_stages = (int)((n + kFusedStage - 1) / kFusedStage);
+    int32_t t[8][2];                                   // the tokens of the warp's next eight blocks, on their way
+    auto load = [&](int s) {
+        const int64_t first = (int64_t)s * kFusedStage + dw * 8;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int k = 32 * u + lane;
+                t[j][u] = (k < block_size && first + j < n) ? __ldg(src + (first + j) * block_size + k) : 0;
+            }
+    };
     auto digest = [&](int s) {
         const int64_t first = (int64_t)s * kFusedStage + dw * 8;
         uint64_t d[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) d[j] = 0;
-        for (int k0 = 0; k0 < block_size; k0 += 64) {
-            int32_t t[8][2];
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
+        for (int u = 0; u < 2; ++u) {
+            const int k = 32 * u + lane;
+            if (32 * u >= block_size) break;
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int k = k0 + 32 * u + lane;
-                    t[j][u] = (k < block_size && first + j < n) ? __ldg(src + (first + j) * block_size + k) : 0;
-                }
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int k = k0 + 32 * u + lane;
-                if (k0 + 32 * u >= block_size) break;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) d[j] += k < block_size ? token_term(t[j][u], (uint32_t)k) : 0ull;
-            }
+            for (int j = 0; j < 8; ++j) d[j] += k < block_size ? token_term(t[j][u], (uint32_t)k) : 0ull;
         }
+        load(s + 1);
         uint64_t mine = 0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -211,7 +239,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) wpp_hash_fused_kernel(const 
             s_m[s & 1][dw * 8 + lane] = c ^ (c >> 30);
         }
     };
-    if (warp != 3 && n_stages > 0) digest(0);
+    if (warp != 3 && n_stages > 0) {
+        load(0);
+        digest(0);
+    }
     sync();
     uint64_t z = 0;
     for (int s = 0; s <= n_stages; ++s) {
@@ -220,11 +251,15 @@ __global__ void __launch_bounds__(kFusedThreads, 1) wpp_hash_fused_kernel(const 
                 const uint64_t* m = s_m[s & 1];
                 uint64_t* h = s_h[s & 1];
                 const int cnt = (int)min((int64_t)kFusedStage, n - (int64_t)s * kFusedStage);
+                uint64_t c[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) c[j] = m[j];
 #pragma unroll 1
                 for (int i = 0; i < cnt; i += 8) {
-                    uint64_t c[8];
+                    uint64_t next[8];                  // (past the stage: the first ones again, not used)
+                    const int at = i + 8 < kFusedStage ? i + 8 : 0;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) c[j] = m[i + j];
+                    for (int j = 0; j < 8; ++j) next[j] = m[at + j];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         z = chain_product(z, c[j]);
@@ -232,6 +267,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) wpp_hash_fused_kernel(const 
                     }
 #pragma unroll
                     for (int j = 0; j < 8; ++j) h[i + j] = c[j];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) c[j] = next[j];
                 }
             }
             __syncwarp();
@@ -279,8 +316,9 @@ extern "C" int wpp_hash_blocks(const wpp_ctx* ctx, const int32_t* tokens, const 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const uint64_t salt_term = salt * 0x9E3779B97F4A7C15ull;
     // One kernel when every request can have an SM and its twelve warps keep up with the chain (blocks of up to 64 tokens:
-    // an SM makes a block's digest in less than a chain step).  us, one kernel | two: 64 requests x 3,125 blocks of 64
-    // 144 | 172, 64 x 100 11 | 15, 148 x 3,125 156 | 222; blocks of 128: 1 x 1,500 90 | 72, 64 x 3,125 269 | 199.
+    // an SM makes a block's digest in less than a chain step).  us, one kernel | two, both before the chain's step was
+    // shortened for both: 64 requests x 3,125 blocks of 64 144 | 172, 64 x 100 11 | 15, 148 x 3,125 156 | 222; blocks of 128:
+    // 1 x 1,500 90 | 72, 64 x 3,125 269 | 199.
     if (num_requests <= 148 && block_size <= 64) {
         wpp_hash_fused_kernel<<<(unsigned)num_requests, kFusedThreads, 0, st>>>(tokens, token_offsets, block_offsets, block_size,
                                                                                salt_term, extra, hashes_out);
