@@ -92,6 +92,11 @@ constexpr int64_t kTileFixedCost = 3, kPartExtraCost = 2, kCombineCost = 20;
 //     1 x 512           26 |  17        32 x 64 / 1024    96 | 108        32 x 1024      845 | 930
 //     1 x 2048         106 | 147        32 x 1 / 1024     58 |  37        4 x 1024       107 | 126
 //     8 x 256           41 |  31        32 x 64 / 4096   280 | 407        8 x 512 / 4096 523 | 730
+// Where the small shape's items take several rounds and average more than kSmallShapeSteps key steps, its estimate is up to
+// 12 % short (the CTAs of an SM share the tensor pipe and L2) and the SM-wide one is taken: 32 x 4..34 new tokens, 40/8 heads
+// (one head per tile), over 512 / 900 / 1,100 / 1,500 / 4,096 cached ones 142 | 92, 171 | 130, 142 | 148, 169 | 184, 431 | 459;
+// over 256..3,635 ones 214 | 240; 64 x 4..16, 64/8 heads, over 0..1,024 / 0..2,048 72 | 62, 90 | 92 (pass, us).
+constexpr int64_t kSmallShapeSteps = 8;
 struct StepCount {
     int64_t sum = 0;
     int32_t longest = 0, shortest = 0x7fffffff;
@@ -479,7 +484,10 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     int shape = o.shape;
     const int64_t n_items = nonempty_halves > n_units ? 2 * n_units : n_units;       // of the small shape
     if (shape == 0 && few_shape != 0) shape = few_shape;
-    else if (shape == 0) shape = small_shape_us(half_steps, n_items, o.max_ctas) <= wide_shape_us(unit_steps, n_units, nonempty_halves, o.max_ctas) ? 2 : 1;
+    else if (shape == 0)
+        shape = !(n_items > 2 * (int64_t)o.max_ctas && half_steps.sum > kSmallShapeSteps * n_items) &&
+                        small_shape_us(half_steps, n_items, o.max_ctas) <= wide_shape_us(unit_steps, n_units, nonempty_halves, o.max_ctas)
+                    ? 2 : 1;
     const int num_ctas = shape == 2 ? (int)std::max<int64_t>(1, std::min<int64_t>(2 * (int64_t)o.max_ctas, 2 * n_units))
                                     : (int)std::max<int64_t>(1, std::min<int64_t>(o.max_ctas, n_units));
     off += sizeof(WppUnit) * (size_t)n_units;

@@ -281,3 +281,11 @@ def test_kernel_shape_follows_the_mean_key_steps_per_half():
         assert forced.info.shape == shape
     with pytest.raises(wpp.WppError):
         wpp.wpp_plan_tiles(None, d, [0] * 4, [64] * 4, opts=wpp.PlanOpts(0, 0, 0, 0, 0, 3), pin=False)
+
+
+@pytest.mark.parametrize("prefix,shape", [(512, 2), (1024, 1), (1500, 1)])
+def test_several_rounds_of_many_steps_go_to_the_sm_wide_shape(prefix, shape):
+    """32 x 20 new tokens, a head per tile (group of five): 1,280 items, several rounds of the small shape; at 1,024 cached
+    tokens an item has nine key steps, one more than the small shape is taken for."""
+    plan = wpp.wpp_plan_tiles(None, desc(32, 40, 8, 128, 64, 64, 4000), np.full(32, prefix, np.int32), np.full(32, 20, np.int32))
+    assert plan.info.shape == shape and plan.info.num_tiles == 1280
