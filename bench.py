@@ -507,9 +507,9 @@ def run_hints(args):
     hbm = float(peaks.get("hbm_gbs", FALLBACK_PEAKS["hbm_gbs"]))
     line = {"metric": "chained block hashing, tokens/s (64 requests x 200K tokens)", "value": tokens.numel() / (ms * 1e-3),
             "unit": "tokens/s", "n_gpus": 1, "steps": steps, "warmup": max(3, args.warmup), "ms_per_step": ms,
-            "higher_is_better": True, "vs_baseline": None, "dtype": "u64", "data": "synthetic", "gpu_launches": 2 * steps,
+            "higher_is_better": True, "vs_baseline": None, "dtype": "u64", "data": "synthetic", "gpu_launches": steps,
             "config": {"workload": "64 requests of 200,000 tokens, 64-token blocks, first 100,000 tokens common"},
-            "roofline": {"bound": "hbm", "kernel": "wpp_block_digest_kernel + wpp_hash_chain_kernel",
+            "roofline": {"bound": "hbm", "kernel": "wpp_hash_fused_kernel",
                          "achieved": nbytes / (ms * 1e-3) / 1e9, "peak": hbm, "unit": "GB/s",
                          "frac": nbytes / (ms * 1e-3) / 1e9 / hbm, "peak_source": f"of {peak_kind} (copy bandwidth)",
                          "traffic": None},
@@ -586,15 +586,17 @@ def run_kda(args):
         # bandwidth bound it from below (7 d_k d_v flop per token and head are 0.04 ms of tensor time for the default
         # wave, the bytes 0.13 ms); what it actually moves is three times that, because the preparation kernel hands
         # its per-block operands to the chain kernel through the workspace.
-        roofline = {"bound": "hbm", "kernel": "kda_tc_prep_kernel + kda_tc_chain_kernel",
+        # (Layout 0: the library chooses between that and the group form, one kernel that moves little but these bytes.)
+        roofline = {"bound": "hbm", "kernel": "kda_tc_prep_kernel + kda_tc_chain_kernel" if args.kda_layout == 3 else
+                                              "the library's choice: the group kernel, or preparation and chain",
                     "achieved": nbytes / (ms * 1e-3) / 1e9, "peak": hbm, "unit": "GB/s",
                     "frac": nbytes / (ms * 1e-3) / 1e9 / hbm, "peak_source": f"of {peak_kind} (copy bandwidth)",
                     "algorithmic_bytes": nbytes, "flop_per_token_head": 7 * w.d_k * w.d_v,
                     "tflops_algorithmic": flops / (ms * 1e-3) / 1e12,
-                    "traffic": KDA_TC_DRAM_BYTES_PER_TOKEN_HEAD * T * Hh,
+                    "traffic": KDA_TC_DRAM_BYTES_PER_TOKEN_HEAD * T * Hh if args.kda_layout == 3 else None,
                     "traffic_source": "estimate: dram read + write bytes of one preparation and one chain launch on the "
                                       "8 x 2,048-token wave (ncu), per (token, head), x this wave's pairs; not measured "
-                                      "in this run"}
+                                      "in this run" if args.kda_layout == 3 else "none"}
     else:
         peak = 148 * 128 * 2 * 1965e6 / 1e12
         roofline = {"bound": "alu", "kernel": "wpp_kda_chunk_kernel", "achieved": flops / (ms * 1e-3) / 1e12,
@@ -606,7 +608,7 @@ def run_kda(args):
     line = {"metric": "recurrent-state (KDA) layer, new tokens/s through one layer", "value": T / (ms * 1e-3),
             "unit": "tokens/s", "n_gpus": 1, "steps": steps, "warmup": warm, "ms_per_step": ms, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "bf16 x 2 terms, fp32 accumulate" if tensor_form else "f32",
-            "data": "synthetic", "gpu_launches": steps * (3 if tensor_form else 1),
+            "data": "synthetic", "gpu_launches": steps * (3 if args.kda_layout == 3 else 1),      # (layout 0: at least)
             "config": {"workload": w.name, "requests": int(w.chunk_lens.size), "chunk": int(w.chunk_lens[0]),
                        "state_heads": Hh, "d_k": w.d_k, "d_v": w.d_v, "layout": args.kda_layout,
                        "form": "chunk-parallel on tensor cores" if tensor_form else "token by token on CUDA cores",
