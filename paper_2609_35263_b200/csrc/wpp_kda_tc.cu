@@ -850,7 +850,7 @@ struct ChainSmem {
     static constexpr int kOffVec = kOffOut + kL * kD * 2;     // per ring slot: alpha of the step's first token, decay product at its end
     static constexpr int kOffRec = kOffVec + kStepRing * 2 * kD * 4;
     static constexpr int kOffBars = kOffRec + kStepRing * (int)sizeof(StepRec);
-    static constexpr int kNumBars = 2 * kStepRing + 8 + 7;
+    static constexpr int kNumBars = 2 * kStepRing + 8 + 8;
     static constexpr int kOffMisc = kOffBars + 8 * kNumBars;
     static constexpr int kBytes = kOffMisc + 64 + 1024;
 };
@@ -879,10 +879,14 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
     const uint32_t bWQFull = b0, bWQEmpty = b0 + 8, bU0Full = b0 + 16, bU0Empty = b0 + 24, bKbFull = b0 + 32,
                    bKbEmpty = b0 + 40, bMFull = b0 + 48, bMEmpty = b0 + 56;
     const uint32_t b1 = b0 + 64;
-    const uint32_t bShlReady = b1, bXReady = b1 + 8, bUhlReady = b1 + 16, bSReady = b1 + 24, bOReady = b1 + 32;
-    // o_free, one per result region: a waiter may lag a barrier by at most one phase, and the issuing thread asks for
-    // the read-out of two steps back while the row threads may already have signalled the one after it
-    auto bOFree = [&](int n) { return b1 + 40 + 8 * (uint32_t)(n & 1); };
+    const uint32_t bShlReady = b1, bXReady = b1 + 8, bUhlReady = b1 + 16, bSReady = b1 + 24;
+    // o_ready and o_free, one per result region: a waiter may lag a barrier by at most one phase.  The issuing thread asks
+    // for the read-out of two steps back while the row threads may already have signalled the one after it; and the row
+    // threads ask for a step's outputs after they have released the products of the next, whose own outputs are then ready
+    // 0.8 us later whether the first were waited for or not (with one barrier for both regions a warp that was held up that
+    // long, by a miss in the instruction cache for instance, waited for a phase that its own read-out had to come before).
+    auto bOReady = [&](int n) { return b1 + 32 + 8 * (uint32_t)(n & 1); };
+    auto bOFree = [&](int n) { return b1 + 48 + 8 * (uint32_t)(n & 1); };
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sm + CS::kOffMisc);
     volatile uint32_t* abort_flag = tmem_slot + 1;
     const float* s_vec = reinterpret_cast<const float*>(sm + CS::kOffVec);
@@ -922,7 +926,7 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
         mbar_init(bU0Full, 1);
         mbar_init(bU0Empty, 256);          // the U0 tile is released by the 256 row threads
         mbar_init(bShlReady, 256); mbar_init(bXReady, 1); mbar_init(bUhlReady, 256); mbar_init(bSReady, 1);
-        mbar_init(bOReady, 1); mbar_init(bOFree(0), 128); mbar_init(bOFree(1), 128);
+        mbar_init(bOReady(0), 1); mbar_init(bOReady(1), 1); mbar_init(bOFree(0), 128); mbar_init(bOFree(1), 128);
         *abort_flag = 0u;
         fence_barrier_init();
     }
@@ -1090,7 +1094,7 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
                 for (int kk = 0; kk < 4; ++kk)
                     mma_ts_accumulate(tD + 64, tD + (kk >> 1) * 32 + (kk & 1) * 8 + (term == 2 ? 16u : 0u), bd + (uint64_t)(kk * 2), idesc64);
             }
-            mma_commit(bOReady);
+            mma_commit(bOReady(n));
             if (last) mma_commit(bMEmpty);
             ++n;
         }
@@ -1130,12 +1134,12 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
         // outputs of a finished step (second warpgroup): rows [a, b) of the block, from result region `n`.  A thread
         // holds one value column of all 64 tokens; the tile is turned round in shared memory so that global memory
         // sees 16-byte stores of whole rows.
-        uint32_t ph_o = 0;
+        uint32_t ph_o = 0;                             // bit i: phase of result region i
         __nv_bfloat16* s_out = reinterpret_cast<__nv_bfloat16*>(sm + CS::kOffOut);
         auto write_outputs = [&](int a, int b, int64_t row_t0, int n) -> bool {
-            const bool oko = mbar_wait(bOReady, ph_o, abort_flag);
+            const bool oko = mbar_wait(bOReady(n), (ph_o >> (n & 1)) & 1u, abort_flag);
             if (!__all_sync(0xffffffffu, oko)) return false;
-            ph_o ^= 1u;
+            ph_o ^= 1u << (n & 1);
             tc_fence_after();
             float o[64];
             tmem_ld32(lane_addr + col_d(n) + 64, reinterpret_cast<uint32_t*>(o));

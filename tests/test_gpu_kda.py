@@ -336,3 +336,30 @@ def test_long_chunks_in_segments_match_the_oracle(lens, prefix, interval):
             pool = torch.from_numpy(new_pool).float()
         assert np.array_equal(np.concatenate(parts), got_o)
         assert np.array_equal(pool.double().numpy(), got_pool)
+
+
+def test_calls_of_few_long_chains_end_alike_however_cold_the_caches_are():
+    """Few long chains start the chain kernel six times a call, beside a preparation that fills the memory system: three
+    hundred calls, each from an idle device with its caches overwritten, end without a wait that ran out and with one
+    result."""
+    w = W.kda_workload("cold", 97, [6000], 8, [128])
+    t = w.tensors()
+    dev = torch.device("cuda")
+    d = {k: v.to(dev) for k, v in t.items()}
+    i32 = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).to(dev)
+    rows, s_in, s_out, prefix = torch.from_numpy(w.row_offsets).to(dev), i32(w.state_in), i32(w.state_out), i32(w.prefix_lens)
+    ws = torch.empty(wpp.wpp_kda_workspace_bytes(1, 8, 6000), dtype=torch.uint8, device=dev)
+    cold = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    out, bad, first = torch.empty_like(d["v"]), torch.zeros(1, dtype=torch.int64, device=dev), None
+    launches = H.ctx().launch_count()
+    for i in range(300):
+        cold.fill_(i & 1)
+        torch.cuda.synchronize()
+        wpp.wpp_kda_chunk(H.ctx(), d["q"], d["k"], d["v"], d["alpha"], d["beta"], rows, d["state_pool"], s_in, s_out, out=out,
+                          prefix_lens=prefix, status=status, layout=3, workspace=ws)
+        if first is None:
+            first = out.clone()
+        bad += (out.view(torch.int16) != first.view(torch.int16)).any()
+    assert int(status.item()) == 0 and int(bad.item()) == 0
+    assert H.ctx().launch_count() - launches > 300 * 3                 # in segments
