@@ -896,7 +896,6 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int head = blockIdx.x, req = blockIdx.y, H = p.num_heads;
     const ReqBlocks g = req_blocks(p, req);
-    grid_launch_dependents();              // (the next segment's preparation, on the SMs this kernel leaves free)
     const int b_lo = min(p.seg_lo, g.n_blocks), b_hi = min(p.seg_hi, g.n_blocks);
     if (p.seg_lo > 0 && b_lo >= b_hi) return;
 
@@ -937,6 +936,7 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_launch_dependents();              // (the next segment's preparation, on the SMs this kernel leaves free)
     const uint32_t tmem = *tmem_slot;
     const int gb0 = p.blk_off[req];
 

@@ -84,7 +84,9 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 // ------------------------------------------------------------------ overlap with the kernels before and after in the stream
 // Everything a kernel reads or writes in global memory may belong to the kernel before it: wait first.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// The kernel after may be set up on the SMs from here on (it waits for this one's end before it touches memory).
+// The kernel after may be set up on the SMs from here on (it waits for this one's end before it touches memory).  It may
+// hold shared memory and tensor memory while it waits, so a kernel comes here only once it has its own tensor memory: the
+// allocation waits without a limit for what the kernel after would only give back once this one has ended.
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ------------------------------------------------------------------ taking over CTAs of this grid that have not started

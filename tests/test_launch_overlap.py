@@ -1,0 +1,76 @@
+"""Kernels that let the next one in their stream be set up while they run (griddepcontrol): what the sources have to keep."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_35263_b200", "csrc")
+
+
+def _kernels():
+    """(file, kernel name, body up to the next kernel) of every __global__ function."""
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        src = re.sub(r"//[^\n]*", "", open(path).read())
+        starts = [m.start() for m in re.finditer(r"__global__", src)] + [len(src)]
+        for a, b in zip(starts, starts[1:]):
+            name = re.search(r"(\w+)\s*\(\s*const", src[a:b])
+            yield os.path.basename(path), name.group(1) if name else "?", src[a:b]
+
+
+def test_tensor_memory_is_allocated_before_the_next_kernel_is_let_in():
+    """The next kernel may take tensor memory of the SM and keep it until this one has ended; an allocation that comes after
+    the release could wait for it for ever.  Every CTA has to have passed the barrier behind its own allocation first."""
+    seen = 0
+    for path, name, body in _kernels():
+        if "tmem_alloc(" not in body or "grid_launch_dependents()" not in body:
+            continue
+        seen += 1
+        alloc, release = body.index("tmem_alloc("), body.index("grid_launch_dependents()")
+        assert alloc < release, f"{path}: {name} lets the next kernel in before it has its tensor memory"
+        assert "__syncthreads()" in body[alloc:release], f"{path}: {name} releases before all of the CTA has its tensor memory"
+    assert seen >= 3
+
+
+@pytest.mark.gpu
+def test_small_attention_directly_behind_the_two_pass_recurrent_layer():
+    """The chain kernel takes all 512 columns of an SM's tensor memory, the small attention shape 256 per CTA: queued behind
+    one another without anything between, both end with the results they have apart."""
+    import numpy as np
+    import torch
+
+    import paper_2609_35263_b200 as wpp
+    import wpp_workloads as W
+    from tests import gpu_harness as H
+    from tests.test_gpu_kda import _gpu
+
+    w = W.custom_workload([300, 64, 0, 17], [33, 64, 90, 5], 8, 2, 64, 16, seed=23)
+    g = H.device_inputs(w)
+    apart = H.run_wave(w, g, shape=2)
+    assert apart["status"] == 0
+    kw = W.kda_workload("front", 29, [200, 70, 333], 7, [5, 0, 64])
+    t = kw.tensors()
+    o_apart, pool_apart, status = _gpu(kw, t, layout=3)
+    assert status == 0
+    dev = torch.device("cuda")
+    d = {k: v.to(dev) for k, v in t.items()}
+    i32 = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).to(dev)
+    rows, s_in, s_out, prefix, chunks, P, bt = (torch.from_numpy(kw.row_offsets).to(dev), i32(kw.state_in), i32(kw.state_out),
+                                                i32(kw.prefix_lens), i32(w.chunk_lens), i32(w.prefix_lens), i32(w.block_tables))
+    ws = torch.empty(wpp.wpp_kda_workspace_bytes(3, 7, int(t["q"].shape[0])), dtype=torch.uint8, device=dev)
+    plan, status = apart["plan"], torch.zeros(1, dtype=torch.int32, device=dev)
+    ws_attn = torch.empty(int(plan.info.workspace_bytes), dtype=torch.uint8, device=dev)
+    pool0 = d["state_pool"].clone()
+    for _ in range(20):
+        out, out_kda = torch.zeros_like(apart["out"]), torch.zeros_like(d["v"])
+        d["state_pool"].copy_(pool0)
+        torch.cuda.synchronize()
+        wpp.wpp_kda_chunk(H.ctx(), d["q"], d["k"], d["v"], d["alpha"], d["beta"], rows, d["state_pool"], s_in, s_out, out=out_kda,
+                          prefix_lens=prefix, status=status, layout=3, workspace=ws)
+        wpp.wpp_prefill_attention_varlen(H.ctx(), H.desc_of(w), g["q"], out, None, g["k_pool"], g["v_pool"], bt, P, chunks, plan,
+                                         workspace=ws_attn, status=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        assert torch.equal(out, apart["out"])
+        assert np.array_equal(out_kda.float().cpu().double().numpy(), o_apart)
+        assert np.array_equal(d["state_pool"].cpu().double().numpy(), pool_apart)
