@@ -259,14 +259,33 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     };
     int TM = o.tile_m;
     int64_t n_base = build_rows(TM);
+    // partial results the built-in scratch array holds (without the workspace's header)
+    const uint64_t slot_bytes = (uint64_t)2 * WPP_HALF_M * (d.head_dim + 1) * sizeof(float);
+    const uint64_t scratch_slots = (kSplitScratchBytes - WPP_WS_HEADER_BYTES) / slot_bytes;
+    if (o.force_kv_splits != 0 && auto_tile_m && n_base < o.max_ctas) {
+        // Few tiles and the caller's cut: more, smaller ones, unless only the taller tiles' partial results fit the built-in
+        // scratch array.  Attention call in us, 256-row tiles | 128: 1 x 8,192 tokens, one head, never cut 112 | 97, in two
+        // parts 78 | 71; 2 x 1,000 over 3,000, 8/2 heads, never cut 76 | 68.
+        auto forced_slots = [&]() {
+            uint64_t n = 0;
+            for (const RowBlock& rb : rbs) {
+                const int32_t parts = std::min(o.force_kv_splits, rb.steps);
+                if (parts > 1) n += (uint64_t)parts * (uint64_t)(Hq / rb.per_tile);
+            }
+            return n;
+        };
+        const bool tall_fits = forced_slots() <= scratch_slots;
+        n_base = build_rows(WPP_HALF_M);
+        if (tall_fits && forced_slots() > scratch_slots) n_base = build_rows(TM);
+        else TM = WPP_HALF_M;
+    }
     int32_t part_eighths = 0;      // length of a tile's parts in eighths of a key step (0: whole tiles)
     int few_shape = 0;             // the kernel shape these parts were chosen for
     if (o.force_kv_splits == 0 && n_base > 0 && n_base < o.max_ctas) {
         const int tms[2] = {128, 256};
         double best = 0.0;
         int best_tm = TM;
-        uint64_t slots_cap = kSplitScratchBytes / ((uint64_t)2 * WPP_HALF_M * (d.head_dim + 1) * sizeof(float));
-        if (slots_cap > 0) --slots_cap;                                    // (the workspace's header)
+        uint64_t slots_cap = scratch_slots - 1;
         // (or within what cutting the 128-row tiles so that there are at least max_ctas parts takes, if that is more)
         if (auto_tile_m) n_base = build_rows(128);
         uint64_t even_parts = 0;

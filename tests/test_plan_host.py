@@ -289,3 +289,25 @@ def test_several_rounds_of_many_steps_go_to_the_sm_wide_shape(prefix, shape):
     tokens an item has nine key steps, one more than the small shape is taken for."""
     plan = wpp.wpp_plan_tiles(None, desc(32, 40, 8, 128, 64, 64, 4000), np.full(32, prefix, np.int32), np.full(32, 20, np.int32))
     assert plan.info.shape == shape and plan.info.num_tiles == 1280
+
+
+@pytest.mark.parametrize("C,heads,splits,units", [(2048, (8, 2, 64), 1, 128), (8192, (1, 1, 128), 1, 64), (8192, (1, 1, 128), 2, 127)])
+def test_few_tiles_fall_back_to_128_row_tiles_whatever_cut_the_caller_asks_for(C, heads, splits, units):
+    """Fewer 256-row tiles than CTAs and a cut of the caller's (never, or into so many parts): 128-row tiles, so that twice
+    as many CTAs have work (units: the row blocks of 128, in 1 or 2 parts; the first one of the last case has one key step
+    and stays whole)."""
+    d = desc(1, *heads, 64, 200)
+    pl = parse_plan(wpp.wpp_plan_tiles(None, d, [0], [C], opts=wpp.PlanOpts(0, 0, splits, 148), pin=False))
+    assert pl["tile_m"] == 128 and len(pl["units"]) == units and all(u["rows_b"] == 0 for u in pl["units"])
+    tall = parse_plan(wpp.wpp_plan_tiles(None, d, [0], [C], opts=wpp.PlanOpts(256, 0, splits, 148), pin=False))
+    assert tall["tile_m"] == 256 and len(tall["units"]) < units                  # an explicit height is kept
+
+
+def test_a_forced_cut_of_few_tiles_fits_the_scratch_that_taller_tiles_fit():
+    """2 x 900 new tokens over 3,000 cached ones in two parts: 128-row tiles would need 256 partial results, more than the
+    built-in scratch array holds, 256-row ones 128 tiles' worth; one head group less and either fits."""
+    scratch = int(wpp.load_library().wpp_static_scratch_bytes())
+    for heads, tile_m in (((6, 2, 128), 256), ((2, 1, 128), 128)):
+        plan = wpp.wpp_plan_tiles(None, desc(2, *heads, 64, 70), [3000, 3000], [900, 900], opts=wpp.PlanOpts(0, 0, 2, 148), pin=False)
+        assert parse_plan(plan)["tile_m"] == tile_m and plan.info.num_split_tiles > 0
+        assert plan.info.workspace_bytes <= scratch
