@@ -207,7 +207,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     auto steps_for = [](int64_t last_visible_plus1) { return (int32_t)((last_visible_plus1 + WPP_TILE_N - 1) / WPP_TILE_N); };
     std::vector<RowBlock> rbs;
     std::vector<int32_t> rb_first((size_t)R + 1);
-    const bool pair_heads = auto_tile_m && G % 2 == 0 && pairs >= kPairHeadsKeys * T;
+    bool pair_heads = auto_tile_m && G % 2 == 0 && pairs >= kPairHeadsKeys * T;
     auto build_rows = [&](int tile_m) -> int64_t {
         // The halves of a 256-row tile are two consecutive row blocks of a head, or, where the queries see many keys on
         // average, two heads of a KV group over the same 128 rows: those see the same keys, so neither half waits for the
@@ -362,75 +362,100 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     //      order 1: longest tile first (best balance, no regard for which tiles run together).
     struct Tile { int32_t rb, head; };          // row block and first head
     std::vector<Tile> tiles;
-    tiles.reserve((size_t)n_base);
-    if (o.order == 1) {
-        for (int32_t k = 0; k < (int32_t)rbs.size(); ++k)
-            for (int h = 0; h < Hq; h += rbs[(size_t)k].per_tile) tiles.push_back({k, h});
-        std::stable_sort(tiles.begin(), tiles.end(),
-                         [&](const Tile& a, const Tile& b) { return rbs[(size_t)a.rb].cost() > rbs[(size_t)b.rb].cost(); });
-    } else {
-        std::vector<int64_t> req_cost((size_t)std::max(R, 1), 0);
-        for (const RowBlock& rb : rbs) req_cost[(size_t)rb.request] += (int64_t)rb.cost() * (Hq / rb.per_tile);
-        std::vector<int32_t> by_cost((size_t)R);
-        for (int i = 0; i < R; ++i) by_cost[(size_t)i] = i;
-        std::stable_sort(by_cost.begin(), by_cost.end(),
-                         [&](int32_t a, int32_t b) { return req_cost[(size_t)a] > req_cost[(size_t)b]; });
-        for (int kvh = 0; kvh < d.num_kv_heads; ++kvh)
-            for (int rank = 0; rank < R; ++rank) {
-                const int i = by_cost[(size_t)rank];
-                for (int32_t k = rb_first[(size_t)i]; k < rb_first[(size_t)i + 1]; ++k)
-                    for (int h = kvh * G; h < (kvh + 1) * G; h += rbs[(size_t)k].per_tile) tiles.push_back({k, h});
-            }
-    }
+    auto order_tiles = [&]() {
+        tiles.clear();
+        tiles.reserve((size_t)n_base);
+        if (o.order == 1) {
+            for (int32_t k = 0; k < (int32_t)rbs.size(); ++k)
+                for (int h = 0; h < Hq; h += rbs[(size_t)k].per_tile) tiles.push_back({k, h});
+            std::stable_sort(tiles.begin(), tiles.end(),
+                             [&](const Tile& a, const Tile& b) { return rbs[(size_t)a.rb].cost() > rbs[(size_t)b.rb].cost(); });
+        } else {
+            std::vector<int64_t> req_cost((size_t)std::max(R, 1), 0);
+            for (const RowBlock& rb : rbs) req_cost[(size_t)rb.request] += (int64_t)rb.cost() * (Hq / rb.per_tile);
+            std::vector<int32_t> by_cost((size_t)R);
+            for (int i = 0; i < R; ++i) by_cost[(size_t)i] = i;
+            std::stable_sort(by_cost.begin(), by_cost.end(),
+                             [&](int32_t a, int32_t b) { return req_cost[(size_t)a] > req_cost[(size_t)b]; });
+            for (int kvh = 0; kvh < d.num_kv_heads; ++kvh)
+                for (int rank = 0; rank < R; ++rank) {
+                    const int i = by_cost[(size_t)rank];
+                    for (int32_t k = rb_first[(size_t)i]; k < rb_first[(size_t)i + 1]; ++k)
+                        for (int h = kvh * G; h < (kvh + 1) * G; h += rbs[(size_t)k].per_tile) tiles.push_back({k, h});
+                }
+        }
+    };
+    order_tiles();
 
     // ---- split decision: into how many key ranges each tile is cut (1 = not at all)
     int64_t tail = 0;              // tiles of a partly filled last round ...
     int32_t tail_parts = 1;        // ... and the number of key ranges each of them is cut into
-    if (o.force_kv_splits == 0 && few_shape == 0 && n_base % o.max_ctas != 0 && n_base < kTailSplitMaxRounds * (int64_t)o.max_ctas) {
-        // A few rounds of long tiles: the last, partly filled round leaves CTAs idle for a whole tile.  Cutting the
-        // tiles of that round into p key ranges each fills it.  The candidates are compared on a model of the run
-        // (tiles handed out in order to the CTA that is free first; a tile costs its key steps plus a fixed start
-        // and end, a part a little more, the combine pass a constant).  The model flatters the cut: SMs of a partly
-        // filled round run faster than those of a full one (more of the power budget and of L2 each), so that a
-        // modelled gain of 12 % measured as 5-6 % and one of 8 % as a small loss; a cut is made from 10 % up.
-        const int64_t n_tail = n_base % o.max_ctas;
-        int32_t min_steps = 0x7fffffff;
-        for (int64_t k = n_base - n_tail; k < n_base; ++k) min_steps = std::min(min_steps, rbs[(size_t)tiles[(size_t)k].rb].steps);
-        if (min_steps >= 2 * kTailSplitMinSteps) {
-            using MinHeap = std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>>;
-            MinHeap before_tail;                 // when each CTA is free once the full rounds have been handed out
-            for (int c = 0; c < o.max_ctas; ++c) before_tail.push(0);
-            int64_t end_before = 0;
-            for (int64_t k = 0; k < n_base - n_tail; ++k) {
-                const int64_t done = before_tail.top() + rbs[(size_t)tiles[(size_t)k].rb].cost() + kTileFixedCost;
-                before_tail.pop();
-                before_tail.push(done);
-                end_before = std::max(end_before, done);
-            }
-            auto makespan = [&](int32_t p) -> int64_t {
-                MinHeap free_at = before_tail;
-                int64_t end = end_before;
-                for (int64_t k = n_base - n_tail; k < n_base; ++k) {
-                    const RowBlock& t = rbs[(size_t)tiles[(size_t)k].rb];
-                    for (int32_t q = 0; q < p; ++q) {
-                        const int32_t a = (int32_t)((int64_t)t.steps * q / p), b = (int32_t)((int64_t)t.steps * (q + 1) / p);
-                        const int64_t done = free_at.top() + cost_of(t, a, b) + kTileFixedCost + (p > 1 ? kPartExtraCost : 0);
-                        free_at.pop();
-                        free_at.push(done);
-                        end = std::max(end, done);
-                    }
+    auto cut_tail = [&](uint64_t max_slots) {
+        tail = 0;
+        tail_parts = 1;
+        if (o.force_kv_splits == 0 && few_shape == 0 && n_base % o.max_ctas != 0 && n_base < kTailSplitMaxRounds * (int64_t)o.max_ctas) {
+            // A few rounds of long tiles: the last, partly filled round leaves CTAs idle for a whole tile.  Cutting the
+            // tiles of that round into p key ranges each fills it.  The candidates are compared on a model of the run
+            // (tiles handed out in order to the CTA that is free first; a tile costs its key steps plus a fixed start
+            // and end, a part a little more, the combine pass a constant).  The model flatters the cut: SMs of a partly
+            // filled round run faster than those of a full one (more of the power budget and of L2 each), so that a
+            // modelled gain of 12 % measured as 5-6 % and one of 8 % as a small loss; a cut is made from 10 % up.
+            const int64_t n_tail = n_base % o.max_ctas;
+            int32_t min_steps = 0x7fffffff;
+            for (int64_t k = n_base - n_tail; k < n_base; ++k) min_steps = std::min(min_steps, rbs[(size_t)tiles[(size_t)k].rb].steps);
+            if (min_steps >= 2 * kTailSplitMinSteps) {
+                using MinHeap = std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>>;
+                MinHeap before_tail;                 // when each CTA is free once the full rounds have been handed out
+                for (int c = 0; c < o.max_ctas; ++c) before_tail.push(0);
+                int64_t end_before = 0;
+                for (int64_t k = 0; k < n_base - n_tail; ++k) {
+                    const int64_t done = before_tail.top() + rbs[(size_t)tiles[(size_t)k].rb].cost() + kTileFixedCost;
+                    before_tail.pop();
+                    before_tail.push(done);
+                    end_before = std::max(end_before, done);
                 }
-                return end + (p > 1 ? kCombineCost : 0);
-            };
-            const int64_t whole = makespan(1);
-            int64_t best = whole;
-            for (int32_t p = 2; p <= kTailSplitMaxParts && min_steps >= p * kTailSplitMinSteps; ++p) {
-                const int64_t m = makespan(p);
-                if (m < best) { best = m; tail_parts = p; }
+                auto makespan = [&](int32_t p) -> int64_t {
+                    MinHeap free_at = before_tail;
+                    int64_t end = end_before;
+                    for (int64_t k = n_base - n_tail; k < n_base; ++k) {
+                        const RowBlock& t = rbs[(size_t)tiles[(size_t)k].rb];
+                        for (int32_t q = 0; q < p; ++q) {
+                            const int32_t a = (int32_t)((int64_t)t.steps * q / p), b = (int32_t)((int64_t)t.steps * (q + 1) / p);
+                            const int64_t done = free_at.top() + cost_of(t, a, b) + kTileFixedCost + (p > 1 ? kPartExtraCost : 0);
+                            free_at.pop();
+                            free_at.push(done);
+                            end = std::max(end, done);
+                        }
+                    }
+                    return end + (p > 1 ? kCombineCost : 0);
+                };
+                const int64_t whole = makespan(1);
+                int64_t best = whole;
+                for (int32_t p = 2; p <= kTailSplitMaxParts && min_steps >= p * kTailSplitMinSteps && (uint64_t)n_tail * p <= max_slots; ++p) {
+                    const int64_t m = makespan(p);
+                    if (m < best) { best = m; tail_parts = p; }
+                }
+                if (tail_parts > 1 && best * 100 <= whole * (100 - kTailSplitMinGainPct)) tail = n_tail;
+                else tail_parts = 1;
             }
-            if (tail_parts > 1 && best * 100 <= whole * (100 - kTailSplitMinGainPct)) tail = n_tail;
-            else tail_parts = 1;
         }
+    };
+    cut_tail(~0ull);
+    if (pair_heads && (uint64_t)tail * (uint64_t)tail_parts > scratch_slots) {
+        // The cut needs more scratch than the built-in array holds.  Tiles whose halves are two heads are cut in more waves
+        // than tiles of row blocks (the halves end together, so the model sees more to gain), and a wave that those would
+        // not have cut beyond the array must not be refused for it by the entry point that has no other scratch: such a
+        // wave is cut as far as the array allows.  2 requests, 950 over 30,000 and 500 over 16,000, 64/8 heads, us: as row
+        // blocks, whole, 1,007; two heads, whole 981, cut in four 887.
+        pair_heads = false;
+        n_base = build_rows(TM);
+        order_tiles();
+        cut_tail(~0ull);
+        const bool cut_anyway = (uint64_t)tail * (uint64_t)tail_parts > scratch_slots;
+        pair_heads = true;
+        n_base = build_rows(TM);
+        order_tiles();
+        cut_tail(cut_anyway ? ~0ull : scratch_slots);
     }
 
     // ---- the plan: header, row offsets, the spans the plan is made for, units, combine records

@@ -311,3 +311,16 @@ def test_a_forced_cut_of_few_tiles_fits_the_scratch_that_taller_tiles_fit():
         plan = wpp.wpp_plan_tiles(None, desc(2, *heads, 64, 70), [3000, 3000], [900, 900], opts=wpp.PlanOpts(0, 0, 2, 148), pin=False)
         assert parse_plan(plan)["tile_m"] == tile_m and plan.info.num_split_tiles > 0
         assert plan.info.workspace_bytes <= scratch
+
+
+@pytest.mark.parametrize("heads,P,C", [((64, 8, 128, 64), [30000, 16000], [950, 500]), ((32, 8, 128, 64), [50000, 50000, 4000], [700, 300, 950]),
+                                       ((32, 8, 128, 128), [30000, 16000, 8000], [950, 300, 950])])
+def test_a_wave_is_not_cut_beyond_the_built_in_scratch_because_its_halves_are_two_heads(heads, P, C):
+    """Waves whose tiles, as row blocks, would stay whole: planned with two heads per tile their last round must not be cut
+    into more partial results than the built-in scratch array holds, or the entry point without a workspace refuses them."""
+    scratch = int(wpp.load_library().wpp_static_scratch_bytes())
+    d = desc(len(P), *heads, (max(P) + max(C) + heads[3] - 1) // heads[3] + 1)
+    rows = wpp.wpp_plan_tiles(None, d, P, C, opts=wpp.PlanOpts(256, 0, 0, 148), pin=False)
+    auto = wpp.wpp_plan_tiles(None, d, P, C, opts=wpp.PlanOpts(0, 0, 0, 148), pin=False)
+    assert rows.info.workspace_bytes <= scratch and auto.info.workspace_bytes <= scratch
+    assert any(u["head_b"] != u["head_a"] and u["row0_b"] == u["row0_a"] and u["rows_a"] == 128 for u in parse_plan(auto)["units"])
