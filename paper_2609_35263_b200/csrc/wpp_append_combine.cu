@@ -71,7 +71,13 @@ __global__ void __launch_bounds__(32 * kCombineRows) wpp_combine_kernel(const Co
     const int64_t tok = (int64_t)reinterpret_cast<const int32_t*>(plan + p.off_q_offsets)[cu.request] + cu.row0 + r;
     const int64_t row = ((int64_t)cu.slot0 * 2 + cu.half) * 128 + cu.lane0 + r;      // + 256 per part
     float m = -INFINITY, wsum = 0.f;
-    for (int s = lane; s < cu.num_splits; s += 32) m = fmaxf(m, p.ws_lse[row + s * 256]);
+    bool nan = false;                 // some part's scores had one: the row is NaN, as it is when the tile is not cut
+    for (int s = lane; s < cu.num_splits; s += 32) {
+        const float l = p.ws_lse[row + s * 256];
+        nan |= l != l;
+        m = fmaxf(m, l);
+    }
+    nan = __any_sync(0xffffffffu, nan);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     float acc[kV];
@@ -80,14 +86,16 @@ __global__ void __launch_bounds__(32 * kCombineRows) wpp_combine_kernel(const Co
     if (m > -INFINITY) {
         for (int s0 = 0; s0 < cu.num_splits; s0 += 32) {
             const int cnt = min(32, cu.num_splits - s0);
-            // a part that saw no key of this row has lse -inf: weight zero, its O row is not defined and not used
-            const float w_mine = lane < cnt ? exp2f(p.ws_lse[row + (s0 + lane) * 256] - m) : 0.f;
+            // a part that saw no key of this row has lse -inf: its O row is not defined and not used (weight -1 here).  One
+            // whose weight merely underflows to zero is used: what it holds may be infinite or NaN.
+            const float l_mine = lane < cnt ? p.ws_lse[row + (s0 + lane) * 256] : -INFINITY;
+            const float w_mine = l_mine == -INFINITY ? -1.f : exp2f(l_mine - m);
             for (int b0 = 0; b0 < cnt; b0 += kCombineBatch) {
                 float x[kCombineBatch][kV], w[kCombineBatch];
 #pragma unroll
                 for (int u = 0; u < kCombineBatch; ++u) {
                     w[u] = __shfl_sync(0xffffffffu, w_mine, (b0 + u) & 31);
-                    const bool use = b0 + u < cnt && w[u] > 0.f;
+                    const bool use = b0 + u < cnt && !(w[u] < 0.f);
                     const float* src = p.ws_o + (row + (int64_t)(s0 + b0 + u) * 256) * D + lane * kV;
                     if constexpr (kV == 4) {
                         const float4 v = use ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -107,14 +115,14 @@ __global__ void __launch_bounds__(32 * kCombineRows) wpp_combine_kernel(const Co
             }
         }
     }
-    const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
+    const float inv = nan ? NAN : wsum > 0.f ? 1.f / wsum : 0.f;
     __nv_bfloat16* dst = p.out + tok * p.o_token_stride + (int64_t)cu.head * p.o_head_stride + lane * kV;
     if constexpr (kV == 4)
         *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv));
     else
         *reinterpret_cast<uint32_t*>(dst) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
     if (p.lse && lane == 0)
-        p.lse[tok * p.num_q_heads + cu.head] = wsum > 0.f ? (m + log2f(wsum)) * 0.6931471805599453f : -INFINITY;
+        p.lse[tok * p.num_q_heads + cu.head] = wsum > 0.f && !nan ? (m + log2f(wsum)) * 0.6931471805599453f : -INFINITY;
 }
 
 // Self-test of the bounded wait every kernel of the library relies on: one warp waits, with a short limit, on

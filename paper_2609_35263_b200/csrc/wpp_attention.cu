@@ -432,7 +432,7 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 tc_fence_after();
                 const float2 ml = s_final[hf * 128 + r];
                 const float inv_l = (ml.y > 0.f) ? 1.f / ml.y : 0.f;
-                const float lse2 = (ml.y > 0.f) ? (ml.x + log2f(ml.y)) : -INFINITY;
+                const float lse2 = (ml.y <= 0.f) ? -INFINITY : (ml.x + log2f(ml.y));       // (NaN if one of the row's scores was)
                 uint8_t* stage = smem_gen + C::kOffStage + (warp & 3) * 2048;
                 if (un.split_slot < 0) {
                     const __nv_bfloat16* dst = p.out + tok * p.o_token_stride + (int64_t)head * p.o_head_stride;
@@ -451,7 +451,7 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         }
                         warp_store_rows64(stage, lane, w, dst, row_ok, q4 * 64);
                     }
-                    if (p.lse && row_ok) p.lse[tok * p.num_q_heads + head] = lse2 * 0.6931471805599453f;
+                    if (p.lse && row_ok) p.lse[tok * p.num_q_heads + head] = fmaxf(lse2 * 0.6931471805599453f, -INFINITY);
                 } else {
                     const float* dst = p.ws_o + prow * D;
 #pragma unroll

@@ -480,7 +480,7 @@ wpp_attn_small_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             }
             tc_fence_after();
             const float inv_l = (l_run > 0.f) ? 1.f / l_run : 0.f;
-            const float lse2 = (l_run > 0.f) ? (-nmc + log2f(l_run)) : -INFINITY;
+            const float lse2 = (l_run <= 0.f) ? -INFINITY : (-nmc + log2f(l_run));       // (NaN if one of the row's scores was)
             uint8_t* stage = smem_gen + C::kOffStage + warp * 2048;
             if (un.split_slot < 0) {
                 const __nv_bfloat16* dst = p.out + tok * p.o_token_stride + (int64_t)head * p.o_head_stride;
@@ -499,7 +499,7 @@ wpp_attn_small_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                     }
                     warp_store_rows64(stage, lane, w, dst, row_ok, q4 * 64);
                 }
-                if (p.lse && row_ok) p.lse[tok * p.num_q_heads + head] = lse2 * 0.6931471805599453f;
+                if (p.lse && row_ok) p.lse[tok * p.num_q_heads + head] = fmaxf(lse2 * 0.6931471805599453f, -INFINITY);
             } else {
                 const float* dst = p.ws_o + prow * D;
 #pragma unroll 1

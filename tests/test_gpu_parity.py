@@ -402,3 +402,37 @@ def test_small_shape_items_dealt_out_or_counted(C, Hq, ctas):
     w = W.custom_workload([40 * i for i in range(len(C))], C, Hq, 1, 128, 64, seed=61, spare_pages=4)
     for tile_m in (128, 256):
         _full_parity(w, opts=wpp.PlanOpts(tile_m, 0, 1, ctas, 0, 2))
+
+
+@pytest.mark.parametrize("shape", [1, 2])
+@pytest.mark.parametrize("d,splits", [(64, 2), (128, 4), (128, 40)])
+def test_a_cut_tile_shows_the_infinities_and_nans_that_a_whole_one_shows(d, splits, shape):
+    """One request whose first 128 keys all score 512 below the others (their weights underflow to zero once parts are
+    merged).  An infinite value among them, a NaN in a key and a NaN in a query: cut along the keys, exactly the elements are
+    NaN that are NaN when the tile stays whole, and the others agree."""
+    w = W.custom_workload([40 * 128], [40], 2, 1, d, 64, seed=31)
+    inp = cpu_inputs(w)
+    page = lambda n: int(w.block_tables[0, n])
+    for k in ("q", "k_new", "k_pool"):
+        inp[k] = (inp[k].float() * 0.1).bfloat16()
+    inp["q"] += 8
+    for n in range(2):
+        inp["k_pool"][page(n)] = -64 / d ** 0.5               # score: -64 / sqrt(d) * 8 d / sqrt(d) = -512
+    inf_, nan_ = float("inf"), float("nan")
+    for what in ("value", "key", "query"):
+        x = {k: v.clone() for k, v in inp.items()}
+        if what == "value":
+            x["v_pool"][page(0), 0, 3, 5] = inf_
+        elif what == "key":
+            x["k_new"][20, 0, 1] = nan_                          # the rows from 20 on see it
+        else:
+            x["q"][11, 1, 2] = nan_
+        whole = H.run_wave(w, H.device_inputs(w, x), opts=wpp.PlanOpts(0, 0, 1, 0), shape=shape)
+        cut = H.run_wave(w, H.device_inputs(w, x), opts=wpp.PlanOpts(0, 0, splits, 0), shape=shape)
+        assert whole["status"] == 0 and cut["status"] == 0
+        assert cut["plan"].info.num_split_tiles > 0 and whole["plan"].info.num_split_tiles == 0
+        a, b = f64(whole["out"]), f64(cut["out"])
+        bad = ~np.isfinite(a)
+        assert bad.any() and np.array_equal(bad, ~np.isfinite(b)) and np.array_equal(np.isnan(a), np.isnan(b)), what
+        assert np.abs(a[~bad] - b[~bad]).max() <= H.MAX_ABS_TOL
+        assert np.array_equal(np.isneginf(f64(whole["lse"])), np.isneginf(f64(cut["lse"])))
