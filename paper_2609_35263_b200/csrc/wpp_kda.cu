@@ -341,7 +341,10 @@ __device__ __noinline__ void kda_compute_item(const KdaParams& p, KdaSmem& sm, i
     if (it.slot_out >= 0) {
         if (kSplit == 8) {
             store_state(&sm.state_out[0][4 * cq], kGroupPitch);
-            fence_proxy_async_smem();
+            // (a periodic snapshot may have gone to the same slot: then what was written to global memory comes first too, which
+            // costs 3 us of 126 where there is nothing to order)
+            if (interval > 0) fence_proxy_async();
+            else fence_proxy_async_smem();
         } else {
             store_state(state_of(it.slot_out, head, cq), 4 * kDV);
         }

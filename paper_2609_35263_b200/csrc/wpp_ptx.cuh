@@ -81,6 +81,11 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// the same for global memory as well: what this thread wrote before and what bulk copies write after keep their order
+__device__ __forceinline__ void fence_proxy_async() {
+    asm volatile("fence.proxy.async;" ::: "memory");
+}
+
 // ------------------------------------------------------------------ overlap with the kernels before and after in the stream
 // Everything a kernel reads or writes in global memory may belong to the kernel before it: wait first.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -363,3 +363,21 @@ def test_calls_of_few_long_chains_end_alike_however_cold_the_caches_are():
         bad += (out.view(torch.int16) != first.view(torch.int16)).any()
     assert int(status.item()) == 0 and int(bad.item()) == 0
     assert H.ctx().launch_count() - launches > 300 * 3                 # in segments
+
+
+@pytest.mark.parametrize("layout", [0, 1, 2, 3])
+@pytest.mark.parametrize("C,interval", [(33, 32), (65, 64), (100, 7)])
+def test_a_snapshot_slot_may_be_the_slot_of_the_chunk_end(layout, C, interval):
+    """A request's periodic snapshots may go to the slot that its state at the chunk end goes to (no other request's slot):
+    the last one written is the state at the end, however soon after the snapshot it follows and whichever way either is
+    stored."""
+    R, H_ = 40, 4
+    w = W.kda_workload("same slot", 53, [C] * R, H_, [0] * R, snap_interval=interval)
+    w.snap_slots[:] = w.state_out[:, None]
+    t = w.tensors()
+    heads = [0, H_ - 1]
+    _, ref_pool = _oracle(w, t, heads=heads)
+    for _ in range(5):
+        _, got_pool, status = _gpu(w, t, layout=layout)
+        assert status == 0
+        _close_state(got_pool[:, heads], ref_pool, "state pool")
