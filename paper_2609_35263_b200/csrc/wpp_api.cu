@@ -508,7 +508,8 @@ static int kda_segments(const wpp_kda_desc* d, int sms, double* us, int32_t* beg
 //                                  4x32x256    51 /  58 /  105 |  75     1x8x2048   336 / 276 /  178 |  142
 //                                  4x32x4096  635 / 801 / 1374 | 722     2x32x8192 1328 / 1103 / 1369 | 913
 //                                  8x32x64     34 /  36 /   67 |  50     64x32x256  630 / 740 / 1409 | 782
-// Error against the fp32 token-by-token form, rms of the states over their rms: 6.0e-6 (two passes: 4.9e-6); outputs equal.
+// Error against 64 bits, rms of the states over their rms, 8 x 2,048 tokens x 32 heads: 4.35e-6 (two passes: 5.09e-6); outputs
+// 1.6595e-3 for both, the rounding to bf16.
 static int kda_chunk_form(const wpp_kda_desc* d, int sms) {
     const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
     auto rounds = [&](double ctas) { return ceil(ctas / sms); };

@@ -1,10 +1,10 @@
 // Recurrent-state (KDA) layer of a chunk in groups of 16 tokens, the state in registers (Section 3.1 update, Section 3.2
 // snapshots).  Per request and head the update
 //     S_t = (I - beta_t k_t k_t^T) Diag(alpha_t) S_{t-1} + beta_t k_t v_t^T,     o_t = S_t^T q_t
-// over a group of tokens [a, e) that starts from the state S, with the decay products G_t = prod_{a <= r <= t} alpha_r and
-// Kt = K o G, Kh = K / G, Qt = Q o G, is
+// over a group of tokens [a, e) that starts from the state S, with the decay products G_t = prod_{a <= r <= t} alpha_r,
+// Gt_t = G_t / G_{e-1}, Kt = K o Gt, Kh = K / Gt, Qt = Q o Gt, is
 //     A = tril(diag(beta) Kt Kh^T, -1),   T = (I + A)^-1 diag(beta),   M = tril(Qt Kh^T),
-//     U = T (V - Kt S),     O = Qt S + M U,     S <- Diag(G_{e-1}) (S + Kh^T U).
+//     S' = Diag(G_{e-1}) S,     U = T (V - Kt S'),     O = Qt S' + M U,     S <- S' + Kh^T U.
 // (Where the first token's own alpha is too small to divide by, it is applied to the state instead and left out of G.)
 //
 // The columns of S evolve independently, so a warp that owns 16 or 32 columns carries them through the whole chunk
@@ -18,14 +18,19 @@
 // state in tensor memory a step is a chain of hand-overs between the issuing thread, the tensor pipe and the warps that
 // scale, split and store, and its operands need a pass of their own in front (14.5 K clocks of an SM per 64 tokens, 144 KB
 // written and read back).  Here a group's chain stays inside a warp: 21 K clocks of an SM per 64 tokens in all, no second
-// pass.  8 x 2,048 tokens, 32 heads: 733 -> 640 us; 8 x 64: 50 -> 33 us; 1 x 512: 62 -> 51 us (the choice: kda_chunk_form).
-// What bounds a group now (clocks, 5.3 K): the products 3.4 K of which the MMA pipe is busy 2.6 K, U 0.4 K, hand-over and
-// outputs 1.2 K; the producers are idle half the time.  Also tried: four column warps of 32 columns with 216 registers
+// pass.  8 x 2,048 tokens, 32 heads: 740 -> 676 us; 8 x 64: 56 -> 41 us; 1 x 512: 68 -> 57 us (the choice: kda_chunk_form).
+// What bounds a group (clocks, 5.3 K before the third terms below): the products 3.4 K of which the MMA pipe is busy 2.6 K,
+// U 0.4 K, hand-over and outputs 1.2 K; the producers are idle half the time.  Also tried: four column warps of 32 columns with 216 registers
 // (809 us: one warp per scheduler waits), one producer warpgroup (660), a thirteenth warp for T and the copies (711: four
 // warps in a quarter of the SM leave 128 registers each).
 //
-// Precision.  Every operand is split into two bf16 terms, x = hi + lo (16 significant bits), and every product is three
-// MMAs, hi hi + hi lo + lo hi (the dropped lo lo is 2^-17 relative), accumulated in fp32.
+// Precision.  Operands are split into two bf16 terms, x = hi + lo (16 significant bits), a product is three MMAs,
+// hi hi + hi lo + lo hi (the dropped lo lo is 2^-17 relative), accumulated in fp32; V - Kt S' and T have three terms and
+// their small product six MMAs.  The decay products are relative to the group's end because its last keys, whose share in
+// the state has decayed least, then have Kh = K to the bit.  Rms error of the states against 64 bits, over their rms, two
+// passes | here, 8 x 2,048 tokens x 32 heads: alpha = sigmoid(4 + 2 n) with n normal 5.09e-6 | 4.35e-6, sigmoid(8 + 2 n)
+// 6.73e-6 | 5.27e-6, sigmoid(1 + 2 n) 4.30e-6 | 3.60e-6; with products from the group's start and two terms throughout it was
+// 6.33e-6, 7.29e-6 and 5.09e-6 at 645 instead of 676 us.
 //
 // Groups are the 16-token blocks of absolute sequence positions (so a chunk split at such a position reproduces the
 // unsplit result bit for bit), cut wherever the state is needed inside a block (a periodic snapshot) and before every
@@ -57,6 +62,14 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_
     hi = pack_bf16x2(x0, x1);
     const float2 d = __ffma2_rn(make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), make_float2(-1.f, -1.f), make_float2(x0, x1));
     lo = pack_bf16x2(d.x, d.y);
+}
+// three terms: 24 significant bits
+__device__ __forceinline__ void split3(float x0, float x1, uint32_t& hi, uint32_t& lo, uint32_t& third) {
+    hi = pack_bf16x2(x0, x1);
+    const float2 d = __ffma2_rn(make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), make_float2(-1.f, -1.f), make_float2(x0, x1));
+    lo = pack_bf16x2(d.x, d.y);
+    const float2 e = __ffma2_rn(make_float2(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u)), make_float2(-1.f, -1.f), d);
+    third = pack_bf16x2(e.x, e.y);
 }
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
@@ -141,7 +154,7 @@ struct StageT {
     static constexpr int kKtH = 0, kKtL = kTile, kQtH = 2 * kTile, kQtL = 3 * kTile, kKhH = 4 * kTile, kKhL = 5 * kTile;
     static constexpr int kV = 6 * kTile;                   // 64-column halves of 128-byte rows (TMA's swizzle)
     static constexpr int kSq = 16 * 32;                    // a 16 x 16 bf16 matrix
-    static constexpr int kTH = kV + kVH * (kTile / 2), kTL = kTH + kSq, kMH = kTL + kSq, kML = kMH + kSq;
+    static constexpr int kTH = kV + kVH * (kTile / 2), kTL = kTH + kSq, kT3 = kTL + kSq, kMH = kT3 + kSq, kML = kMH + kSq;
     static constexpr int kEnd = kML + kSq;                 // fp32 [128]: decay product of the whole group
     static constexpr int kPre = kEnd + kD * 4;             // fp32 [128]: alpha of the first token (if `pre`)
     static constexpr int kRec = kPre + kD * 4;
@@ -363,6 +376,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                 // ---- Kt, Qt and Kh as hi/lo bf16 operands; rows outside the group are zero.  (The stores carry no memory
                 //      clobber: behind one, every token's loads would wait for the stores of the token before.)
                 const uint32_t row_c = st + half * 2048 + cp * 4;
+                const float2 r_end = make_float2(rcp_approx(g_end.x), rcp_approx(g_end.y));              // g_end >= 2^-40: finite
                 if (half == 0) sts2f(st + Stage::kEnd + cp * 8, g_end);
                 if (pre && half == (a >> 3)) sts2f(st + Stage::kPre + cp * 8, lds2f(r_alpha + (a & 7) * kD * 4));
 #pragma unroll
@@ -380,8 +394,8 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                         const int i = i0 + u;
                         const float2 k2 = make_float2(__uint_as_float(kr[u] << 16), __uint_as_float(kr[u] & 0xffff0000u));
                         const float2 q2 = make_float2(__uint_as_float(qr[u] << 16), __uint_as_float(qr[u] & 0xffff0000u));
-                        const float2 gt = __fmul2_rn(g[i], carry);
-                        const float2 inv = make_float2(rcp_approx(gt.x), rcp_approx(gt.y));      // gt >= 2^-40: finite
+                        const float2 gs = __fmul2_rn(g[i], carry), gt = __fmul2_rn(gs, r_end);
+                        const float2 inv = __fmul2_rn(g_end, make_float2(rcp_approx(gs.x), rcp_approx(gs.y)));      // gs >= 2^-40
                         const uint32_t at = (row_c ^ (i << 4)) + i * 256;                        // row_off(8 half + i, cp >> 2)
                         auto put = [&](int at_hi, int at_lo, float2 x) {
                             uint32_t hi, lo;
@@ -478,10 +492,12 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                     for (int r = 0; r < 8; ++r) {
                         const float v = x[r] * bt;
                         const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-                        const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
+                        const float d = v - __bfloat162float(hi);
+                        const __nv_bfloat16 lo = __float2bfloat16_rn(d), third = __float2bfloat16_rn(d - __bfloat162float(lo));
                         const uint32_t at = dst + sq_off(r, c >> 3);             // (the swizzle of row r0 + r is that of row r)
                         asm volatile("st.shared.b16 [%0], %1;" ::"r"(at), "h"(__bfloat16_as_ushort(hi)));
                         asm volatile("st.shared.b16 [%0], %1;" ::"r"(at + Stage::kTL - Stage::kTH), "h"(__bfloat16_as_ushort(lo)));
+                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(at + Stage::kT3 - Stage::kTH), "h"(__bfloat16_as_ushort(third)));
                     }
                 }
                 __syncwarp();
@@ -570,7 +586,16 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                         }
                     }
                 }
-                uint32_t th[4], tl[4], mh[4], ml[4];
+#pragma unroll
+                for (int j = 0; j < kNT; ++j) {
+                    const float2 f = lds2f(st + Stage::kEnd + (ch0 + 8 * j + 2 * gc) * 4);
+#pragma unroll
+                    for (int m = 0; m < kMT; ++m) {
+                        const float2 lo = __fmul2_rn(make_float2(S[m][j][0], S[m][j][1]), f), hi = __fmul2_rn(make_float2(S[m][j][2], S[m][j][3]), f);
+                        S[m][j][0] = lo.x; S[m][j][1] = lo.y; S[m][j][2] = hi.x; S[m][j][3] = hi.y;
+                    }
+                }
+                uint32_t th[4], tl[4], t3[4], mh[4], ml[4];
                 // lane addresses of the operands of 16 channels 16 k: row_off(.., 2k + ..) is an exclusive or of the low bits
                 // (one register per operand family instead of one per k)
                 const uint32_t row_a = st + (l16 * 8 + ln7) * 256 + ((l8 ^ ln7) << 4), row_b = st + (l8 * 8 + ln7) * 256 + ((l16 ^ ln7) << 4);
@@ -683,13 +708,14 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                     if (m == 0) {
                         ldsm4(th, st + Stage::kTH + sq);
                         ldsm4(tl, st + Stage::kTL + sq);
+                        ldsm4(t3, st + Stage::kT3 + sq);
                         ldsm4(mh, st + Stage::kMH + sq);
                         ldsm4(ml, st + Stage::kML + sq);
                     }
                     uint32_t uh[4], ul[4];
                     {
                         const int vc = col0 + m * 16 + l8 * 8;               // 8 columns of V from here, tokens l16 * 8 + ln7
-                        uint32_t vv[4], yh[4], yl[4];
+                        uint32_t vv[4], yh[4], yl[4], y3[4];
                         ldsm4t(vv, st + Stage::kV + (kVH == 2 ? vc >> 6 : 0) * (Stage::kTile / 2) + (l16 * 8 + ln7) * 128 + ((((vc & 63) >> 3) ^ ln7) << 4));
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
@@ -697,7 +723,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                             const int t = (i >> 1) * 8 + 2 * gc;
                             const float y0 = (t >= a && t < e) ? __uint_as_float(vv[i] << 16) - X[i >> 1][(i & 1) * 2] : 0.f;
                             const float y1 = (t + 1 >= a && t + 1 < e) ? __uint_as_float(vv[i] & 0xffff0000u) - X[i >> 1][(i & 1) * 2 + 1] : 0.f;
-                            split2(y0, y1, yh[i], yl[i]);
+                            split3(y0, y1, yh[i], yl[i], y3[i]);
                         }
                         float U[2][4], Ul[2][4];
 #pragma unroll
@@ -705,10 +731,18 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                             U[n][0] = U[n][1] = U[n][2] = U[n][3] = 0.f;
                             Ul[n][0] = Ul[n][1] = Ul[n][2] = Ul[n][3] = 0.f;
                             mma16(U[n], yh, th[2 * n], th[2 * n + 1]);
-                            mma16(Ul[n], yh, tl[2 * n], tl[2 * n + 1]);
+                            mma16(Ul[n], yh, t3[2 * n], t3[2 * n + 1]);
                         }
 #pragma unroll
-                        for (int n = 0; n < 2; ++n) mma16(U[n], yl, th[2 * n], th[2 * n + 1]);
+                        for (int n = 0; n < 2; ++n) {
+                            mma16(U[n], yl, th[2 * n], th[2 * n + 1]);
+                            mma16(Ul[n], yl, tl[2 * n], tl[2 * n + 1]);
+                        }
+#pragma unroll
+                        for (int n = 0; n < 2; ++n) {
+                            mma16(Ul[n], y3, th[2 * n], th[2 * n + 1]);
+                            mma16(U[n], yh, tl[2 * n], tl[2 * n + 1]);
+                        }
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
                             split2(U[i >> 1][2 * (i & 1)] + Ul[i >> 1][2 * (i & 1)], U[i >> 1][2 * (i & 1) + 1] + Ul[i >> 1][2 * (i & 1) + 1], uh[i], ul[i]);
@@ -731,7 +765,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                         if (wn == w && ++sn == SM::kStages) { sn = 0; pn ^= 1u; }
                         ready = mbar_test(bFull(wn, sn), pn);
                     }
-                    // ---- S <- Diag(G_end) (S + (U^T Kh)^T)
+                    // ---- S <- S' + (U^T Kh)^T
 #pragma unroll
                     for (int j2 = 0; j2 < kNT / 2; ++j2) {
                         const uint32_t at = chunk(row_b, j2);
@@ -744,12 +778,6 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
                         mma16(S[m][2 * j2 + 1], ul, bh[2], bh[3]);
                         mma16(S[m][2 * j2], uh, bl[0], bl[1]);
                         mma16(S[m][2 * j2 + 1], uh, bl[2], bl[3]);
-                    }
-#pragma unroll
-                    for (int j = 0; j < kNT; ++j) {
-                        const float2 f = lds2f(st + Stage::kEnd + (ch0 + 8 * j + 2 * gc) * 4);
-                        const float2 lo = __fmul2_rn(make_float2(S[m][j][0], S[m][j][1]), f), hi = __fmul2_rn(make_float2(S[m][j][2], S[m][j][3]), f);
-                        S[m][j][0] = lo.x; S[m][j][1] = lo.y; S[m][j][2] = hi.x; S[m][j][3] = hi.y;
                     }
                     if (m == kMT - 1) {
                         __syncwarp();

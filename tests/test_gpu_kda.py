@@ -381,3 +381,25 @@ def test_a_snapshot_slot_may_be_the_slot_of_the_chunk_end(layout, C, interval):
         _, got_pool, status = _gpu(w, t, layout=layout)
         assert status == 0
         _close_state(got_pool[:, heads], ref_pool, "state pool")
+
+
+@pytest.mark.parametrize("shift", [None, 8.0, 1.0])                     # decays: the workload's, long memory, short memory
+@pytest.mark.parametrize("H_", [9, 17, 33])                             # CTAs of 32, 64 and 128 columns
+def test_groups_of_sixteen_positions_are_no_further_from_64_bits_than_the_two_passes(H_, shift):
+    """What the library chooses for 4 x 192 tokens against the form that it stands in for (layout 3): the root mean square
+    error of the states against 64 bits is no larger.  That the choice was the group form shows in the states' last bits."""
+    w = W.kda_workload("error", 60 + H_, [192] * 4, H_, [0, 64, 5, 100])
+    t = w.tensors()
+    if shift is not None:
+        g = torch.Generator().manual_seed(H_)
+        t["alpha"] = torch.sigmoid(shift + 2 * torch.randn(t["alpha"].shape, generator=g))
+    heads = [0, H_ - 1]
+    _, ref_pool = _oracle(w, t, heads=heads)
+    err, pools = [], []
+    for layout in (0, 3):
+        _, pool, status = _gpu(w, t, layout=layout)
+        assert status == 0
+        pools.append(pool)
+        err.append(np.sqrt(np.mean((pool[w.state_out][:, heads] - ref_pool[w.state_out]) ** 2)))
+    assert not np.array_equal(pools[0], pools[1])
+    assert err[0] <= err[1], err
