@@ -504,24 +504,45 @@ static int kda_segments(const wpp_kda_desc* d, int sms, double* us, int32_t* beg
 // The two-pass form reads and writes 144 KB of operands per block but its chain is the fastest per token; the group form
 // has nothing in front of its chain and moves nothing but inputs and outputs.  The estimates below are microseconds for
 // C tokens per request, measured on 148 SMs (us; group with 128 / 64 / 32 columns | two passes):
-//     requests x heads x tokens    8x32x2048  640 / 801 / 1224 | 733     1x32x512    91 /  75 /   51 |   62
-//                                  4x32x256    51 /  58 /  105 |  75     1x8x2048   336 / 276 /  178 |  142
-//                                  4x32x4096  635 / 801 / 1374 | 722     2x32x8192 1328 / 1103 / 1369 | 913
-//                                  8x32x64     34 /  36 /   67 |  50     64x32x256  630 / 740 / 1409 | 782
+//     requests x heads x tokens    8x32x2048  669 / 853 / 1285 | 744     1x32x512    93 /  77 /   56 |   71
+//                                  4x32x256    56 /  67 /  116 |  79     1x8x2048   333 / 273 /  188 |  153
+//                                  4x32x4096  661 / 857 / 1443 | 732     2x32x2048  335 / 280 /  378 |  259
+//                                  8x32x64     42 /  44 /   75 |  58     64x32x256  652 / 775 / 1469 |  798
 // Error against 64 bits, rms of the states over their rms, 8 x 2,048 tokens x 32 heads: 4.35e-6 (two passes: 5.09e-6); outputs
 // 1.6595e-3 for both, the rounding to bf16.
-static int kda_chunk_form(const wpp_kda_desc* d, int sms) {
+//
+// These are waves of equal chunks, and a wave lasts at least as long as its longest chain, which costs three times as much per
+// token here as in the two passes.  The lengths are on the device: the group form's CTAs look at them, and a wave with a chunk
+// longer than *longest is left to the two passes queued behind (which end at once if it is not).  *longest is the length up
+// to which the group form is the faster one however the rest is distributed: no order of its CTAs takes longer than its rounds
+// all of the longest chunk, nor than the chunks spread evenly and the longest on top; the two passes are taken for equal chunks,
+// where they are fastest.  us, two passes | group form whatever the lengths | now:
+//     8 x 32 heads, 14,000 and 7 x 340 tokens 1261 | 2108 | 1263     8 x 32, 8,192 and 7 x 1,170 960 | 1248 | 959
+//     9 x 8 heads, 16,000 and 8 x 48 tokens 1004 | 2055 | 1004        4 x 32, 512 and 3 x 64 85 | 92 | 83
+// The empty launches behind a wave of equal chunks: 8 x 2,048 669 -> 676, 4 x 256 56 -> 64, 8 x 64 42 -> 50, 64 x 256 652 -> 673.
+constexpr double kGroupUs = 12.0;       // what a launch takes before and after its chains
+static int kda_chunk_form(const wpp_kda_desc* d, int sms, int64_t* longest) {
     const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
-    auto rounds = [&](double ctas) { return ceil(ctas / sms); };
     double two_passes = 0.0;
     kda_segments(d, sms, &two_passes, nullptr);
-    const double t[4] = {35 + two_passes,
-                         rounds(n) * C * 0.157,                                                       // one CTA per SM
-                         2 * n <= sms ? C * 0.135 : rounds(n) * C * 0.195,                            // two per SM
-                         rounds(4 * n) * C * 0.084};
+    two_passes += 35.0;
+    const struct { double ctas, at_once, us_per_token; } form[4] = {{},
+                                                                    {n, (double)sms, 0.165},                                 // one CTA per SM
+                                                                    {2 * n, 2.0 * sms, 2 * n <= sms ? 0.14 : 0.2},           // two per SM
+                                                                    {4 * n, (double)sms, 0.088}};
     int best = 0;
-    for (int i = 1; i < 4; ++i)
-        if (t[i] < t[best]) best = i;
+    double best_us = two_passes;
+    for (int i = 1; i < 4; ++i) {
+        const double us = ceil(form[i].ctas / form[i].at_once) * C * form[i].us_per_token;
+        if (us < best_us) { best = i; best_us = us; }
+    }
+    if (best > 0) {
+        const double budget = (two_passes - kGroupUs) / form[best].us_per_token;                 // tokens one after the other
+        const double all_longest = budget / ceil(form[best].ctas / form[best].at_once);
+        const double spread = budget - form[best].ctas * C / form[best].at_once;
+        *longest = (int64_t)(all_longest > spread ? all_longest : spread);
+        if (d->num_requests > 1 && (double)*longest < C) best = 0;
+    }
     return best;
 }
 
@@ -553,8 +574,58 @@ extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const
         if (w.n_bh * 64 > 0x7fffffffll || desc->total_tokens > 0x7fffffffll) return WPP_ERR_UNSUPPORTED;
     }
     // (layout 3 is always the two passes: their result does not depend on how long the rest of the chunk is)
-    const int form = tensor_form && desc->layout == 0 ? kda_chunk_form(desc, ctx->sm_count) : 0;
-    if (tensor_form && form == 0) {
+    int64_t longest = 0;
+    const int form = tensor_form && desc->layout == 0 ? kda_chunk_form(desc, ctx->sm_count, &longest) : 0;
+    // a single chunk's length is known here: nothing has to stand behind the group form
+    const bool gated = form > 0 && desc->num_requests > 1;
+    int e;
+    if (!tensor_form || form > 0) {
+        wpp::KdaGroupParams p;
+        memset(&p, 0, sizeof(p));
+        p.q = static_cast<const __nv_bfloat16*>(q);
+        p.k = static_cast<const __nv_bfloat16*>(k);
+        p.v = static_cast<const __nv_bfloat16*>(v);
+        p.alpha = alpha;
+        p.beta = beta;
+        p.row_offsets = row_offsets;
+        p.prefix_lens = prefix_lens;
+        p.state_pool = state_pool;
+        p.state_in = state_in;
+        p.state_out = state_out;
+        p.snap_slots = desc->max_snaps > 0 ? snap_slots : nullptr;
+        p.out = static_cast<__nv_bfloat16*>(out);
+        p.status = status_dev;
+        p.num_requests = desc->num_requests;
+        p.num_heads = desc->num_heads;
+        p.num_slots = desc->num_slots;
+        p.snap_interval = desc->snap_interval;
+        p.max_snaps = desc->max_snaps;
+        if (tensor_form) {
+            p.longest = longest;
+            p.blk_off = gated ? reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + w.off_blk) : nullptr;
+            CUtensorMap maps[4];
+            memset(maps, 0, sizeof(maps));
+            int rc;
+            if (desc->total_tokens > 0) {
+                // boxes of the 16 rows of a group: whole rows of q, k and alpha (fp32 as a bf16 map with twice the elements:
+                // the copies move bytes), 64-column swizzled halves of v
+                const uint64_t H = (uint64_t)desc->num_heads, T = (uint64_t)desc->total_tokens;
+                const uint64_t dims[3] = {128, H, T}, dims_a[3] = {256, H, T};
+                const uint64_t strides[2] = {256, 256 * H}, strides_a[2] = {512, 512 * H};
+                const uint32_t box[3] = {128, 1, 16}, box_v[3] = {64, 1, 16}, box_a[3] = {256, 1, 16};
+                if ((rc = make_map(ctx, &maps[0], q, 3, dims, strides, box, false)) != WPP_OK) return rc;
+                if ((rc = make_map(ctx, &maps[1], k, 3, dims, strides, box, false)) != WPP_OK) return rc;
+                if ((rc = make_map(ctx, &maps[2], v, 3, dims, strides, box_v)) != WPP_OK) return rc;
+                if ((rc = make_map(ctx, &maps[3], alpha, 3, dims_a, strides_a, box_a, false)) != WPP_OK) return rc;
+            }
+            e = wpp_launch_kda_group(&p, maps, form, cuda_stream);
+        } else {
+            e = wpp_launch_kda(&p, ctx->sm_count, desc->layout, cuda_stream);
+        }
+        if (e != 0) return cuda_fail(ctx, e);
+        const_cast<wpp_ctx*>(ctx)->launches += 1;
+    }
+    if (tensor_form && (form == 0 || gated)) {
         char* ws = static_cast<char*>(workspace);
         wpp::KdaTcParams p;
         memset(&p, 0, sizeof(p));
@@ -618,57 +689,15 @@ extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const
             const uint64_t strides[2] = {512, 512 * H};
             if ((rc = make_map(ctx, &maps[12], alpha, 3, dims, strides, box)) != WPP_OK) return rc;
         }
-        // few long chains leave most SMs to the next segment's preparation
+        // few long chains leave most SMs to the next segment's preparation (not behind the group form: each segment is two
+        // launches that usually have nothing to do)
+        p.gated = gated;
         int32_t seg_begin[kMaxSegments] = {0};
-        const int segments = kda_segments(desc, ctx->sm_count, nullptr, seg_begin);
-        int e = wpp_launch_kda_tc(&p, maps, desc->total_tokens > 0 ? (int)w.max_blocks : 0, ctx->sm_count, segments, seg_begin,
-                                  cuda_stream);
+        const int segments = gated ? 1 : kda_segments(desc, ctx->sm_count, nullptr, seg_begin);
+        e = wpp_launch_kda_tc(&p, maps, desc->total_tokens > 0 ? (int)w.max_blocks : 0, ctx->sm_count, segments, seg_begin,
+                              cuda_stream);
         if (e != 0) return cuda_fail(ctx, e);
-        const_cast<wpp_ctx*>(ctx)->launches += 1 + 2 * segments;
-        return WPP_OK;
+        const_cast<wpp_ctx*>(ctx)->launches += (gated ? 0 : 1) + 2 * segments;
     }
-    wpp::KdaParams p;
-    memset(&p, 0, sizeof(p));
-    p.q = static_cast<const __nv_bfloat16*>(q);
-    p.k = static_cast<const __nv_bfloat16*>(k);
-    p.v = static_cast<const __nv_bfloat16*>(v);
-    p.alpha = alpha;
-    p.beta = beta;
-    p.row_offsets = row_offsets;
-    p.prefix_lens = prefix_lens;
-    p.state_pool = state_pool;
-    p.state_in = state_in;
-    p.state_out = state_out;
-    p.snap_slots = desc->max_snaps > 0 ? snap_slots : nullptr;
-    p.out = static_cast<__nv_bfloat16*>(out);
-    p.status = status_dev;
-    p.num_requests = desc->num_requests;
-    p.num_heads = desc->num_heads;
-    p.num_slots = desc->num_slots;
-    p.snap_interval = desc->snap_interval;
-    p.max_snaps = desc->max_snaps;
-    int e;
-    if (tensor_form) {
-        CUtensorMap maps[4];
-        memset(maps, 0, sizeof(maps));
-        int rc;
-        if (desc->total_tokens > 0) {
-            // boxes of the 16 rows of a group: whole rows of q, k and alpha (fp32 as a bf16 map with twice the elements:
-            // the copies move bytes), 64-column swizzled halves of v
-            const uint64_t H = (uint64_t)desc->num_heads, T = (uint64_t)desc->total_tokens;
-            const uint64_t dims[3] = {128, H, T}, dims_a[3] = {256, H, T};
-            const uint64_t strides[2] = {256, 256 * H}, strides_a[2] = {512, 512 * H};
-            const uint32_t box[3] = {128, 1, 16}, box_v[3] = {64, 1, 16}, box_a[3] = {256, 1, 16};
-            if ((rc = make_map(ctx, &maps[0], q, 3, dims, strides, box, false)) != WPP_OK) return rc;
-            if ((rc = make_map(ctx, &maps[1], k, 3, dims, strides, box, false)) != WPP_OK) return rc;
-            if ((rc = make_map(ctx, &maps[2], v, 3, dims, strides, box_v)) != WPP_OK) return rc;
-            if ((rc = make_map(ctx, &maps[3], alpha, 3, dims_a, strides_a, box_a, false)) != WPP_OK) return rc;
-        }
-        e = wpp_launch_kda_group(&p, maps, form, cuda_stream);
-    } else {
-        e = wpp_launch_kda(&p, ctx->sm_count, desc->layout, cuda_stream);
-    }
-    if (e != 0) return cuda_fail(ctx, e);
-    const_cast<wpp_ctx*>(ctx)->launches += 1;
     return WPP_OK;
 }

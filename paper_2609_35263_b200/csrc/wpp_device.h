@@ -81,6 +81,12 @@ struct KdaParams {
 
 // Chunk-parallel (tensor-core) form of the recurrent layer: the inputs of KdaParams plus the workspace arrays the
 // preparation kernel fills for the chain kernel.  bh = (global block index) * num_heads + head.
+struct KdaGroupParams : KdaParams {
+    int64_t longest;                // longest chunk this form takes; a wave with a longer one is left to the two passes behind it
+    int32_t* blk_off;               // [R+1] for the two passes: their block offsets, or blk_off[0] = -1 if there is nothing left
+                                    // for them; null: nothing is behind, the wave is this form's whatever its lengths
+};
+
 struct KdaTcParams {
     const __nv_bfloat16* q;
     const __nv_bfloat16* k;
@@ -98,6 +104,7 @@ struct KdaTcParams {
     int32_t num_requests, num_heads, num_slots, snap_interval, max_snaps;
     int32_t seg_lo, seg_hi;         // blocks [seg_lo, seg_hi) of every request belong to this launch
     int32_t beside;                 // preparation: launched beside the chain of the segment before
+    int32_t gated;                  // behind the group form: nothing to do if that did the wave (blk_off[0] < 0)
     int32_t* blk_off;               // [R+1] exclusive scan of the requests' block counts
     unsigned long long* ws_mask;    // [bh] bit t: token t of the block starts a sub-block
     float* ws_e;                    // [bh][64][128] decay product at a sub-block's last token (other rows unused)
@@ -119,7 +126,7 @@ int wpp_launch_attention_small(int head_dim, const CUtensorMap* tq, const CUtens
 int wpp_launch_append(const wpp::AppendParams* p, int num_sms, void* stream);
 int wpp_launch_combine(const wpp::CombineParams* p, int num_combine, void* stream);
 // maps: q, k, v, alpha; form: 1, 2, 3 = CTAs of 128, 64, 32 columns of the state
-int wpp_launch_kda_group(const wpp::KdaParams* p, const CUtensorMap* maps, int form, void* stream);
+int wpp_launch_kda_group(const wpp::KdaGroupParams* p, const CUtensorMap* maps, int form, void* stream);
 int wpp_launch_kda(const wpp::KdaParams* p, int num_sms, int layout, void* stream);
 int wpp_launch_selftest_wait(long long limit_cycles, int32_t* status, long long* waited_cycles, void* stream);
 }

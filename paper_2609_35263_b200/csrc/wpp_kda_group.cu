@@ -18,7 +18,7 @@
 // state in tensor memory a step is a chain of hand-overs between the issuing thread, the tensor pipe and the warps that
 // scale, split and store, and its operands need a pass of their own in front (14.5 K clocks of an SM per 64 tokens, 144 KB
 // written and read back).  Here a group's chain stays inside a warp: 21 K clocks of an SM per 64 tokens in all, no second
-// pass.  8 x 2,048 tokens, 32 heads: 740 -> 676 us; 8 x 64: 56 -> 41 us; 1 x 512: 68 -> 57 us (the choice: kda_chunk_form).
+// pass.  8 x 2,048 tokens, 32 heads: 744 -> 669 us; 8 x 64: 58 -> 42 us; 1 x 512: 71 -> 56 us (the choice: kda_chunk_form).
 // What bounds a group (clocks, 5.3 K before the third terms below): the products 3.4 K of which the MMA pipe is busy 2.6 K,
 // U 0.4 K, hand-over and outputs 1.2 K; the producers are idle half the time.  Also tried: four column warps of 32 columns with 216 registers
 // (809 us: one warp per scheduler waits), one producer warpgroup (660), a thirteenth warp for T and the copies (711: four
@@ -42,6 +42,7 @@
 
 #include "../../include/wpp.h"
 #include "wpp_device.h"
+#include "wpp_kda_blocks.cuh"
 #include "wpp_ptx.cuh"
 
 namespace wpp {
@@ -187,7 +188,7 @@ struct Smem {
 __host__ __device__ constexpr int col_warps(int slice, int mt, int ks) { return slice / 16 / mt * ks; }
 template <int kSlice, int kMT, int kKS, int kP, int kMinCtas>
 __global__ void __launch_bounds__(32 * col_warps(kSlice, kMT, kKS) + 128 * kP, kMinCtas)
-kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
+kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
     constexpr int kNC = col_warps(kSlice, kMT, kKS);
     static_assert(kNC % 4 == 0 && (kKS == 1 || (kKS == 2 && kMT == 1 && kNC == 4)), "whole warpgroups of column warps");
     constexpr int kVH = kSlice == kD ? 2 : 1;
@@ -206,6 +207,19 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
     auto bEmpty = [&](int w, int s) { return bFull(w, SM::kStages + s); };
     auto bRaw = [&](int w, int s) { return bFull(w, 2 * SM::kStages + s); };
     auto stage_off = [&](int w, int s) { return SM::kOffStage + (w * SM::kStages + s) * Stage::kBytes; };
+
+    // A wave lasts as long as its longest chain, and only the device knows the lengths: every CTA looks at all of them and
+    // comes to the same answer.
+    if (p.blk_off) {
+        bool longer = false;
+        for (int i = tid; i < p.num_requests; i += blockDim.x) longer |= p.row_offsets[i + 1] - p.row_offsets[i] > p.longest;
+        const bool first_cta = blockIdx.x == 0 && blockIdx.y == 0;
+        if (__syncthreads_or(longer)) {
+            if (first_cta) scan_block_offsets(p, reinterpret_cast<int*>(sm));
+            return;
+        }
+        if (first_cta && tid == 0) p.blk_off[0] = -1;
+    }
 
     const int64_t row0 = p.row_offsets[req];
     const int C = (int)(p.row_offsets[req + 1] - row0);
@@ -834,7 +848,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaParams p) {
 }
 
 template <int kSlice, int kMT, int kKS, int kP, int kMinCtas>
-static int launch(const Maps& maps, const KdaParams& p, cudaStream_t st) {
+static int launch(const Maps& maps, const KdaGroupParams& p, cudaStream_t st) {
     auto kernel = kda_group_kernel<kSlice, kMT, kKS, kP, kMinCtas>;
     constexpr int kNC = col_warps(kSlice, kMT, kKS), smem = Smem<kP, (kSlice == kD ? 2 : 1), kNC, kKS>::kBytes;
     static bool attr_set[64] = {};
@@ -858,7 +872,7 @@ static int launch(const Maps& maps, const KdaParams& p, cudaStream_t st) {
 //         made once per chain; for waves with enough (request, head) pairs to fill the SMs.
 // form 2: 64 columns (four column warps, one producer warpgroup, two CTAs per SM).
 // form 3: 32 columns, the channels halved between paired warps: the shortest chain per group, for a few long chains.
-extern "C" int wpp_launch_kda_group(const wpp::KdaParams* p, const CUtensorMap* maps, int form, void* stream) {
+extern "C" int wpp_launch_kda_group(const wpp::KdaGroupParams* p, const CUtensorMap* maps, int form, void* stream) {
     using namespace wpp::kdag;
     Maps m;
     m.q = maps[0]; m.k = maps[1]; m.v = maps[2]; m.alpha = maps[3];

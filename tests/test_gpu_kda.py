@@ -403,3 +403,60 @@ def test_groups_of_sixteen_positions_are_no_further_from_64_bits_than_the_two_pa
         err.append(np.sqrt(np.mean((pool[w.state_out][:, heads] - ref_pool[w.state_out]) ** 2)))
     assert not np.array_equal(pools[0], pools[1])
     assert err[0] <= err[1], err
+
+
+@pytest.mark.parametrize("H_", [1, 7, 17, 30])       # 6 requests: CTAs of 32 columns, of 64, of 128, and two rounds of them
+@pytest.mark.parametrize("interval,decays", [(0, False), (7, True), (64, False), (1000, True)])
+def test_the_group_form_matches_the_oracle_and_is_the_one_that_ran(H_, interval, decays):
+    """Chunks around the group size and up to nine groups, none so long that the wave is left to the two passes: outputs and
+    states against the oracle, and states whose last bits are not those of the two passes."""
+    lens, prefix = [0, 17, 130, 144, 100, 128], [5, 16, 31, 0, 4097, 63]
+    w = W.kda_workload("group form", 80 + H_, lens, H_, prefix, resume=[True, False, True, False, True, True], snap_interval=interval)
+    t = w.tensors()
+    if decays:
+        rng = np.random.default_rng(H_)
+        a = t["alpha"].numpy()
+        for val, count in ((0.0, 6), (1e-9, 6), (1e-30, 4), (0.2, 200)):
+            a[rng.integers(0, a.shape[0], count), rng.integers(0, H_, count), rng.integers(0, 128, count)] = val
+    got_o, got_pool, status = _gpu(w, t)
+    _, two_passes, _ = _gpu(w, t, layout=3)
+    assert status == 0 and not np.array_equal(got_pool, two_passes)
+    heads = [0, H_ - 1]
+    ref_o, ref_pool = _oracle(w, t, heads=heads)
+    _close_out(got_o[:, heads], ref_o, "outputs")
+    _close_state(got_pool[:, heads], ref_pool, "state pool")
+
+
+@pytest.mark.parametrize("H_", [9, 17, 33])                             # CTAs of 32, 64 and 128 columns
+@pytest.mark.parametrize("lens,two_passes", [([192] * 4, False), ([1500, 64, 64, 64], True), ([64, 64, 64, 1500], True), ([2000, 0, 0, 0], True)])
+def test_a_wave_of_one_long_chunk_is_left_to_the_two_passes(H_, lens, two_passes):
+    """The library's choice sees the lengths on the device: a wave much longer than its mean takes the form whose chain is
+    the faster one per token (the same bits as when it is asked for), equal chunks take the groups (other bits)."""
+    w = W.kda_workload("unequal", 41, lens, H_, [0, 100, 64, 7], snap_interval=100)
+    t = w.tensors()
+    got_o, got_pool, status = _gpu(w, t)
+    ref_o, ref_pool, _ = _gpu(w, t, layout=3)
+    assert status == 0
+    assert np.array_equal(got_pool, ref_pool) == two_passes
+    assert np.array_equal(got_o, ref_o) or not two_passes
+    _close_state(got_pool, ref_pool, "state pool")
+
+
+@pytest.mark.parametrize("H_", [9, 17, 33])                             # CTAs of 32, 64 and 128 columns
+def test_the_group_form_is_bit_identical_when_chunks_are_cut_at_a_multiple_of_sixteen(H_):
+    """256 tokens a request in one call, and 112 and then 144: both take the groups in CTAs of the same width, and groups are
+    blocks of absolute positions, so outputs and states have the same bits."""
+    whole = W.kda_workload("whole", 37, [256] * 4, H_, [0, 16, 64, 160])
+    t = whole.tensors()
+    want_o, want_pool, status = _gpu(whole, t)
+    assert status == 0 and not np.array_equal(_gpu(whole, t, layout=3)[1], want_pool)
+    pool, got_o = t["state_pool"], np.zeros_like(want_o)
+    for lo, hi, s_in in ((0, 112, whole.state_in), (112, 256, whole.state_out)):
+        rows = np.concatenate([np.arange(r + lo, r + hi) for r in whole.row_offsets[:-1]])
+        part = W.kda_workload("part", 37, [hi - lo] * 4, H_, [int(x) + lo for x in whole.prefix_lens])
+        part.num_slots = whole.num_slots
+        o, pool_, status = _gpu(part, {k: (v[rows].contiguous() if k != "state_pool" else pool) for k, v in t.items()},
+                                state_in=s_in, state_out=whole.state_out)
+        assert status == 0
+        got_o[rows], pool = o, torch.from_numpy(pool_).float()
+    assert np.array_equal(got_o, want_o) and np.array_equal(pool.double().numpy(), want_pool)
