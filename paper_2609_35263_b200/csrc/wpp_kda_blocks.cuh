@@ -25,9 +25,10 @@ __device__ __forceinline__ ReqBlocks req_blocks(const Params& p, int req) {
 }
 
 // Exclusive scan of the requests' block counts to p.blk_off [R + 1], by one whole CTA; `part`: an int per thread in shared memory.
-template <class Params>
+template <int kThreads, class Params>
 __device__ __forceinline__ void scan_block_offsets(const Params& p, int* part) {
-    const int R = p.num_requests, tid = threadIdx.x, n = blockDim.x;
+    constexpr int n = kThreads;
+    const int R = p.num_requests, tid = threadIdx.x;
     const int per = (R + n - 1) / n;
     const int i0 = min(R, tid * per), i1 = min(R, i0 + per);
     int sum = 0;

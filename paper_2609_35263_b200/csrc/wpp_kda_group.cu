@@ -215,7 +215,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
         for (int i = tid; i < p.num_requests; i += blockDim.x) longer |= p.row_offsets[i + 1] - p.row_offsets[i] > p.longest;
         const bool first_cta = blockIdx.x == 0 && blockIdx.y == 0;
         if (__syncthreads_or(longer)) {
-            if (first_cta) scan_block_offsets(p, reinterpret_cast<int*>(sm));
+            if (first_cta) scan_block_offsets<32 * kNC + 128 * kP>(p, reinterpret_cast<int*>(sm));
             return;
         }
         if (first_cta && tid == 0) p.blk_off[0] = -1;

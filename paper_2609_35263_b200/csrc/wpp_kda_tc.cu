@@ -85,7 +85,7 @@ __device__ __forceinline__ int sub_end(uint64_t mask, int t, int hi) {     // ex
 // Set-up: exclusive scan of the requests' block counts (one CTA).
 __global__ void __launch_bounds__(1024) kda_tc_setup_kernel(const KdaTcParams p) {
     __shared__ int part[1024];
-    scan_block_offsets(p, part);
+    scan_block_offsets<1024>(p, part);
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -172,6 +172,8 @@ __device__ __forceinline__ PrepItem prep_item(const KdaTcParams& p, int item) {
     return it;
 }
 
+// kGated: behind the group form
+template <bool kGated>
 __global__ void __launch_bounds__(kPrepThreads, 2)
 kda_tc_prep_kernel(const __grid_constant__ PrepMaps maps, const KdaTcParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -201,7 +203,7 @@ kda_tc_prep_kernel(const __grid_constant__ PrepMaps maps, const KdaTcParams p) {
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int H = p.num_heads;
-    if (p.gated && p.blk_off[0] < 0) return;               // the group form has done the wave
+    if (kGated && p.blk_off[0] < 0) return;                // the group form has done the wave
     int n_items = p.blk_off[p.num_requests] * H;
     if (p.seg_hi != 0x7fffffff || p.seg_lo != 0) {
         n_items = 0;
@@ -828,6 +830,8 @@ struct ChainSmem {
 constexpr uint32_t kColS = 0, kColShl = 128, kColD = 256;
 __device__ __forceinline__ uint32_t col_d(int step) { return kColD + 128u * (uint32_t)(step & 1); }
 
+// kGated: behind the group form
+template <bool kGated>
 __global__ void __launch_bounds__(352, 1)
 kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_constant__ CUtensorMap tm_w0_l,
                     const __grid_constant__ CUtensorMap tm_qt_h, const __grid_constant__ CUtensorMap tm_qt_l,
@@ -862,7 +866,7 @@ kda_tc_chain_kernel(const __grid_constant__ CUtensorMap tm_w0_h, const __grid_co
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int head = blockIdx.x, req = blockIdx.y, H = p.num_heads;
-    if (p.gated) {
+    if constexpr (kGated) {
         grid_dependency_wait();
         if (p.blk_off[0] < 0) return;                      // the group form has done the wave
     }
@@ -1277,9 +1281,13 @@ extern "C" int wpp_launch_kda_tc(const wpp::KdaTcParams* params, const CUtensorM
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(kda_tc_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PrepSmem::kBytes);
+        cudaError_t e = cudaFuncSetAttribute(kda_tc_prep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PrepSmem::kBytes);
         if (e != cudaSuccess) return (int)e;
-        e = cudaFuncSetAttribute(kda_tc_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainSmem::kBytes);
+        e = cudaFuncSetAttribute(kda_tc_prep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PrepSmem::kBytes);
+        if (e != cudaSuccess) return (int)e;
+        e = cudaFuncSetAttribute(kda_tc_chain_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainSmem::kBytes);
+        if (e != cudaSuccess) return (int)e;
+        e = cudaFuncSetAttribute(kda_tc_chain_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainSmem::kBytes);
         if (e != cudaSuccess) return (int)e;
         attr_set[dev] = true;
     }
@@ -1311,7 +1319,7 @@ extern "C" int wpp_launch_kda_tc(const wpp::KdaTcParams* params, const CUtensorM
             cfg.stream = st;
             cfg.attrs = &overlap;
             cfg.numAttrs = s > 0 ? 1 : 0;
-            cudaError_t e = cudaLaunchKernelEx(&cfg, kda_tc_prep_kernel, pm, p);
+            cudaError_t e = cudaLaunchKernelEx(&cfg, p.gated ? kda_tc_prep_kernel<true> : kda_tc_prep_kernel<false>, pm, p);
             if (e != cudaSuccess) return (int)e;
         }
         cudaLaunchConfig_t cfg = {};
@@ -1321,7 +1329,7 @@ extern "C" int wpp_launch_kda_tc(const wpp::KdaTcParams* params, const CUtensorM
         cfg.stream = st;
         cfg.attrs = &overlap;
         cfg.numAttrs = p.gated ? 1 : 0;
-        cudaError_t e = cudaLaunchKernelEx(&cfg, kda_tc_chain_kernel, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], maps[6],
+        cudaError_t e = cudaLaunchKernelEx(&cfg, p.gated ? kda_tc_chain_kernel<true> : kda_tc_chain_kernel<false>, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], maps[6],
                                            maps[7], p);
         if (e != cudaSuccess) return (int)e;
     }
