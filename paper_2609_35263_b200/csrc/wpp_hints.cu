@@ -319,13 +319,14 @@ extern "C" int wpp_hash_blocks(const wpp_ctx* ctx, const int32_t* tokens, const 
     // an SM makes a block's digest in less than a chain step).  us, one kernel | two, both before the chain's step was
     // shortened for both: 64 requests x 3,125 blocks of 64 144 | 172, 64 x 100 11 | 15, 148 x 3,125 156 | 222; blocks of 128:
     // 1 x 1,500 90 | 72, 64 x 3,125 269 | 199.
-    if (num_requests <= 148 && block_size <= 64) {
+    const int sms = wpp_ctx_sm_count(ctx);
+    if (num_requests <= sms && block_size <= 64) {
         wpp_hash_fused_kernel<<<(unsigned)num_requests, kFusedThreads, 0, st>>>(tokens, token_offsets, block_offsets, block_size,
                                                                                salt_term, extra, hashes_out);
         return cudaGetLastError() == cudaSuccess ? WPP_OK : WPP_ERR_CUDA;
     }
     // eight blocks per warp once that still gives every SM 32 warps; one below, where a warp's latency is all that counts
-    const bool wide = total_blocks >= 8ll * 32 * 148;
+    const bool wide = total_blocks >= 8ll * 32 * sms;
     const int64_t ctas = (total_blocks + (wide ? 63 : 7)) / (wide ? 64 : 8);
     if (ctas > 0x7fffffffll) return WPP_ERR_INVALID_ARG;
     if (wide)
