@@ -523,8 +523,8 @@ def run_kda(args):
     """The recurrent-state (KDA) layer of one wave (Section 3.1 update, Section 3.2 snapshots): `--kda-lanes`
     requests of `--kda-chunk` tokens, 32 state heads of 128 x 128, every request resuming from a snapshot and
     storing one at the chunk end.  Timed with CUDA events over back-to-back launches on inputs larger than L2;
-    the library's choice (--kda-layout 0) is the chunk-parallel tensor-core form, bounded by the algorithmic bytes at
-    HBM bandwidth; the token-by-token forms (--kda-layout 1, 2) are plain fp32 arithmetic: 7 flop per state element
+    the library's choice (--kda-layout 0) is one of the two chunk-parallel tensor-core forms, bounded by the algorithmic bytes
+    at HBM bandwidth; the token-by-token forms (--kda-layout 1, 2) are plain fp32 arithmetic: 7 flop per state element
     and token against 148 SMs x 128 lanes x 2 flop x the maximum SM clock."""
     if int(os.environ.get("RANK", "0")) != 0:
         return
@@ -553,10 +553,12 @@ def run_kda(args):
     sampler = ClockSampler(0)
     sampler.start()
     a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    launches = ctx.launch_count()
     a.record()
     for _ in range(steps):
         step()
     b.record()
+    launches = ctx.launch_count() - launches
     torch.cuda.synchronize()
     clocks = sampler.stop()
     ms = a.elapsed_time(b) / steps
@@ -608,10 +610,11 @@ def run_kda(args):
     line = {"metric": "recurrent-state (KDA) layer, new tokens/s through one layer", "value": T / (ms * 1e-3),
             "unit": "tokens/s", "n_gpus": 1, "steps": steps, "warmup": warm, "ms_per_step": ms, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "bf16 x 2 terms, fp32 accumulate" if tensor_form else "f32",
-            "data": "synthetic", "gpu_launches": steps * (3 if args.kda_layout == 3 else 1),      # (layout 0: at least)
+            "data": "synthetic", "gpu_launches": int(launches),
             "config": {"workload": w.name, "requests": int(w.chunk_lens.size), "chunk": int(w.chunk_lens[0]),
                        "state_heads": Hh, "d_k": w.d_k, "d_v": w.d_v, "layout": args.kda_layout,
-                       "form": "chunk-parallel on tensor cores" if tensor_form else "token by token on CUDA cores",
+                       "form": "token by token on CUDA cores" if not tensor_form else "chunk-parallel in two passes on tensor cores"
+                               if args.kda_layout == 3 else "the library's choice: groups of 16 tokens or two passes, on tensor cores",
                        "l2": "inputs larger than L2"},
             "clocks": clocks, "roofline": roofline,
             "cpu_baseline": {"value": (sl.stop - sl.start) / t_cpu / Hh, "unit": "tokens/s", "cores": 1, "kind": "oracle",
