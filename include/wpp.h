@@ -22,6 +22,8 @@
  *     `cuda_stream` (a cudaStream_t passed as void*) has completed.
  *   - bf16 tensors are passed as void*; inner (head_dim) elements are contiguous and
  *     every row start and stride must be a multiple of 16 bytes.
+ *   - Calls may be captured in a CUDA graph.  A captured call keeps what its plan_host said (counts, cut, kernel shape): replay
+ *     it with that plan's bytes in plan_dev; for another plan, capture again.
  *   - Problems the host can see are reported before anything is launched.  Problems
  *     only the device can see (a page id outside [0, num_pages), a bounded wait that
  *     ran out, lengths on the device that differ from the plan's) set *status_dev (first error wins, never cleared by the library), the
@@ -103,9 +105,10 @@ typedef struct {
     int32_t tile_m;           /* query rows per work tile: 128 or 256 (default 256: two 128-row halves) */
     int32_t tile_n;           /* keys per inner step: 128 */
     int32_t force_kv_splits;  /* >= 2: split every tile's key range into this many parts (when it has that many
-                                 key steps); 1: never split; 0: library decides (all tiles when there are fewer of
-                                 them than CTAs; the tiles of a partly filled last round when the tiles are long and
-                                 the rounds few; wpp_plan_info.workspace_bytes says what the partials need) */
+                                 key steps); 1: never split; 0: library decides (fewer tiles than CTAs: by estimated
+                                 time over tile heights, part lengths and kernel shapes, whole tiles among them; else the
+                                 tiles of a partly filled last round when the tiles are long and the rounds few;
+                                 wpp_plan_info.workspace_bytes says what the partials need) */
     int32_t max_ctas;         /* persistent CTAs to launch (default: SM count of the context, 148 without one) */
     int32_t order;            /* order in which the persistent CTAs take the tiles at run time.  0: stream order -
                                  tiles that read the same (request, KV head) pages are neighbours and so run at the
@@ -243,7 +246,8 @@ int wpp_selftest_bounded_wait(const wpp_ctx* ctx, int64_t limit_cycles, int32_t*
 /* Number of kernels the library has launched through this context so far (for launch accounting). */
 int64_t wpp_launch_count(const wpp_ctx* ctx);
 
-/* The attention kernel keeps a reference per query row for its exponentials and rescales the row's accumulator when
+/* The SM-wide attention kernel (wpp_plan_opts.shape 1; the small one rescales before, whatever the mode, and counts nothing)
+ * keeps a reference per query row for its exponentials and rescales the row's accumulator when
  * the reference has to move.  It exists in two orders of work: rescale before the step's exponentials (best when
  * references move now and then: every workload whose scores do not keep growing along the sequence) or after them
  * (best when most steps move a reference).  Both are within the tolerance; they differ in rounding order.
@@ -334,7 +338,7 @@ int wpp_plan_waves(const wpp_wave_config* cfg, wpp_wave_state* state, const int6
  *   digest_i = sum_k term_k (mod 2^64)
  *   H_i = mix64(H_{i-1} xor mix64(digest_i + extraKeys_i) xor (salt * 0x9E3779B97F4A7C15)). */
 
-/* Chained block hashes of a batch of requests, on the GPU (two small kernels on `cuda_stream`).
+/* Chained block hashes of a batch of requests, on the GPU (one or two small kernels on `cuda_stream`).
  *   tokens        : device int32 [token_offsets[R]], the requests' token ids back to back.
  *   token_offsets : device int64 [R+1], start of each request in `tokens`.
  *   block_offsets : device int64 [R+1], exclusive scan of floor(n_i / block_size): where each request's hashes go.
@@ -384,11 +388,12 @@ int wpp_hint_probe_recurrent(const wpp_hint_index* idx, int32_t window, const ui
  * with S (d_k x d_v, fp32) resumed from the state after exactly the reused prefix - a recurrent layer cannot
  * resume from anything else - and written back at the chunk end and, optionally, at sparse periodic boundaries.
  * Heads are independent.  No normalisation or scaling of q or k is applied here (the update has none).
- * Two forms compute it.  The chunk-parallel form (layout 3) works on blocks of 64 sequence positions: per block the
- * products Kt Kh^T, Qt Kh^T (Kt, Kh, Qt: keys and queries scaled by the decay products inside the block), Kt S_0,
+ * Three forms compute it.  The chunk-parallel form in two passes (layout 3) works on blocks of 64 sequence positions: per
+ * block the products Kt Kh^T, Qt Kh^T (Kt, Kh, Qt: keys and queries scaled by the decay products inside the block), Kt S_0,
  * T (V - Kt S_0), Qt S_0, tril(Qt Kh^T) U and Kb^T U run on the tensor cores with the fp32 state in tensor memory;
  * every operand is split into two bf16 terms (16 significant bits, three MMAs per product), accumulation is fp32.
- * It needs a workspace (wpp_kda_workspace_bytes).  The token-by-token forms (layouts 1, 2) use fp32 fused
+ * It needs a workspace (wpp_kda_workspace_bytes).  The same algebra over groups of 16 positions with the state in registers is
+ * one of the library's choices (layout 0).  The token-by-token forms (layouts 1, 2) use fp32 fused
  * multiply-adds on CUDA cores in token order and need no workspace.  Outputs are rounded to bf16, states stay fp32. */
 typedef struct {
     int32_t num_requests;   /* R >= 0 */
@@ -399,9 +404,11 @@ typedef struct {
     int32_t snap_interval;  /* > 0: snapshot whenever the tokens folded into S reach a multiple of it; 0: none */
     int32_t max_snaps;      /* row length of snap_slots (0 when snap_interval is 0) */
     int32_t layout;         /* 0: the library chooses (when a large enough workspace is given and the wave has at least
-                             * 64 tokens per request on average, the chunk-parallel form or the same arithmetic in
-                             * groups of 16 positions with the state in registers, whichever is estimated to be faster
-                             * for these sizes; else 1 or 2);
+                             * 64 tokens per request on average, the two passes or the groups of 16 positions, by
+                             * the estimated time for these sizes and, on the device, by the longest chunk; else 1
+                             * or 2).  A request's last bits then depend on the wave it is in; with a layout named
+                             * they do not, nor on cuts of its chunk (1, 2: anywhere; 3: at multiples of 64
+                             * positions);
                              * 1: token by token, one CTA per (request, head); 2: token by token, four CTAs per
                              * (request, head) of 32 columns each; 3: chunk-parallel on the tensor cores */
     int64_t total_tokens;   /* T = row_offsets[R] */
@@ -428,8 +435,10 @@ typedef struct {
  *                 and that request's state is neither read (zero state used) nor written there.
  * A request with an empty chunk copies state_in to state_out.  Returns WPP_ERR_INVALID_ARG for null or misaligned
  * pointers or negative sizes, WPP_ERR_UNSUPPORTED for d_k, d_v other than 128, WPP_ERR_WORKSPACE_TOO_SMALL when
- * layout 3 is asked for without enough workspace, WPP_ERR_CUDA for a launch failure.  The chunk-parallel form
- * of layout 3 enqueues three kernels (block offsets, per-block preparation, the chain over the blocks), the others one. */
+ * layout 3 is asked for without enough workspace, WPP_ERR_CUDA for a launch failure.  Layout 3 enqueues block offsets and,
+ * for one to six segments of the chunks, per-block preparation and the chain over the blocks; layouts 1 and 2 one kernel;
+ * layout 0 either, or the group kernel, with the two passes of one segment behind it when there are several requests (they end
+ * at once unless a chunk is too long for the groups). */
 int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const void* q, const void* k, const void* v,
                   const float* alpha, const float* beta, const int64_t* row_offsets, const int32_t* prefix_lens,
                   float* state_pool, const int32_t* state_in, const int32_t* state_out, const int32_t* snap_slots,
