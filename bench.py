@@ -786,7 +786,7 @@ def main():
     # the bound is the slower of FLOPs at the tensor peak and compulsory bytes at HBM bandwidth
     t_flops, t_bytes, kv_bytes, qo_bytes = roofline_times(w, flops, peaks)
     traffic = DRAM_BYTES_PER_KEY_STEP * float(info.key_steps)
-    roofline = {"bound": "tensor" if t_flops >= t_bytes else "hbm", "kernel": "wpp_attn_kernel",
+    roofline = {"bound": "tensor" if t_flops >= t_bytes else "hbm", "kernel": "wpp_attn_kernel" if info.shape == 1 else "wpp_attn_small_kernel",
                 "achieved": achieved, "peak": roof_peak, "unit": "TFLOP/s", "frac": achieved / roof_peak,
                 "peak_source": f"of {peak_kind} (burst bf16 matmul)", "frac_of_sustained": achieved / roof_sus,
                 "traffic": traffic, "traffic_source": DRAM_SOURCE, "compulsory_bytes": kv_bytes + qo_bytes,
