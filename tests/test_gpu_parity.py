@@ -436,3 +436,35 @@ def test_a_cut_tile_shows_the_infinities_and_nans_that_a_whole_one_shows(d, spli
         assert bad.any() and np.array_equal(bad, ~np.isfinite(b)) and np.array_equal(np.isnan(a), np.isnan(b)), what
         assert np.abs(a[~bad] - b[~bad]).max() <= H.MAX_ABS_TOL
         assert np.array_equal(np.isneginf(f64(whole["lse"])), np.isneginf(f64(cut["lse"])))
+
+
+@pytest.mark.parametrize("B,d,P,C,splits", [
+    (16, 128, [511, 512, 513, 1040, 2100, 0], [1, 64, 65, 130, 40, 300], 1),      # around one and two windows of 32 pages
+    (16, 64, [3000, 5, 1023], [17, 1200, 129], 3),                                # parts that start inside a window
+    (32, 64, [1023, 2049, 4100], [33, 7, 90], 1), (64, 128, [2047, 6200], [65, 3], 2), (128, 128, [4095, 8300, 64], [66, 5, 64], 5),
+])
+def test_small_shape_follows_the_block_table_32_pages_at_a_time(B, d, P, C, splits):
+    """Its producer holds the page ids of 32 pages at a time: prefixes on both sides of one and two of these windows, every page
+    size, parts whose first page is odd; the table's rows are exactly as long as the longest request needs."""
+    _full_parity(W.custom_workload(P, C, 4, 2, d, B, seed=B + d), opts=wpp.PlanOpts(0, 0, splits, 0), shapes=(2,))
+
+
+@pytest.mark.parametrize("pad", [0, 8, 24])
+def test_small_shape_stores_rows_on_16_byte_boundaries(pad):
+    """Output rows that do not start on 32-byte boundaries are stored in 16-byte pieces; nothing between the rows is written."""
+    w = W.custom_workload([40, 0], [70, 129], 4, 2, 64, 16, seed=71)
+    inp = cpu_inputs(w)
+    ref = H.run_wave(w, H.device_inputs(w, inp), shape=2)
+    g, dev, pitch = H.device_inputs(w, inp), torch.device("cuda"), 64 + pad
+    desc = wpp.make_desc(w.num_requests, 4, 2, 64, 16, w.max_blocks_per_req, w.num_pages, o_head_stride=pitch, o_token_stride=4 * pitch)
+    plan = wpp.wpp_plan_tiles(H.ctx(), desc, w.prefix_lens, w.chunk_lens, opts=wpp.PlanOpts(0, 0, 0, 0, 0, 2)).to_device()
+    i32 = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).to(dev)
+    bt, P, C, status = i32(w.block_tables), i32(w.prefix_lens), i32(w.chunk_lens), torch.zeros(1, dtype=torch.int32, device=dev)
+    out = torch.full((w.total_new_tokens, 4, pitch), 7.0, dtype=torch.bfloat16, device=dev)
+    ws = torch.empty(int(plan.info.workspace_bytes), dtype=torch.uint8, device=dev)
+    wpp.wpp_kv_append(H.ctx(), desc, g["k_new"], g["v_new"], g["k_pool"], g["v_pool"], bt, P, C, plan, status=status)
+    wpp.wpp_prefill_attention_varlen(H.ctx(), desc, g["q"], out, None, g["k_pool"], g["v_pool"], bt, P, C, plan, workspace=ws,
+                                     status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(out[..., :64], ref["out"]) and bool((out[..., 64:] == 7.0).all())
