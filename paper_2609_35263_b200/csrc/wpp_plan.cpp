@@ -87,15 +87,17 @@ constexpr int64_t kTileFixedCost = 3, kPartExtraCost = 2, kCombineCost = 20;
 // Estimated microseconds of a wave on either kernel shape: tiles (or halves) handed out in order to the CTA free first,
 // each with a start and end and a time per 128-key step.  Constants from waves timed on 148 SMs, attention call in us, SM-wide |
 // small (requests x new tokens over cached ones, 64/8 heads of 128):
-//     1 x 64            20 |   7        32 x 64           45 |  21        32 x 256       117 | 105
-//     1 x 64 / 2048     34 |  22        32 x 64 / 256     61 |  43        32 x 512       306 | 290
-//     1 x 512           26 |  17        32 x 64 / 1024    96 | 108        32 x 1024      845 | 930
-//     1 x 2048         106 | 147        32 x 1 / 1024     58 |  37        4 x 1024       107 | 126
-//     8 x 256           41 |  31        32 x 64 / 4096   280 | 407        8 x 512 / 4096 523 | 730
+//     32 x 64            44 |  21       32 x 300..1000       525 | 445      32 x 64 / 1024          102 | 117
+//     32 x 128           60 |  45       32 x 1024            781 | 789      32 x 256 / 1024         309 | 443
+//     32 x 256          117 |  97       16 x 2048           1199 | 1466     16 x 512 / 2048         556 | 878
+//     32 x 512          303 | 246       64 x 1..300 / 0..500  83 |  69      8 x 300 / 700            68 |  70
+// (the last two in the middle and on the right with 16/4 heads of 64 and 32/8 of 128).  The line lies where both are equal.  With
+// 3.3 and 3.0 us, the constants of one thread per query row, 32 x 300..1000 and 64 x 1..300 / 0..500 went to the SM-wide shape;
+// with one slope for all lengths 4 x 1407, 2 x 196..1950 and 7 x 1250..1751 went to the small one (pass, us, SM-wide | small:
+// 132 | 147, 69 | 86, 62 | 74; but 80 x 228 over 119..239 271 | 214, 12 x 210..393 over 127..212 132 | 108).
 // Where the small shape's items take several rounds and average more than kSmallShapeSteps key steps, its estimate is up to
 // 12 % short (the CTAs of an SM share the tensor pipe and L2) and the SM-wide one is taken: 32 x 4..34 new tokens, 40/8 heads
-// (one head per tile), over 512 / 900 / 1,100 / 1,500 / 4,096 cached ones 142 | 92, 171 | 130, 142 | 148, 169 | 184, 431 | 459;
-// over 256..3,635 ones 214 | 240; 64 x 4..16, 64/8 heads, over 0..1,024 / 0..2,048 72 | 62, 90 | 92 (pass, us).
+// (one head per tile), over 1,100 / 1,500 / 4,096 cached ones 142 | 148, 169 | 184, 431 | 459 (pass, us, one thread per row).
 constexpr int64_t kSmallShapeSteps = 8;
 struct StepCount {
     int64_t sum = 0;
@@ -106,17 +108,19 @@ struct StepCount {
         shortest = std::min(shortest, n);
     }
 };
-static double wave_us(const StepCount& s, int64_t n, int64_t slots, double fixed, double per_step) {
+// `more` us for each step beyond kShortSteps that the items of several rounds average
+constexpr double kShortSteps = 4.0;
+static double wave_us(const StepCount& s, int64_t n, int64_t slots, double fixed, double per_step, double more = 0.0) {
     const double longest = fixed + per_step * s.longest;
     if (n <= slots) return longest;
-    const double mean = fixed + per_step * (double)s.sum / (double)n;
+    const double steps = (double)s.sum / (double)n, mean = fixed + per_step * steps + more * std::max(0.0, steps - kShortSteps);
     return std::max(longest, mean * ((double)n / (double)slots + (n % slots ? 0.5 : 0.0)));    // a partly filled last round
 }
 static double wide_shape_us(const StepCount& units, int64_t n_units, int64_t nonempty_halves, int max_ctas) {
     return 10.0 + wave_us(units, n_units, max_ctas, 5.0, nonempty_halves > n_units ? 1.9 : 1.4);
 }
 static double small_shape_us(const StepCount& halves, int64_t n_items, int max_ctas) {
-    return 0.5 + wave_us(halves, n_items, 2 * (int64_t)max_ctas, 3.3, 3.0);
+    return 0.5 + wave_us(halves, n_items, 2 * (int64_t)max_ctas, 3.0, 2.75, 1.0);
 }
 
 // Few tiles are cut along the keys so that the CTAs have work: the part length, the tile height and the kernel shape are
