@@ -515,13 +515,32 @@ static int kda_segments(const wpp_kda_desc* d, int sms, double* us, int32_t* beg
 // token here as in the two passes.  The lengths are on the device: the group form's CTAs look at them, and a wave with a chunk
 // longer than *longest is left to the two passes queued behind (which end at once if it is not).  *longest is the length up
 // to which the group form is the faster one however the rest is distributed: no order of its CTAs takes longer than its rounds
-// all of the longest chunk, nor than the chunks spread evenly and the longest on top; the two passes are taken for equal chunks,
-// where they are fastest.  us, two passes | group form whatever the lengths | now:
+// all of the longest chunk, nor than the chunks spread evenly and the longest on top (where the chains are cut, half of its piece
+// on top, or it alone); the two passes are taken for equal chunks, where they are fastest.  us, two passes | group form whatever the lengths | now:
 //     8 x 32 heads, 14,000 and 7 x 340 tokens 1261 | 2108 | 1263     8 x 32, 8,192 and 7 x 1,170 960 | 1248 | 959
 //     9 x 8 heads, 16,000 and 8 x 48 tokens 1004 | 2055 | 1004        4 x 32, 512 and 3 x 64 85 | 92 | 83
 // The empty launches behind a wave of equal chunks: 8 x 2,048 669 -> 676, 4 x 256 56 -> 64, 8 x 64 42 -> 50, 64 x 256 652 -> 673.
 constexpr double kGroupUs = 12.0;       // what a launch takes before and after its chains
-static int kda_chunk_form(const wpp_kda_desc* d, int sms, int64_t* longest) {
+constexpr double kPieceUs = 8.0;        // what a piece of a chain takes besides its tokens
+constexpr int kMaxPieces = 8;
+// Pieces per chain of the 128-column CTAs, one CTA per SM: whole chains leave the last of few rounds partly empty (256 chains on
+// 148 SMs take two rounds of which the second is 73 % full).  A piece of a chain waits for the one before, which started a
+// whole round of chains earlier: only with at least as many chains as SMs.  Measured, us, in 1 / 2 / 4 / 5 / 8 pieces (32 heads):
+// 8 x 2,048 676 / 721 / 657 / 684 / 698, 8 x 1,024 354 / 383 / 361 / 379 / 403, 5 x 1,000 300 / 283 / 251 / 249 / 257,
+// 6 x 2,048 622 / 545 / 560 / 531 / 546 (3 pieces: 495), 64 x 256 697 / 828 / 1020: cut where it gives 3 % by this estimate.
+static int kda_pieces(double n, double C, int sms, double us_per_token, double* us) {
+    int best = 1;
+    double best_us = ceil(n / sms) * C * us_per_token;
+    const double whole = best_us + ceil(n / sms) * kPieceUs;
+    double least = 0.97 * whole;
+    for (int k = 2; k <= kMaxPieces && n >= sms && C >= 64.0 * k; ++k) {
+        const double t = ceil(n * k / sms) * (C / k * us_per_token + kPieceUs);
+        if (t < least) { best = k; least = t; best_us = t - ceil(n / sms) * kPieceUs; }
+    }
+    *us = best_us;
+    return best;
+}
+static int kda_chunk_form(const wpp_kda_desc* d, int sms, int64_t* longest, int* pieces) {
     const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
     double two_passes = 0.0;
     kda_segments(d, sms, &two_passes, nullptr);
@@ -532,14 +551,26 @@ static int kda_chunk_form(const wpp_kda_desc* d, int sms, int64_t* longest) {
                                                                     {4 * n, (double)sms, 0.088}};
     int best = 0;
     double best_us = two_passes;
+    double whole_us = 0.0;                  // form 1 with its chains cut
+    *pieces = kda_pieces(n, C, sms, form[1].us_per_token, &whole_us);
     for (int i = 1; i < 4; ++i) {
-        const double us = ceil(form[i].ctas / form[i].at_once) * C * form[i].us_per_token;
+        const double us = i == 1 ? whole_us : ceil(form[i].ctas / form[i].at_once) * C * form[i].us_per_token;
         if (us < best_us) { best = i; best_us = us; }
     }
     if (best > 0) {
-        const double budget = (two_passes - kGroupUs) / form[best].us_per_token;                 // tokens one after the other
-        const double all_longest = budget / ceil(form[best].ctas / form[best].at_once);
-        const double spread = budget - form[best].ctas * C / form[best].at_once;
+        const double per_token = form[best].us_per_token, budget = two_passes - kGroupUs;
+        double all_longest, spread;
+        if (best == 1 && *pieces > 1) {
+            // cut chains: the wave is done when the longest is, or when the SMs are through with everything and half a piece
+            const double k = *pieces, work = n * C / sms * per_token + ceil(n * k / sms) * kPieceUs;
+            all_longest = C * budget / whole_us;
+            spread = (budget - work) * 2.0 * k / per_token;
+            const double alone = (budget - k * kPieceUs) / per_token;
+            if (alone < spread) spread = alone;
+        } else {
+            all_longest = budget / per_token / ceil(form[best].ctas / form[best].at_once);
+            spread = budget / per_token - form[best].ctas * C / form[best].at_once;
+        }
         *longest = (int64_t)(all_longest > spread ? all_longest : spread);
         if (d->num_requests > 1 && (double)*longest < C) best = 0;
     }
@@ -575,7 +606,8 @@ extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const
     }
     // (layout 3 is always the two passes: their result does not depend on how long the rest of the chunk is)
     int64_t longest = 0;
-    const int form = tensor_form && desc->layout == 0 ? kda_chunk_form(desc, ctx->sm_count, &longest) : 0;
+    int pieces = 1;
+    const int form = tensor_form && desc->layout == 0 ? kda_chunk_form(desc, ctx->sm_count, &longest, &pieces) : 0;
     // a single chunk's length is known here: nothing has to stand behind the group form
     const bool gated = form > 0 && desc->num_requests > 1;
     int e;
@@ -602,6 +634,9 @@ extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const
         p.max_snaps = desc->max_snaps;
         if (tensor_form) {
             p.longest = longest;
+            p.pieces = form == 1 ? pieces : 1;
+            p.hand = reinterpret_cast<float4*>(static_cast<char*>(workspace) + w.off_e);              // (n_bh >= 2 R H rows of 32 KB)
+            p.hand_seen = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + w.off_u0);
             p.blk_off = gated ? reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + w.off_blk) : nullptr;
             CUtensorMap maps[4];
             memset(maps, 0, sizeof(maps));

@@ -19,6 +19,12 @@
 // scale, split and store, and its operands need a pass of their own in front (14.5 K clocks of an SM per 64 tokens, 144 KB
 // written and read back).  Here a group's chain stays inside a warp: 21 K clocks of an SM per 64 tokens in all, no second
 // pass.  8 x 2,048 tokens, 32 heads: 744 -> 669 us; 8 x 64: 58 -> 42 us; 1 x 512: 71 -> 56 us (the choice: kda_chunk_form).
+// Whole chains leave the last of few rounds of CTAs partly empty, and a longer chain makes the wave late.  Waves of at least
+// as many chains as SMs are therefore cut into pieces of whole blocks (the same bits), dealt out a round of chains after the
+// other; a CTA's start costs 7 to 8 us, so few of them (kda_pieces).  32 heads, us, whole | cut: 8 x 2,048 676 | 657,
+// 6 x 2,048 622 | 495, 5 x 1,000 300 | 249; with lengths that whole chains left to the two passes 16 x 512..1,024 607 | 529,
+// 8 x 1,024..2,048 609 | 538, 5 x 1,500..3,000 622 | 525.  In one kernel with the uncut chains the few more registers spilled
+// (64 x 256 tokens, uncut, 697 -> 739), so the cut ones have their own.
 // What bounds a group (clocks, 5.3 K before the third terms below): the products 3.4 K of which the MMA pipe is busy 2.6 K,
 // U 0.4 K, hand-over and outputs 1.2 K; the producers are idle half the time.  Also tried: four column warps of 32 columns with 216 registers
 // (809 us: one warp per scheduler waits), one producer warpgroup (660), a thirteenth warp for T and the copies (711: four
@@ -119,6 +125,12 @@ __device__ __forceinline__ float4 lds4f(uint32_t addr) {
 __device__ __forceinline__ void sts1f(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v)); }
 __device__ __forceinline__ void sts1u(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v)); }
 __device__ __forceinline__ void sts2f(uint32_t addr, float2 v) { asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y)); }
+__device__ __forceinline__ int32_t ld_acquire(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release(int32_t* p, int32_t v) { asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
 __device__ __forceinline__ void named_bar(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
@@ -186,7 +198,8 @@ struct Smem {
 // kSlice value columns per CTA; a column warp owns kMT x 16 of them, or kKS warps share 16 of them and half the channels
 // each.  The column warps first, then kP producer warpgroups that take blocks in turn.
 __host__ __device__ constexpr int col_warps(int slice, int mt, int ks) { return slice / 16 / mt * ks; }
-template <int kSlice, int kMT, int kKS, int kP, int kMinCtas>
+// kCut: the chains are cut into gridDim.z pieces.
+template <int kSlice, int kMT, int kKS, int kP, int kMinCtas, bool kCut>
 __global__ void __launch_bounds__(32 * col_warps(kSlice, kMT, kKS) + 128 * kP, kMinCtas)
 kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
     constexpr int kNC = col_warps(kSlice, kMT, kKS);
@@ -213,7 +226,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
     if (p.blk_off) {
         bool longer = false;
         for (int i = tid; i < p.num_requests; i += blockDim.x) longer |= p.row_offsets[i + 1] - p.row_offsets[i] > p.longest;
-        const bool first_cta = blockIdx.x == 0 && blockIdx.y == 0;
+        const bool first_cta = blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
         if (__syncthreads_or(longer)) {
             if (first_cta) scan_block_offsets<32 * kNC + 128 * kP>(p, reinterpret_cast<int*>(sm));
             return;
@@ -224,8 +237,18 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
     const int64_t row0 = p.row_offsets[req];
     const int C = (int)(p.row_offsets[req + 1] - row0);
     const int P = p.prefix_lens ? p.prefix_lens[req] : 0;
-    const int first_block = P / kL;
-    const int n_blocks = C > 0 ? (P + C + kL - 1) / kL - first_block : 0;
+    int first_block = P / kL;
+    int n_blocks = C > 0 ? (P + C + kL - 1) / kL - first_block : 0;
+    bool resumed = false;
+    if constexpr (kCut) {
+        // this CTA's piece of the chain.  The pieces of a chain follow one another in the grid, a whole round of chains apart (z
+        // is the slowest index), and the state goes from one to the next through memory.
+        const int begin = (int)((int64_t)n_blocks * blockIdx.z / gridDim.z), end = (int)((int64_t)n_blocks * (blockIdx.z + 1) / gridDim.z);
+        if (begin == end && (C > 0 || blockIdx.z > 0)) return;       // (fewer blocks than pieces; an empty chain is the first CTA's)
+        resumed = begin > 0;
+        first_block += begin;
+        n_blocks = end - begin;
+    }
 
     // slot ids: anything outside [-1, num_slots) is reported and treated as -1
     int slot_in = p.state_in[req], slot_out = p.state_out[req];
@@ -543,7 +566,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
         // S[m][j]: rows (columns of the state) gr, gr + 8 of m-tile m; channels ch0 + 8j + 2gc, + 1
         float S[kMT][kNT][4];
         {
-            const float* src = slot_in >= 0 ? p.state_pool + ((size_t)slot_in * H + head) * head_floats + col0 + gr : nullptr;
+            const float* src = slot_in >= 0 && !(kCut && resumed) ? p.state_pool + ((size_t)slot_in * H + head) * head_floats + col0 + gr : nullptr;
 #pragma unroll
             for (int m = 0; m < kMT; ++m)
 #pragma unroll
@@ -562,6 +585,38 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
                     for (int i = 0; i < 4; ++i)
                         dst[(size_t)(ch0 + 8 * j + 2 * gc + (i & 1)) * kD + m * 16 + (i >> 1) * 8] = S[m][j][i];
         };
+        bool dead = false;
+        // The state between pieces, as this warp's threads hold it, and the last block that it has seen.  (Worked out anew at
+        // either end: kept across the chain, the addresses cost registers that the groups need.)
+        auto between = [&](float4*& hand, int32_t*& seen) {
+            uint32_t z = 0;
+            asm volatile("" : "+r"(z));
+            const size_t cta = ((size_t)(blockIdx.y + z) * H + head) * kSlices + slice;
+            hand = p.hand + cta * (head_floats / (4 * kSlices)) + warp * (kMT * kNT * 32) + lane;
+            seen = p.hand_seen + cta * kNC + warp;
+        };
+        if (kCut && resumed) {
+            // (the piece before was started before this one)
+            float4* hand;
+            int32_t* seen;
+            between(hand, seen);
+            const long long t0 = clock64();
+            for (uint32_t n = 0; ld_acquire(seen) != first_block;) {
+                if ((++n & 31u) == 0u && (*abort_flag || clock64() - t0 > WPP_WAIT_LIMIT)) {
+                    *abort_flag = 1u;
+                    dead = true;
+                    break;
+                }
+            }
+            dead = __any_sync(0xffffffffu, dead);
+#pragma unroll
+            for (int m = 0; m < kMT; ++m)
+#pragma unroll
+                for (int j = 0; j < kNT; ++j) {
+                    const float4 v = __ldcg(hand + (m * kNT + j) * 32);
+                    S[m][j][0] = v.x; S[m][j][1] = v.y; S[m][j][2] = v.z; S[m][j][3] = v.w;
+                }
+        }
         const uint32_t s_out = base + SM::kOffOut + warp * 1024;
         // lane parts of the operand addresses
         const int ln7 = lane & 7, l8 = (lane >> 3) & 1, l16 = lane >> 4;
@@ -570,7 +625,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
 #pragma unroll
         for (int w = 0; w < kP; ++w) { stage[w] = 0; ph[w] = 0; }
         uint32_t n_group = 0;
-        bool dead = false, ready = false;
+        bool ready = false;
         for (int b = 0; b < n_blocks && !dead; ++b) {
             const int w = b % kP;
             const int64_t row_t0 = row0 + ((int64_t)(first_block + b) * kL - P);
@@ -834,7 +889,22 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
                 if (store_slot >= 0) store_state(store_slot);
             }
         }
-        if (!dead && slot_out >= 0) store_state(slot_out);
+        if (kCut && blockIdx.z + 1 < gridDim.z) {
+            if (!dead) {
+                float4* hand;
+                int32_t* seen;
+                between(hand, seen);
+#pragma unroll
+                for (int m = 0; m < kMT; ++m)
+#pragma unroll
+                    for (int j = 0; j < kNT; ++j) __stcg(hand + (m * kNT + j) * 32, make_float4(S[m][j][0], S[m][j][1], S[m][j][2], S[m][j][3]));
+                __threadfence();
+                __syncwarp();
+                if (lane == 0) st_release(seen, first_block + n_blocks);
+            }
+        } else if (!dead && slot_out >= 0) {
+            store_state(slot_out);
+        }
     }
 
     // ---- teardown: every wait above is bounded, so every thread gets here
@@ -847,9 +917,9 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
     }
 }
 
-template <int kSlice, int kMT, int kKS, int kP, int kMinCtas>
+template <int kSlice, int kMT, int kKS, int kP, int kMinCtas, bool kCut = false>
 static int launch(const Maps& maps, const KdaGroupParams& p, cudaStream_t st) {
-    auto kernel = kda_group_kernel<kSlice, kMT, kKS, kP, kMinCtas>;
+    auto kernel = kda_group_kernel<kSlice, kMT, kKS, kP, kMinCtas, kCut>;
     constexpr int kNC = col_warps(kSlice, kMT, kKS), smem = Smem<kP, (kSlice == kD ? 2 : 1), kNC, kKS>::kBytes;
     static bool attr_set[64] = {};
     int dev = 0;
@@ -859,7 +929,11 @@ static int launch(const Maps& maps, const KdaGroupParams& p, cudaStream_t st) {
         if (e != cudaSuccess) return (int)e;
         attr_set[dev] = true;
     }
-    dim3 grid((unsigned)p.num_heads * (kD / kSlice), (unsigned)p.num_requests);
+    dim3 grid((unsigned)p.num_heads * (kD / kSlice), (unsigned)p.num_requests, kCut ? (unsigned)p.pieces : 1u);
+    if (kCut) {
+        const cudaError_t e = cudaMemsetAsync(p.hand_seen, 0, sizeof(int32_t) * kNC * (size_t)p.num_heads * (kD / kSlice) * p.num_requests, st);
+        if (e != cudaSuccess) return (int)e;
+    }
     kernel<<<grid, 32 * kNC + 128 * kP, smem, st>>>(maps, p);
     return (int)cudaGetLastError();
 }
@@ -879,5 +953,6 @@ extern "C" int wpp_launch_kda_group(const wpp::KdaGroupParams* p, const CUtensor
     cudaStream_t st = (cudaStream_t)stream;
     if (form == 3) return launch<32, 1, 2, 2, 1>(m, *p, st);
     if (form == 2) return launch<64, 1, 1, 1, 2>(m, *p, st);
+    if (p->pieces > 1) return launch<128, 1, 1, 2, 1, true>(m, *p, st);
     return launch<128, 1, 1, 2, 1>(m, *p, st);
 }

@@ -462,3 +462,26 @@ def test_the_group_form_is_bit_identical_when_chunks_are_cut_at_a_multiple_of_si
         assert status == 0
         got_o[rows], pool = o, torch.from_numpy(pool_).float()
     assert np.array_equal(got_o, want_o) and np.array_equal(pool.double().numpy(), want_pool)
+
+
+@pytest.mark.parametrize("lens,prefix,interval", [
+    ([640, 0, 33, 600, 640], [5, 3, 0, 31, 64], 0),
+    ([640, 1, 16, 600, 640], [100, 7, 15, 0, 1000], 100),      # snapshots inside the pieces; a chunk of fewer blocks than pieces
+])
+def test_chains_cut_into_pieces_match_the_oracle(lens, prefix, interval):
+    """160 chains on 148 SMs: each is cut into pieces whose states pass through the workspace (a sample of the heads against the
+    oracle; every head against the two passes).  That the group form ran shows in the last bits, which are not layout 3's."""
+    w = W.kda_workload("pieces", 19, lens, 32, prefix, snap_interval=interval)
+    t = w.tensors()
+    heads = [0, 13, 31]
+    ref_o, ref_pool = _oracle(w, t, heads)
+    got_o, got_pool, status = _gpu(w, t)
+    assert status == 0
+    _close_out(got_o[:, heads], ref_o, "outputs")
+    _close_state(got_pool[:, heads], ref_pool, "state pool")
+    two_o, two_pool, status = _gpu(w, t, layout=3)
+    assert status == 0
+    _close_state(got_pool, two_pool, "state pool of all heads")
+    assert not np.array_equal(got_pool, two_pool)
+    again_o, again_pool, _ = _gpu(w, t)
+    assert np.array_equal(got_o, again_o) and np.array_equal(got_pool, again_pool)
