@@ -1,4 +1,4 @@
-"""ctypes binding of libwpp.so: argument marshalling only — every step of the path runs in the library.
+"""Binding of libwpp.so (ctypes, and _wpp_call for the calls of every layer): argument marshalling only — every step of the path runs in the library.
 
 The functions carry the C names (wpp_plan_tiles, wpp_kv_append, wpp_prefill_attention_varlen).  Tensors are
 torch tensors used as device memory; streams are torch streams.  There is no fallback: if the library cannot be
@@ -93,11 +93,12 @@ EXPORTS = ["wpp_create", "wpp_destroy", "wpp_status_string", "wpp_last_cuda_erro
            "wpp_hint_probe_recurrent", "wpp_kda_chunk", "wpp_kda_workspace_bytes"]
 
 _lib = None
+_call = None          # the calls of every layer, marshalled in C (csrc/wpp_call.c)
 
 
 def load_library() -> ctypes.CDLL:
     """Load libwpp.so (built in-tree by paper_2609_35263_b200.build); raises if it is missing."""
-    global _lib
+    global _lib, _call
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError(f"{LIB_PATH} is missing: run `python -m paper_2609_35263_b200.build` "
@@ -147,7 +148,9 @@ def load_library() -> ctypes.CDLL:
         lib.wpp_kda_chunk.argtypes = [vp, ctypes.POINTER(KdaDesc)] + [vp] * 13 + [ctypes.c_size_t, vp, vp]
         lib.wpp_kda_workspace_bytes.restype = ctypes.c_size_t
         lib.wpp_kda_workspace_bytes.argtypes = [ctypes.POINTER(KdaDesc)]
-        _lib = lib
+        from . import _wpp_call as call          # (built beside the library; there is no other path)
+        call.init(*(ctypes.cast(f, vp).value for f in (lib.wpp_kv_append, lib.wpp_prefill_attention_varlen, lib.wpp_kda_chunk)))
+        _call, _lib = call, lib
     return _lib
 
 
@@ -274,8 +277,10 @@ def wpp_validate_batch(desc: BatchDesc, block_tables, prefix_lens, chunk_lens) -
     return int(load_library().wpp_validate_batch(ctypes.byref(desc), bt.ctypes.data, P.ctypes.data, C.ctypes.data))
 
 
-# Addresses and streams go to the library as plain integers (the argument types convert them): an object per argument
-# and a torch.cuda.Stream per call were a third of the host time of a small wave.
+# Addresses and streams go to the library as plain integers: an object per argument and a torch.cuda.Stream per call were a
+# third of the host time of a small wave.  The calls a stage makes once per layer take the tensors themselves and are
+# marshalled in C (csrc/wpp_call.c): through ctypes an append and an attention call cost 7.8 us of host time before the library
+# was entered, 3.2 us so.
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
@@ -288,11 +293,10 @@ def _stream(ctx: Context, stream) -> int:
 def wpp_kv_append(ctx: Context, desc: BatchDesc, k_new, v_new, k_cache, v_cache, block_tables, prefix_lens,
                   chunk_lens, plan: Plan, status=None, stream=None) -> None:
     """Queue the KV append of one wave on `stream` (device tensors; int32 metadata on the device)."""
-    st = load_library().wpp_kv_append(ctx.handle, ctypes.byref(desc), _ptr(k_new), _ptr(v_new), _ptr(k_cache),
-                                      _ptr(v_cache), _ptr(block_tables), _ptr(prefix_lens), _ptr(chunk_lens),
-                                      plan.host.data_ptr(), _ptr(plan.dev), _ptr(status),
-                                      _stream(ctx, stream))
-    _check(st, "wpp_kv_append")
+    st = _call.kv_append(ctx.handle.value, desc, k_new, v_new, k_cache, v_cache, block_tables, prefix_lens, chunk_lens, plan.host,
+                         plan.dev, status, _stream(ctx, stream))
+    if st:
+        _check(st, "wpp_kv_append")
 
 
 def wpp_prefill_attention_varlen(ctx: Context, desc: BatchDesc, q, out, lse, k_cache, v_cache, block_tables,
@@ -300,11 +304,10 @@ def wpp_prefill_attention_varlen(ctx: Context, desc: BatchDesc, q, out, lse, k_c
                                  stream=None) -> None:
     """Queue chunked-prefill attention of one wave on `stream`; results land in `out` (and `lse` if given)."""
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    st = load_library().wpp_prefill_attention_varlen(
-        ctx.handle, ctypes.byref(desc), _ptr(q), _ptr(out), _ptr(lse), _ptr(k_cache), _ptr(v_cache),
-        _ptr(block_tables), _ptr(prefix_lens), _ptr(chunk_lens), plan.host.data_ptr(),
-        _ptr(plan.dev), _ptr(workspace), ws_bytes, _ptr(status), _stream(ctx, stream))
-    _check(st, "wpp_prefill_attention_varlen")
+    st = _call.attention(ctx.handle.value, desc, q, out, lse, k_cache, v_cache, block_tables, prefix_lens, chunk_lens, plan.host,
+                         plan.dev, workspace, ws_bytes, status, _stream(ctx, stream))
+    if st:
+        _check(st, "wpp_prefill_attention_varlen")
 
 
 def wpp_static_scratch_bytes() -> int:
@@ -477,9 +480,8 @@ def wpp_kda_chunk(ctx: Context, q, k, v, alpha, beta, row_offsets, state_pool, s
     max_snaps = 0 if snap_slots is None else int(snap_slots.shape[1])
     desc = KdaDesc(R, H, dk, dv, int(state_pool.shape[0]), int(snap_interval), max_snaps, int(layout), T)
     ws_bytes = 0 if workspace is None else int(workspace.numel() * workspace.element_size())
-    st = load_library().wpp_kda_chunk(ctx.handle, ctypes.byref(desc), _ptr(q), _ptr(k), _ptr(v), _ptr(alpha), _ptr(beta),
-                                      _ptr(row_offsets), _ptr(prefix_lens), _ptr(state_pool), _ptr(state_in),
-                                      _ptr(state_out), _ptr(snap_slots), _ptr(out), _ptr(workspace), ws_bytes,
-                                      _ptr(status), _stream(ctx, stream))
-    _check(st, "wpp_kda_chunk")
+    st = _call.kda_chunk(ctx.handle.value, desc, q, k, v, alpha, beta, row_offsets, prefix_lens, state_pool, state_in, state_out,
+                         snap_slots, out, workspace, ws_bytes, status, _stream(ctx, stream))
+    if st:
+        _check(st, "wpp_kda_chunk")
     return out

@@ -3,12 +3,15 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libwpp.so")
 SOURCES = ["wpp_plan.cpp", "wpp_waves.cpp", "wpp_hints.cu", "wpp_api.cu", "wpp_append_combine.cu", "wpp_attention.cu", "wpp_attention_small.cu",
            "wpp_kda.cu", "wpp_kda_tc.cu", "wpp_kda_group.cu"]
+CALL_SOURCE = os.path.join(CSRC, "wpp_call.c")          # Python module that marshals the calls of every layer
+CALL = os.path.join(HERE, "_wpp_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 HEADERS = ["wpp_host.h", "wpp_plan_format.h", "wpp_device.h", "wpp_ptx.cuh", "wpp_kda_blocks.cuh", os.path.join("..", "..", "include", "wpp.h")]
 
 
@@ -20,10 +23,10 @@ def _nvcc() -> str:
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALL))
+    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS] + [CALL_SOURCE]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -31,6 +34,11 @@ def build(force: bool = False, verbose: bool = False, defines=(), out: str = Non
     """Compile the library; `defines` (a list of NAME=VALUE strings) and `out` build a variant beside it."""
     if out is None and not force and not is_stale():
         return LIB
+    if out is None:
+        tmp = CALL + f".tmp{os.getpid()}"
+        subprocess.check_call(["gcc", "-O2", "-Wall", "-Wextra", "-shared", "-fPIC", "-fvisibility=hidden",
+                               "-I", sysconfig.get_paths()["include"], CALL_SOURCE, "-o", tmp])
+        os.replace(tmp, CALL)
     target = out or LIB
     tmp = target + f".tmp{os.getpid()}"
     cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
