@@ -465,8 +465,8 @@ def test_the_group_form_is_bit_identical_when_chunks_are_cut_at_a_multiple_of_si
 
 
 @pytest.mark.parametrize("lens,prefix,interval", [
-    ([640, 0, 33, 600, 640], [5, 3, 0, 31, 64], 0),
-    ([640, 1, 16, 600, 640], [100, 7, 15, 0, 1000], 100),      # snapshots inside the pieces; a chunk of fewer blocks than pieces
+    ([500, 0, 480, 300, 510], [5, 3, 0, 31, 64], 0),
+    ([500, 1, 480, 300, 510], [100, 7, 15, 0, 1000], 100),      # snapshots inside the pieces; a chunk of fewer blocks than pieces
 ])
 def test_chains_cut_into_pieces_match_the_oracle(lens, prefix, interval):
     """160 chains on 148 SMs: each is cut into pieces whose states pass through the workspace (a sample of the heads against the
