@@ -149,7 +149,8 @@ def load_library() -> ctypes.CDLL:
         lib.wpp_kda_workspace_bytes.restype = ctypes.c_size_t
         lib.wpp_kda_workspace_bytes.argtypes = [ctypes.POINTER(KdaDesc)]
         from . import _wpp_call as call          # (built beside the library; there is no other path)
-        call.init(*(ctypes.cast(f, vp).value for f in (lib.wpp_kv_append, lib.wpp_prefill_attention_varlen, lib.wpp_kda_chunk)))
+        call.init(*(ctypes.cast(f, vp).value for f in (lib.wpp_kv_append, lib.wpp_prefill_attention_varlen, lib.wpp_kda_chunk)),
+                  BatchDesc, KdaDesc)
         _call, _lib = call, lib
     return _lib
 
