@@ -148,7 +148,12 @@ def load_library() -> ctypes.CDLL:
         lib.wpp_kda_chunk.argtypes = [vp, ctypes.POINTER(KdaDesc)] + [vp] * 13 + [ctypes.c_size_t, vp, vp]
         lib.wpp_kda_workspace_bytes.restype = ctypes.c_size_t
         lib.wpp_kda_workspace_bytes.argtypes = [ctypes.POINTER(KdaDesc)]
-        from . import _wpp_call as call          # (built beside the library; there is no other path)
+        try:
+            from . import _wpp_call as call
+        except ImportError as e:
+            raise ImportError(f"the module _wpp_call is missing in {_HERE} (it belongs to one Python version and is needed for a "
+                              "library named by WPP_LIB_PATH too): run `python -m paper_2609_35263_b200.build` "
+                              "(there is no fallback path)") from e
         call.init(*(ctypes.cast(f, vp).value for f in (lib.wpp_kv_append, lib.wpp_prefill_attention_varlen, lib.wpp_kda_chunk)),
                   BatchDesc, KdaDesc)
         _call, _lib = call, lib

@@ -1,5 +1,6 @@
 """Builds libwpp.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
 import os
+import shlex
 import shutil
 import subprocess
 import sys
@@ -22,6 +23,14 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def _cc() -> list:
+    """The C compiler's command: CC (with its options), else gcc or cc."""
+    for cand in (shlex.split(os.environ.get("CC", "")), ["gcc"], ["cc"]):
+        if cand and shutil.which(cand[0]):
+            return cand
+    raise RuntimeError("no C compiler found (CC, gcc, cc)")
+
+
 def is_stale() -> bool:
     if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
@@ -36,7 +45,7 @@ def build(force: bool = False, verbose: bool = False, defines=(), out: str = Non
         return LIB
     if out is None:
         tmp = CALL + f".tmp{os.getpid()}"
-        subprocess.check_call(["gcc", "-O2", "-Wall", "-Wextra", "-shared", "-fPIC", "-fvisibility=hidden",
+        subprocess.check_call(_cc() + ["-O2", "-Wall", "-Wextra", "-shared", "-fPIC", "-fvisibility=hidden",
                                "-I", sysconfig.get_paths()["include"], CALL_SOURCE, "-o", tmp])
         os.replace(tmp, CALL)
     target = out or LIB

@@ -1,6 +1,7 @@
 """The calls marshalled in C (csrc/wpp_call.c) refuse on the host what the ctypes calls refuse: no GPU is touched, the context
 is null throughout and the library itself answers WPP_ERR_INVALID_ARG to what passes."""
 import ctypes
+import sys
 
 import pytest
 import torch
@@ -111,3 +112,29 @@ class _Pointer:
 def test_an_address_is_an_integer_of_the_machine(value, error):
     with pytest.raises(error):
         _append(k_new=_Pointer(value))
+
+
+def test_a_missing_module_is_answered_with_the_build_instruction(monkeypatch):
+    B.load_library()
+    name = B.__package__ + "._wpp_call"
+    monkeypatch.setattr(B, "_lib", None)
+    monkeypatch.delattr(sys.modules[B.__package__], "_wpp_call", raising=False)
+    monkeypatch.setitem(sys.modules, name, None)                        # what a failed search leaves
+    with pytest.raises(ImportError, match="python -m paper_2609_35263_b200.build"):
+        B.load_library()
+    assert B._lib is None
+
+
+def test_the_compiler_is_looked_for(monkeypatch, tmp_path):
+    from paper_2609_35263_b200 import build
+    mine = tmp_path / "mine"
+    mine.write_text("#!/bin/sh\n")
+    mine.chmod(0o755)
+    monkeypatch.setenv("CC", str(mine))
+    assert build._cc() == [str(mine)]
+    monkeypatch.setenv("CC", str(mine) + " -m64")
+    assert build._cc() == [str(mine), "-m64"]
+    monkeypatch.setenv("CC", "")
+    monkeypatch.setenv("PATH", str(tmp_path))
+    with pytest.raises(RuntimeError, match="C compiler"):
+        build._cc()
