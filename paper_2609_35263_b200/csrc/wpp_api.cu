@@ -636,7 +636,8 @@ extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const
             p.longest = longest;
             p.pieces = form == 1 ? pieces : 1;
             p.hand = reinterpret_cast<float4*>(static_cast<char*>(workspace) + w.off_e);              // (n_bh >= 2 R H rows of 32 KB)
-            p.hand_seen = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + w.off_u0);
+            p.ticket = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + w.off_u0);
+            p.hand_seen = p.ticket + 1;
             p.blk_off = gated ? reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + w.off_blk) : nullptr;
             CUtensorMap maps[4];
             memset(maps, 0, sizeof(maps));

@@ -85,9 +85,10 @@ struct KdaGroupParams : KdaParams {
     int64_t longest;                // longest chunk this form takes; a wave with a longer one is left to the two passes behind it
     int32_t* blk_off;               // [R+1] for the two passes: their block offsets, or blk_off[0] = -1 if there is nothing left
                                     // for them; null: nothing is behind, the wave is this form's whatever its lengths
-    int32_t pieces;                 // a chain is cut into so many, one after the other in the grid
+    int32_t pieces;                 // a chain is cut into so many, a CTA each
+    int32_t* ticket;                // next piece to be taken: first pieces of all chains, then second ones, ...
     float4* hand;                   // [R][H] states of 64 KB between pieces, and per column warp how many blocks they have seen
-    int32_t* hand_seen;             // [R][H][8]
+    int32_t* hand_seen;             // [R][H][8], behind the ticket
 };
 
 struct KdaTcParams {

@@ -21,8 +21,8 @@
 // pass.  8 x 2,048 tokens, 32 heads: 744 -> 669 us; 8 x 64: 58 -> 42 us; 1 x 512: 71 -> 56 us (the choice: kda_chunk_form).
 // Whole chains leave the last of few rounds of CTAs partly empty, and a longer chain makes the wave late.  Waves of at least
 // as many chains as SMs are therefore cut into pieces of whole blocks (the same bits), dealt out a round of chains after the
-// other; a CTA's start costs 7 to 8 us, so few of them (kda_pieces).  32 heads, us, whole | cut: 8 x 2,048 676 | 657,
-// 6 x 2,048 622 | 495, 5 x 1,000 300 | 249; with lengths that whole chains left to the two passes 16 x 512..1,024 607 | 529,
+// other by tickets that the CTAs take as they start; a CTA's start costs 7 to 8 us, so few of them (kda_pieces).  32 heads, us,
+// whole | cut: 8 x 2,048 676 | 632 (657 with the piece from the CTA's index), 6 x 2,048 622 | 495, 5 x 1,000 300 | 249; with lengths that whole chains left to the two passes 16 x 512..1,024 607 | 529,
 // 8 x 1,024..2,048 609 | 538, 5 x 1,500..3,000 622 | 525.  In one kernel with the uncut chains the few more registers spilled
 // (64 x 256 tokens, uncut, 697 -> 739), so the cut ones have their own.
 // What bounds a group (clocks, 5.3 K before the third terms below): the products 3.4 K of which the MMA pipe is busy 2.6 K,
@@ -198,7 +198,7 @@ struct Smem {
 // kSlice value columns per CTA; a column warp owns kMT x 16 of them, or kKS warps share 16 of them and half the channels
 // each.  The column warps first, then kP producer warpgroups that take blocks in turn.
 __host__ __device__ constexpr int col_warps(int slice, int mt, int ks) { return slice / 16 / mt * ks; }
-// kCut: the chains are cut into gridDim.z pieces.
+// kCut: the chains are cut into p.pieces pieces.
 template <int kSlice, int kMT, int kKS, int kP, int kMinCtas, bool kCut>
 __global__ void __launch_bounds__(32 * col_warps(kSlice, kMT, kKS) + 128 * kP, kMinCtas)
 kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
@@ -212,9 +212,11 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
     constexpr int kSlices = kD / kSlice;
-    const int head = blockIdx.x / kSlices, slice = blockIdx.x % kSlices, req = blockIdx.y, H = p.num_heads;
+    const int H = p.num_heads;
+    int head = blockIdx.x / kSlices, slice = blockIdx.x % kSlices, req = blockIdx.y;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(sm + SM::kOffMisc);
+    volatile int32_t* ticket = reinterpret_cast<volatile int32_t*>(sm + SM::kOffMisc + 4);
     const uint32_t bars = base + SM::kOffBars;
     auto bFull = [&](int w, int s) { return bars + 8 * (w * (2 * SM::kStages + SM::kRaw) + s); };
     auto bEmpty = [&](int w, int s) { return bFull(w, SM::kStages + s); };
@@ -226,7 +228,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
     if (p.blk_off) {
         bool longer = false;
         for (int i = tid; i < p.num_requests; i += blockDim.x) longer |= p.row_offsets[i + 1] - p.row_offsets[i] > p.longest;
-        const bool first_cta = blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
+        const bool first_cta = blockIdx.x == 0 && blockIdx.y == 0;
         if (__syncthreads_or(longer)) {
             if (first_cta) scan_block_offsets<32 * kNC + 128 * kP>(p, reinterpret_cast<int*>(sm));
             return;
@@ -234,6 +236,18 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
         if (first_cta && tid == 0) p.blk_off[0] = -1;
     }
 
+    int piece = 0;
+    if constexpr (kCut) {
+        // A piece waits for the one before it, so that one has to have started: the CTAs take tickets as they start, all first
+        // pieces first, and whatever a ticket waits for is a smaller ticket's.  (CUDA does not say in which order CTAs start.)
+        if (tid == 0) *ticket = atomicAdd(p.ticket, 1);
+        __syncthreads();
+        piece = *ticket / (H * p.num_requests);
+        const int chain = *ticket % (H * p.num_requests);
+        head = chain % H;
+        req = chain / H;
+        slice = 0;
+    }
     const int64_t row0 = p.row_offsets[req];
     const int C = (int)(p.row_offsets[req + 1] - row0);
     const int P = p.prefix_lens ? p.prefix_lens[req] : 0;
@@ -241,10 +255,10 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
     int n_blocks = C > 0 ? (P + C + kL - 1) / kL - first_block : 0;
     bool resumed = false;
     if constexpr (kCut) {
-        // this CTA's piece of the chain.  The pieces of a chain follow one another in the grid, a whole round of chains apart (z
-        // is the slowest index), and the state goes from one to the next through memory.
-        const int begin = (int)((int64_t)n_blocks * blockIdx.z / gridDim.z), end = (int)((int64_t)n_blocks * (blockIdx.z + 1) / gridDim.z);
-        if (begin == end && (C > 0 || blockIdx.z > 0)) return;       // (fewer blocks than pieces; an empty chain is the first CTA's)
+        // this CTA's piece of the chain.  The pieces of a chain are a whole round of chains apart, and the state goes from one to
+        // the next through memory.
+        const int begin = (int)((int64_t)n_blocks * piece / p.pieces), end = (int)((int64_t)n_blocks * (piece + 1) / p.pieces);
+        if (begin == end && (C > 0 || piece > 0)) return;            // (fewer blocks than pieces; an empty chain is the first CTA's)
         resumed = begin > 0;
         first_block += begin;
         n_blocks = end - begin;
@@ -589,14 +603,11 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
         // The state between pieces, as this warp's threads hold it, and the last block that it has seen.  (Worked out anew at
         // either end: kept across the chain, the addresses cost registers that the groups need.)
         auto between = [&](float4*& hand, int32_t*& seen) {
-            uint32_t z = 0;
-            asm volatile("" : "+r"(z));
-            const size_t cta = ((size_t)(blockIdx.y + z) * H + head) * kSlices + slice;
-            hand = p.hand + cta * (head_floats / (4 * kSlices)) + warp * (kMT * kNT * 32) + lane;
-            seen = p.hand_seen + cta * kNC + warp;
+            const size_t chain = *ticket % (H * p.num_requests);
+            hand = p.hand + chain * (head_floats / 4) + warp * (kMT * kNT * 32) + lane;
+            seen = p.hand_seen + chain * kNC + warp;
         };
         if (kCut && resumed) {
-            // (the piece before was started before this one)
             float4* hand;
             int32_t* seen;
             between(hand, seen);
@@ -889,7 +900,7 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
                 if (store_slot >= 0) store_state(store_slot);
             }
         }
-        if (kCut && blockIdx.z + 1 < gridDim.z) {
+        if (kCut && *ticket < (p.pieces - 1) * H * p.num_requests) {
             if (!dead) {
                 float4* hand;
                 int32_t* seen;
@@ -929,9 +940,12 @@ static int launch(const Maps& maps, const KdaGroupParams& p, cudaStream_t st) {
         if (e != cudaSuccess) return (int)e;
         attr_set[dev] = true;
     }
-    dim3 grid((unsigned)p.num_heads * (kD / kSlice), (unsigned)p.num_requests, kCut ? (unsigned)p.pieces : 1u);
+    dim3 grid((unsigned)p.num_heads * (kD / kSlice), (unsigned)p.num_requests);
     if (kCut) {
-        const cudaError_t e = cudaMemsetAsync(p.hand_seen, 0, sizeof(int32_t) * kNC * (size_t)p.num_heads * (kD / kSlice) * p.num_requests, st);
+        static_assert(!kCut || (kSlice == kD && kNC == 8), "a CTA per piece; the layout of hand_seen");
+        grid = dim3((unsigned)p.num_heads * (unsigned)p.num_requests * (unsigned)p.pieces);
+        const size_t words = 1 + (size_t)kNC * p.num_heads * p.num_requests;         // the ticket, then what has been seen
+        const cudaError_t e = cudaMemsetAsync(p.ticket, 0, sizeof(int32_t) * words, st);
         if (e != cudaSuccess) return (int)e;
     }
     kernel<<<grid, 32 * kNC + 128 * kP, smem, st>>>(maps, p);
