@@ -612,8 +612,9 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
             int32_t* seen;
             between(hand, seen);
             const long long t0 = clock64();
-            for (uint32_t n = 0; ld_acquire(seen) != first_block;) {
-                if ((++n & 31u) == 0u && (*abort_flag || clock64() - t0 > WPP_WAIT_LIMIT)) {
+            int32_t at = 0;                  // (negative: the piece before gave up)
+            for (uint32_t n = 0; (at = ld_acquire(seen)) != first_block;) {
+                if (at < 0 || ((++n & 31u) == 0u && (*abort_flag || clock64() - t0 > WPP_WAIT_LIMIT))) {
                     *abort_flag = 1u;
                     dead = true;
                     break;
@@ -901,18 +902,19 @@ kda_group_kernel(const __grid_constant__ Maps maps, const KdaGroupParams p) {
             }
         }
         if (kCut && *ticket < (p.pieces - 1) * H * p.num_requests) {
+            float4* hand;
+            int32_t* seen;
+            between(hand, seen);
             if (!dead) {
-                float4* hand;
-                int32_t* seen;
-                between(hand, seen);
 #pragma unroll
                 for (int m = 0; m < kMT; ++m)
 #pragma unroll
                     for (int j = 0; j < kNT; ++j) __stcg(hand + (m * kNT + j) * 32, make_float4(S[m][j][0], S[m][j][1], S[m][j][2], S[m][j][3]));
                 __threadfence();
                 __syncwarp();
-                if (lane == 0) st_release(seen, first_block + n_blocks);
             }
+            // (a piece that gave up says so: the ones behind it end at once instead of waiting for their own limit one after the other)
+            if (lane == 0) st_release(seen, dead ? -1 : first_block + n_blocks);
         } else if (!dead && slot_out >= 0) {
             store_state(slot_out);
         }

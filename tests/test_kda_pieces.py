@@ -51,3 +51,20 @@ def test_no_order_of_starting_leaves_a_piece_waiting():
     for chains, pieces, sms in ((20, 4, 16), (16, 8, 16), (37, 2, 5)):
         for order in _orders(chains * pieces):
             assert not _stuck(order, chains, pieces, sms, by_ticket)
+
+
+def _limits_until_the_end(pieces, failure_is_told):
+    """How many limits of a wait pass, one after the other, until the pieces of a chain have ended whose first one gave up."""
+    limits, told = 1, failure_is_told
+    for _ in range(pieces - 1):
+        if not told:
+            limits += 1
+    return limits
+
+
+def test_the_pieces_behind_one_that_gave_up_do_not_wait_for_their_limits():
+    """Half a second each: eight pieces in fourteen rounds of CTAs would keep the GPU for minutes."""
+    body = _kernel_source()
+    told = re.search(r"st_release\(seen, dead \? -1 :", body) is not None and re.search(r"if \(at < 0 \|\|", body) is not None
+    assert _limits_until_the_end(8, False) == 8
+    assert _limits_until_the_end(8, told) == 1
