@@ -513,27 +513,37 @@ static int kda_segments(const wpp_kda_desc* d, int sms, double* us, int32_t* beg
 //
 // These are waves of equal chunks, and a wave lasts at least as long as its longest chain, which costs three times as much per
 // token here as in the two passes.  The lengths are on the device: the group form's CTAs look at them, and a wave with a chunk
-// longer than *longest is left to the two passes queued behind (which end at once if it is not).  *longest is the length up
-// to which the group form is the faster one however the rest is distributed: no order of its CTAs takes longer than its rounds
-// all of the longest chunk, nor than the chunks spread evenly and the longest on top (where the chains are cut, half of its piece
-// on top, or it alone); the two passes are taken for equal chunks, where they are fastest.  us, two passes | group form whatever the lengths | now:
+// longer than *longest is left to the two passes queued behind (which end at once if it is not).  For whole chains *longest is the
+// length up to which the group form is the faster one however the rest is distributed: no order of its CTAs takes longer than
+// its rounds all of the longest chunk, nor than the chunks spread evenly and the longest on top; the two passes are taken for
+// equal chunks, where they are fastest.  us, two passes | group form whatever the lengths | now:
 //     8 x 32 heads, 14,000 and 7 x 340 tokens 1261 | 2108 | 1263     8 x 32, 8,192 and 7 x 1,170 960 | 1248 | 959
 //     9 x 8 heads, 16,000 and 8 x 48 tokens 1004 | 2055 | 1004        4 x 32, 512 and 3 x 64 85 | 92 | 83
-// The empty launches behind a wave of equal chunks: 8 x 2,048 669 -> 676, 4 x 256 56 -> 64, 8 x 64 42 -> 50, 64 x 256 652 -> 673.
+// For cut chains *longest is an estimate and no bound: an even spread with half of the longest piece on top, or the longest chain
+// alone.  It leaves out that waiting pieces hold an SM and that several chunks may have that length: 7 x 1,590 and 9 x 8 tokens
+// (32 heads), just not too long for 2 pieces, 556 | 553, the worst of 240 drawn waves of unequal chunks 1 % behind the two
+// passes, 4 x 1,000 and 2 x 2,330 480 | 453, 8 x 1,024..2,048 533 | 480.
+// What it costs to ask: the empty launches behind a wave of equal chunks (whole chains) 8 x 2,048 669 -> 676, 4 x 256 56 -> 64,
+// 8 x 64 42 -> 50, 64 x 256 652 -> 673; the group kernel's empty CTAs, one per piece, in front of a wave that is then left to the
+// two passes, 1 to 4 us (1,290 + 3 x 60 + 40 tokens 151 -> 152, 11 x 1..433 210 -> 214, 20 x 1..524 (8 heads) 111 -> 113).
 constexpr double kGroupUs = 12.0;       // what a launch takes before and after its chains
-constexpr double kPieceUs = 8.0;        // what a piece of a chain takes besides its tokens
+constexpr double kPieceUs = 8.0;        // what a piece of a chain takes besides its tokens (6 measured: not cut where it hardly gains)
+constexpr double kPieceTokens = 96.0;   // tokens that a piece has at least, on average
 constexpr int kMaxPieces = 8;
 // Pieces per chain of the 128-column CTAs, one CTA per SM: whole chains leave the last of few rounds partly empty (256 chains on
 // 148 SMs take two rounds of which the second is 73 % full).  A piece of a chain waits for the one before, which started a
 // whole round of chains earlier: only with at least as many chains as SMs.  Measured, us, in 1 / 2 / 4 / 5 / 8 pieces (32 heads):
-// 8 x 2,048 676 / 721 / 657 / 684 / 698, 8 x 1,024 354 / 383 / 361 / 379 / 403, 5 x 1,000 300 / 283 / 251 / 249 / 257,
-// 6 x 2,048 622 / 545 / 560 / 531 / 546 (3 pieces: 495), 64 x 256 697 / 828 / 1020: cut where it gives 3 % by this estimate.
+// 8 x 2,048 672 / 693 / 637 / 666 / 683, 8 x 1,024 350 / 369 / 352 / 371 / 398, 5 x 1,000 345 / 279 / 250 / 249 / 257,
+// 6 x 2,048 670 / 528 / 542 / 520 / 531 (3 pieces: 479), 64 x 256 667 / 787 / 988: cut where it gives 3 % by this estimate.
+// It takes all chunks for equally long.  Where some are far shorter, the long chains alone may fit the SMs at once, and short
+// pieces cost more than they even out: 4 x 166 and 22 tokens whole 45 us, in 2 pieces 53 (equal chunks, 5 x 160: 72 | 70).
+// Hence kPieceTokens: what shorter pieces would gain on equal chunks is 3 to 4 %, 5 x 200 tokens 86 | 82.
 static int kda_pieces(double n, double C, int sms, double us_per_token, double* us) {
     int best = 1;
     double best_us = ceil(n / sms) * C * us_per_token;
     const double whole = best_us + ceil(n / sms) * kPieceUs;
     double least = 0.97 * whole;
-    for (int k = 2; k <= kMaxPieces && n >= sms && C >= 64.0 * k; ++k) {
+    for (int k = 2; k <= kMaxPieces && n >= sms && C >= kPieceTokens * k; ++k) {
         const double t = ceil(n * k / sms) * (C / k * us_per_token + kPieceUs);
         if (t < least) { best = k; least = t; best_us = t - ceil(n / sms) * kPieceUs; }
     }
@@ -575,6 +585,14 @@ static int kda_chunk_form(const wpp_kda_desc* d, int sms, int64_t* longest, int*
         if (d->num_requests > 1 && (double)*longest < C) best = 0;
     }
     return best;
+}
+// (the choice by itself, for the tests: no GPU needed)
+extern "C" int wpp_kda_choice(const wpp_kda_desc* d, int sms, int64_t* longest, int* pieces) {
+    if (!kda_desc_ok(d) || d->num_requests < 1 || d->total_tokens < 64 * (int64_t)d->num_requests || sms < 1) return -1;
+    *longest = 0;
+    const int form = kda_chunk_form(d, sms, longest, pieces);
+    if (form != 1) *pieces = 1;
+    return form;
 }
 
 extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const void* q, const void* k, const void* v,

@@ -1,10 +1,13 @@
-"""The recurrent layer's group form with its chains cut into pieces (wpp_kda_group.cu): who waits for whom, as a model of the
-launch on the CPU."""
+"""The recurrent layer's group form with its chains cut into pieces (wpp_kda_group.cu): which waves are cut, and who waits for
+whom, as a model of the launch on the CPU."""
+import ctypes
 import os
 import random
 import re
 
 import pytest
+
+import paper_2609_35263_b200.binding as B
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_35263_b200", "csrc")
 
@@ -68,3 +71,39 @@ def test_the_pieces_behind_one_that_gave_up_do_not_wait_for_their_limits():
     told = re.search(r"st_release\(seen, dead \? -1 :", body) is not None and re.search(r"if \(at < 0 \|\|", body) is not None
     assert _limits_until_the_end(8, False) == 8
     assert _limits_until_the_end(8, told) == 1
+
+
+def choice(requests, heads, tokens, sms=148):
+    """(form, pieces, longest chunk) that the library chooses for layout 0; form 1 is the one that is cut."""
+    fn = B.load_library().wpp_kda_choice
+    fn.argtypes = [ctypes.POINTER(B.KdaDesc), ctypes.c_int, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int)]
+    longest, pieces = ctypes.c_int64(0), ctypes.c_int(0)
+    form = fn(ctypes.byref(B.KdaDesc(requests, heads, 128, 128, 0, 0, 0, 0, tokens)), sms, ctypes.byref(longest), ctypes.byref(pieces))
+    return form, pieces.value, longest.value
+
+
+@pytest.mark.parametrize("lens,heads", [([166] * 4 + [22], 32), ([186] * 4 + [93, 19], 32), ([130] * 5, 32), ([190] * 5, 32)])
+def test_short_chains_are_not_cut(lens, heads):
+    """Cut in two, the first wave takes 53 us and not 45, the second 67 and not 59."""
+    assert choice(len(lens), heads, sum(lens))[:2] == (1, 1)
+
+
+def test_a_piece_has_96_tokens_and_its_chains_fill_the_sms():
+    seen = set()
+    for sms in (148, 132, 64):
+        for heads in (1, 7, 8, 16, 32, 64, 300):
+            for requests in (1, 2, 5, 6, 8, 13, 20, 64):
+                for mean in (64, 100, 150, 191, 192, 250, 400, 1000, 2048, 5000):
+                    form, pieces, longest = choice(requests, heads, requests * mean, sms)
+                    assert 1 <= pieces <= 8
+                    if pieces > 1:
+                        seen.add(pieces)
+                        assert form == 1 and requests * heads >= sms and mean >= 96 * pieces
+                        assert requests == 1 or longest >= mean
+    assert seen >= {2, 3, 4, 5}
+
+
+@pytest.mark.parametrize("requests,heads,mean,pieces", [(8, 32, 2048, 4), (6, 32, 2048, 3), (5, 32, 1000, 5), (20, 8, 800, 4), (64, 32, 256, 1),
+                                                        (5, 32, 256, 2), (8, 32, 1024, 1)])
+def test_waves_whose_cut_was_measured(requests, heads, mean, pieces):
+    assert choice(requests, heads, requests * mean)[:2] == (1, pieces)
