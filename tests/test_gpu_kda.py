@@ -14,6 +14,7 @@ import paper_2609_35263_b200 as wpp
 import wpp_workloads as W
 from oracle import kda as O
 from tests import gpu_harness as H
+from tests.test_kda_pieces import choice
 
 pytestmark = pytest.mark.gpu
 
@@ -464,14 +465,21 @@ def test_the_group_form_is_bit_identical_when_chunks_are_cut_at_a_multiple_of_si
     assert np.array_equal(got_o, want_o) and np.array_equal(pool.double().numpy(), want_pool)
 
 
+def _cut(w, pieces):
+    """Asserts that the library cuts this wave's chains into so many pieces (on 148 SMs, as all tests of this file assume)."""
+    form, k, longest = choice(len(w.chunk_lens), int(w.num_heads), int(w.total_tokens), torch.cuda.get_device_properties(0).multi_processor_count)
+    assert (form, k) == (1, pieces) and w.chunk_lens.max() <= longest, (form, k, longest)
+
+
 @pytest.mark.parametrize("lens,prefix,interval", [
     ([500, 0, 480, 300, 510], [5, 3, 0, 31, 64], 0),
     ([500, 1, 480, 300, 510], [100, 7, 15, 0, 1000], 100),      # snapshots inside the pieces; a chunk of fewer blocks than pieces
 ])
 def test_chains_cut_into_pieces_match_the_oracle(lens, prefix, interval):
-    """160 chains on 148 SMs: each is cut into pieces whose states pass through the workspace (a sample of the heads against the
-    oracle; every head against the two passes).  That the group form ran shows in the last bits, which are not layout 3's."""
+    """160 chains on 148 SMs in three pieces each, whose states pass through the workspace (a sample of the heads against the
+    oracle; every head against the two passes)."""
     w = W.kda_workload("pieces", 19, lens, 32, prefix, snap_interval=interval)
+    _cut(w, 3)
     t = w.tensors()
     heads = [0, 13, 31]
     ref_o, ref_pool = _oracle(w, t, heads)
@@ -485,3 +493,100 @@ def test_chains_cut_into_pieces_match_the_oracle(lens, prefix, interval):
     assert not np.array_equal(got_pool, two_pool)
     again_o, again_pool, _ = _gpu(w, t)
     assert np.array_equal(got_o, again_o) and np.array_equal(got_pool, again_pool)
+
+
+@pytest.mark.parametrize("lens,H_,pieces,step", [
+    ([256, 250, 240, 256, 251], 32, 2, 128), ([384, 330, 400, 369, 390], 32, 3, 144), ([640, 600, 633, 655, 580], 32, 4, 176),
+    ([992, 976, 987], 50, 5, 176), ([1500, 1479, 1488], 50, 6, 176),
+])
+def test_cut_chains_have_the_bits_of_whole_ones(lens, H_, pieces, step):
+    """A wave whose chains are cut against the same tokens in calls of up to `step` tokens a request, which the library does not
+    cut and gives to CTAs of the same width: groups are blocks of 16 absolute positions, so outputs and states have the same
+    bits."""
+    w = W.kda_workload("cut", 61 + pieces, lens, H_, [16 * i for i in range(len(lens))])
+    _cut(w, pieces)
+    t = w.tensors()
+    want_o, want_pool, status = _gpu(w, t)
+    assert status == 0
+    pool, got_o, done = t["state_pool"], np.zeros_like(want_o), 0
+    while done < max(lens):
+        part_lens = [min(step, n - done) for n in lens]
+        rows = np.concatenate([np.arange(r + done, r + done + n) for r, n in zip(w.row_offsets[:-1], part_lens)])
+        part = W.kda_workload("part", 61 + pieces, part_lens, H_, [int(x) + done for x in w.prefix_lens])
+        part.num_slots = w.num_slots
+        _cut(part, 1)
+        o, pool_, status = _gpu(part, {k: (v[rows].contiguous() if k != "state_pool" else pool) for k, v in t.items()},
+                                state_in=w.state_in if done == 0 else w.state_out, state_out=w.state_out)
+        assert status == 0
+        got_o[rows], pool = o, torch.from_numpy(pool_).float()
+        done += step
+    assert np.array_equal(got_o, want_o) and np.array_equal(pool.double().numpy(), want_pool)
+
+
+@pytest.mark.parametrize("lens,interval", [([640, 0, 33, 600, 640], 0), ([33, 640, 0, 640, 600], 100)])
+def test_a_cut_wave_that_is_turned_away_on_the_device_is_the_two_passes(lens, interval):
+    """The host would cut the chains in three; the CTAs find a chunk longer than the choice allows and leave the wave, whichever
+    piece they would have been, to the two passes behind: their bits."""
+    w = W.kda_workload("turned away", 43, lens, 32, [5, 3, 0, 31, 64], snap_interval=interval)
+    form, pieces, longest = choice(5, 32, w.total_tokens)
+    assert (form, pieces) == (1, 3) and max(lens) > longest
+    t = w.tensors()
+    got_o, got_pool, status = _gpu(w, t)
+    two_o, two_pool, two_status = _gpu(w, t, layout=3)
+    assert status == 0 and two_status == 0
+    assert np.array_equal(got_o, two_o) and np.array_equal(got_pool, two_pool)
+
+
+@pytest.mark.parametrize("same_slot", [False, True])         # periodic snapshots in slots of their own, or in the chunk end's
+def test_cut_chains_with_states_in_place_strong_decays_and_snapshots(same_slot):
+    """The first piece reads the slot that the last one writes, snapshots are stored by the piece that passes them, decays end
+    groups or go to the state directly (a sample of the heads against the oracle)."""
+    lens, heads = [500, 0, 480, 300, 510], [0, 21, 31]
+    w = W.kda_workload("in place", 67, lens, 32, [5, 3, 16, 31, 64], snap_interval=100)
+    _cut(w, 3)
+    w.state_in = w.state_out
+    if same_slot:
+        w.snap_slots[:] = w.state_out[:, None]
+    t = w.tensors()
+    rng, a = np.random.default_rng(3), t["alpha"].numpy()
+    for val, count in ((0.0, 6), (1e-9, 6), (1e-30, 4), (0.2, 200)):
+        a[rng.integers(0, a.shape[0], count), rng.choice(heads, count), rng.integers(0, 128, count)] = val
+    ref_o, ref_pool = _oracle(w, t, heads)
+    for _ in range(5):
+        got_o, got_pool, status = _gpu(w, t)
+        assert status == 0
+        _close_out(got_o[:, heads], ref_o, "outputs")
+        _close_state(got_pool[:, heads], ref_pool, "state pool")
+
+
+def test_a_captured_call_of_cut_chains_replays_with_the_same_bits():
+    """The clearing of the counter and of the hand-over flags is part of the graph: every replay starts from the first piece."""
+    w = W.kda_workload("captured", 71, [500, 30, 480, 300, 510], 32, [5, 3, 0, 31, 64])
+    _cut(w, 3)
+    t = w.tensors()
+    want_o, want_pool, status = _gpu(w, t)
+    assert status == 0
+    dev = torch.device("cuda")
+    d = {k: v.to(dev) for k, v in t.items()}
+    i32 = lambda x: torch.from_numpy(np.ascontiguousarray(x, dtype=np.int32)).to(dev)
+    rows, s_in, s_out, prefix = torch.from_numpy(w.row_offsets).to(dev), i32(w.state_in), i32(w.state_out), i32(w.prefix_lens)
+    ws = torch.empty(wpp.wpp_kda_workspace_bytes(5, 32, w.total_tokens), dtype=torch.uint8, device=dev)
+    status, out, pool = torch.zeros(1, dtype=torch.int32, device=dev), torch.empty_like(d["v"]), d["state_pool"].clone()
+    call = lambda: wpp.wpp_kda_chunk(H.ctx(), d["q"], d["k"], d["v"], d["alpha"], d["beta"], rows, pool, s_in, s_out, out=out,
+                                     prefix_lens=prefix, status=status, workspace=ws)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        call()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            call()
+    for _ in range(3):
+        pool.copy_(d["state_pool"])
+        out.zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        assert np.array_equal(out.float().cpu().double().numpy(), want_o)
+        assert np.array_equal(pool.cpu().double().numpy(), want_pool)
