@@ -521,8 +521,8 @@ static int kda_segments(const wpp_kda_desc* d, int sms, double* us, int32_t* beg
 //     9 x 8 heads, 16,000 and 8 x 48 tokens 1004 | 2055 | 1004        4 x 32, 512 and 3 x 64 85 | 92 | 83
 // For cut chains *longest is an estimate and no bound: an even spread with half of the longest piece on top, or the longest chain
 // alone.  It leaves out that waiting pieces hold an SM and that several chunks may have that length: 7 x 1,590 and 9 x 8 tokens
-// (32 heads), just not too long for 2 pieces, 556 | 553, the worst of 240 drawn waves of unequal chunks 1 % behind the two
-// passes, 4 x 1,000 and 2 x 2,330 480 | 453, 8 x 1,024..2,048 533 | 480.
+// (32 heads), just not too long for 2 pieces, two passes | cut 554 | 550, 4 x 1,000 and 2 x 2,330 476 | 450, 8 x 1,024..2,048
+// 537 | 480.
 // What it costs to ask: the empty launches behind a wave of equal chunks (whole chains) 8 x 2,048 669 -> 676, 4 x 256 56 -> 64,
 // 8 x 64 42 -> 50, 64 x 256 652 -> 673; the group kernel's empty CTAs, one per piece, in front of a wave that is then left to the
 // two passes, 1 to 4 us (1,290 + 3 x 60 + 40 tokens 151 -> 152, 11 x 1..433 210 -> 214, 20 x 1..524 (8 heads) 111 -> 113).

@@ -21,9 +21,10 @@
 // pass.  8 x 2,048 tokens, 32 heads: 744 -> 669 us; 8 x 64: 58 -> 42 us; 1 x 512: 71 -> 56 us (the choice: kda_chunk_form).
 // Whole chains leave the last of few rounds of CTAs partly empty, and a longer chain makes the wave late.  Waves of at least
 // as many chains as SMs are therefore cut into pieces of whole blocks (the same bits), dealt out a round of chains after the
-// other by tickets that the CTAs take as they start; a CTA's start costs 7 to 8 us, so few of them (kda_pieces).  32 heads, us,
-// whole | cut: 8 x 2,048 676 | 632 (657 with the piece from the CTA's index), 6 x 2,048 622 | 495, 5 x 1,000 300 | 249; with lengths that whole chains left to the two passes 16 x 512..1,024 607 | 529,
-// 8 x 1,024..2,048 609 | 538, 5 x 1,500..3,000 622 | 525.  In one kernel with the uncut chains the few more registers spilled
+// other by tickets that the CTAs take as they start; a piece costs about 6 us besides its tokens, so few of them (kda_pieces).  32
+// heads, us, whole (or the two passes, where those were taken instead) | cut: 8 x 2,048 672 | 635 (651 with the piece from the
+// CTA's index), 6 x 2,048 610 | 476, 5 x 1,000 297 | 248, 16 x 512..1,024 568 | 490, 8 x 1,024..2,048 537 | 480,
+// 5 x 1,500..3,000 545 | 500.  In one kernel with the uncut chains the few more registers spilled
 // (64 x 256 tokens, uncut, 697 -> 739), so the cut ones have their own.
 // What bounds a group (clocks, 5.3 K before the third terms below): the products 3.4 K of which the MMA pipe is busy 2.6 K,
 // U 0.4 K, hand-over and outputs 1.2 K; the producers are idle half the time.  Also tried: four column warps of 32 columns with 216 registers

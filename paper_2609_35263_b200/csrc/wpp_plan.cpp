@@ -91,13 +91,19 @@ constexpr int64_t kTileFixedCost = 3, kPartExtraCost = 2, kCombineCost = 20;
 //     32 x 128           60 |  45       32 x 1024            781 | 789      32 x 256 / 1024         309 | 443
 //     32 x 256          117 |  97       16 x 2048           1199 | 1466     16 x 512 / 2048         556 | 878
 //     32 x 512          303 | 246       64 x 1..300 / 0..500  83 |  69      8 x 300 / 700            68 |  70
-// (the last two in the middle and on the right with 16/4 heads of 64 and 32/8 of 128).  The line lies where both are equal.  With
+// (the last two in the middle and on the right with 16/4 heads of 64 and 32/8 of 128; the least of five runs of ten calls.  The
+// median of nine on another B200: 32 x 512 326 | 263, 32 x 1024 847 | 818, 32 x 256 / 1024 328 | 440, 8 x 300 / 700 68 | 70).  The
+// line lies where both are about equal: 32 x 1024, 3 % better on the small shape there, is on the SM-wide side.  With
 // 3.3 and 3.0 us, the constants of one thread per query row, 32 x 300..1000 and 64 x 1..300 / 0..500 went to the SM-wide shape;
 // with one slope for all lengths 4 x 1407, 2 x 196..1950 and 7 x 1250..1751 went to the small one (pass, us, SM-wide | small:
 // 132 | 147, 69 | 86, 62 | 74; but 80 x 228 over 119..239 271 | 214, 12 x 210..393 over 127..212 132 | 108).
-// Where the small shape's items take several rounds and average more than kSmallShapeSteps key steps, its estimate is up to
-// 12 % short (the CTAs of an SM share the tensor pipe and L2) and the SM-wide one is taken: 32 x 4..34 new tokens, 40/8 heads
-// (one head per tile), over 1,100 / 1,500 / 4,096 cached ones 142 | 148, 169 | 184, 431 | 459 (pass, us, one thread per row).
+// Where the small shape's items take several rounds and average more than kSmallShapeSteps key steps, the SM-wide one is taken
+// whatever the estimate says, because that is too short for some of these waves by up to a third: items whose lengths differ
+// much, and the shorter steps of heads of 64.  Of 55 drawn waves that only this rule sends to the SM-wide shape the small one
+// is slower on 11, by up to a half, and faster on 44, by up to 32 % (pass, us, SM-wide | small: 69 x 14..39 over 160..3,524
+// cached tokens, 32/8 heads, 146 | 219; 51 x 25..34 over 2,234..3,626 146 | 201; 120 x 3..35 over 2,520..4,368, 16/4 of 64,
+// 153 | 201; 42 x 5 over 253..2,477, 64/8, 80 | 99; but 22 x 7..15 over 987..1,080, 40/8, 118 | 80; 32 x 4..34, 40/8, over 1,100 /
+// 1,500 / 4,096 140 | 126, 167 | 162, 430 | 406).  An estimate that tells them apart could take its place.
 constexpr int64_t kSmallShapeSteps = 8;
 struct StepCount {
     int64_t sum = 0;
@@ -217,7 +223,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
         // average, two heads of a KV group over the same 128 rows: those see the same keys, so neither half waits for the
         // other's last step.  Attention call, us, row blocks | heads: 16 x 256..2,048 over 0..8,192 (32 heads) 1156 | 1130,
         // 8 x 512 over 4,096 522 | 507, 128 requests behind a shared prefix 123.1 | 122.2 ms; but 32 x 1,024 without prefix
-        // 845 | 853 and 32 x 256 on the small shape 110 | 112.  (An explicit tile height keeps the row blocks.)
+        // 845 | 853 and 32 x 256 on the small shape 97.4 | 98.2.  (An explicit tile height keeps the row blocks.)
         const int block_m = pair_heads ? WPP_HALF_M : tile_m;
         rbs.clear();
         int64_t n_tiles = 0;
