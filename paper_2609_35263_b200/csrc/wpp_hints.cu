@@ -97,19 +97,24 @@ __global__ void __launch_bounds__(256) wpp_block_digest_kernel(const int32_t* __
     }
 }
 
-// The chain H_i = mix64(H_{i-1} ^ mix64(digest_i + extraKeys_i) ^ salt term) is sequential by definition: one lane of a
+// The chain H_i = mix64(H_{i-1} ^ mix64(digest_i + extraKeys_i) ^ salt term) is sequential by definition: a
 // warp walks a request's blocks, and what bounds it is the step's own dependent arithmetic.
 // With z the value before mix64's last shift, h = z ^ z >> 31, the next step starts from
 //     h ^ c ^ (h ^ c) >> 30  =  z ^ z >> 30 ^ z >> 31 ^ z >> 61 ^ (c ^ c >> 30),
 // whose shifts are independent of one another and whose last term the digests left ready: two dependent operations
 // between the multiplications instead of four.  The step works on 32-bit halves, because a 64-bit product's low half is
 // there long before its high half: all of a shift that comes from the low half is folded in while the high half is on its
-// way, and the high half is the sum of three products that do not wait for one another.  64 requests x 3,125 blocks, the
-// fused kernel with its tokens in L2: 64-bit operations 143 us, halves with wide products 129, this order 125.
+// way, and the high half is the sum of three products that do not wait for one another.  Its shifts and exclusive ors are
+// issued every other clock at most, so their number counts as well: one funnel shift takes what z >> 30 needs of both
+// halves, and z ^ z >> 31, the hash itself, is left to whoever stores it.  64 requests x 3,125 blocks, the fused kernel with
+// its tokens in L2: 64-bit operations 143 us, halves with wide products 129, in this order 127.5, with the funnel shift, the
+// hash left out and four steps a turn 117 (69 clocks a step; eight steps a turn 123, two 126, the same without the funnel
+// shift 123).
 // The warp moves kStage blocks at a time through shared memory - the next
 // stage's loads are in flight while this one is chained, the finished hashes leave as coalesced stores - so that the
-// walk never waits on global memory; inside a stage eight terms are read before and eight hashes written after the
-// eight steps between them (a load that may alias the store before it would put shared-memory latency into every step).
+// walk never waits on global memory; inside a stage a turn's terms are read a turn ahead and its results written after its
+// steps (a load that may alias the store before it would put shared-memory latency into every step).  All lanes walk alike:
+// one lane alone takes 1 % longer.
 __device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) {
     uint32_t r;
     asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
@@ -128,17 +133,41 @@ __device__ __forceinline__ uint32_t mul_lo(uint32_t a, uint32_t b) {
 __device__ __forceinline__ uint64_t chain_product(uint64_t z, uint64_t c) {
     constexpr uint32_t k1l = 0x1CE4E5B9u, k1h = 0xBF58476Du, k2l = 0x133111EBu, k2h = 0x94D049BBu;
     const uint32_t l = (uint32_t)z, h = (uint32_t)(z >> 32), cl = (uint32_t)c, ch = (uint32_t)(c >> 32);
-    const uint32_t early = xor3(l, cl, l >> 30) ^ (l >> 31);
-    const uint32_t xl = xor3(h << 2, h << 1, h >> 29) ^ early, xh = xor3(h ^ ch, h >> 30, h >> 31);
+    const uint32_t early = xor3(l, cl, l >> 31);                               // ... ^ the low halves of z >> 61, 31 and 30
+    const uint32_t xl = xor3(early, h >> 29, h << 1) ^ __funnelshift_l(l, h, 2), xh = xor3(h ^ ch, h >> 30, h >> 31);
     const uint32_t pl = mul_lo(xl, k1l), ph = mul_hi(xl, k1l) + mul_lo(xl, k1h) + mul_lo(xh, k1l);
     const uint32_t yl = xor3(pl, pl >> 27, ph << 5), yh = ph ^ (ph >> 27);
     const uint32_t ql = mul_lo(yl, k2l), qh = mul_hi(yl, k2l) + mul_lo(yl, k2h) + mul_lo(yh, k2l);
     return ((uint64_t)qh << 32) | ql;
 }
+__device__ __forceinline__ uint64_t chain_hash(uint64_t z) { return z ^ (z >> 31); }
+// The steps of the terms m[0, cnt), whose products go to h; both have room for kMost values.  (Steps past the last term
+// compute on values nobody reads.)
+template <int kMost>
+__device__ __forceinline__ void chain_steps(uint64_t& z, const uint64_t* m, uint64_t* h, int cnt) {
+    constexpr int kTurn = 4;
+    static_assert(kMost % kTurn == 0, "whole turns");
+    uint64_t c[kTurn];
+#pragma unroll
+    for (int j = 0; j < kTurn; ++j) c[j] = m[j];
+#pragma unroll 1
+    for (int i = 0; i < cnt; i += kTurn) {
+        uint64_t next[kTurn];                              // (past the last turn: the first one's again, not used)
+        const int at = i + kTurn < kMost ? i + kTurn : 0;
+#pragma unroll
+        for (int j = 0; j < kTurn; ++j) next[j] = m[at + j];
+#pragma unroll
+        for (int j = 0; j < kTurn; ++j) c[j] = z = chain_product(z, c[j]);
+#pragma unroll
+        for (int j = 0; j < kTurn; ++j) h[i + j] = c[j];
+#pragma unroll
+        for (int j = 0; j < kTurn; ++j) c[j] = next[j];
+    }
+}
 constexpr int kStage = 128, kPerLane = kStage / 32;
 __global__ void __launch_bounds__(32) wpp_hash_chain_kernel(const int64_t* __restrict__ block_offsets,
                                                             uint64_t* __restrict__ hashes) {
-    __shared__ uint64_t buf[kStage];
+    __shared__ uint64_t buf[kStage], done[kStage];
     const int lane = threadIdx.x;
     const int64_t b0 = block_offsets[blockIdx.x], n = block_offsets[blockIdx.x + 1] - b0;
     uint64_t* h = hashes + b0;
@@ -155,39 +184,23 @@ __global__ void __launch_bounds__(32) wpp_hash_chain_kernel(const int64_t* __res
             const int64_t i = first + kStage + u * 32 + lane;
             nxt[u] = i < n ? h[i] : 0ull;
         }
-        if (lane == 0) {
-            const int cnt = (int)min((int64_t)kStage, n - first);
-#pragma unroll 1
-            for (int i = 0; i < cnt; i += 8) {          // (steps past the last block compute on zeros nobody reads)
-                uint64_t c[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) c[j] = buf[i + j];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    z = chain_product(z, c[j]);
-                    c[j] = z ^ (z >> 31);
-                }
-#pragma unroll
-                for (int j = 0; j < 8; ++j) buf[i + j] = c[j];
-            }
-        }
+        chain_steps<kStage>(z, buf, done, (int)min((int64_t)kStage, n - first));
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < kPerLane; ++u) {
             const int64_t i = first + u * 32 + lane;
-            if (i < n) h[i] = buf[u * 32 + lane];
+            if (i < n) h[i] = chain_hash(done[u * 32 + lane]);
         }
         __syncwarp();
     }
 }
 
 // Digests and chain of long prompts in one kernel, a CTA per request: twelve warps work on the digests of the next stage of
-// 96 blocks while one lane chains the current ones out of shared memory, so that only the first stage's digests stand in
+// 96 blocks while one warp chains the current ones out of shared memory, so that only the first stage's digests stand in
 // front of the chain.  The chain's warp is the only one of its scheduler (warps 7, 11 and 15 leave at once): beside digest
 // warps its dependent steps waited for issue slots (170 us instead of 144 for 64 requests x 3,125 blocks of 64 tokens).
 // The tokens of a stage are requested a stage ahead (requested with their use, a stage of tokens that come from HBM took
-// longer than its chain: 154 us however short the chain's step), the chain's next eight terms eight steps ahead (137 us
-// without, 129 with).
+// longer than its chain: 154 us however short the chain's step), the chain's next terms a turn ahead.
 constexpr int kFusedWarps = 12, kFusedStage = 8 * kFusedWarps, kFusedThreads = 512;
 __global__ void __launch_bounds__(kFusedThreads, 1) wpp_hash_fused_kernel(const int32_t* __restrict__ tokens,
                                                                           const int64_t* __restrict__ token_offsets,
@@ -227,13 +240,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1) wpp_hash_fused_kernel(const 
             for (int j = 0; j < 8; ++j) d[j] += k < block_size ? token_term(t[j][u], (uint32_t)k) : 0ull;
         }
         load(s + 1);
-        uint64_t mine = 0;
+        // lane l ends with the sum of block l & 7: with every exchange it hands over the half of its blocks that it does not
+        // keep (nine exchanges instead of forty; a stage's digests 4.0 K clocks instead of 4.9 K)
+        const bool hi4 = lane & 4, hi2 = lane & 2, hi1 = lane & 1;
+        uint64_t e4[4], e2[2];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 4; ++j) e4[j] = (hi4 ? d[j + 4] : d[j]) + __shfl_xor_sync(0xffffffffu, hi4 ? d[j] : d[j + 4], 4);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) d[j] += __shfl_xor_sync(0xffffffffu, d[j], o);
-            if (lane == j) mine = d[j];
-        }
+        for (int j = 0; j < 2; ++j) e2[j] = (hi2 ? e4[j + 2] : e4[j]) + __shfl_xor_sync(0xffffffffu, hi2 ? e4[j] : e4[j + 2], 2);
+        uint64_t mine = (hi1 ? e2[1] : e2[0]) + __shfl_xor_sync(0xffffffffu, hi1 ? e2[0] : e2[1], 1);
+        mine += __shfl_xor_sync(0xffffffffu, mine, 8);
+        mine += __shfl_xor_sync(0xffffffffu, mine, 16);
         if (lane < 8) {                     // (entries past the request's last block are never used)
             const uint64_t c = mix64(mine + ((extra && first + lane < n) ? extra[b0 + first + lane] : 0ull)) ^ salt_term;
             s_m[s & 1][dw * 8 + lane] = c ^ (c >> 30);
@@ -247,35 +264,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) wpp_hash_fused_kernel(const 
     uint64_t z = 0;
     for (int s = 0; s <= n_stages; ++s) {
         if (warp == 3) {
-            if (lane == 0 && s < n_stages) {
-                const uint64_t* m = s_m[s & 1];
-                uint64_t* h = s_h[s & 1];
-                const int cnt = (int)min((int64_t)kFusedStage, n - (int64_t)s * kFusedStage);
-                uint64_t c[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) c[j] = m[j];
-#pragma unroll 1
-                for (int i = 0; i < cnt; i += 8) {
-                    uint64_t next[8];                  // (past the stage: the first ones again, not used)
-                    const int at = i + 8 < kFusedStage ? i + 8 : 0;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) next[j] = m[at + j];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        z = chain_product(z, c[j]);
-                        c[j] = z ^ (z >> 31);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) h[i + j] = c[j];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) c[j] = next[j];
-                }
-            }
+            if (s < n_stages) chain_steps<kFusedStage>(z, s_m[s & 1], s_h[s & 1], (int)min((int64_t)kFusedStage, n - (int64_t)s * kFusedStage));
             __syncwarp();
         } else {
             if (s > 0) {
                 const int64_t i = (int64_t)(s - 1) * kFusedStage + dw * 8 + lane;
-                if (lane < 8 && i < n) out[b0 + i] = s_h[(s - 1) & 1][dw * 8 + lane];
+                if (lane < 8 && i < n) out[b0 + i] = chain_hash(s_h[(s - 1) & 1][dw * 8 + lane]);
             }
             if (s + 1 < n_stages) digest(s + 1);
         }
