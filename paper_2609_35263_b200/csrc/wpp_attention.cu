@@ -276,8 +276,9 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         const int hf = b / per_half, k = (b % per_half) / C::kHalves, h = b % C::kHalves;
                         const int n_hf = hf ? v.n[1] : v.n[0];
                         if (n_hf == 0) continue;
+                        // (more places than heads in the group: the last head again, into rows that nobody stores)
                         tma_load_3d(sQ + hf * C::kTileBytes + h * C::kHalfBytes + k * rph * 128, qm, bQFull, h * 64,
-                                    (hf ? un.head[1] : un.head[0]) + k, v.q_off + (hf ? un.row0[1] : un.row0[0]));
+                                    (hf ? un.head[1] : un.head[0]) + min(k, p.group - 1), v.q_off + (hf ? un.row0[1] : un.row0[0]));
                     }
                 }
                 __syncwarp();
@@ -415,7 +416,7 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 if (un.rows[hf] == 0) continue;
                 const int rph = 128 / un.pack, rr = r & (rph - 1);       // row inside its head's block
                 const int head = un.head[hf] + r / rph;
-                const bool row_ok = rr < un.rows[hf];
+                const bool row_ok = rr < un.rows[hf] && r / rph < p.group;
                 const int64_t tok = (int64_t)v.q_off + un.row0[hf] + rr;
                 const int64_t prow = ((int64_t)un.split_slot * 2 + hf) * 128 + r;
                 if (v.n[hf] == 0) {

@@ -296,7 +296,8 @@ wpp_attn_small_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 const CUtensorMap* qm = log_pack == 0 ? &tm_q : log_pack == 1 ? &tm_q64 : log_pack == 2 ? &tm_q32 : &tm_q16;
                 if (lane < (C::kHalves << log_pack)) {
                     const int k = lane / C::kHalves, h = lane % C::kHalves;
-                    tma_load_3d(sQ + h * C::kQHalfBytes + k * (128 >> log_pack) * 128, qm, bQFull, h * 64, head + k, q_off + row0);
+                    // (more places than heads in the group: the last head again, into rows that nobody stores)
+                    tma_load_3d(sQ + h * C::kQHalfBytes + k * (128 >> log_pack) * 128, qm, bQFull, h * 64, head + min(k, p.group - 1), q_off + row0);
                 }
                 return true;
             };
@@ -419,7 +420,7 @@ wpp_attn_small_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             const int n = rec[0].y, step0 = rec[0].z, kv_len = rec[0].w, first_pos = rec[1].x;
             const int rr = r & ((1 << rec[1].z) - 1);                    // row inside its head's block
             const int head = rec[2].x + (r >> rec[1].z);
-            const bool row_ok = rr < rec[1].y, split = rec[2].y >= 0;
+            const bool row_ok = rr < rec[1].y && (r >> rec[1].z) < p.group, split = rec[2].y >= 0;
             const int64_t tok = (int64_t)rec[1].w + rr, prow = (int64_t)rec[2].y + r;
             if (n == 0) {
                 // a split part that lies wholly above this half's diagonal (or a refused request): no key is visible

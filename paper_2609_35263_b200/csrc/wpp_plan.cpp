@@ -217,6 +217,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     auto steps_for = [](int64_t last_visible_plus1) { return (int32_t)((last_visible_plus1 + WPP_TILE_N - 1) / WPP_TILE_N); };
     std::vector<RowBlock> rbs;
     std::vector<int32_t> rb_first((size_t)R + 1);
+    bool whole_groups = false;
     bool pair_heads = auto_tile_m && G % 2 == 0 && pairs >= kPairHeadsKeys * T;
     auto build_rows = [&](int tile_m) -> int64_t {
         // The halves of a 256-row tile are two consecutive row blocks of a head, or, where the queries see many keys on
@@ -226,6 +227,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
         // 845 | 853 and 32 x 256 on the small shape 97.4 | 98.2.  (An explicit tile height keeps the row blocks.)
         const int block_m = pair_heads ? WPP_HALF_M : tile_m;
         rbs.clear();
+        whole_groups = false;
         int64_t n_tiles = 0;
         for (int i = 0; i < R; ++i) {
             rb_first[(size_t)i] = (int32_t)rbs.size();
@@ -242,8 +244,19 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
                     // per head); with 256-row tiles the second half takes the next heads of the group
                     int pack = 1;
                     while (pack < 8 && G % (2 * pack) == 0 && WPP_HALF_M / (2 * pack) >= rows) pack *= 2;
-                    rb.pack = pack;
                     rb.per_tile = (tile_m == 256 && G % (2 * pack) == 0) ? 2 * pack : pack;
+                    // a group of 3, 5, 6 or 7 heads: whole in one half where that has a place for each of them, so that its keys
+                    // are walked once and not a head at a time.  Pass, us, as many heads as divide the group | whole (40/8
+                    // heads): 104 x 3 tokens 50 | 18.5, 32 x 1..16 over 1,000 cached ones 121 | 37, 64 x 1 over 2,000..8,000
+                    // 1,094 | 280.  (17 to 64 rows leave room for 2 or 4 heads: as many as divide the group, as ever.)
+                    int whole = 1;
+                    while (whole < G) whole *= 2;
+                    if (pack < whole && whole <= 8 && WPP_HALF_M / whole >= rows) {
+                        pack = whole;
+                        rb.per_tile = G;
+                        whole_groups = true;
+                    }
+                    rb.pack = pack;
                     rb.rows[0] = rows;
                     rb.rows[1] = rb.per_tile == 2 * pack ? rows : 0;
                     rb.row0_b = (int32_t)r0;
@@ -515,7 +528,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
             count_steps(0, t.steps);
         } else {
             for (int hf = 0; hf < 2; ++hf)
-                for (int kk = 0; kk < t.pack && t.rows[hf] > 0; ++kk)
+                for (int kk = 0; kk < std::min(t.pack, G) && t.rows[hf] > 0; ++kk)
                     combines.push_back({t.request, u.row0[hf], t.rows[hf], u.head[hf] + kk, slots, parts, hf,
                                         kk * (WPP_HALF_M / t.pack)});
             for (int32_t q = 0; q < parts; ++q) {
@@ -554,7 +567,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     std::memset(p + off, 0, hd.plan_bytes - off);
 
     hd.magic = WPP_PLAN_MAGIC;
-    hd.version = WPP_PLAN_VERSION;
+    hd.version = whole_groups ? WPP_PLAN_VERSION_WHOLE_GROUPS : WPP_PLAN_VERSION;
     hd.desc_hash = wpp_desc_hash(&d);
     hd.num_requests = R;
     hd.num_ctas = num_ctas;
@@ -599,7 +612,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
 int wpp_check_plan(const void* plan_host, const wpp_batch_desc* resolved, const WppPlanHeader** out) {
     if (!plan_host) return WPP_ERR_INVALID_ARG;
     const WppPlanHeader* h = static_cast<const WppPlanHeader*>(plan_host);
-    if (h->magic != WPP_PLAN_MAGIC || h->version != WPP_PLAN_VERSION) return WPP_ERR_PLAN_MISMATCH;
+    if (h->magic != WPP_PLAN_MAGIC || (h->version != WPP_PLAN_VERSION && h->version != WPP_PLAN_VERSION_WHOLE_GROUPS)) return WPP_ERR_PLAN_MISMATCH;
     if (h->desc_hash != wpp_desc_hash(resolved) || h->num_requests != resolved->num_requests ||
         h->head_dim != resolved->head_dim)
         return WPP_ERR_PLAN_MISMATCH;

@@ -5,6 +5,7 @@
 
 #define WPP_PLAN_MAGIC 0x31505057u /* "WPP1" */
 #define WPP_PLAN_VERSION 8u
+#define WPP_PLAN_VERSION_WHOLE_GROUPS 9u     /* as 8, with units whose pack is larger than the group */
 #define WPP_TILE_N 128             /* keys per step */
 #define WPP_WS_HEADER_BYTES 256
 #define WPP_HALF_M 128             /* query rows per tensor-core tile (one TMEM lane per row) */
@@ -33,16 +34,17 @@ struct WppPlanHeader {
 // is rows [row0, row0+rows) of the request's chunk for `pack` consecutive query heads of that KV group
 // (head, head+1, ...): head k of the half sits in tensor rows [k*128/pack, k*128/pack + rows).  pack is 1
 // for row blocks longer than 64 rows; shorter blocks pack 2, 4 or 8 heads so that the 128-row MMA tile is not
-// mostly padding.  rows == 0 marks an unused half.  Usually the halves are consecutive row blocks of one
-// head; a short block gives the second half the next heads of the group instead.  The tile covers key steps
-// [kv_begin, kv_end) of 128 keys (absolute key = step*128 + column); each half additionally stops at its own
-// causal end.
+// mostly padding.  Where a whole KV group of 3, 5, 6 or 7 heads fits into a half, pack is 4 or 8, more than there are heads:
+// the places behind the group's last head hold nothing.  rows == 0 marks an unused half.  Usually the halves are
+// consecutive row blocks of one head; a short block gives the second half the next heads of the group instead.  The tile
+// covers key steps [kv_begin, kv_end) of 128 keys (absolute key = step*128 + column); each half additionally stops at its
+// own causal end.
 struct WppUnit {
     int32_t request, kv_begin, kv_end;
     int32_t split_slot;             // -1: writes the final output; else partial slot in the workspace
     int32_t row0[2], rows[2], head[2];
     int32_t cost;                   // 128x128 steps over both halves
-    int32_t pack;                   // query heads per half: 1, 2, 4 or 8
+    int32_t pack;                   // places for query heads per half: 1, 2, 4 or 8
 };
 
 // One half tile whose key range was split: partial slots [slot0, slot0+num_splits) merged in increasing order.

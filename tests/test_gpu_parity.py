@@ -74,6 +74,14 @@ def test_short_chunks_pack_heads(C, Hq, Hkv, d, B, splits):
     _full_parity(w, opts=wpp.PlanOpts(128, 0, splits, 0))
 
 
+@pytest.mark.parametrize("Hq,Hkv,d,B", [(5, 1, 128, 64), (10, 2, 64, 16), (12, 2, 128, 128), (7, 1, 128, 32), (6, 2, 64, 64)])
+@pytest.mark.parametrize("shape,splits", [(1, 0), (2, 0), (1, 2), (2, 3)])
+def test_whole_groups_of_three_to_seven_heads(Hq, Hkv, d, B, shape, splits):
+    """More places in a half than the group has heads: the last places compute on a head that is there already."""
+    w = W.custom_workload([300, 0, 129, 64, 5], [16, 1, 17, 32, 7], Hq, Hkv, d, B, seed=27, spare_pages=4)
+    _full_parity(w, opts=wpp.PlanOpts(0, 0, splits, 0, 0, shape))
+
+
 @pytest.mark.parametrize("tile_m,splits,ctas", [(256, 2, 3), (128, 3, 2), (256, 1, 1), (128, 1, 5)])
 def test_many_tiles_per_cta_back_to_back(tile_m, splits, ctas):
     """Few persistent CTAs walk long tile lists: a tile's first product must not overwrite the accumulator

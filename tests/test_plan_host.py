@@ -185,6 +185,29 @@ def test_short_row_blocks_pack_heads_of_one_kv_group():
     assert all(u["pack"] == 1 and u["head_b"] == u["head_a"] + 1 for u in pl100["units"]) and len(pl100["units"]) == 4
 
 
+@pytest.mark.parametrize("Hq,Hkv,C,places", [(5, 1, [1, 16, 17], 8), (40, 8, [3] * 4, 8), (12, 2, [16, 33], 8), (7, 1, [2], 8), (6, 2, [3, 32, 40], 4),
+                                             (3, 1, [32, 33, 1], 4), (9, 1, [1], 1)])
+@pytest.mark.parametrize("splits", [0, 2])
+def test_a_group_that_is_no_power_of_two_is_whole_in_a_half_that_has_room(Hq, Hkv, C, places, splits):
+    G, P = Hq // Hkv, [300] * len(C)
+    pl = parse_plan(wpp.wpp_plan_tiles(None, desc(len(C), Hq, Hkv, 128, 64, 8), P, C, opts=wpp.PlanOpts(0, 0, splits, 148), pin=False))
+    heads = {}
+    for u in pl["units"]:
+        for hf in "ab":
+            if u["rows_" + hf]:
+                n = min(u["pack"], G)
+                assert u["head_" + hf] % G + n <= G and u["rows_" + hf] <= 128 // u["pack"]
+                assert (u["pack"] == places and n == G) == (places > 1 and u["rows_" + hf] <= 128 // places)
+                for h in range(u["head_" + hf], u["head_" + hf] + n):
+                    key = (u["request"], u["row0_" + hf], h)
+                    heads[key] = heads.get(key, 0) + u["rows_" + hf] * (min(u["kv_end"], (300 + u["row0_" + hf] + u["rows_" + hf] + 127) // 128) - u["kv_begin"])
+    assert heads == {(i, 0, h): c * ((300 + c + 127) // 128) for i, c in enumerate(C) for h in range(Hq)}
+    for req, row0, rows, head, slot0, ns, half, lane0 in pl["comb"].tolist():
+        u = next(u for u in pl["units"] if u["split_slot"] == slot0)
+        assert u["head_" + "ab"[half]] + lane0 // (128 // u["pack"]) == head
+    assert len(pl["comb"]) == sum(Hq for c in C) if splits else True
+
+
 def test_few_tiles_fall_back_to_128_row_tiles_and_split_keys():
     d = desc(1, 8, 2, 64, 16, 64)
     pl = parse_plan(wpp.wpp_plan_tiles(None, d, [256], [128], pin=False))       # the single-request configuration
