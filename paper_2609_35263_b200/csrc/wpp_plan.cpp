@@ -108,8 +108,8 @@ constexpr int64_t kSmallShapeSteps = 8;
 struct StepCount {
     int64_t sum = 0;
     int32_t longest = 0, shortest = 0x7fffffff;
-    void add(int32_t n) {
-        sum += n;
+    void add(int32_t n, int64_t times = 1) {
+        sum += times * n;
         longest = std::max(longest, n);
         shortest = std::min(shortest, n);
     }
@@ -128,6 +128,24 @@ static double wide_shape_us(const StepCount& units, int64_t n_units, int64_t non
 static double small_shape_us(const StepCount& halves, int64_t n_items, int max_ctas) {
     return 0.5 + wave_us(halves, n_items, 2 * (int64_t)max_ctas, 3.0, 2.75, 1.0);
 }
+// 1: SM-wide, 2: small; `items` of the small shape
+static int shape_of(const StepCount& units, const StepCount& halves, int64_t n_units, int64_t nonempty_halves, int64_t items, int max_ctas) {
+    if (items > 2 * (int64_t)max_ctas && halves.sum > kSmallShapeSteps * items) return 1;
+    return small_shape_us(halves, items, max_ctas) <= wide_shape_us(units, n_units, nonempty_halves, max_ctas) ? 2 : 1;
+}
+
+// Tiles by length, the longest first, instead of stream order, where they are short or few.  Two things gain: the last tiles to be
+// started are the shortest, and CTAs that start their tiles together end them together, so that the heads of a group, side by
+// side in the order, go on reading the same keys at the same time; among tiles of mixed lengths they drift apart (rounds of
+// 148 equal tiles whose length alternates from round to round are as fast as sorted ones, 37 at a time are not).  Attention
+// call or pass, us, stream order | by length (new tokens over cached ones; mean key steps of a half):
+//     32 x 1,024, 64/8 heads      911 | 766 (5)       64 x 1,000 / 1,000, 32/8    1,843 | 1,683 (12)    32 x 1,000 / 2,000  1,329 | 1,340 (20)
+//     87 x 1,908, 32/8          3,835 | 3,070 (8)     40 x 500 / 1,500, 64/8      1,258 | 1,267 (14)    6 x 2,500 / 5,000   2,851 | 2,967 (50)
+//     43 x 957..1,294, 64/8     1,702 | 1,533 (5)     24 x 4,096, 64/8            6,229 | 6,209 (17)    18 x 1,217 / 3,700  1,444 | 1,564 (34)
+// Long tiles have to run beside those that read the same stream, unless they make few rounds, where the last ones count: 95 x
+// 11..76 / 655..10,600, 8/2 heads of 64, 1.6 rounds, 175 | 146, but 92 x 12 / 1,125..3,016, 16/4, 2.5 rounds, 82 | 84.  On the
+// small shape, too, only the last tiles count: 9 x 992, 40/8, ten rounds of items, 195 | 159, but 27 rounds, 32 x 512, 254 | 275.
+constexpr int64_t kLengthOrderSteps = 12, kLengthOrderTiles = 2, kLengthOrderItems = 24;       // (tiles and items: per CTA of max_ctas)
 
 // Few tiles are cut along the keys so that the CTAs have work: the part length, the tile height and the kernel shape are
 // those with the smallest estimated time.  Measured, attention call in us, every CTA given a part whatever that costs | now:
@@ -383,8 +401,35 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     //      so a page comes from DRAM once and is then hit in L2 by the other tiles; a prefix shared by many
     //      requests stays L2-resident while its KV head is being worked on.
     //      order 1: longest tile first (best balance, no regard for which tiles run together).
+    //      Where every choice is the planner's and tiles are short or few it takes that order too, equally long tiles in
+    //      stream order (see kLengthOrderSteps).
     struct Tile { int32_t rb, head; };          // row block and first head
     std::vector<Tile> tiles;
+    auto for_each_request = [&](auto&& visit) {        // the costliest first
+        std::vector<int64_t> req_cost((size_t)std::max(R, 1), 0);
+        for (const RowBlock& rb : rbs) req_cost[(size_t)rb.request] += (int64_t)rb.cost() * (Hq / rb.per_tile);
+        std::vector<int32_t> by_cost((size_t)R);
+        for (int i = 0; i < R; ++i) by_cost[(size_t)i] = i;
+        std::stable_sort(by_cost.begin(), by_cost.end(),
+                         [&](int32_t a, int32_t b) { return req_cost[(size_t)a] > req_cost[(size_t)b]; });
+        for (int i : by_cost) visit(i);
+    };
+    bool by_length = false;
+    if (o.order == 0 && o.shape == 0 && auto_tile_m && o.force_kv_splits == 0 && few_shape == 0) {
+        int64_t halves = 0;
+        StepCount unit, half;
+        for (const RowBlock& rb : rbs) {
+            const int64_t times = Hq / rb.per_tile;
+            halves += times * (rb.rows[1] > 0 ? 2 : 1);
+            unit.add(std::max(rb.end[0], rb.end[1]), times);
+            half.add(rb.end[0], times);
+            if (rb.rows[1] > 0) half.add(rb.end[1], times);
+        }
+        const int64_t items = halves > n_base ? 2 * n_base : n_base;
+        const int shape = shape_of(unit, half, n_base, halves, items, o.max_ctas);
+        by_length = shape == 2 ? items <= kLengthOrderItems * o.max_ctas
+                               : half.sum <= kLengthOrderSteps * halves || n_base <= kLengthOrderTiles * o.max_ctas;
+    }
     auto order_tiles = [&]() {
         tiles.clear();
         tiles.reserve((size_t)n_base);
@@ -393,19 +438,26 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
                 for (int h = 0; h < Hq; h += rbs[(size_t)k].per_tile) tiles.push_back({k, h});
             std::stable_sort(tiles.begin(), tiles.end(),
                              [&](const Tile& a, const Tile& b) { return rbs[(size_t)a.rb].cost() > rbs[(size_t)b.rb].cost(); });
+        } else if (by_length) {
+            std::vector<int32_t> longest_first;
+            longest_first.reserve(rbs.size());
+            for_each_request([&](int i) {
+                for (int32_t k = rb_first[(size_t)i]; k < rb_first[(size_t)i + 1]; ++k) longest_first.push_back(k);
+            });
+            std::stable_sort(longest_first.begin(), longest_first.end(),
+                             [&](int32_t a, int32_t b) { return rbs[(size_t)a].cost() > rbs[(size_t)b].cost(); });
+            for (size_t a = 0, b; a < longest_first.size(); a = b) {         // equally long ones in stream order
+                for (b = a; b < longest_first.size() && rbs[(size_t)longest_first[b]].cost() == rbs[(size_t)longest_first[a]].cost();) ++b;
+                for (int kvh = 0; kvh < d.num_kv_heads; ++kvh)
+                    for (size_t j = a; j < b; ++j)
+                        for (int h = kvh * G; h < (kvh + 1) * G; h += rbs[(size_t)longest_first[j]].per_tile) tiles.push_back({longest_first[j], h});
+            }
         } else {
-            std::vector<int64_t> req_cost((size_t)std::max(R, 1), 0);
-            for (const RowBlock& rb : rbs) req_cost[(size_t)rb.request] += (int64_t)rb.cost() * (Hq / rb.per_tile);
-            std::vector<int32_t> by_cost((size_t)R);
-            for (int i = 0; i < R; ++i) by_cost[(size_t)i] = i;
-            std::stable_sort(by_cost.begin(), by_cost.end(),
-                             [&](int32_t a, int32_t b) { return req_cost[(size_t)a] > req_cost[(size_t)b]; });
             for (int kvh = 0; kvh < d.num_kv_heads; ++kvh)
-                for (int rank = 0; rank < R; ++rank) {
-                    const int i = by_cost[(size_t)rank];
+                for_each_request([&](int i) {
                     for (int32_t k = rb_first[(size_t)i]; k < rb_first[(size_t)i + 1]; ++k)
                         for (int h = kvh * G; h < (kvh + 1) * G; h += rbs[(size_t)k].per_tile) tiles.push_back({k, h});
-                }
+                });
         }
     };
     order_tiles();
@@ -551,10 +603,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     int shape = o.shape;
     const int64_t n_items = nonempty_halves > n_units ? 2 * n_units : n_units;       // of the small shape
     if (shape == 0 && few_shape != 0) shape = few_shape;
-    else if (shape == 0)
-        shape = !(n_items > 2 * (int64_t)o.max_ctas && half_steps.sum > kSmallShapeSteps * n_items) &&
-                        small_shape_us(half_steps, n_items, o.max_ctas) <= wide_shape_us(unit_steps, n_units, nonempty_halves, o.max_ctas)
-                    ? 2 : 1;
+    else if (shape == 0) shape = shape_of(unit_steps, half_steps, n_units, nonempty_halves, n_items, o.max_ctas);
     const int num_ctas = shape == 2 ? (int)std::max<int64_t>(1, std::min<int64_t>(2 * (int64_t)o.max_ctas, 2 * n_units))
                                     : (int)std::max<int64_t>(1, std::min<int64_t>(o.max_ctas, n_units));
     off += sizeof(WppUnit) * (size_t)n_units;

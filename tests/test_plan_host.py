@@ -169,6 +169,22 @@ def test_stream_order_runs_the_tiles_of_one_kv_stream_together():
     assert all(u["request"] == 0 and u["head_a"] // 4 == 0 for u in firsts)
 
 
+@pytest.mark.parametrize("R,P,C,heads,sorted_", [(32, 0, 1024, (64, 8, 128, 64), True), (16, 0, 2048, (64, 8, 128, 64), True), (34, 1000, 500, (32, 8, 128, 64), True),
+                                                 (32, 0, 512, (64, 8, 128, 64), False),      # many rounds of the small shape
+                                                 (18, 3700, 1217, (32, 8, 128, 64), False),  # long tiles, many rounds
+                                                 (5, 1600, 300, (32, 8, 128, 64), True)])    # not two rounds of tiles
+def test_tiles_go_by_length_where_they_are_short_or_few(R, P, C, heads, sorted_):
+    d = desc(R, *heads, (P + C + heads[3] - 1) // heads[3], 10 ** 6)
+    pl = parse_plan(wpp.wpp_plan_tiles(None, d, [P] * R, [C] * R, pin=False))
+    cost = [u["cost"] for u in pl["units"]]
+    stream = parse_plan(wpp.wpp_plan_tiles(None, d, [P] * R, [C] * R, opts=wpp.PlanOpts(0, 0, 0, 0, 0, pl["shape"]), pin=False))
+    kv = [u["head_a"] // (heads[0] // heads[1]) for u in stream["units"]]
+    assert kv == sorted(kv)                              # a shape of the caller's choice keeps stream order
+    key = lambda u: sorted(u.items())
+    assert sorted(map(key, pl["units"])) == sorted(map(key, stream["units"]))
+    assert (pl["units"] != stream["units"]) == sorted_ and (not sorted_ or cost == sorted(cost, reverse=True))
+
+
 def test_short_row_blocks_pack_heads_of_one_kv_group():
     d = desc(1, 8, 2, 128, 64, 10)                  # G = 4
     pl = parse_plan(wpp.wpp_plan_tiles(None, d, [0], [300], opts=wpp.PlanOpts(256, 0, 1, 148), pin=False))
