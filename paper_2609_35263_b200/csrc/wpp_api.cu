@@ -44,9 +44,10 @@ struct wpp_ctx {
     EncodeTiledFn encode_tiled;
     void* static_scratch;           // device address of the built-in scratch array on this context's device
     // Where a moved row reference rescales O (see the attention kernel's kLate) is chosen per launch from what the
-    // kernels of earlier launches counted: key steps and steps that rescaled, added up in mapped host memory.
-    unsigned long long* stats_host; // [0] key steps, [1] rescaling steps (pinned, mapped; the kernels add to it)
-    unsigned long long* stats_dev;  // the same two words as the device sees them
+    // kernels of earlier launches counted: key steps and steps that rescaled, added up in device memory and stored to
+    // mapped host memory at a launch's end.
+    unsigned long long* stats_host; // [0] key steps, [1] rescaling steps (pinned, mapped)
+    unsigned long long* stats_dev;  // device memory: the same two, the CTAs that run, the device address of stats_host
     unsigned long long seen_steps, seen_moves;   // the counters when the choice was last looked at
     int rescale_mode;               // 0: always before the exponentials (default), 1: always after, 2: chosen from the counters
     int late_rescale;               // the current choice
@@ -130,17 +131,32 @@ extern "C" int wpp_create(wpp_ctx** out, int cuda_device) {
     }
     // two counters the attention kernels add to and the next call reads without synchronising (a missing mapping
     // only means that the choice they feed stays at its default)
+    // (a context may be made while some stream is being captured: neither may disturb the other)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     void* hp = nullptr;
     if (cudaHostAlloc(&hp, 64, cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) {
         memset(hp, 0, 64);
-        void* dp = nullptr;
-        if (cudaHostGetDevicePointer(&dp, hp, 0) == cudaSuccess) {
+        void *dp = nullptr, *words = nullptr;
+        int before = -1;
+        bool ok = cudaGetDevice(&before) == cudaSuccess && cudaSetDevice(cuda_device) == cudaSuccess &&
+                  cudaHostGetDevicePointer(&dp, hp, 0) == cudaSuccess && cudaMalloc(&words, 64) == cudaSuccess;
+        cudaStream_t st = nullptr;
+        if (ok && (ok = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess)) {
+            const unsigned long long start[4] = {0, 0, 0, (unsigned long long)reinterpret_cast<uintptr_t>(dp)};
+            ok = cudaMemcpyAsync(words, start, sizeof(start), cudaMemcpyHostToDevice, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+            cudaStreamDestroy(st);
+        }
+        if (before >= 0) cudaSetDevice(before);
+        if (ok) {
             c->stats_host = static_cast<unsigned long long*>(hp);
-            c->stats_dev = static_cast<unsigned long long*>(dp);
+            c->stats_dev = static_cast<unsigned long long*>(words);
         } else {
+            if (words) cudaFree(words);
             cudaFreeHost(hp);
         }
     }
+    cudaThreadExchangeStreamCaptureMode(&mode);
     (void)cudaGetLastError();
     *out = c;
     return WPP_OK;
@@ -149,6 +165,7 @@ extern "C" int wpp_create(wpp_ctx** out, int cuda_device) {
 extern "C" int wpp_destroy(wpp_ctx* ctx) {
     if (ctx) {
         delete ctx->map_lock;
+        if (ctx->stats_dev) cudaFree(ctx->stats_dev);
         if (ctx->stats_host) cudaFreeHost(ctx->stats_host);
     }
     free(ctx);
@@ -371,20 +388,22 @@ extern "C" int wpp_prefill_attention_varlen(const wpp_ctx* ctx, const wpp_batch_
     p.off_units = hd->off_units;
     p.num_units = hd->num_units;
     // The counter the CTAs take their tiles from starts at zero (a memset node on the caller's stream).  The small shape
-    // needs none when its items are dealt out: then nothing stands between it and the kernel before it.
+    // needs none when its items are dealt out, the SM-wide one when every tile has a CTA: then nothing stands between the
+    // kernel and the one before it.  SM-wide attention call of 2 x 4 tokens, us, with the memset and counters added on the
+    // host's side of the bus 21.0, without the latter 16.6, without either 15.3.
     int e = 0;
     p.item_shift = hd->nonempty_halves > hd->num_units ? 1 : 0;
     const int64_t items = (int64_t)hd->num_units << p.item_shift;
-    if (hd->shape == 2 && hd->deal_items) {
+    const int num_ctas = hd->shape == 2 ? (int)(items < hd->num_ctas ? items : hd->num_ctas) : hd->num_ctas;
+    if (hd->shape == 2 ? hd->deal_items != 0 : hd->num_units <= num_ctas) {
         p.tile_counter = nullptr;
     } else {
         e = (int)cudaMemsetAsync(workspace, 0, WPP_WS_HEADER_BYTES, (cudaStream_t)cuda_stream);
         if (e != 0) return cuda_fail(ctx, e);
     }
     p.stats = ctx->stats_dev;
-    e = hd->shape == 2 ? wpp_launch_attention_small(d.head_dim, tq, &tk, &tv, &p, (int)(items < hd->num_ctas ? items : hd->num_ctas), cuda_stream)
-                       : wpp_launch_attention(d.head_dim, tq, &tk, &tv, &p, hd->num_ctas, choose_late_rescale(ctx),
-                                              cuda_stream);
+    e = hd->shape == 2 ? wpp_launch_attention_small(d.head_dim, tq, &tk, &tv, &p, num_ctas, cuda_stream)
+                       : wpp_launch_attention(d.head_dim, tq, &tk, &tv, &p, num_ctas, choose_late_rescale(ctx), cuda_stream);
     if (e != 0) return cuda_fail(ctx, e);
     const_cast<wpp_ctx*>(ctx)->launches += 1;
     if (hd->num_combine > 0) {

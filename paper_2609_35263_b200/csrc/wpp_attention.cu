@@ -142,7 +142,10 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // Work tiles are not preassigned: the producer warp takes the next tile of the planner's order from a counter
     // in global memory and publishes its index to the other roles through a small queue in shared memory, so the
     // CTAs of the grid always work on neighbouring tiles of that order (which share K/V pages, see the planner)
-    // however their speeds differ, and the tail balances itself.
+    // however their speeds differ, and the tail balances itself.  (Tiles of CTAs that the hardware has not started, taken over
+    // with launch_cancel_request, need no counter, but come in another order: 32 x 1,024 tokens 787 us | 833.)  A wave
+    // with a CTA for every tile needs none: nothing has to be zeroed in front of it, and it is set up while the
+    // kernel before it runs.
     const uint32_t bTileFull = bHalf + 96, bTileEmpty = bTileFull + 8 * C::kTileQ;
     float2* s_final = reinterpret_cast<float2*>(smem_gen + C::kOffFinal);     // [2][128] (reference in log2 units, l)
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + C::kOffMisc);
@@ -178,6 +181,8 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     grid_launch_dependents();
+    grid_dependency_wait();           // (launched while the kernel before may still be running)
+    if (p.stats && threadIdx.x == 0) atomicAdd(p.stats + 2, 1ull);
 
     const char* plan = static_cast<const char*>(p.plan);
     const WppPlanHeader* hd = reinterpret_cast<const WppPlanHeader*>(plan);
@@ -212,7 +217,7 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 // take the next tile of the planner's order (the first one is this CTA's own) and tell the other roles
                 int u = (int)blockIdx.x;
                 if (!first) {
-                    if (lane == 0) u = (int)(gridDim.x + atomicAdd(p.tile_counter, 1u));
+                    if (lane == 0) u = p.tile_counter ? (int)(gridDim.x + atomicAdd(p.tile_counter, 1u)) : num_units;
                     u = __shfl_sync(0xffffffffu, u, 0);
                 }
                 first = false;
@@ -656,11 +661,9 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             s_final[hf * 128 + r] = make_float2(-nmc, l_run);
             mbar_arrive(bFinalReady(hf));
         }
-        // the launch's counters live behind the tile counter in the workspace header (zeroed with it)
         if (p.stats && lane == 0 && n_steps_seen) {
-            unsigned long long* ws_stats = reinterpret_cast<unsigned long long*>(p.tile_counter) + 1;
-            atomicAdd(ws_stats, (unsigned long long)n_steps_seen);
-            atomicAdd(ws_stats + 1, (unsigned long long)n_moves_seen);
+            atomicAdd(p.stats, (unsigned long long)n_steps_seen);
+            atomicAdd(p.stats + 1, (unsigned long long)n_moves_seen);
         }
     }
 
@@ -678,15 +681,21 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         tc_fence_after();
         tmem_dealloc(tmem, kTmemCols);
     }
-    // the last CTA to get here hands the launch's two counters to the caller's words (mapped host memory: two
-    // transactions per launch, where one per warp would cost milliseconds)
+    // The context's counters go to the two words that the host sees when the last CTA that runs has counted: plain stores, and
+    // not additions, whose answers would come back over the bus (4 us of every launch).  Launches in several streams may get
+    // here together: whoever stored what has changed meanwhile stores again.
     if (p.stats && threadIdx.x == 0) {
-        unsigned long long* ws_stats = reinterpret_cast<unsigned long long*>(p.tile_counter) + 1;
         __threadfence();
-        if (atomicAdd(reinterpret_cast<unsigned int*>(ws_stats + 2), 1u) == gridDim.x - 1) {
-            __threadfence();
-            atomicAdd_system(p.stats, atomicAdd(ws_stats, 0ull));
-            atomicAdd_system(p.stats + 1, atomicAdd(ws_stats + 1, 0ull));
+        if (atomicAdd(p.stats + 2, ~0ull) == 1ull) {
+            volatile unsigned long long* host = reinterpret_cast<volatile unsigned long long*>(p.stats[3]);
+            unsigned long long steps = atomicAdd(p.stats, 0ull), moves = atomicAdd(p.stats + 1, 0ull), seen;
+            do {
+                seen = steps;
+                host[0] = steps;
+                host[1] = moves;
+                moves = atomicAdd(p.stats + 1, 0ull);
+                steps = atomicAdd(p.stats, 0ull);
+            } while (steps != seen);
         }
     }
 }
@@ -703,8 +712,17 @@ static cudaError_t launch(const CUtensorMap* tq, const CUtensorMap& tk, const CU
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
     }
-    wpp_attn_kernel<D, kLate><<<num_ctas, kThreads, Cfg<D>::kSmemBytes, stream>>>(tq[0], tq[1], tq[2], tq[3], tk, tv, p);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)num_ctas);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Cfg<D>::kSmemBytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute overlap;
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &overlap;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, wpp_attn_kernel<D, kLate>, tq[0], tq[1], tq[2], tq[3], tk, tv, p);
 }
 
 }  // namespace wpp

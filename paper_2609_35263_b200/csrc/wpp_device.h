@@ -19,8 +19,10 @@ struct AttnParams {
     float* ws_lse;                   // [slots][2][128], log2 units
     int32_t* status;                 // sticky device status word or null
     uint32_t* tile_counter;          // zeroed before the launch: how many tiles have been taken beyond the first one per CTA;
-                                     // or null (small shape): round k of the CTAs takes tiles k gridDim .., rotated by k
-    unsigned long long* stats;       // or null: [0] += key steps of the softmax warps, [1] += those that rescaled O
+                                     // or null: every CTA has one tile; (small shape) round k of the CTAs takes tiles k gridDim ..,
+                                     // rotated by k
+    unsigned long long* stats;       // or null: [0] += key steps of the softmax warps, [1] += those that rescaled O, [2] CTAs
+                                     // that run, [3] where the host sees the first two
     int64_t o_token_stride, o_head_stride;
     int32_t num_q_heads, group, page_size, max_blocks, num_pages;
     float scale_log2;                // sm_scale * log2(e)
@@ -47,6 +49,7 @@ struct AppendParams {
     int64_t kvnew_token_stride, kvnew_head_stride;       // in 16-byte units
     int64_t kv_page_stride, kv_head_stride, kv_token_stride;
     int32_t num_requests, num_kv_heads, vec_per_row, page_size, max_blocks, num_pages;
+    int32_t few;                     // the SMs hold the whole grid at once
     int64_t total_new_tokens;
 };
 

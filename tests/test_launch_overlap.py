@@ -74,3 +74,44 @@ def test_small_attention_directly_behind_the_two_pass_recurrent_layer():
         assert torch.equal(out, apart["out"])
         assert np.array_equal(out_kda.float().cpu().double().numpy(), o_apart)
         assert np.array_equal(d["state_pool"].cpu().double().numpy(), pool_apart)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [1, 2])
+@pytest.mark.parametrize("P,C", [([300, 64], [33, 90]), ([0, 70, 5], [700, 600, 130]), ([5000], [40])])
+def test_passes_one_behind_the_other_see_their_own_keys(P, C, shape):
+    """Append and attention of successive passes are set up while the kernel before them runs, append over the same pages each
+    time: every pass has the results it has alone.  (Waves of one tile per CTA, of several, and cut along the keys.)"""
+    import torch
+
+    import paper_2609_35263_b200 as wpp
+    import wpp_workloads as W
+    from tests import gpu_harness as H
+
+    w = W.custom_workload(P, C, 8, 2, 128, 64, seed=31, spare_pages=4)
+    g, d, dev = H.device_inputs(w), H.desc_of(w), torch.device("cuda")
+    plan = wpp.wpp_plan_tiles(H.ctx(), d, w.prefix_lens, w.chunk_lens, opts=wpp.PlanOpts(0, 0, 0, 0, 0, shape)).to_device(dev)
+    i32 = lambda a: torch.from_numpy(a.astype("int32")).to(dev)
+    Pd, Cd, bt = i32(w.prefix_lens), i32(w.chunk_lens), i32(w.block_tables)
+    ws = torch.empty(int(plan.info.workspace_bytes), dtype=torch.uint8, device=dev)
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    new = [(g["k_new"] * f, g["v_new"] * f) for f in (1.0, -0.5, 0.25, 2.0)]
+
+    def one(k, v, out):
+        wpp.wpp_kv_append(H.ctx(), d, k, v, g["k_pool"], g["v_pool"], bt, Pd, Cd, plan, status=status)
+        wpp.wpp_prefill_attention_varlen(H.ctx(), d, g["q"], out, None, g["k_pool"], g["v_pool"], bt, Pd, Cd, plan, workspace=ws, status=status)
+
+    alone = []
+    for k, v in new:
+        out = torch.zeros_like(g["q"])
+        one(k, v, out)
+        torch.cuda.synchronize()
+        alone.append(out)
+    for _ in range(5):
+        outs = [torch.zeros_like(g["q"]) for _ in new]
+        torch.cuda.synchronize()
+        for (k, v), out in zip(new, outs):
+            one(k, v, out)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0 and all(torch.equal(a, b) for a, b in zip(alone, outs))
+    assert not torch.equal(alone[0], alone[1])
