@@ -61,7 +61,7 @@ struct Cfg {
     static constexpr int kOffKV = 2 * kTileBytes;
     static constexpr int kOffBars = kOffKV + kSlots * kTileBytes;
     static constexpr int kTileQ = 2;                       // tile ids the producer may publish ahead
-    static constexpr int kNumBars = 2 + 2 * kSlots + 1 + 6 * 2 + 2 * kTileQ;
+    static constexpr int kNumBars = 2 + 2 * kSlots + 1 + 6 * 2 + 2 * kTileQ + 2;
     static constexpr int kOffFinal = kOffBars + 8 * kNumBars;          // float2 (m, l)[2][128]
     static constexpr int kOffStage = (kOffFinal + 2 * 128 * 8 + 15) / 16 * 16;   // 4 x 2 KB: the epilogue warps' store staging (16-byte chunks)
     static constexpr int kOffMisc = kOffStage + 4 * 2048;              // tmem ptr, abort flag, tile ids
@@ -147,9 +147,13 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // with a CTA for every tile needs none: nothing has to be zeroed in front of it, and it is set up while the
     // kernel before it runs.
     const uint32_t bTileFull = bHalf + 96, bTileEmpty = bTileFull + 8 * C::kTileQ;
+    // v_ask: the last V of a sequence has landed and is next (which slot, how many rows: v_rows), or there are no more; v_end: its
+    // rows past the sequence are zero
+    const uint32_t bVAsk = bTileEmpty + 8 * C::kTileQ, bVEnd = bVAsk + 8;
     float2* s_final = reinterpret_cast<float2*>(smem_gen + C::kOffFinal);     // [2][128] (reference in log2 units, l)
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_gen + C::kOffMisc);
     volatile uint32_t* abort_flag = tmem_slot + 1;
+    volatile int32_t* v_rows = reinterpret_cast<volatile int32_t*>(tmem_slot + 2);        // [2]: slot (-1: no more), rows
     volatile int32_t* tile_ids = reinterpret_cast<volatile int32_t*>(tmem_slot + 4);      // [kTileQ]
     constexpr uint32_t kTileConsumers = 2 + 256 + 128;   // two issuing threads, softmax threads, epilogue threads
 
@@ -165,6 +169,7 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             mbar_init(bFinalReady(h), 128); mbar_init(bOFinal(h), 1); mbar_init(bOFree(h), 128);
         }
         for (int i = 0; i < C::kTileQ; ++i) { mbar_init(bTileFull + 8 * i, 1); mbar_init(bTileEmpty + 8 * i, kTileConsumers); }
+        mbar_init(bVAsk, 1); mbar_init(bVEnd, 1);
         *abort_flag = 0u;
         fence_barrier_init();
     }
@@ -348,7 +353,7 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             // ================================================================ issuer of O += P V (one thread)
             // O_A += P_A V(0), O_B += P_B V(0), O_A += P_A V(1), ...: each product waits for its P.
             Ring ring = {0, 0};
-            uint32_t p_phase[2] = {0, 0}, of_phase[2] = {0, 0};
+            uint32_t p_phase[2] = {0, 0}, of_phase[2] = {0, 0}, ve_phase = 0;
             constexpr uint32_t idesc_pv = idesc_bf16(D, 0, 1);
             const uint64_t v_desc0 = smem_desc_sw128(sKV, C::kHalfBytes, 1024);       // + stage * (kTileBytes >> 4)
             bool dead = false;
@@ -364,14 +369,13 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         if (!ok) { dead = true; break; }
                     }
                     const int valid = v.kv_len - (v.kv_begin + k) * 128;      // keys of this step that exist
-                    if (valid < 128) {
-                        // rows past the end of the sequence may hold anything (stale slots, never-loaded
-                        // pages): zero them so that 0 * garbage cannot reach O
-                        uint8_t* vg = smem_gen + C::kOffKV + ring.stage * C::kTileBytes;
-                        for (int h = 0; h < C::kHalves; ++h)
-                            for (int i = valid * 8; i < 128 * 8; ++i)
-                                *reinterpret_cast<uint4*>(vg + h * C::kHalfBytes + i * 16) = make_uint4(0, 0, 0, 0);
-                        fence_proxy_async_smem();
+                    if (valid < 128) {                                        // warp 15 zeroes the rows past them
+                        v_rows[0] = (int32_t)ring.stage;
+                        v_rows[1] = valid;
+                        mbar_arrive(bVAsk);
+                        const bool ok = mbar_wait(bVEnd, ve_phase, abort_flag);
+                        if (!ok) { dead = true; break; }
+                        ve_phase ^= 1u;
                     }
                     const uint64_t vd = v_desc0 + (uint64_t)(ring.stage * (C::kTileBytes >> 4));
 #pragma unroll
@@ -401,6 +405,33 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     mma_commit(bSlotEmpty + 8 * ring.stage);                          // V(k) has been read
                     ring.advance(n_v);
                 }
+            }
+            v_rows[0] = -1;
+            mbar_arrive(bVAsk);
+        } else if (warp == 15) {
+            // ================================================================ the end of a sequence
+            // Rows of V past it may hold anything (stale slots, pages never loaded): they are zeroed so that 0 * garbage cannot
+            // reach O.  A warp does it for the issuing thread, while the softmax of the step is under way: by itself that took up
+            // to 2,000 stores in front of its product (2 x 4 tokens, attention call, 15.3 us | 10.1; pass, 34 x 427..576 over
+            // 1,000, 32/8 heads, 499 | 450).  It is asked, and does not follow the tiles itself: one more role in the hand-over of
+            // tiles cost long waves 2 to 5 %.
+            uint32_t va_phase = 0;
+            while (true) {
+                bool ok = false;
+                const long long t0 = clock64();
+                // (nothing to do may last as long as the launch; the issuing thread's own waits have the usual limit)
+                while (!(ok = mbar_try_wait(bVAsk, va_phase) != 0u) && !*abort_flag && clock64() - t0 < 64 * WPP_WAIT_LIMIT) { }
+                if (!__all_sync(0xffffffffu, ok)) break;
+                va_phase ^= 1u;
+                const int slot = v_rows[0], valid = v_rows[1];
+                if (slot < 0) break;
+                uint8_t* vg = smem_gen + C::kOffKV + slot * C::kTileBytes;
+                for (int h = 0; h < C::kHalves; ++h)
+                    for (int i = valid * 8 + lane; i < 128 * 8; i += 32)
+                        *reinterpret_cast<uint4*>(vg + h * C::kHalfBytes + i * 16) = make_uint4(0, 0, 0, 0);
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bVEnd);
             }
         }
     } else if (wg == 2) {

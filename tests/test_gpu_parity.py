@@ -248,6 +248,31 @@ def test_results_do_not_depend_on_which_cta_takes_which_tile(shape):
                 assert torch.equal(ref[key][1], r["lse"]), (order, splits)
 
 
+@pytest.mark.parametrize("d,B", [(128, 64), (64, 16)])
+@pytest.mark.parametrize("ctas", [1, 3])
+def test_the_end_of_every_sequence_is_zeroed_before_its_product(d, B, ctas):
+    """The SM-wide shape hands the rows of V past a sequence's end to a warp of their own: ends after 1, 16, 63, 64, 127 and 128
+    keys of a step, in tiles of one step and of several, one behind the other in a CTA, NaN patterns behind every end."""
+    ends = [1, 127, 64, 63, 128, 16, 127, 1]
+    P = [0, 0, 200, 300, 0, 129, 500, 640]
+    C = [e if p == 0 else (e - p) % 128 or 128 for e, p in zip(ends, P)]
+    w = W.custom_workload(P, C, 4, 2, d, B, seed=33, spare_pages=6)
+    inp = cpu_inputs(w)
+    kp, vp = bits(inp["k_pool"]).copy(), bits(inp["v_pool"]).copy()
+    live = np.zeros((w.num_pages, w.page_size), dtype=bool)
+    for i in range(w.num_requests):
+        for pos in range(int(w.prefix_lens[i])):
+            live[w.block_tables[i, pos // w.page_size], pos % w.page_size] = True
+    dead = np.broadcast_to(~live[:, None, :, None], kp.shape)
+    kp[dead], vp[dead] = 0x7FC0, 0xFFFF
+    inp = dict(inp, k_pool=from_bits(kp), v_pool=from_bits(vp))
+    _, _, ref, _ = run_oracle(w, inp)
+    for rep in range(4):
+        res = H.run_wave(w, H.device_inputs(w, inp), opts=wpp.PlanOpts(256 if rep % 2 else 128, 0, 1, ctas), shape=1)
+        assert res["status"] == 0
+        H.assert_close(f64(res["out"]), ref, f"ends of sequences, {ctas} CTAs, repeat {rep}")
+
+
 def test_stale_slots_unused_pages_and_scratch_poison_do_not_matter():
     """NaN bit patterns everywhere the method must not look: slots past the sequence end, unreferenced pages."""
     w = W.custom_workload([90, 3, 0], [40, 200, 5], 4, 2, 128, 64, seed=13, spare_pages=6)
