@@ -312,6 +312,8 @@ extern "C" int wpp_kv_append(const wpp_ctx* ctx, const wpp_batch_desc* desc, con
     p.max_blocks = d.max_blocks_per_req;
     p.num_pages = d.num_pages;
     p.total_new_tokens = hd->total_new_tokens;
+    p.off_q_offsets = hd->off_q_offsets;
+    p.off_prefix = hd->off_prefix;
     int e = wpp_launch_append(&p, ctx->sm_count, cuda_stream);
     if (e != 0) return cuda_fail(ctx, e);
     const_cast<wpp_ctx*>(ctx)->launches += 1;

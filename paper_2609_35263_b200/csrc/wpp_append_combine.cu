@@ -9,53 +9,79 @@
 
 namespace wpp {
 
-// One thread moves one 16-byte vector of K and the matching vector of V.  A vector index decomposes as
-// (token, kv head, vector within the head row); the request is found by bisection in the row offsets.
+// One thread moves one 16-byte vector of K and the matching vector of V, or kVec of each.  A vector index decomposes as
+// (token, kv head, vector within the head row).
 // A request whose span on the device (prefix_lens, chunk_lens) is not the span the plan was made for is refused:
 // nothing of it is written and the status word becomes WPP_ERR_PLAN_MISMATCH (Section 4.6: a position mismatch
 // fails execution instead of writing against the wrong cache state).
+//
+// What bounds a small append is its chain of dependent loads, a large one HBM.  The new rows, which depend on nothing, are
+// asked for first; the request is found by a search whose every step is one load of 32 offsets by the warp (a bisection by
+// each thread was up to seven dependent loads), the plan's offsets come with the launch, and a token is divided out once per
+// warp.  Append in a graph, us, a bisection in front of the loads | now: 128 x 3 tokens (64/8 heads) 3.4 | 2.7, 32 x 64 4.3 |
+// 4.2, 32 x 256 11.8 | 10.4, 32 x 1,024 47.5 | 47.2 (5.7 TB/s).
 //
 // A grid that the SMs hold at once (`few`) is set up while the kernel before it runs, which is worth 2 us, and lets the
 // attention kernel in as its CTAs end; a larger one starts behind the kernel before and lets the attention kernel in at once.
 // Pass, us, the latter for all | the former for all: 1 x 128 tokens over 256 (8/2 heads) 14.3 | 12.5, 32 x 64 (64/8) 25.5 |
 // 24.6, 5 x 32..276 over 100..4,000 63.3 | 59.7, but 32 x 512 304 | 309.
+constexpr int kAppendVec = 4;          // of a large grid (1: 11.2 us for 32 x 256 tokens, 2: 10.5, 8: 13.5)
+template <int kVec>
 __global__ void __launch_bounds__(256) wpp_append_kernel(const AppendParams p) {
     if (!p.few) grid_launch_dependents();
     grid_dependency_wait();
     const char* plan = static_cast<const char*>(p.plan);
-    const WppPlanHeader* hd = reinterpret_cast<const WppPlanHeader*>(plan);
-    const int32_t* q_offsets = reinterpret_cast<const int32_t*>(plan + hd->off_q_offsets);
-    const int32_t* plan_prefix = reinterpret_cast<const int32_t*>(plan + hd->off_prefix);
-    const int64_t per_token = (int64_t)p.num_kv_heads * p.vec_per_row;
+    const int32_t* q_offsets = reinterpret_cast<const int32_t*>(plan + p.off_q_offsets);
+    const int32_t* plan_prefix = reinterpret_cast<const int32_t*>(plan + p.off_prefix);
+    const uint32_t per_token = (uint32_t)(p.num_kv_heads * p.vec_per_row);
     const int64_t total = p.total_new_tokens * per_token;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < total; v += stride) {
-        const int64_t tok = v / per_token;
-        const int rem = (int)(v - tok * per_token);
-        const int h = rem / p.vec_per_row, c = rem - h * p.vec_per_row;
-        int lo = 0, hi = p.num_requests;          // largest i with q_offsets[i] <= tok
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * kVec;
+    for (int64_t first = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) * kVec; first < total; first += stride) {
+        const int64_t tok0 = first / per_token;                           // of the warp's first vector
+        const uint32_t rem0 = (uint32_t)(first - tok0 * per_token);
+        int tok[kVec];
+        uint32_t h[kVec], c[kVec];
+        uint4 kv[kVec], vv[kVec];
+#pragma unroll
+        for (int u = 0; u < kVec; ++u) {
+            const uint32_t r = rem0 + u * 32 + lane, t = r / per_token, in_token = r - t * per_token;
+            tok[u] = first + u * 32 + lane < total ? (int)(tok0 + t) : -1;
+            h[u] = in_token / (uint32_t)p.vec_per_row;
+            c[u] = in_token - h[u] * (uint32_t)p.vec_per_row;
+            if (tok[u] < 0) continue;
+            const int64_t src = (int64_t)tok[u] * p.kvnew_token_stride + h[u] * p.kvnew_head_stride + c[u];
+            kv[u] = p.k_new[src];
+            vv[u] = p.v_new[src];
+        }
+        int lo = 0, hi = p.num_requests;          // largest i with q_offsets[i] <= tok0
         while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (q_offsets[mid] <= tok) lo = mid; else hi = mid;
+            const int width = (hi - lo + 31) / 32, i = lo + lane * width;
+            const unsigned le = __ballot_sync(0xffffffffu, i < hi && q_offsets[i] <= tok0) | 1u;
+            const int last = 31 - __clz((int)le);
+            hi = min(hi, lo + (last + 1) * width);
+            lo += last * width;
         }
-        const int P = p.prefix_lens[lo];
-        if (P != plan_prefix[lo] || p.chunk_lens[lo] != q_offsets[lo + 1] - q_offsets[lo]) {
-            if (p.status) atomicCAS(p.status, 0, WPP_ERR_PLAN_MISMATCH);
-            continue;
+#pragma unroll
+        for (int u = 0; u < kVec; ++u) {
+            if (tok[u] < 0) continue;
+            while (lo + 1 < p.num_requests && q_offsets[lo + 1] <= tok[u]) ++lo;          // (a thread's tokens ascend)
+            const int P = p.prefix_lens[lo], at = q_offsets[lo];
+            if (P != plan_prefix[lo] || p.chunk_lens[lo] != q_offsets[lo + 1] - at) {
+                if (p.status) atomicCAS(p.status, 0, WPP_ERR_PLAN_MISMATCH);
+                continue;
+            }
+            const int pos = P + (tok[u] - at);
+            const int blk = pos / p.page_size, slot = pos - blk * p.page_size;
+            const int page = (blk < p.max_blocks) ? p.block_tables[(int64_t)lo * p.max_blocks + blk] : -1;
+            if (page < 0 || page >= p.num_pages) {
+                if (p.status) atomicCAS(p.status, 0, WPP_ERR_BOUNDS);
+                continue;
+            }
+            const int64_t dst = page * p.kv_page_stride + h[u] * p.kv_head_stride + slot * p.kv_token_stride + c[u];
+            p.k_cache[dst] = kv[u];
+            p.v_cache[dst] = vv[u];
         }
-        const int pos = P + (int)(tok - q_offsets[lo]);
-        const int blk = pos / p.page_size, slot = pos - blk * p.page_size;
-        const int page = (blk < p.max_blocks) ? p.block_tables[(int64_t)lo * p.max_blocks + blk] : -1;
-        if (page < 0 || page >= p.num_pages) {
-            if (p.status) atomicCAS(p.status, 0, WPP_ERR_BOUNDS);
-            continue;
-        }
-        const int64_t src = tok * p.kvnew_token_stride + h * p.kvnew_head_stride + c;
-        const int64_t dst = page * p.kv_page_stride + h * p.kv_head_stride + slot * p.kv_token_stride + c;
-        const uint4 kv = p.k_new[src];
-        const uint4 vv = p.v_new[src];
-        p.k_cache[dst] = kv;
-        p.v_cache[dst] = vv;
     }
 }
 
@@ -164,8 +190,11 @@ extern "C" int wpp_launch_selftest_wait(long long limit_cycles, int32_t* status,
 extern "C" int wpp_launch_append(const wpp::AppendParams* p, int num_sms, void* stream) {
     const int64_t total = p->total_new_tokens * p->num_kv_heads * p->vec_per_row;
     if (total == 0) return 0;
-    int64_t blocks = (total + 255) / 256;
-    const int64_t cap = (int64_t)num_sms * 16;
+    wpp::AppendParams q = *p;
+    q.few = total <= (int64_t)num_sms * 8 * 256;
+    const int per_block = q.few ? 256 : 256 * wpp::kAppendVec;
+    int64_t blocks = (total + per_block - 1) / per_block;
+    const int64_t cap = (int64_t)num_sms * 8;
     if (blocks > cap) blocks = cap;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
@@ -174,11 +203,9 @@ extern "C" int wpp_launch_append(const wpp::AppendParams* p, int num_sms, void* 
     cudaLaunchAttribute overlap;
     overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     overlap.val.programmaticStreamSerializationAllowed = 1;
-    wpp::AppendParams q = *p;
-    q.few = blocks <= (int64_t)num_sms * 8;
     cfg.attrs = &overlap;
     cfg.numAttrs = q.few ? 1 : 0;
-    return (int)cudaLaunchKernelEx(&cfg, wpp::wpp_append_kernel, q);
+    return (int)cudaLaunchKernelEx(&cfg, q.few ? wpp::wpp_append_kernel<1> : wpp::wpp_append_kernel<wpp::kAppendVec>, q);
 }
 
 extern "C" int wpp_launch_combine(const wpp::CombineParams* p, int num_combine, void* stream) {

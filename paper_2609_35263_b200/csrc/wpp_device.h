@@ -50,6 +50,7 @@ struct AppendParams {
     int64_t kv_page_stride, kv_head_stride, kv_token_stride;
     int32_t num_requests, num_kv_heads, vec_per_row, page_size, max_blocks, num_pages;
     int32_t few;                     // the SMs hold the whole grid at once
+    uint32_t off_q_offsets, off_prefix;                  // of the plan's arrays (as in its header: one dependent read less)
     int64_t total_new_tokens;
 };
 

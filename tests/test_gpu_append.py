@@ -33,6 +33,21 @@ def test_append_is_bit_exact(P, C, Hkv, d, B):
     assert np.array_equal(bits(res["v_pool"]), vp)
 
 
+@pytest.mark.parametrize("R,most,Hkv,d,B", [(33, 5, 1, 64, 16), (1100, 3, 1, 64, 16), (70, 40, 3, 128, 32), (700, 30, 5, 64, 16), (45, 170, 8, 128, 64)])
+def test_append_finds_every_request(R, most, Hkv, d, B):
+    """More requests than one search step tells apart, empty chunks among them, several requests' tokens in a warp, and sizes on
+    both sides of the one from which a thread moves several vectors (303,104 vectors on 148 SMs; the last two)."""
+    rng = np.random.default_rng(R)
+    C = rng.integers(0, most + 1, R).tolist()
+    C[0], C[-1] = 0, max(1, C[-1])
+    w = W.custom_workload(rng.integers(0, 50, R).tolist(), C, Hkv, Hkv, d, B, seed=R, spare_pages=3)
+    inp = cpu_inputs(w)
+    kp, vp = oracle.oracle_append(inp["k_new"], inp["v_new"], inp["k_pool"], inp["v_pool"], w.block_tables, w.prefix_lens, w.chunk_lens)
+    res = H.run_wave(w, H.device_inputs(w, inp), do_attention=False)
+    assert res["status"] == 0
+    assert np.array_equal(bits(res["k_pool"]), kp) and np.array_equal(bits(res["v_pool"]), vp)
+
+
 def test_append_shared_prefix_pages_are_left_alone():
     rng = np.random.default_rng(22)
     w = W.make_workload("shared", 22, rng, [128, 150, 128], [64, 10, 100], 4, 2, 128, 64, shared_tokens=128,
