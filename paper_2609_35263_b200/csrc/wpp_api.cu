@@ -488,33 +488,59 @@ extern "C" size_t wpp_kda_workspace_bytes(const wpp_kda_desc* desc) {
 constexpr double kPrepUs = 0.9e-3, kChainUs = 0.0525, kOperandsUs = 0.49e-3, kSegmentUs = 12.0;
 
 // Segments of the two-pass form.  Few long chains leave most SMs idle: the chunk is cut so that a segment's preparation runs
-// beside the chain of the segment before.  Each segment is longer than the one before by what the chain takes longer per
-// block than the preparation on the SMs left, so that only the first segment's preparation is waited for.  Returns the
-// number of segments with the smallest estimated time, which comes back in *us, and where they begin, in blocks.
-// 1 x 16,384 tokens x 32 heads: in one piece 1340 us, 4 equal segments 1060, 8 equal ones 1068.
-constexpr int kMaxSegments = 6;
+// beside the chain of the segment before.  A preparation takes whole rounds of items on its CTAs (two per SM; kRoundUs each
+// on all SMs, kBesideUs beside a chain) and a start; a segment has as many rounds as fit beside the chain before it, so that
+// only the first segment's preparation is waited for, whose rounds are those with the smallest total.  Returns the number of
+// segments and where they begin, in blocks; *us: the estimate that the choice between the forms goes by.
+// 1 x 16,384 tokens x 32 heads, us: in one piece 1,340, 4 equal segments 1,060, six that grow by the ratio of the two rates from
+// 14 blocks on 1,093 (every chain but the last was done 20 to 37 us before the preparation beside it), so, five from 37 blocks on,
+// 1,034 with no chain waiting; 1 x 8,192 579 | 562, 1 x 4,096 318 | 309, 1 x 2,048 190 | 181, 1 x 12,000 x 16 heads 771 | 743,
+// 3,000 and 5,000 tokens x 16 heads 369 | 355.
+constexpr int kMaxSegments = 8, kMaxFirstRounds = 8;
+constexpr double kRoundUs = 18.0, kBesideUs = 20.0, kStartUs = 6.0, kGapUs = 12.0;      // (kGapUs: from a chain's last step to the next one's first)
 static int kda_segments(const wpp_kda_desc* d, int sms, double* us, int32_t* begin) {
     const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
     const double prep = n * C * kPrepUs * 148 / sms, operands = n * C * kOperandsUs, chain = ceil(n / sms) * C * kChainUs;
     const int64_t blocks = d->total_tokens / d->num_requests / 64 + 1;
-    int best = 1;
-    double best_us = prep + (chain > operands ? chain : operands);
     const double growth = 2 * n <= sms ? chain / (prep * sms / (sms - n)) : 0.0;
-    double best_first = 1.0;
-    for (int s = 2; growth > 1.05 && s <= kMaxSegments; ++s) {
-        const double g = growth < 4.0 ? growth : 4.0, first = (g - 1.0) / (pow(g, s) - 1.0);
-        if (first * (double)blocks < 4.0) break;
-        const double t = prep * first + chain + kSegmentUs * (s - 1);
-        if (t < best_us) { best = s; best_us = t; best_first = first; }
+    if (us) {
+        *us = prep + (chain > operands ? chain : operands);
+        for (int s = 2; growth > 1.05 && s <= 6; ++s) {
+            const double g = growth < 4.0 ? growth : 4.0, first = (g - 1.0) / (pow(g, s) - 1.0);
+            if (first * (double)blocks < 4.0) break;
+            const double t = prep * first + chain + kSegmentUs * (s - 1);
+            if (t < *us) *us = t;
+        }
     }
-    if (us) *us = best_us;
-    if (begin) {
-        const double g = growth < 4.0 ? growth : 4.0;
-        double at = 0.0, len = best_first;
-        for (int s = 0; s < best; ++s) {
-            begin[s] = (int32_t)(at * (double)blocks);
-            at += len;
-            len *= g;
+    int best = 1;
+    if (begin) begin[0] = 0;
+    if (!begin || !(growth > 1.05)) return best;
+    const double step = 64 * kChainUs, all = 2.0 * sms, beside = 2.0 * (sms - n);
+    double best_us = ceil((double)blocks * n / all) * kRoundUs + (double)blocks * step;
+    for (int candidate = 0; candidate < kMaxFirstRounds * (kMaxSegments - 1); ++candidate) {
+        const int rounds = 1 + candidate / (kMaxSegments - 1), most = 2 + candidate % (kMaxSegments - 1);      // of the first one; segments
+        if (rounds * all >= (double)blocks * n) break;
+        int32_t at[kMaxSegments] = {0};
+        int64_t len = (int64_t)(rounds * all / n), done = 0;
+        double t = rounds * kRoundUs;
+        int s = 0;
+        while (true) {
+            if (len < 1 || s == most - 1 || len > blocks - done) len = blocks - done;
+            if (s > 0) {
+                const double ready = ceil((double)len * n / beside) * kBesideUs + kStartUs, busy = (double)(done - at[s - 1]) * step + kGapUs;
+                t += ready > busy ? ready : busy;
+            }
+            at[s++] = (int32_t)done;
+            done += len;
+            if (done >= blocks) break;
+            const double fit = floor(((double)len * step + kGapUs - kStartUs) / kBesideUs);
+            len = (int64_t)((fit > 1.0 ? fit : 1.0) * beside / n);
+        }
+        t += (double)(blocks - at[s - 1]) * step;
+        if (t < best_us) {
+            best = s;
+            best_us = t;
+            for (int i = 0; i < s; ++i) begin[i] = at[i];
         }
     }
     return best;
