@@ -212,7 +212,37 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // that the thread issuing S = Q K^T and the thread issuing O += P V walk their own ring.  (A third K
         // slot, which would still fit, was measured and makes no difference.)
         const uint32_t n_v = C::kSlots / 2, n_k = C::kSlots - n_v;
-        if (warp == 13) {
+        if (warp == 15) {
+            // ================================================================ the end of a sequence
+            // Rows of V past it may hold anything (stale slots, pages never loaded): they are zeroed so that 0 * garbage cannot
+            // reach O.  A warp does it for the issuing thread, while the softmax of the step is under way: by itself that took up
+            // to 2,000 stores in front of its product (2 x 4 tokens, attention call, 15.3 us | 10.1; pass, 34 x 427..576 over
+            // 1,000, 32/8 heads, 499 | 450).  It is asked, and does not follow the tiles itself: one more role in the hand-over of
+            // tiles cost long waves 2 to 5 %.  It stands in front of the other roles and looks every 256 ns instead of waiting at the
+            // barrier, which costs nothing measurable at the short end: behind them and waiting, 2 x 8,192 tokens over 98,304, 64/8
+            // heads, 43.25 ms | 42.90 (without the role 42.87), 25 x 3,505..6,285 over 3,000..9,000, 32/8, 14.96 | 14.89 (14.91);
+            // in front and waiting 43.06 and 14.90, every 1,000 ns 43.01 and 14.89; 40 x 200..500 over 3,000..6,000, 2,152 us |
+            // 2,136.
+            uint32_t va_phase = 0;
+            while (true) {
+                bool ok = false;
+                const long long t0 = clock64();
+                // (nothing to do may last as long as the launch; the issuing thread's own waits have the usual limit)
+                while (!(ok = mbar_test(bVAsk, va_phase) != 0u) && !*abort_flag && clock64() - t0 < 64 * WPP_WAIT_LIMIT)
+                    __nanosleep(256);
+                if (!__all_sync(0xffffffffu, ok)) break;
+                va_phase ^= 1u;
+                const int slot = v_rows[0], valid = v_rows[1];
+                if (slot < 0) break;
+                uint8_t* vg = smem_gen + C::kOffKV + slot * C::kTileBytes;
+                for (int h = 0; h < C::kHalves; ++h)
+                    for (int i = valid * 8 + lane; i < 128 * 8; i += 32)
+                        *reinterpret_cast<uint4*>(vg + h * C::kHalfBytes + i * 16) = make_uint4(0, 0, 0, 0);
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bVEnd);
+            }
+        } else if (warp == 13) {
             // ================================================================ producer
             // Tiles are requested in the order the issuers first touch them: K(0), K(1), V(0), K(2), V(1), ...
             Ring ring_k = {0, 0}, ring_v = {0, 0};
@@ -408,31 +438,6 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             }
             v_rows[0] = -1;
             mbar_arrive(bVAsk);
-        } else if (warp == 15) {
-            // ================================================================ the end of a sequence
-            // Rows of V past it may hold anything (stale slots, pages never loaded): they are zeroed so that 0 * garbage cannot
-            // reach O.  A warp does it for the issuing thread, while the softmax of the step is under way: by itself that took up
-            // to 2,000 stores in front of its product (2 x 4 tokens, attention call, 15.3 us | 10.1; pass, 34 x 427..576 over
-            // 1,000, 32/8 heads, 499 | 450).  It is asked, and does not follow the tiles itself: one more role in the hand-over of
-            // tiles cost long waves 2 to 5 %.
-            uint32_t va_phase = 0;
-            while (true) {
-                bool ok = false;
-                const long long t0 = clock64();
-                // (nothing to do may last as long as the launch; the issuing thread's own waits have the usual limit)
-                while (!(ok = mbar_try_wait(bVAsk, va_phase) != 0u) && !*abort_flag && clock64() - t0 < 64 * WPP_WAIT_LIMIT) { }
-                if (!__all_sync(0xffffffffu, ok)) break;
-                va_phase ^= 1u;
-                const int slot = v_rows[0], valid = v_rows[1];
-                if (slot < 0) break;
-                uint8_t* vg = smem_gen + C::kOffKV + slot * C::kTileBytes;
-                for (int h = 0; h < C::kHalves; ++h)
-                    for (int i = valid * 8 + lane; i < 128 * 8; i += 32)
-                        *reinterpret_cast<uint4*>(vg + h * C::kHalfBytes + i * 16) = make_uint4(0, 0, 0, 0);
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bVEnd);
-            }
         }
     } else if (wg == 2) {
         // ================================================================ epilogue (one thread per output row)
