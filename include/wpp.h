@@ -70,8 +70,8 @@ typedef struct wpp_ctx wpp_ctx;
  * fallback).  *out is host memory owned by the library until wpp_destroy.  Every launching entry point must be
  * called with the context's device current (WPP_ERR_INVALID_ARG otherwise).  The context caches the tensor maps
  * it encodes, keyed by (pointer, extents, strides); it may be used from several host threads.  It also owns 64
- * bytes of pinned host memory mapped for the device, to which the attention kernels add two counters (see
- * wpp_set_rescale_mode): everything enqueued through the context must have completed before wpp_destroy. */
+ * bytes of device memory, in which the attention kernels add up two counters (see wpp_set_rescale_mode), and 64 of pinned
+ * host memory mapped for the device, to which they store the totals: everything enqueued through the context must have completed before wpp_destroy. */
 int wpp_create(wpp_ctx** out, int cuda_device);
 int wpp_destroy(wpp_ctx* ctx);
 const char* wpp_status_string(int status);
@@ -192,13 +192,13 @@ int wpp_kv_append(const wpp_ctx* ctx, const wpp_batch_desc* desc, const void* k_
  *   k_cache, v_cache, block_tables, prefix_lens, chunk_lens : device, read only.
  *   plan_host / plan_dev : as for wpp_kv_append.
  *   workspace     : device scratch of >= info.workspace_bytes bytes, 256-byte aligned, required: holds the
- *                   counter the persistent CTAs take their tiles from (zeroed by this call on the stream) and
+ *                   counter the persistent CTAs take their tiles from (zeroed by this call on the stream if used) and
  *                   the split-KV partial results; contents are undefined afterwards.  Two calls that may run
  *                   at the same time need a workspace each.
  * A request whose prefix_lens[i] or chunk_lens[i] on the device differ from the plan's sets *status_dev =
  * WPP_ERR_PLAN_MISMATCH; its tiles are skipped (its output rows are not computed; rows of split tiles read as zero).
  * Enqueues one persistent kernel (the shape the plan names), a 256-byte memset in front of it when the tiles are taken
- * from the counter (the small shape deals few or equally long tiles out instead), and one combine kernel iff the
+ * from the counter (not where every tile has a CTA; the small shape deals few or equally long tiles out instead), and one combine kernel iff the
  * plan has split tiles.  The kernels may be set up on the GPU while the kernel before them in the stream still runs;
  * they wait for its end before they touch memory.
  * Results are bit-reproducible for a given plan, whichever CTA takes which tile (no atomics on outputs; partials
@@ -226,7 +226,7 @@ int wpp_prefill_attention_varlen(const wpp_ctx* ctx, const wpp_batch_desc* desc,
  *     (Like any CUDA kernel, the attention kernels are loaded onto the device by their first launch; this entry
  *     point adds nothing to that.)
  *   - All calls on a device share the one array and it keeps whatever the last call left in it.  The call zeroes
- *     the tile counter itself (a memset node on the stream) and every partial row is written before the combine
+ *     the tile counter itself where it uses it (a memset node on the stream) and every partial row is written before the combine
  *     pass reads it, but two calls whose kernels overlap on the GPU, e.g. on different streams, race on it:
  *     serialise them. */
 int wpp_prefill_attention_varlen_static(const wpp_ctx* ctx, const wpp_batch_desc* desc, const void* q, void* out,
@@ -255,9 +255,9 @@ int64_t wpp_launch_count(const wpp_ctx* ctx);
  *   wpp_set_rescale_mode : 0 = always before (default: outputs are bit-reproducible from call to call),
  *                          1 = always after,
  *                          2 = chosen per call from what the kernels of earlier launches on this context counted -
- *                              their key steps and the steps that rescaled, added up in two words of pinned host
- *                              memory that wpp_create maps for the device and that the call reads without
- *                              synchronising: at least 30 % of the steps rescaling: after; under 15 %: before; in
+ *                              their key steps and the steps that rescaled, whose totals a launch leaves at its end in
+ *                              two words of pinned host memory that wpp_create maps for the device and that the call
+ *                              reads without synchronising: at least 30 % of the steps rescaling: after; under 15 %: before; in
  *                              between: as it was.  Outputs may then differ in the last bit from call to call.
  *   wpp_rescale_stats    : the counters so far (either pointer may be null) and the order the next call would use. */
 int wpp_set_rescale_mode(wpp_ctx* ctx, int mode);
