@@ -105,8 +105,9 @@ constexpr int64_t kTileFixedCost = 3, kPartExtraCost = 2, kCombineCost = 20;
 // 153 | 201; 42 x 5 over 253..2,477, 64/8, 80 | 99; but 22 x 7..15 over 987..1,080, 40/8, 118 | 80; 32 x 4..34, 40/8, over 1,100 /
 // 1,500 / 4,096 140 | 126, 167 | 162, 430 | 406).  An estimate that tells them apart could take its place.
 // All of these figures are from before tiles were ordered by length and a launch cost 4 us less (32 x 1024 on the SM-wide shape, a
-// call at a time: 774 us before, 650 since).  With both, over 170 drawn waves the choice loses 0.6 % in the geometric mean against the better shape of each wave; a
-// fixed cost of 6 us for the SM-wide shape and no kSmallShapeSteps would lose 0.3 %: not enough to move plans for.
+// call at a time: 774 us before, 650 since).  With both, over 170 drawn waves the choice loses 0.6 % in the geometric mean
+// against the better shape of each wave; a fixed cost of 6 us for the SM-wide shape and no kSmallShapeSteps would lose 0.3 %: not
+// enough to move plans for.
 constexpr int64_t kSmallShapeSteps = 8;
 struct StepCount {
     int64_t sum = 0;
