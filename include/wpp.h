@@ -69,9 +69,11 @@ typedef struct wpp_ctx wpp_ctx;
  * the KV pool is sized from the free memory.  WPP_ERR_CUDA if the device or driver is unusable (there is no CPU
  * fallback).  *out is host memory owned by the library until wpp_destroy.  Every launching entry point must be
  * called with the context's device current (WPP_ERR_INVALID_ARG otherwise).  The context caches the tensor maps
- * it encodes, keyed by (pointer, extents, strides); it may be used from several host threads.  It also owns 64
- * bytes of device memory, in which the attention kernels add up two counters (see wpp_set_rescale_mode), and 64 of pinned
- * host memory mapped for the device, to which they store the totals: everything enqueued through the context must have completed before wpp_destroy. */
+ * it encodes, keyed by (pointer, extents, strides); it may be used from several host threads.  The first context on a device
+ * also allocates 128 KB of pinned host memory mapped for the device, kept until the process exits, in which the attention
+ * kernels leave two counters of each of up to 256 contexts at a time (see wpp_set_rescale_mode; contexts beyond them have
+ * none).  Contexts may be created and destroyed while a stream is being captured; everything enqueued through a context must
+ * have completed before wpp_destroy. */
 int wpp_create(wpp_ctx** out, int cuda_device);
 int wpp_destroy(wpp_ctx* ctx);
 const char* wpp_status_string(int status);
@@ -256,10 +258,12 @@ int64_t wpp_launch_count(const wpp_ctx* ctx);
  *                          1 = always after,
  *                          2 = chosen per call from what the kernels of earlier launches on this context counted -
  *                              their key steps and the steps that rescaled, whose totals a launch leaves at its end in
- *                              two words of pinned host memory that wpp_create maps for the device and that the call
- *                              reads without synchronising: at least 30 % of the steps rescaling: after; under 15 %: before; in
+ *                              pinned host memory that is mapped for the device and that the call reads without
+ *                              synchronising: at least 30 % of the steps rescaling: after; under 15 %: before; in
  *                              between: as it was.  Outputs may then differ in the last bit from call to call.
- *   wpp_rescale_stats    : the counters so far (either pointer may be null) and the order the next call would use. */
+ *   wpp_rescale_stats    : the counters so far, with those of every launch that has ended (either pointer may be null), and
+ *                          the order the next call would use.  (The counters of a launch that overlaps one made a multiple of
+ *                          sixteen launches before it may be among them only when that one has ended too.) */
 int wpp_set_rescale_mode(wpp_ctx* ctx, int mode);
 int wpp_rescale_stats(const wpp_ctx* ctx, uint64_t* key_steps, uint64_t* rescaling_steps, int* late);
 

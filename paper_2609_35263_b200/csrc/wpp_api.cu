@@ -44,10 +44,13 @@ struct wpp_ctx {
     EncodeTiledFn encode_tiled;
     void* static_scratch;           // device address of the built-in scratch array on this context's device
     // Where a moved row reference rescales O (see the attention kernel's kLate) is chosen per launch from what the
-    // kernels of earlier launches counted: key steps and steps that rescaled, added up in device memory and stored to
-    // mapped host memory at a launch's end.
-    unsigned long long* stats_host; // [0] key steps, [1] rescaling steps (pinned, mapped)
-    unsigned long long* stats_dev;  // device memory: the same two, the CTAs that run, the device address of stats_host
+    // kernels of earlier launches counted: key steps and steps that rescaled.
+    int counters;                   // which of the device's counters are this context's, -1: none
+    volatile unsigned long long* totals_host;    // [kCounterSlots][2]: totals that launches have left, as the host sees them
+    char* totals_dev;               // the same as the device sees them
+    uint32_t next_slot;             // launches in turn
+    unsigned long long steps, moves;             // the largest totals seen so far ...
+    unsigned long long base_steps, base_moves;   // ... and those at the context's creation
     unsigned long long seen_steps, seen_moves;   // the counters when the choice was last looked at
     int rescale_mode;               // 0: always before the exponentials (default), 1: always after, 2: chosen from the counters
     int late_rescale;               // the current choice
@@ -91,6 +94,75 @@ static cudaError_t static_scratch_address(int device, void** out) {
     return cudaSuccess;
 }
 
+// The counters of the contexts on a device: device memory of the attention kernel's module, and pinned memory mapped for the
+// device, to which the kernels store totals: allocated with the first context on a device, kept, and aligned to its size, so that
+// an address in it says which context's counters and which slot it stands for.  Contexts beyond kCounterContexts at a time on
+// a device have none (their choice of order stays at its default).
+struct CounterPool {
+    char *host, *dev;
+    bool used[wpp::kCounterContexts];
+};
+static CounterPool g_counters[64];
+
+// (no CUDA call but for the first context on a device)
+static void take_counters(wpp_ctx* c) {
+    c->counters = -1;
+    std::lock_guard<std::mutex> guard(g_scratch_lock);
+    if (c->device < 0 || c->device >= 64) return;
+    CounterPool& pool = g_counters[c->device];
+    if (!pool.host) {
+        constexpr uintptr_t size = wpp::kCounterBytes;
+        int before = -1;
+        void *host = nullptr, *dev = nullptr;
+        if (cudaGetDevice(&before) != cudaSuccess) return;
+        if (before != c->device && cudaSetDevice(c->device) != cudaSuccess) return;
+        if (cudaHostAlloc(&host, 2 * size, cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) {
+            char* at = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(host) + size - 1) / size * size);
+            if (cudaHostGetDevicePointer(&dev, at, 0) == cudaSuccess && reinterpret_cast<uintptr_t>(dev) % size == 0) {
+                memset(at, 0, size);
+                pool.host = at;
+                pool.dev = static_cast<char*>(dev);
+            } else {
+                cudaFreeHost(host);
+            }
+        }
+        if (before != c->device) cudaSetDevice(before);
+        (void)cudaGetLastError();
+    }
+    for (int i = 0; pool.host && i < wpp::kCounterContexts; ++i) {
+        if (pool.used[i]) continue;
+        pool.used[i] = true;
+        c->counters = i;
+        const size_t off = (size_t)i * wpp::kCounterSlots * 16;
+        c->totals_host = reinterpret_cast<volatile unsigned long long*>(pool.host + off);
+        c->totals_dev = pool.dev + off;
+        return;
+    }
+}
+static void give_counters_back(const wpp_ctx* c) {
+    if (c->counters < 0) return;
+    std::lock_guard<std::mutex> guard(g_scratch_lock);
+    g_counters[c->device].used[c->counters] = false;
+}
+
+// The totals now: every launch leaves them at its end, in a slot of its own, so the largest are the newest (map_lock is held).
+static void read_counters(wpp_ctx* c) {
+    for (int i = 0; c->counters >= 0 && i < wpp::kCounterSlots; ++i) {
+        const unsigned long long steps = c->totals_host[2 * i], moves = c->totals_host[2 * i + 1];
+        if (steps > c->steps || (steps == c->steps && moves > c->moves)) {
+            c->steps = steps;
+            if (moves > c->moves) c->moves = moves;
+        }
+    }
+}
+
+// Creating a context must neither disturb a stream that is being captured nor be refused for it.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 extern "C" int wpp_ctx_sm_count(const wpp_ctx* ctx) { return ctx ? ctx->sm_count : 148; }
 
 static int cuda_fail(const wpp_ctx* ctx, int err) {
@@ -101,6 +173,7 @@ static int cuda_fail(const wpp_ctx* ctx, int err) {
 extern "C" int wpp_create(wpp_ctx** out, int cuda_device) {
     if (!out) return WPP_ERR_INVALID_ARG;
     *out = nullptr;
+    RelaxedCapture relaxed;
     int n = 0;
     cudaError_t e = cudaGetDeviceCount(&n);
     if (e != cudaSuccess || cuda_device < 0 || cuda_device >= n) return WPP_ERR_CUDA;
@@ -129,44 +202,19 @@ extern "C" int wpp_create(wpp_ctx** out, int cuda_device) {
         free(c);
         return WPP_ERR_INVALID_ARG;
     }
-    // two counters the attention kernels add to and the next call reads without synchronising (a missing mapping
-    // only means that the choice they feed stays at its default)
-    // (a context may be made while some stream is being captured: neither may disturb the other)
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    void* hp = nullptr;
-    if (cudaHostAlloc(&hp, 64, cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) {
-        memset(hp, 0, 64);
-        void *dp = nullptr, *words = nullptr;
-        int before = -1;
-        bool ok = cudaGetDevice(&before) == cudaSuccess && cudaSetDevice(cuda_device) == cudaSuccess &&
-                  cudaHostGetDevicePointer(&dp, hp, 0) == cudaSuccess && cudaMalloc(&words, 64) == cudaSuccess;
-        cudaStream_t st = nullptr;
-        if (ok && (ok = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess)) {
-            const unsigned long long start[4] = {0, 0, 0, (unsigned long long)reinterpret_cast<uintptr_t>(dp)};
-            ok = cudaMemcpyAsync(words, start, sizeof(start), cudaMemcpyHostToDevice, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
-            cudaStreamDestroy(st);
-        }
-        if (before >= 0) cudaSetDevice(before);
-        if (ok) {
-            c->stats_host = static_cast<unsigned long long*>(hp);
-            c->stats_dev = static_cast<unsigned long long*>(words);
-        } else {
-            if (words) cudaFree(words);
-            cudaFreeHost(hp);
-        }
-    }
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    (void)cudaGetLastError();
+    take_counters(c);
+    read_counters(c);
+    c->base_steps = c->seen_steps = c->steps;
+    c->base_moves = c->seen_moves = c->moves;
     *out = c;
     return WPP_OK;
 }
 
+// (no CUDA call: a context may be collected while a stream is being captured)
 extern "C" int wpp_destroy(wpp_ctx* ctx) {
     if (ctx) {
+        give_counters_back(ctx);
         delete ctx->map_lock;
-        if (ctx->stats_dev) cudaFree(ctx->stats_dev);
-        if (ctx->stats_host) cudaFreeHost(ctx->stats_host);
     }
     free(ctx);
     return WPP_OK;
@@ -181,28 +229,29 @@ extern "C" int wpp_set_rescale_mode(wpp_ctx* ctx, int mode) {
 
 extern "C" int wpp_rescale_stats(const wpp_ctx* ctx, uint64_t* key_steps, uint64_t* rescaling_steps, int* late) {
     if (!ctx) return WPP_ERR_INVALID_ARG;
-    volatile unsigned long long* s = ctx->stats_host;
-    if (key_steps) *key_steps = s ? s[0] : 0;
-    if (rescaling_steps) *rescaling_steps = s ? s[1] : 0;
+    std::lock_guard<std::mutex> guard(*ctx->map_lock);
+    read_counters(const_cast<wpp_ctx*>(ctx));
+    if (key_steps) *key_steps = ctx->steps - ctx->base_steps;
+    if (rescaling_steps) *rescaling_steps = ctx->moves - ctx->base_moves;
     if (late) *late = ctx->rescale_mode == 1 || (ctx->rescale_mode == 2 && ctx->late_rescale);
     return WPP_OK;
 }
 
-// The choice for the next launch: with the counters' increase since the last look, once there are enough steps to
-// judge by; between the two thresholds the choice stays what it was.
-static int choose_late_rescale(const wpp_ctx* cctx) {
+// The choice for the next launch, and in *totals where it leaves the totals: with the counters' increase since the last look,
+// once there are enough steps to judge by; between the two thresholds the choice stays what it was.
+static int choose_late_rescale(const wpp_ctx* cctx, unsigned long long** totals) {
     wpp_ctx* c = const_cast<wpp_ctx*>(cctx);
     std::lock_guard<std::mutex> guard(*c->map_lock);
+    *totals = nullptr;
+    if (c->counters >= 0) *totals = reinterpret_cast<unsigned long long*>(c->totals_dev + 16 * (c->next_slot++ % wpp::kCounterSlots));
     if (c->rescale_mode != 2) return c->rescale_mode == 1;
-    if (!c->stats_host) return 0;
-    volatile unsigned long long* s = c->stats_host;
-    const unsigned long long steps = s[0], moves = s[1];
-    const unsigned long long ds = steps - c->seen_steps, dm = moves - c->seen_moves;
+    read_counters(c);
+    const unsigned long long ds = c->steps - c->seen_steps, dm = c->moves - c->seen_moves;
     if (ds >= 4096) {
         if (dm * 100 >= ds * kLateRescaleOnPct) c->late_rescale = 1;
         else if (dm * 100 < ds * kLateRescaleOffPct) c->late_rescale = 0;
-        c->seen_steps = steps;
-        c->seen_moves = moves;
+        c->seen_steps = c->steps;
+        c->seen_moves = c->moves;
     }
     return c->late_rescale;
 }
@@ -403,9 +452,9 @@ extern "C" int wpp_prefill_attention_varlen(const wpp_ctx* ctx, const wpp_batch_
         e = (int)cudaMemsetAsync(workspace, 0, WPP_WS_HEADER_BYTES, (cudaStream_t)cuda_stream);
         if (e != 0) return cuda_fail(ctx, e);
     }
-    p.stats = ctx->stats_dev;
+    const int late = hd->shape == 2 ? 0 : choose_late_rescale(ctx, &p.totals);
     e = hd->shape == 2 ? wpp_launch_attention_small(d.head_dim, tq, &tk, &tv, &p, num_ctas, cuda_stream)
-                       : wpp_launch_attention(d.head_dim, tq, &tk, &tv, &p, num_ctas, choose_late_rescale(ctx), cuda_stream);
+                       : wpp_launch_attention(d.head_dim, tq, &tk, &tv, &p, num_ctas, late, cuda_stream);
     if (e != 0) return cuda_fail(ctx, e);
     const_cast<wpp_ctx*>(ctx)->launches += 1;
     if (hd->num_combine > 0) {

@@ -38,6 +38,12 @@
 
 namespace wpp {
 
+// key steps and those that rescaled, per context; what of the launches in a slot has ended, in units of 2^-32 launches
+__device__ unsigned long long g_counts[kCounterContexts][2], g_ended[kCounterContexts * kCounterSlots];
+__device__ __forceinline__ int counter_slot(const unsigned long long* totals) {
+    return (int)(reinterpret_cast<uintptr_t>(totals) % kCounterBytes / 16);
+}
+
 constexpr int kThreads = 512;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColS = 0;                                                        // landing buffer of S
@@ -187,7 +193,6 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const uint32_t tmem = *tmem_slot;
     grid_launch_dependents();
     grid_dependency_wait();           // (launched while the kernel before may still be running)
-    if (p.stats && threadIdx.x == 0) atomicAdd(p.stats + 2, 1ull);
 
     const char* plan = static_cast<const char*>(p.plan);
     const WppPlanHeader* hd = reinterpret_cast<const WppPlanHeader*>(plan);
@@ -697,9 +702,10 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             s_final[hf * 128 + r] = make_float2(-nmc, l_run);
             mbar_arrive(bFinalReady(hf));
         }
-        if (p.stats && lane == 0 && n_steps_seen) {
-            atomicAdd(p.stats, (unsigned long long)n_steps_seen);
-            atomicAdd(p.stats + 1, (unsigned long long)n_moves_seen);
+        if (p.totals && lane == 0 && n_steps_seen) {
+            unsigned long long* count = g_counts[counter_slot(p.totals) / kCounterSlots];
+            atomicAdd(count, (unsigned long long)n_steps_seen);
+            atomicAdd(count + 1, (unsigned long long)n_moves_seen);
         }
     }
 
@@ -717,21 +723,21 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         tc_fence_after();
         tmem_dealloc(tmem, kTmemCols);
     }
-    // The context's counters go to the two words that the host sees when the last CTA that runs has counted: plain stores, and
-    // not additions, whose answers would come back over the bus (4 us of every launch).  Launches in several streams may get
-    // here together: whoever stored what has changed meanwhile stores again.
-    if (p.stats && threadIdx.x == 0) {
+    // The CTA that ends the launch leaves the totals where the host sees them: a plain store, not additions, whose answers would
+    // come back over the bus (4 us of every launch).  Which CTA that is says a sum of shares that make up 1 for every launch:
+    // it passes a whole number.  (Launches on several streams have slots of their own; should two that overlap have the same
+    // one, it still passes a whole number with the end of the last.)
+    if (p.totals && threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(p.stats + 2, ~0ull) == 1ull) {
-            volatile unsigned long long* host = reinterpret_cast<volatile unsigned long long*>(p.stats[3]);
-            unsigned long long steps = atomicAdd(p.stats, 0ull), moves = atomicAdd(p.stats + 1, 0ull), seen;
-            do {
-                seen = steps;
-                host[0] = steps;
-                host[1] = moves;
-                moves = atomicAdd(p.stats + 1, 0ull);
-                steps = atomicAdd(p.stats, 0ull);
-            } while (steps != seen);
+        const int slot = counter_slot(p.totals);
+        const uint32_t each = 0xffffffffu / gridDim.x;
+        const unsigned long long share = blockIdx.x ? each : 0x100000000ull - (unsigned long long)each * (gridDim.x - 1);
+        const unsigned long long before = atomicAdd(&g_ended[slot], share);
+        if (((before & 0xffffffffull) + share) >> 32) {
+            __threadfence();
+            unsigned long long* count = g_counts[slot / kCounterSlots];
+            const unsigned long long steps = atomicAdd(count, 0ull), moves = atomicAdd(count + 1, 0ull);
+            *reinterpret_cast<ulonglong2*>(p.totals) = make_ulonglong2(steps, moves);
         }
     }
 }

@@ -8,6 +8,11 @@
 
 namespace wpp {
 
+// Counters of the SM-wide attention kernel, per context: key steps of the softmax warps and those that rescaled O, added up in
+// device memory; a launch leaves the totals in one of the context's kCounterSlots pairs of words in mapped host memory.
+constexpr int kCounterContexts = 256, kCounterSlots = 16;
+constexpr int kCounterBytes = kCounterContexts * kCounterSlots * 16;      // of the host side, which is aligned to its size
+
 struct AttnParams {
     const void* plan;                // device copy of the plan
     const int32_t* block_tables;     // [R][max_blocks]
@@ -21,8 +26,7 @@ struct AttnParams {
     uint32_t* tile_counter;          // zeroed before the launch: how many tiles have been taken beyond the first one per CTA;
                                      // or null: every CTA has one tile; (small shape) round k of the CTAs takes tiles k gridDim ..,
                                      // rotated by k
-    unsigned long long* stats;       // or null: [0] += key steps of the softmax warps, [1] += those that rescaled O, [2] CTAs
-                                     // that run, [3] where the host sees the first two
+    unsigned long long* totals;      // or null: the launch's slot of the counters' host side (see kCounterContexts)
     int64_t o_token_stride, o_head_stride;
     int32_t num_q_heads, group, page_size, max_blocks, num_pages;
     float scale_log2;                // sm_scale * log2(e)
