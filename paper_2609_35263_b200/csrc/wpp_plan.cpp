@@ -239,6 +239,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     auto steps_for = [](int64_t last_visible_plus1) { return (int32_t)((last_visible_plus1 + WPP_TILE_N - 1) / WPP_TILE_N); };
     std::vector<RowBlock> rbs;
     std::vector<int32_t> rb_first((size_t)R + 1);
+    bool newer = true;              // whole groups and tiles by length are allowed (see lay_out)
     bool whole_groups = false;
     bool pair_heads = auto_tile_m && G % 2 == 0 && pairs >= kPairHeadsKeys * T;
     auto build_rows = [&](int tile_m) -> int64_t {
@@ -273,7 +274,7 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
                     // 1,094 | 280.  (17 to 64 rows leave room for 2 or 4 heads: as many as divide the group, as ever.)
                     int whole = 1;
                     while (whole < G) whole *= 2;
-                    if (pack < whole && whole <= 8 && WPP_HALF_M / whole >= rows) {
+                    if (newer && pack < whole && whole <= 8 && WPP_HALF_M / whole >= rows) {
                         pack = whole;
                         rb.per_tile = G;
                         whole_groups = true;
@@ -303,96 +304,101 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
         return n_tiles;
     };
     int TM = o.tile_m;
-    int64_t n_base = build_rows(TM);
+    int64_t n_base = 0;
     // partial results the built-in scratch array holds (without the workspace's header)
     const uint64_t slot_bytes = (uint64_t)2 * WPP_HALF_M * (d.head_dim + 1) * sizeof(float);
     const uint64_t scratch_slots = (kSplitScratchBytes - WPP_WS_HEADER_BYTES) / slot_bytes;
-    if (o.force_kv_splits != 0 && auto_tile_m && n_base < o.max_ctas) {
-        // Few tiles and the caller's cut: more, smaller ones, unless only the taller tiles' partial results fit the built-in
-        // scratch array.  Attention call in us, 256-row tiles | 128: 1 x 8,192 tokens, one head, never cut 112 | 97, in two
-        // parts 78 | 71; 2 x 1,000 over 3,000, 8/2 heads, never cut 76 | 68.
-        auto forced_slots = [&]() {
-            uint64_t n = 0;
-            for (const RowBlock& rb : rbs) {
-                const int32_t parts = std::min(o.force_kv_splits, rb.steps);
-                if (parts > 1) n += (uint64_t)parts * (uint64_t)(Hq / rb.per_tile);
-            }
-            return n;
-        };
-        const bool tall_fits = forced_slots() <= scratch_slots;
-        n_base = build_rows(WPP_HALF_M);
-        if (tall_fits && forced_slots() > scratch_slots) n_base = build_rows(TM);
-        else TM = WPP_HALF_M;
-    }
     int32_t part_eighths = 0;      // length of a tile's parts in eighths of a key step (0: whole tiles)
     int few_shape = 0;             // the kernel shape these parts were chosen for
-    if (o.force_kv_splits == 0 && n_base > 0 && n_base < o.max_ctas) {
-        const int tms[2] = {128, 256};
-        double best = 0.0;
-        int best_tm = TM;
-        uint64_t slots_cap = scratch_slots - 1;
-        // (or within what cutting the 128-row tiles so that there are at least max_ctas parts takes, if that is more)
-        if (auto_tile_m) n_base = build_rows(128);
-        uint64_t even_parts = 0;
+    auto forced_slots = [&]() {
+        uint64_t n = 0;
         for (const RowBlock& rb : rbs) {
-            const int32_t parts = std::min((int32_t)((o.max_ctas + n_base - 1) / n_base), rb.steps / kMinPartSteps);
-            if (n_base < o.max_ctas && parts > 1) even_parts += (uint64_t)parts * (uint64_t)(Hq / rb.per_tile);
+            const int32_t parts = std::min(o.force_kv_splits, rb.steps);
+            if (parts > 1) n += (uint64_t)parts * (uint64_t)(Hq / rb.per_tile);
         }
-        slots_cap = std::max(slots_cap, even_parts);
-        for (int ti = 0; ti < 2; ++ti) {
-            if (!auto_tile_m && tms[ti] != TM) continue;
-            if (build_rows(tms[ti]) == 0) continue;
-            // tiles cut into parts of `ps` eighths of a key step: items of either shape and their steps
-            struct Count { int64_t units, halves, cut; StepCount unit, half; };
-            auto count = [&](int32_t ps, bool steps_too) {
-                Count c = {0, 0, 0, StepCount(), StepCount()};
-                for (const RowBlock& rb : rbs) {
-                    const int32_t parts = parts_of(rb.steps, ps);
-                    const int64_t times = Hq / rb.per_tile;
-                    c.units += parts * times;
-                    c.halves += parts * times * (rb.rows[1] > 0 ? 2 : 1);
-                    c.cut += parts > 1 ? parts * times : 0;
-                    if (!steps_too) continue;
-                    const int32_t part = (rb.steps + parts - 1) / parts;
-                    c.unit.sum += times * std::max(rb.end[0], rb.end[1]);
-                    c.half.sum += times * ((int64_t)rb.end[0] + rb.end[1]);
-                    c.unit.longest = std::max(c.unit.longest, part);
-                    c.half.longest = std::max(c.half.longest, part);
-                }
-                return c;
-            };
-            int32_t longest = 0;
-            for (const RowBlock& rb : rbs) longest = std::max(longest, rb.steps);
-            for (int shape = 2; shape >= 1; --shape) {
-                if (o.shape != 0 && o.shape != shape) continue;
-                for (int rounds = 0; rounds <= 2; ++rounds) {
-                    // the shortest parts that make at most `rounds` rounds of items (0: whole tiles)
-                    int32_t ps = 0;
-                    if (rounds > 0) {
-                        const int64_t slots = (int64_t)rounds * o.max_ctas * (shape == 2 ? 2 : 1);
-                        int32_t lo = 8 * kMinPartSteps, hi = 8 * longest;
-                        if (hi < lo) continue;
-                        while (lo < hi) {
-                            const int32_t mid = lo + (hi - lo) / 2;
-                            const Count c = count(mid, false);
-                            const int64_t items = shape == 2 ? (c.halves > c.units ? 2 * c.units : c.units) : c.units;
-                            if (items <= slots && (uint64_t)c.cut <= slots_cap) hi = mid; else lo = mid + 1;
-                        }
-                        ps = lo;
+        return n;
+    };
+    auto cut_few = [&](uint64_t max_slots) {
+        TM = o.tile_m;
+        n_base = build_rows(TM);
+        part_eighths = 0;
+        few_shape = 0;
+        if (o.force_kv_splits != 0 && auto_tile_m && n_base < o.max_ctas) {
+            // Few tiles and the caller's cut: more, smaller ones, unless only the taller tiles' partial results fit the built-in
+            // scratch array.  Attention call in us, 256-row tiles | 128: 1 x 8,192 tokens, one head, never cut 112 | 97, in two
+            // parts 78 | 71; 2 x 1,000 over 3,000, 8/2 heads, never cut 76 | 68.
+            const bool tall_fits = forced_slots() <= scratch_slots;
+            n_base = build_rows(WPP_HALF_M);
+            if (tall_fits && forced_slots() > scratch_slots) n_base = build_rows(TM);
+            else TM = WPP_HALF_M;
+        }
+        if (o.force_kv_splits == 0 && n_base > 0 && n_base < o.max_ctas) {
+            const int tms[2] = {128, 256};
+            double best = 0.0;
+            int best_tm = TM;
+            uint64_t slots_cap = scratch_slots - 1;
+            // (or within what cutting the 128-row tiles so that there are at least max_ctas parts takes, if that is more)
+            if (auto_tile_m) n_base = build_rows(128);
+            uint64_t even_parts = 0;
+            for (const RowBlock& rb : rbs) {
+                const int32_t parts = std::min((int32_t)((o.max_ctas + n_base - 1) / n_base), rb.steps / kMinPartSteps);
+                if (n_base < o.max_ctas && parts > 1) even_parts += (uint64_t)parts * (uint64_t)(Hq / rb.per_tile);
+            }
+            slots_cap = std::min(std::max(slots_cap, even_parts), max_slots);
+            for (int ti = 0; ti < 2; ++ti) {
+                if (!auto_tile_m && tms[ti] != TM) continue;
+                if (build_rows(tms[ti]) == 0) continue;
+                // tiles cut into parts of `ps` eighths of a key step: items of either shape and their steps
+                struct Count { int64_t units, halves, cut; StepCount unit, half; };
+                auto count = [&](int32_t ps, bool steps_too) {
+                    Count c = {0, 0, 0, StepCount(), StepCount()};
+                    for (const RowBlock& rb : rbs) {
+                        const int32_t parts = parts_of(rb.steps, ps);
+                        const int64_t times = Hq / rb.per_tile;
+                        c.units += parts * times;
+                        c.halves += parts * times * (rb.rows[1] > 0 ? 2 : 1);
+                        c.cut += parts > 1 ? parts * times : 0;
+                        if (!steps_too) continue;
+                        const int32_t part = (rb.steps + parts - 1) / parts;
+                        c.unit.sum += times * std::max(rb.end[0], rb.end[1]);
+                        c.half.sum += times * ((int64_t)rb.end[0] + rb.end[1]);
+                        c.unit.longest = std::max(c.unit.longest, part);
+                        c.half.longest = std::max(c.half.longest, part);
                     }
-                    const Count c = count(ps, true);
-                    if (c.cut > 0 && (uint64_t)c.cut > slots_cap) continue;
-                    double us = shape == 2 ? small_shape_us(c.half, c.halves > c.units ? 2 * c.units : c.units, o.max_ctas)
-                                           : wide_shape_us(c.unit, c.units, c.halves, o.max_ctas);
-                    if (c.cut > 0) us += kCombineUs + kPartUs * (double)c.cut;
-                    if (few_shape == 0 || us < best) { best = us; best_tm = tms[ti]; part_eighths = ps; few_shape = shape; }
+                    return c;
+                };
+                int32_t longest = 0;
+                for (const RowBlock& rb : rbs) longest = std::max(longest, rb.steps);
+                for (int shape = 2; shape >= 1; --shape) {
+                    if (o.shape != 0 && o.shape != shape) continue;
+                    for (int rounds = 0; rounds <= 2; ++rounds) {
+                        // the shortest parts that make at most `rounds` rounds of items (0: whole tiles)
+                        int32_t ps = 0;
+                        if (rounds > 0) {
+                            const int64_t slots = (int64_t)rounds * o.max_ctas * (shape == 2 ? 2 : 1);
+                            int32_t lo = 8 * kMinPartSteps, hi = 8 * longest;
+                            if (hi < lo) continue;
+                            while (lo < hi) {
+                                const int32_t mid = lo + (hi - lo) / 2;
+                                const Count c = count(mid, false);
+                                const int64_t items = shape == 2 ? (c.halves > c.units ? 2 * c.units : c.units) : c.units;
+                                if (items <= slots && (uint64_t)c.cut <= slots_cap) hi = mid; else lo = mid + 1;
+                            }
+                            ps = lo;
+                        }
+                        const Count c = count(ps, true);
+                        if (c.cut > 0 && (uint64_t)c.cut > slots_cap) continue;
+                        double us = shape == 2 ? small_shape_us(c.half, c.halves > c.units ? 2 * c.units : c.units, o.max_ctas)
+                                               : wide_shape_us(c.unit, c.units, c.halves, o.max_ctas);
+                        if (c.cut > 0) us += kCombineUs + kPartUs * (double)c.cut;
+                        if (few_shape == 0 || us < best) { best = us; best_tm = tms[ti]; part_eighths = ps; few_shape = shape; }
+                    }
                 }
             }
+            TM = best_tm;
+            n_base = build_rows(TM);
         }
-        TM = best_tm;
-        n_base = build_rows(TM);
-    }
-    if (n_base > 0x3fffffff) return WPP_ERR_INVALID_ARG;
+    };
     // cost of key steps [a, b) of a tile = 128x128 steps over its halves, each cut at its own causal end
     auto cost_of = [](const RowBlock& t, int32_t a, int32_t b) -> int32_t {
         return std::max(0, std::min(b, t.end[0]) - a) + std::max(0, std::min(b, t.end[1]) - a);
@@ -419,21 +425,24 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
         for (int i : by_cost) visit(i);
     };
     bool by_length = false;
-    if (o.order == 0 && o.shape == 0 && auto_tile_m && o.force_kv_splits == 0 && few_shape == 0) {
-        int64_t halves = 0;
-        StepCount unit, half;
-        for (const RowBlock& rb : rbs) {
-            const int64_t times = Hq / rb.per_tile;
-            halves += times * (rb.rows[1] > 0 ? 2 : 1);
-            unit.add(std::max(rb.end[0], rb.end[1]), times);
-            half.add(rb.end[0], times);
-            if (rb.rows[1] > 0) half.add(rb.end[1], times);
+    auto choose_order = [&]() {
+        by_length = false;
+        if (newer && o.order == 0 && o.shape == 0 && auto_tile_m && o.force_kv_splits == 0 && few_shape == 0) {
+            int64_t halves = 0;
+            StepCount unit, half;
+            for (const RowBlock& rb : rbs) {
+                const int64_t times = Hq / rb.per_tile;
+                halves += times * (rb.rows[1] > 0 ? 2 : 1);
+                unit.add(std::max(rb.end[0], rb.end[1]), times);
+                half.add(rb.end[0], times);
+                if (rb.rows[1] > 0) half.add(rb.end[1], times);
+            }
+            const int64_t items = halves > n_base ? 2 * n_base : n_base;
+            const int shape = shape_of(unit, half, n_base, halves, items, o.max_ctas);
+            by_length = shape == 2 ? items <= kLengthOrderItems * o.max_ctas
+                                   : half.sum <= kLengthOrderSteps * halves || n_base <= kLengthOrderTiles * o.max_ctas;
         }
-        const int64_t items = halves > n_base ? 2 * n_base : n_base;
-        const int shape = shape_of(unit, half, n_base, halves, items, o.max_ctas);
-        by_length = shape == 2 ? items <= kLengthOrderItems * o.max_ctas
-                               : half.sum <= kLengthOrderSteps * halves || n_base <= kLengthOrderTiles * o.max_ctas;
-    }
+    };
     auto order_tiles = [&]() {
         tiles.clear();
         tiles.reserve((size_t)n_base);
@@ -464,7 +473,6 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
                 });
         }
     };
-    order_tiles();
 
     // ---- split decision: into how many key ranges each tile is cut (1 = not at all)
     int64_t tail = 0;              // tiles of a partly filled last round ...
@@ -519,8 +527,9 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
             }
         }
     };
-    cut_tail(~0ull);
-    if (pair_heads && (uint64_t)tail * (uint64_t)tail_parts > scratch_slots) {
+    auto cut_tail_pairs = [&](uint64_t most) {
+        cut_tail(most);
+        if (!pair_heads || (uint64_t)tail * (uint64_t)tail_parts <= scratch_slots) return;
         // The cut needs more scratch than the built-in array holds.  Tiles whose halves are two heads are cut in more waves
         // than tiles of row blocks (the halves end together, so the model sees more to gain), and a wave that those would
         // not have cut beyond the array must not be refused for it by the entry point that has no other scratch: such a
@@ -529,13 +538,38 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
         pair_heads = false;
         n_base = build_rows(TM);
         order_tiles();
-        cut_tail(~0ull);
+        cut_tail(most);
         const bool cut_anyway = (uint64_t)tail * (uint64_t)tail_parts > scratch_slots;
         pair_heads = true;
         n_base = build_rows(TM);
         order_tiles();
-        cut_tail(cut_anyway ? ~0ull : scratch_slots);
+        cut_tail(cut_anyway ? most : scratch_slots);
+    };
+    // Tiles, their order and their cuts, with at most `max_slots` partial results; how many there are comes back.
+    auto lay_out = [&](bool allow_newer, uint64_t max_slots) -> uint64_t {
+        newer = allow_newer;
+        cut_few(max_slots);
+        if (n_base > 0x3fffffff) return 0;
+        choose_order();
+        order_tiles();
+        cut_tail_pairs(max_slots);
+        if (o.force_kv_splits >= 2) return forced_slots();
+        uint64_t n = (uint64_t)tail * (uint64_t)tail_parts;
+        for (const RowBlock& rb : rbs) {
+            const int32_t parts = few_shape != 0 ? parts_of(rb.steps, part_eighths) : 1;
+            if (parts > 1) n += (uint64_t)parts * (uint64_t)(Hq / rb.per_tile);
+        }
+        return n;
+    };
+    // Fewer tiles (whole groups) and tiles in another order may be cut into more parts than the built-in scratch array holds.  A
+    // wave whose parts it would hold without them must not be refused for them by the entry point that has no other scratch: it is
+    // cut as far as the array allows.  1 x 1 token over 20,000, 40/8 heads of 128: 120 parts a head at a time, 144 of whole
+    // groups, of which the array holds 127.
+    if (lay_out(true, ~0ull) > scratch_slots && o.force_kv_splits == 0 && (whole_groups || by_length)) {
+        const bool fits = lay_out(false, ~0ull) <= scratch_slots;
+        lay_out(true, fits ? scratch_slots : ~0ull);
     }
+    if (n_base > 0x3fffffff) return WPP_ERR_INVALID_ARG;
 
     // ---- the plan: header, row offsets, the spans the plan is made for, units, combine records
     WppPlanHeader hd;

@@ -224,6 +224,19 @@ def test_a_group_that_is_no_power_of_two_is_whole_in_a_half_that_has_room(Hq, Hk
     assert len(pl["comb"]) == sum(Hq for c in C) if splits else True
 
 
+@pytest.mark.parametrize("Hq,Hkv,P,C", [(40, 8, [20000], [1]), (40, 8, [20000] * 4, [1] * 4), (40, 8, [8192], [8]),
+                                        (64, 8, [12151, 18919, 18919], [1072, 19, 19]), (64, 8, [14453, 20188], [521, 225]), (8, 2, [15968], [5851])])
+def test_whole_groups_and_order_by_length_take_no_more_scratch_than_there_is(Hq, Hkv, P, C):
+    """Waves that fit the built-in scratch array with as many heads as divide the group, and in stream order, still fit it (with fewer
+    tiles there is more to cut: 144 parts where the array holds 127, for one)."""
+    mb = max((p + c + 63) // 64 for p, c in zip(P, C))
+    plan = wpp.wpp_plan_tiles(None, desc(len(P), Hq, Hkv, 128, 64, mb), P, C, pin=False)
+    assert plan.info.workspace_bytes <= wpp.wpp_static_scratch_bytes()
+    if Hq // Hkv in (3, 5, 6, 7):
+        pl = parse_plan(plan)
+        assert all(u["pack"] > Hq // Hkv for u in pl["units"]) and pl["slots"] > 0          # whole groups, and cut
+
+
 def test_few_tiles_fall_back_to_128_row_tiles_and_split_keys():
     d = desc(1, 8, 2, 64, 16, 64)
     pl = parse_plan(wpp.wpp_plan_tiles(None, d, [256], [128], pin=False))       # the single-request configuration
