@@ -415,14 +415,14 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
     //      stream order (see kLengthOrderSteps).
     struct Tile { int32_t rb, head; };          // row block and first head
     std::vector<Tile> tiles;
-    auto for_each_request = [&](auto&& visit) {        // the costliest first
+    auto requests_by_cost = [&]() {        // the costliest first
         std::vector<int64_t> req_cost((size_t)std::max(R, 1), 0);
         for (const RowBlock& rb : rbs) req_cost[(size_t)rb.request] += (int64_t)rb.cost() * (Hq / rb.per_tile);
         std::vector<int32_t> by_cost((size_t)R);
         for (int i = 0; i < R; ++i) by_cost[(size_t)i] = i;
         std::stable_sort(by_cost.begin(), by_cost.end(),
                          [&](int32_t a, int32_t b) { return req_cost[(size_t)a] > req_cost[(size_t)b]; });
-        for (int i : by_cost) visit(i);
+        return by_cost;
     };
     bool by_length = false;
     auto choose_order = [&]() {
@@ -454,9 +454,8 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
         } else if (by_length) {
             std::vector<int32_t> longest_first;
             longest_first.reserve(rbs.size());
-            for_each_request([&](int i) {
+            for (int32_t i : requests_by_cost())
                 for (int32_t k = rb_first[(size_t)i]; k < rb_first[(size_t)i + 1]; ++k) longest_first.push_back(k);
-            });
             std::stable_sort(longest_first.begin(), longest_first.end(),
                              [&](int32_t a, int32_t b) { return rbs[(size_t)a].cost() > rbs[(size_t)b].cost(); });
             for (size_t a = 0, b; a < longest_first.size(); a = b) {         // equally long ones in stream order
@@ -466,11 +465,11 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
                         for (int h = kvh * G; h < (kvh + 1) * G; h += rbs[(size_t)longest_first[j]].per_tile) tiles.push_back({longest_first[j], h});
             }
         } else {
+            const std::vector<int32_t> by_cost = requests_by_cost();
             for (int kvh = 0; kvh < d.num_kv_heads; ++kvh)
-                for_each_request([&](int i) {
+                for (int32_t i : by_cost)
                     for (int32_t k = rb_first[(size_t)i]; k < rb_first[(size_t)i + 1]; ++k)
                         for (int h = kvh * G; h < (kvh + 1) * G; h += rbs[(size_t)k].per_tile) tiles.push_back({k, h});
-                });
         }
     };
 

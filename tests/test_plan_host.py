@@ -8,6 +8,7 @@ import ctypes
 import os
 import re
 import struct
+import time
 
 import numpy as np
 import pytest
@@ -167,6 +168,20 @@ def test_stream_order_runs_the_tiles_of_one_kv_stream_together():
     # the first tiles (one per CTA) belong to KV head 0 of the costliest request (request 0: 4 row blocks x 4 heads)
     firsts = pl["units"][:pl["num_ctas"]]
     assert all(u["request"] == 0 and u["head_a"] // 4 == 0 for u in firsts)
+
+
+def test_stream_order_sorts_the_requests_once():
+    """Not once per KV head: ordering 4,096 requests of 64 KV heads takes less than sorting their 262,144 tiles (which it did
+    not, 17.5 ms against 13.7, with a sort per KV head; 8.0 against 12.7 with one)."""
+    rng = np.random.default_rng(3)
+    P, C = rng.integers(0, 2000, 4096), np.ones(4096, np.int64)
+    d, best = desc(4096, 64, 64, 128, 64, 32), {}
+    for _ in range(5):
+        for order in (0, 1):
+            t0 = time.perf_counter()
+            wpp.wpp_plan_tiles(None, d, P, C, opts=wpp.PlanOpts(0, 0, 0, 0, order, 1), pin=False)
+            best[order] = min(best.get(order, 9.0), time.perf_counter() - t0)
+    assert best[0] < best[1], best
 
 
 @pytest.mark.parametrize("R,P,C,heads,sorted_", [(32, 0, 1024, (64, 8, 128, 64), True), (16, 0, 2048, (64, 8, 128, 64), True), (34, 1000, 500, (32, 8, 128, 64), True),
