@@ -116,7 +116,7 @@ typedef struct {
                                  tiles that read the same (request, KV head) pages are neighbours and so run at the
                                  same time: the pages are fetched from DRAM once and shared through L2 - or, where
                                  tile_m, force_kv_splits and shape are 0 as well and the tiles are short or few, by
-                                 length; 1: longest tile first */
+                                 length; 1: longest tile first; 2: stream order in any case */
     int32_t shape;            /* which attention kernel runs the plan.  1: one CTA per SM working on both 128-row halves
                                  of a tile against 128-key steps (long tiles: the two halves and the tensor pipe overlap
                                  inside the CTA); 2: two small CTAs per SM, each working on one half against 64-key

@@ -173,7 +173,7 @@ static int resolve_opts(const wpp_ctx* ctx, const wpp_plan_opts* in, wpp_plan_op
     if (o->tile_m > WPP_MAX_TILE_M) return WPP_ERR_UNSUPPORTED;
     if (o->tile_n != WPP_TILE_N) return WPP_ERR_UNSUPPORTED;
     if (o->force_kv_splits < 0 || o->force_kv_splits > 64 || o->max_ctas < 1 || o->max_ctas > 4096 ||
-        o->order < 0 || o->order > 1 || o->shape < 0 || o->shape > 2)
+        o->order < 0 || o->order > 2 || o->shape < 0 || o->shape > 2)
         return WPP_ERR_INVALID_ARG;
     return WPP_OK;
 }
@@ -406,13 +406,13 @@ int wpp_plan_tiles(const wpp_ctx* ctx, const wpp_batch_desc* desc, const int32_t
 
     // ---- order of execution.  The persistent CTAs take tiles in this order at run time (a counter in the
     //      workspace), so tiles adjacent in the order run at the same time on different SMs.
-    //      order 0 (default), "stream order": KV head major, then requests (longest first), then row blocks and
+    //      order 0 (default) and 2, "stream order": KV head major, then requests (longest first), then row blocks and
     //      heads.  All tiles that read one (request, KV head) stream start together and walk its pages in step,
     //      so a page comes from DRAM once and is then hit in L2 by the other tiles; a prefix shared by many
     //      requests stays L2-resident while its KV head is being worked on.
     //      order 1: longest tile first (best balance, no regard for which tiles run together).
-    //      Where every choice is the planner's and tiles are short or few it takes that order too, equally long tiles in
-    //      stream order (see kLengthOrderSteps).
+    //      With order 0, where every other choice is the planner's too and tiles are short or few, it takes that order,
+    //      equally long tiles in stream order (see kLengthOrderSteps); order 2 is stream order in any case.
     struct Tile { int32_t rb, head; };          // row block and first head
     std::vector<Tile> tiles;
     auto requests_by_cost = [&]() {        // the costliest first

@@ -170,6 +170,13 @@ def test_stream_order_runs_the_tiles_of_one_kv_stream_together():
     assert all(u["request"] == 0 and u["head_a"] // 4 == 0 for u in firsts)
 
 
+@pytest.mark.parametrize("order", [-1, 3])
+def test_there_are_three_orders(order):
+    with pytest.raises(wpp.WppError) as e:
+        wpp.wpp_plan_tiles(None, desc(1, 8, 2, 128, 64, 10), [0], [300], opts=wpp.PlanOpts(0, 0, 0, 0, order, 0), pin=False)
+    assert e.value.status == 1                                                             # WPP_ERR_INVALID_ARG
+
+
 def test_stream_order_sorts_the_requests_once():
     """Not once per KV head: ordering 4,096 requests of 64 KV heads takes less than sorting their 262,144 tiles (which it did
     not, 17.5 ms against 13.7, with a sort per KV head; 8.0 against 12.7 with one)."""
@@ -195,6 +202,8 @@ def test_tiles_go_by_length_where_they_are_short_or_few(R, P, C, heads, sorted_)
     stream = parse_plan(wpp.wpp_plan_tiles(None, d, [P] * R, [C] * R, opts=wpp.PlanOpts(0, 0, 0, 0, 0, pl["shape"]), pin=False))
     kv = [u["head_a"] // (heads[0] // heads[1]) for u in stream["units"]]
     assert kv == sorted(kv)                              # a shape of the caller's choice keeps stream order
+    asked = parse_plan(wpp.wpp_plan_tiles(None, d, [P] * R, [C] * R, opts=wpp.PlanOpts(0, 0, 0, 0, 2, 0), pin=False))
+    assert asked["shape"] == pl["shape"] and asked["tile_m"] == pl["tile_m"] and asked["units"] == stream["units"]
     key = lambda u: sorted(u.items())
     assert sorted(map(key, pl["units"])) == sorted(map(key, stream["units"]))
     assert (pl["units"] != stream["units"]) == sorted_ and (not sorted_ or cost == sorted(cost, reverse=True))
