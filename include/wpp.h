@@ -441,7 +441,7 @@ typedef struct {
  * A request with an empty chunk copies state_in to state_out.  Returns WPP_ERR_INVALID_ARG for null or misaligned
  * pointers or negative sizes, WPP_ERR_UNSUPPORTED for d_k, d_v other than 128, WPP_ERR_WORKSPACE_TOO_SMALL when
  * layout 3 is asked for without enough workspace, WPP_ERR_CUDA for a launch failure.  Layout 3 enqueues block offsets and,
- * for one to six segments of the chunks, per-block preparation and the chain over the blocks; layouts 1 and 2 one kernel;
+ * for one to sixteen segments of the chunks, per-block preparation and the chain over the blocks; layouts 1 and 2 one kernel;
  * layout 0 either, or the group kernel (a memset of its counter and flags in front where the chains are cut into pieces), with the two passes
  * of one segment behind it when there are several requests (they end at once unless a chunk is too long for the groups). */
 int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const void* q, const void* k, const void* v,

@@ -535,64 +535,109 @@ extern "C" size_t wpp_kda_workspace_bytes(const wpp_kda_desc* desc) {
 // Microseconds of the two passes over C tokens per request, measured on 148 SMs: preparation of a token of a chain on all SMs,
 // a token of a chain that has an SM to itself, and what a token's operands take at the memory's rate.
 constexpr double kPrepUs = 0.9e-3, kChainUs = 0.0525, kOperandsUs = 0.49e-3, kSegmentUs = 12.0;
+struct KdaRates {
+    double chains, tokens, prep, operands, chain;          // tokens: per request; us: on all SMs, of all chains
+    double growth;                                         // what a chain takes over the preparation beside it; 0: no SMs for that
+    KdaRates(const wpp_kda_desc* d, int sms) {
+        chains = (double)d->num_requests * d->num_heads;
+        tokens = (double)d->total_tokens / d->num_requests;
+        prep = chains * tokens * kPrepUs * 148 / sms;
+        operands = chains * tokens * kOperandsUs;
+        chain = ceil(chains / sms) * tokens * kChainUs;
+        growth = 2 * chains <= sms && tokens > 0 ? chain / (prep * sms / (sms - chains)) : 0.0;
+    }
+};
 
 // Segments of the two-pass form.  Few long chains leave most SMs idle: the chunk is cut so that a segment's preparation runs
 // beside the chain of the segment before.  A preparation takes whole rounds of items on its CTAs (two per SM; kRoundUs each
 // on all SMs, kBesideUs beside a chain) and a start; a segment has as many rounds as fit beside the chain before it, so that
-// only the first segment's preparation is waited for, whose rounds are those with the smallest total.  Returns the number of
-// segments and where they begin, in blocks; *us: the estimate that the choice between the forms goes by.
+// only the first segment's preparation is waited for, and the last segment takes the rest.  Numbers of segments and of the first
+// one's rounds (up to eight each of them, then in steps of a quarter) are those with the smallest total: the longer the chunk and
+// the more chains, the more of both, so that no long preparation is left to the last segment; or segments that grow by the ratio of
+// the two rates, where whole rounds do not come out (31 heads x 2,900 tokens).  Returns the number of segments and where they
+// begin, in blocks; *us: the total.
 // 1 x 16,384 tokens x 32 heads, us: in one piece 1,340, 4 equal segments 1,060, six that grow by the ratio of the two rates from
-// 14 blocks on 1,093 (every chain but the last was done 20 to 37 us before the preparation beside it), so, five from 37 blocks on,
-// 1,034 with no chain waiting; 1 x 8,192 579 | 562, 1 x 4,096 318 | 309, 1 x 2,048 190 | 181, 1 x 12,000 x 16 heads 771 | 743,
-// 3,000 and 5,000 tokens x 16 heads 369 | 355.
-constexpr int kMaxSegments = 8, kMaxFirstRounds = 8;
-constexpr double kRoundUs = 18.0, kBesideUs = 20.0, kStartUs = 6.0, kGapUs = 12.0;      // (kGapUs: from a chain's last step to the next one's first)
+// 14 blocks on 1,084 (every chain but the last was done 20 to 37 us before the preparation beside it), so, five from 37 blocks on,
+// 1,024 with no chain waiting; 1 x 8,192 584 | 556, 1 x 4,096 320 | 305, 1 x 2,048 189 | 178, 1 x 12,000 x 16 heads 738 | 701.
+// Six growing segments | at most eight, the first of eight rounds at most | so: 1 x 65,536 x 32 heads 3,775 | 3,727 | 3,727,
+// 98,304 5,577 | 6,174 | 5,486, 131,072 7,338 | 9,018 | 7,279, 65,536 x 36 3,889 | 4,973 | 3,889, 32,768 x 40 2,140 | 2,589 | 2,127,
+// 2,900 x 31 236 | 244 | 236.
+// Each segment beyond the eighth has to gain kMoreUs: it takes longer than by this count, 1 x 98,304 x 24 heads with nine 5,453, with
+// eight 5,432, and 65,536 x 32 with eleven 3,733, where the count has gains of 6 and 18 us.
+constexpr int kMaxSegments = 16;
+constexpr double kRoundUs = 18.0, kBesideUs = 20.0, kStartUs = 6.0, kMoreUs = 8.0;
+constexpr double kGapUs = 12.0;         // from a chain's last step to the next one's first
 static int kda_segments(const wpp_kda_desc* d, int sms, double* us, int32_t* begin) {
-    const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
-    const double prep = n * C * kPrepUs * 148 / sms, operands = n * C * kOperandsUs, chain = ceil(n / sms) * C * kChainUs;
+    const KdaRates w(d, sms);
     const int64_t blocks = d->total_tokens / d->num_requests / 64 + 1;
-    const double growth = 2 * n <= sms ? chain / (prep * sms / (sms - n)) : 0.0;
-    if (us) {
-        *us = prep + (chain > operands ? chain : operands);
-        for (int s = 2; growth > 1.05 && s <= 6; ++s) {
-            const double g = growth < 4.0 ? growth : 4.0, first = (g - 1.0) / (pow(g, s) - 1.0);
-            if (first * (double)blocks < 4.0) break;
-            const double t = prep * first + chain + kSegmentUs * (s - 1);
-            if (t < *us) *us = t;
+    const double n = w.chains, step = 64 * kChainUs, all = 2.0 * sms, beside = 2.0 * (sms - n);
+    double best_us = ceil((double)blocks * n / all) * kRoundUs + ceil(n / sms) * (double)blocks * step;
+    begin[0] = 0;
+    *us = best_us;
+    if (w.growth <= 1.05) return 1;
+    // of the segment behind one of `len` blocks: how many it has (two at least: it leaves its state in their operands' place), ...
+    auto behind = [&](int64_t len) {
+        const double fit = floor(((double)len * step + kGapUs - kStartUs) / kBesideUs);
+        return (int64_t)fmax(2.0, floor(fmax(fit, 1.0) * beside / n));
+    };
+    // ... and from the start of the chain of `before` blocks to that of its own, if it has `len`
+    auto wait = [&](int64_t len, int64_t before) {
+        return fmax(ceil((double)len * n / beside) * kBesideUs + kStartUs, (double)before * step + kGapUs);
+    };
+    int best = 1;
+    int64_t best_first = 0;
+    for (int64_t rounds = 1; (double)rounds * all < (double)blocks * n; rounds += rounds < 8 ? 1 : rounds / 4) {
+        const int64_t first = (int64_t)((double)rounds * all / n);
+        double t = (double)rounds * kRoundUs;              // up to the start of the chain of the last segment so far
+        int64_t len = first, done = first;
+        for (int s = 2; s <= kMaxSegments && done < blocks; ++s) {
+            const double rest = (double)(blocks - done), more = s > 8 ? kMoreUs * (s - 8) : 0.0;
+            const double total = t + wait(blocks - done, len) + rest * step + more;
+            if (total < best_us) { best_us = total; best = s; best_first = first; }
+            const int64_t next = behind(len);
+            t += wait(next, len);
+            len = next;
+            done += next;
         }
     }
-    int best = 1;
-    if (begin) begin[0] = 0;
-    if (!begin || !(growth > 1.05)) return best;
-    const double step = 64 * kChainUs, all = 2.0 * sms, beside = 2.0 * (sms - n);
-    double best_us = ceil((double)blocks * n / all) * kRoundUs + (double)blocks * step;
-    for (int candidate = 0; candidate < kMaxFirstRounds * (kMaxSegments - 1); ++candidate) {
-        const int rounds = 1 + candidate / (kMaxSegments - 1), most = 2 + candidate % (kMaxSegments - 1);      // of the first one; segments
-        if (rounds * all >= (double)blocks * n) break;
-        int32_t at[kMaxSegments] = {0};
-        int64_t len = (int64_t)(rounds * all / n), done = 0;
-        double t = rounds * kRoundUs;
-        int s = 0;
-        while (true) {
-            if (len < 1 || s == most - 1 || len > blocks - done) len = blocks - done;
-            if (s > 0) {
-                const double ready = ceil((double)len * n / beside) * kBesideUs + kStartUs, busy = (double)(done - at[s - 1]) * step + kGapUs;
-                t += ready > busy ? ready : busy;
-            }
-            at[s++] = (int32_t)done;
-            done += len;
-            if (done >= blocks) break;
-            const double fit = floor(((double)len * step + kGapUs - kStartUs) / kBesideUs);
-            len = (int64_t)((fit > 1.0 ? fit : 1.0) * beside / n);
+    int64_t len = best_first;
+    for (int s = 1; s < best; ++s, len = behind(len)) begin[s] = begin[s - 1] + (int32_t)len;
+    for (int s = 2; s <= 6; ++s) {                         // segments that grow by the ratio of the two rates
+        const double g = fmin(w.growth, 4.0), one = (double)blocks * (g - 1.0) / (pow(g, s) - 1.0);
+        if (one < 4.0) break;
+        int32_t at[7] = {0};
+        double t = ceil(floor(one) * n / all) * kRoundUs;
+        for (int i = 1; i <= s; ++i) {
+            at[i] = i < s ? (int32_t)(one * (pow(g, i) - 1.0) / (g - 1.0)) : (int32_t)blocks;
+            if (i > 1) t += wait(at[i] - at[i - 1], at[i - 1] - at[i - 2]);
         }
-        t += (double)(blocks - at[s - 1]) * step;
+        t += (double)(at[s] - at[s - 1]) * step;
         if (t < best_us) {
-            best = s;
             best_us = t;
+            best = s;
             for (int i = 0; i < s; ++i) begin[i] = at[i];
         }
     }
+    *us = best_us;
     return best;
+}
+
+// What the choice between the forms takes for the time of the two passes, without their launches: one piece, or the preparation of
+// the first of a few growing segments and the chains.  Apart from kda_segments' total, which is for comparing cuts with one
+// another: with one constant for the launches, this meets the measured times on either side of where the forms cross (us, this
+// and 35 | two passes | group form: 1 x 2,048 x 32 heads 179 | 178 | 186, 2,048 x 24 169 | 168 | 185, 1,024 x 16 104 | 87 | 96; two
+// chunks of 2,048 x 32 260 | 259) and stays within 5 % of them behind it (1 x 4,096 x 32 300 | 305, 16,384 982 | 1,024, 131,072
+// 7,192 | 7,279).
+static double kda_two_passes_us(const wpp_kda_desc* d, int sms) {
+    const KdaRates w(d, sms);
+    const double blocks = (double)(d->total_tokens / d->num_requests / 64 + 1), g = w.growth < 4.0 ? w.growth : 4.0;
+    double us = w.prep + (w.chain > w.operands ? w.chain : w.operands);
+    for (int s = 2; w.growth > 1.05 && s <= 6; ++s) {
+        const double first = (g - 1.0) / (pow(g, s) - 1.0);
+        if (first * blocks < 4.0) break;
+        us = fmin(us, w.prep * first + w.chain + kSegmentUs * (s - 1));
+    }
+    return us;
 }
 
 // Which chunk-parallel kernel: 0 = blocks of 64 tokens in two passes (preparation for all blocks in parallel, then the
@@ -648,9 +693,7 @@ static int kda_pieces(double n, double C, int sms, double us_per_token, double* 
 }
 static int kda_chunk_form(const wpp_kda_desc* d, int sms, int64_t* longest, int* pieces) {
     const double n = (double)d->num_requests * d->num_heads, C = (double)d->total_tokens / d->num_requests;
-    double two_passes = 0.0;
-    kda_segments(d, sms, &two_passes, nullptr);
-    two_passes += 35.0;
+    const double two_passes = kda_two_passes_us(d, sms) + 35.0;
     const struct { double ctas, at_once, us_per_token; } form[4] = {{},
                                                                     {n, (double)sms, 0.165},                                 // one CTA per SM
                                                                     {2 * n, 2.0 * sms, 2 * n <= sms ? 0.14 : 0.2},           // two per SM
@@ -682,13 +725,17 @@ static int kda_chunk_form(const wpp_kda_desc* d, int sms, int64_t* longest, int*
     }
     return best;
 }
-// (the choice by itself, for the tests: no GPU needed)
+// (the choices by themselves, for the tests: no GPU needed)
 extern "C" int wpp_kda_choice(const wpp_kda_desc* d, int sms, int64_t* longest, int* pieces) {
     if (!kda_desc_ok(d) || d->num_requests < 1 || d->total_tokens < 64 * (int64_t)d->num_requests || sms < 1) return -1;
     *longest = 0;
     const int form = kda_chunk_form(d, sms, longest, pieces);
     if (form != 1) *pieces = 1;
     return form;
+}
+extern "C" int wpp_kda_cut(const wpp_kda_desc* d, int sms, double* us, int32_t* begin /* [16] */) {
+    if (!kda_desc_ok(d) || d->num_requests < 1 || sms < 1) return -1;
+    return kda_segments(d, sms, us, begin);
 }
 
 extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const void* q, const void* k, const void* v,
@@ -843,7 +890,8 @@ extern "C" int wpp_kda_chunk(const wpp_ctx* ctx, const wpp_kda_desc* desc, const
         // launches that usually have nothing to do)
         p.gated = gated;
         int32_t seg_begin[kMaxSegments] = {0};
-        const int segments = gated ? 1 : kda_segments(desc, ctx->sm_count, nullptr, seg_begin);
+        double us = 0.0;
+        const int segments = gated ? 1 : kda_segments(desc, ctx->sm_count, &us, seg_begin);
         e = wpp_launch_kda_tc(&p, maps, desc->total_tokens > 0 ? (int)w.max_blocks : 0, ctx->sm_count, segments, seg_begin,
                               cuda_stream);
         if (e != 0) return cuda_fail(ctx, e);

@@ -15,6 +15,7 @@ import wpp_workloads as W
 from oracle import kda as O
 from tests import gpu_harness as H
 from tests.test_kda_pieces import choice
+from tests.test_kda_segments import cut
 
 pytestmark = pytest.mark.gpu
 
@@ -339,6 +340,53 @@ def test_long_chunks_in_segments_match_the_oracle(lens, prefix, interval):
             pool = torch.from_numpy(new_pool).float()
         assert np.array_equal(np.concatenate(parts), got_o)
         assert np.array_equal(pool.double().numpy(), got_pool)
+
+
+@pytest.mark.parametrize("lens,prefix,interval,H_,segments", [([4096], [70], 0, 32, 3), ([4096], [0], 1152, 32, 3), ([4100], [129], 1000, 32, 3),
+                                                              ([4500, 3692], [63, 0], 640, 16, 3), ([9000, 10, 0], [0, 5, 64], 1000, 11, 3),
+                                                              ([16384], [0], 4096, 32, 5)])
+def test_three_segments_and_more_match_the_oracle(lens, prefix, interval, H_, segments):
+    """As above with chains enough for more than a few segments: how many ran is asserted, and snapshots lie on the cuts (block 18
+    of 64 tokens: 1,152) and off them."""
+    assert len(cut(len(lens), H_, sum(lens))) == segments
+    w = W.kda_workload("segments", 92, lens, H_, prefix, snap_interval=interval)
+    t = w.tensors()
+    launches = H.ctx().launch_count()
+    got_o, got_pool, status = _gpu(w, t, layout=3)
+    assert status == 0 and H.ctx().launch_count() - launches == 1 + 2 * segments
+    heads = [0, H_ - 1]
+    ref_o, ref_pool = _oracle(w, t, heads=heads)
+    _close_out(got_o[:, heads], ref_o, "outputs")
+    _close_state(got_pool[:, heads], ref_pool, "state pool")
+
+
+@pytest.mark.parametrize("tokens,H_,at_least", [(16384, 32, 5), (32768, 40, 9)])
+def test_any_number_of_segments_has_the_bits_of_two_resumed_calls(tokens, H_, at_least):
+    dev = torch.device("cuda")
+    g = torch.Generator(device=dev).manual_seed(tokens)
+    normal = lambda *shape: torch.empty(*shape, device=dev).normal_(generator=g)
+    q, k, v = (normal(tokens, H_, 128).mul_(f).bfloat16() for f in (0.088, 0.088, 1.0))
+    alpha, beta = torch.sigmoid(normal(tokens, H_, 128) + 4.0), torch.sigmoid(normal(tokens, H_))
+    start = normal(2, H_, 128, 128).mul_(0.1)
+    status, i32 = torch.zeros(1, dtype=torch.int32, device=dev), lambda *x: torch.tensor(x, dtype=torch.int32, device=dev)
+
+    def run(pool, lo, hi, s_in):
+        n, launches = hi - lo, H.ctx().launch_count()
+        ws = torch.full((wpp.wpp_kda_workspace_bytes(1, H_, n),), 0xFF, dtype=torch.uint8, device=dev)
+        out = wpp.wpp_kda_chunk(H.ctx(), q[lo:hi], k[lo:hi], v[lo:hi], alpha[lo:hi], beta[lo:hi],
+                                torch.tensor([0, n], dtype=torch.int64, device=dev), pool, i32(s_in), i32(1), prefix_lens=i32(lo),
+                                status=status, layout=3, workspace=ws)
+        segments = (H.ctx().launch_count() - launches - 1) // 2
+        assert segments == len(cut(1, H_, n))
+        return out, segments
+
+    whole, parts = start.clone(), start.clone()
+    out, segments = run(whole, 0, tokens, 0)
+    assert segments >= at_least
+    middle = tokens // 3 // 64 * 64
+    first, second = run(parts, 0, middle, 0)[0], run(parts, middle, tokens, 1)[0]
+    assert int(status.item()) == 0
+    assert torch.equal(torch.cat([first, second]).view(torch.int16), out.view(torch.int16)) and torch.equal(parts, whole)
 
 
 def test_calls_of_few_long_chains_end_alike_however_cold_the_caches_are():
