@@ -4,6 +4,7 @@ import pytest
 import torch
 
 import oracle
+import paper_2609_35263_b200 as wpp
 import wpp_workloads as W
 from tests.helpers import bits, cpu_inputs, from_bits
 from tests import gpu_harness as H
@@ -46,6 +47,48 @@ def test_append_finds_every_request(R, most, Hkv, d, B):
     res = H.run_wave(w, H.device_inputs(w, inp), do_attention=False)
     assert res["status"] == 0
     assert np.array_equal(bits(res["k_pool"]), kp) and np.array_equal(bits(res["v_pool"]), vp)
+
+
+def test_append_does_not_walk_over_empty_chunks():
+    """The second token of a warp may belong to a request far behind that of its first one: no slower than with the next one (a
+    walk from request to request over 30,000 of them takes a hundred times as long)."""
+    R, dev = 30000, torch.device("cuda")
+    k = torch.randn(2, 1, 64, device=dev).bfloat16()
+    pool = torch.zeros(2, 1, 16, 64, dtype=torch.bfloat16, device=dev)
+    d = wpp.make_desc(R, 1, 1, 64, 16, 1, 2)
+    P, status, best = np.zeros(R, np.int32), torch.zeros(1, dtype=torch.int32, device=dev), {}
+    for behind in (1, R - 1):
+        C = np.zeros(R, np.int32)
+        C[0] = C[behind] = 1
+        bt = torch.zeros(R, 1, dtype=torch.int32, device=dev)
+        bt[behind] = 1
+        plan = wpp.wpp_plan_tiles(H.ctx(), d, P, C).to_device()
+        Pd, Cd = torch.from_numpy(P).to(dev), torch.from_numpy(C).to(dev)
+        for _ in range(20):
+            pool.zero_()
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            wpp.wpp_kv_append(H.ctx(), d, k, k, pool, pool, bt, Pd, Cd, plan, status=status)
+            b.record()
+            torch.cuda.synchronize()
+            best[behind] = min(best.get(behind, 1e9), a.elapsed_time(b))
+            assert torch.equal(pool[:, 0, 0], k[:, 0]) and int(status.item()) == 0
+    assert best[R - 1] < 5 * best[1], best
+
+
+@pytest.mark.parametrize("gaps", [(0, 1, 2, 3), (4, 5, 7, 8), (15, 16, 17, 31), (63, 64, 100, 333)])
+def test_append_steps_over_any_number_of_empty_chunks(gaps):
+    C = []
+    for n in gaps + gaps:
+        C += [2] + [0] * n + [1]
+    for tail in (0, 1, 6):
+        lens = C + [0] * tail
+        w = W.custom_workload([i % 7 for i in range(len(lens))], lens, 1, 1, 64, 16, seed=len(lens), spare_pages=3)
+        inp = cpu_inputs(w)
+        kp, vp = oracle.oracle_append(inp["k_new"], inp["v_new"], inp["k_pool"], inp["v_pool"], w.block_tables, w.prefix_lens, w.chunk_lens)
+        res = H.run_wave(w, H.device_inputs(w, inp), do_attention=False)
+        assert res["status"] == 0
+        assert np.array_equal(bits(res["k_pool"]), kp) and np.array_equal(bits(res["v_pool"]), vp)
 
 
 def test_append_shared_prefix_pages_are_left_alone():
