@@ -21,13 +21,15 @@ namespace wpp {
 // warp.  Append in a graph, us, a bisection in front of the loads | now: 128 x 3 tokens (64/8 heads) 3.4 | 2.7, 32 x 64 4.3 |
 // 4.2, 32 x 256 11.8 | 10.4, 32 x 1,024 47.5 | 47.2 (5.7 TB/s).
 //
-// A grid that the SMs hold at once (`few`) is set up while the kernel before it runs, which is worth 2 us, and lets the
-// attention kernel in as its CTAs end; a larger one starts behind the kernel before and lets the attention kernel in at once.
+// A grid that the SMs hold at once (`few`: kAppendCtas per SM, which the launch bounds hold the registers to) is set up while the
+// kernel before it runs, which is worth 2 us, and lets the attention kernel in as its CTAs end; a larger one starts behind the
+// kernel before and lets the attention kernel in once its last CTAs have started (an SM holds half of its eight: 64 registers).
 // Pass, us, the latter for all | the former for all: 1 x 128 tokens over 256 (8/2 heads) 14.3 | 12.5, 32 x 64 (64/8) 25.5 |
 // 24.6, 5 x 32..276 over 100..4,000 63.3 | 59.7, but 32 x 512 304 | 309.
 constexpr int kAppendVec = 4;          // of a large grid (1: 11.2 us for 32 x 256 tokens, 2: 10.5, 8: 13.5)
+constexpr int kAppendCtas = 8;         // per SM
 template <int kVec>
-__global__ void __launch_bounds__(256) wpp_append_kernel(const AppendParams p) {
+__global__ void __launch_bounds__(256, kVec == 1 ? kAppendCtas : kAppendCtas / 2) wpp_append_kernel(const AppendParams p) {
     if (!p.few) grid_launch_dependents();
     grid_dependency_wait();
     const char* plan = static_cast<const char*>(p.plan);
@@ -198,10 +200,10 @@ extern "C" int wpp_launch_append(const wpp::AppendParams* p, int num_sms, void* 
     const int64_t total = p->total_new_tokens * p->num_kv_heads * p->vec_per_row;
     if (total == 0) return 0;
     wpp::AppendParams q = *p;
-    q.few = total <= (int64_t)num_sms * 8 * 256;
+    q.few = total <= (int64_t)num_sms * wpp::kAppendCtas * 256;
     const int per_block = q.few ? 256 : 256 * wpp::kAppendVec;
     int64_t blocks = (total + per_block - 1) / per_block;
-    const int64_t cap = (int64_t)num_sms * 8;
+    const int64_t cap = (int64_t)num_sms * wpp::kAppendCtas;
     if (blocks > cap) blocks = cap;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);

@@ -32,6 +32,13 @@ def test_tensor_memory_is_allocated_before_the_next_kernel_is_let_in():
     assert seen >= 3
 
 
+def test_an_append_grid_that_is_set_up_early_fits_the_sms():
+    """What counts as such a grid is what the launch bounds make room for, whatever registers the kernel would like."""
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "wpp_append_combine.cu")).read())
+    assert re.search(r"__launch_bounds__\(256, kVec == 1 \? kAppendCtas : [^)]*\) wpp_append_kernel", src)
+    assert re.search(r"q\.few = total <= \(int64_t\)num_sms \* wpp::kAppendCtas \* 256;", src)
+
+
 @pytest.mark.gpu
 def test_small_attention_directly_behind_the_two_pass_recurrent_layer():
     """The chain kernel takes all 512 columns of an SM's tensor memory, the small attention shape 256 per CTA: queued behind
