@@ -122,3 +122,65 @@ def test_passes_one_behind_the_other_see_their_own_keys(P, C, shape):
         torch.cuda.synchronize()
         assert int(status.item()) == 0 and all(torch.equal(a, b) for a, b in zip(alone, outs))
     assert not torch.equal(alone[0], alone[1])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("with_append", [False, True])
+@pytest.mark.parametrize("shape", [1, 2])
+@pytest.mark.parametrize("lens,layout", [([200, 70, 333], 3), ([4096], 3), ([200], 0), ([100, 130, 64], 0)])
+def test_append_and_attention_directly_behind_the_recurrent_layer(lens, layout, shape, with_append):
+    """Both are set up while the kernel before them runs: behind the two passes (one segment and several; the chain kernel and the
+    SM-wide attention kernel take all 512 columns of an SM's tensor memory), behind the group form alone and behind the empty two
+    passes that follow it.  Every result is what it is apart."""
+    import numpy as np
+    import torch
+
+    import paper_2609_35263_b200 as wpp
+    import wpp_workloads as W
+    from tests import gpu_harness as H
+    from tests.test_gpu_kda import _gpu
+    from tests.test_kda_pieces import choice
+    from tests.test_kda_segments import cut
+
+    heads = 32 if lens == [4096] else 7
+    if layout == 0:
+        assert choice(len(lens), heads, sum(lens))[0] > 0
+    else:
+        assert len(cut(len(lens), heads, sum(lens))) == (3 if lens == [4096] else 1)
+    dev = torch.device("cuda")
+    w = W.custom_workload([300, 64, 0, 17], [33, 64, 90, 5], 8, 2, 64, 16, seed=23)
+    g = H.device_inputs(w)
+    pools = g["k_pool"].clone(), g["v_pool"].clone()
+    apart = H.run_wave(w, g, shape=shape)
+    after = g["k_pool"].clone(), g["v_pool"].clone()
+    kw = W.kda_workload("front", 29, lens, heads, [5, 0, 64][:len(lens)])
+    t = kw.tensors()
+    o_apart, pool_apart, status = _gpu(kw, t, layout=layout)
+    assert status == 0 and apart["status"] == 0
+    d = {k: v.to(dev) for k, v in t.items()}
+    i32 = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).to(dev)
+    rows, s_in, s_out, prefix = torch.from_numpy(kw.row_offsets).to(dev), i32(kw.state_in), i32(kw.state_out), i32(kw.prefix_lens)
+    chunks, P, bt = i32(w.chunk_lens), i32(w.prefix_lens), i32(w.block_tables)
+    ws = torch.empty(wpp.wpp_kda_workspace_bytes(len(lens), heads, sum(lens)), dtype=torch.uint8, device=dev)
+    plan, status = apart["plan"], torch.zeros(1, dtype=torch.int32, device=dev)
+    ws_attn = torch.empty(int(plan.info.workspace_bytes), dtype=torch.uint8, device=dev)
+    pool0 = d["state_pool"].clone()
+    for _ in range(10):
+        out, out_kda = torch.zeros_like(apart["out"]), torch.zeros_like(d["v"])
+        d["state_pool"].copy_(pool0)
+        for name, before, now in zip(("k_pool", "v_pool"), pools, after):
+            g[name].copy_(before if with_append else now)
+        torch.cuda.synchronize()
+        for _ in range(2):                                          # (the recurrent layer behind the attention kernel as well)
+            d["state_pool"].copy_(pool0)
+            wpp.wpp_kda_chunk(H.ctx(), d["q"], d["k"], d["v"], d["alpha"], d["beta"], rows, d["state_pool"], s_in, s_out, out=out_kda,
+                              prefix_lens=prefix, status=status, layout=layout, workspace=ws)
+            if with_append:
+                wpp.wpp_kv_append(H.ctx(), H.desc_of(w), g["k_new"], g["v_new"], g["k_pool"], g["v_pool"], bt, P, chunks, plan, status=status)
+            wpp.wpp_prefill_attention_varlen(H.ctx(), H.desc_of(w), g["q"], out, None, g["k_pool"], g["v_pool"], bt, P, chunks, plan,
+                                             workspace=ws_attn, status=status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        assert torch.equal(out, apart["out"]) and torch.equal(g["k_pool"], after[0]) and torch.equal(g["v_pool"], after[1])
+        assert np.array_equal(out_kda.float().cpu().double().numpy(), o_apart)
+        assert np.array_equal(d["state_pool"].cpu().double().numpy(), pool_apart)
