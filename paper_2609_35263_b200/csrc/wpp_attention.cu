@@ -231,18 +231,11 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             uint32_t va_phase = 0;
             while (true) {
                 bool ok = false;
-                long long t0 = clock64();
-                int32_t tile = -1;
-                // (nothing to do may last as long as the launch: the limit begins anew as long as tiles are handed on.  The issuing
-                // thread always says that there are no more, its own waits have the usual limit.)
-                while (!(ok = mbar_test(bVAsk, va_phase) != 0u) && !*abort_flag) {
-                    if (clock64() - t0 > 64 * WPP_WAIT_LIMIT) {
-                        if (tile_ids[0] == tile) { *abort_flag = 1u; break; }
-                        tile = tile_ids[0];
-                        t0 = clock64();
-                    }
+                const long long t0 = clock64();
+                // (nothing to do may last as long as the launch: a limit of hours.  The issuing thread always says that there are
+                // no more and its own waits have the usual limit, after which the flag is up.)
+                while (!(ok = mbar_test(bVAsk, va_phase) != 0u) && !*abort_flag && clock64() - t0 < 16384 * WPP_WAIT_LIMIT)
                     __nanosleep(256);
-                }
                 if (!__all_sync(0xffffffffu, ok)) break;
                 va_phase ^= 1u;
                 const int slot = v_rows[0], valid = v_rows[1];
