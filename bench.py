@@ -640,7 +640,7 @@ def main():
                     help="skip the short runs of further workloads reported under other_configs")
     ap.add_argument("--force-kv-splits", type=int, default=0)
     ap.add_argument("--cpu-seconds", type=float, default=15.0)
-    ap.add_argument("--plan-order", type=int, default=0, help="0: stream order (default), 1: longest tile first")
+    ap.add_argument("--plan-order", type=int, default=0, help="0: the planner's (default), 1: longest tile first, 2: stream order")
     ap.add_argument("--max-ctas", type=int, default=0, help="persistent CTAs to launch (0: one per SM)")
     ap.add_argument("--shape", type=int, default=0, help="attention kernel: 0 planner's choice, 1 SM-wide two-half CTAs, "
                                                          "2 small single-half CTAs (two per SM)")

@@ -44,6 +44,12 @@ __device__ __forceinline__ int counter_slot(const unsigned long long* totals) {
     return (int)(reinterpret_cast<uintptr_t>(totals) % kCounterBytes / 16);
 }
 
+__device__ __forceinline__ unsigned long long atomic_add_acquire(unsigned long long* at, unsigned long long v) {
+    unsigned long long before;
+    asm volatile("atom.acquire.gpu.global.add.u64 %0, [%1], %2;" : "=l"(before) : "l"(at), "l"(v) : "memory");
+    return before;
+}
+
 constexpr int kThreads = 512;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColS = 0;                                                        // landing buffer of S
@@ -733,9 +739,9 @@ wpp_attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const int slot = counter_slot(p.totals);
         const uint32_t each = 0xffffffffu / gridDim.x;
         const unsigned long long share = blockIdx.x ? each : 0x100000000ull - (unsigned long long)each * (gridDim.x - 1);
-        const unsigned long long before = atomicAdd(&g_ended[slot], share);
+        // (a fence in place of the acquire: 0.7 us of every launch)
+        const unsigned long long before = atomic_add_acquire(&g_ended[slot], share);
         if (((before & 0xffffffffull) + share) >> 32) {
-            __threadfence();
             unsigned long long* count = g_counts[slot / kCounterSlots];
             const unsigned long long steps = atomicAdd(count, 0ull), moves = atomicAdd(count + 1, 0ull);
             *reinterpret_cast<ulonglong2*>(p.totals) = make_ulonglong2(steps, moves);

@@ -85,29 +85,21 @@ constexpr int64_t kPairHeadsKeys = 2048;     // keys a query sees on average fro
 constexpr int64_t kTileFixedCost = 3, kPartExtraCost = 2, kCombineCost = 20;
 
 // Estimated microseconds of a wave on either kernel shape: tiles (or halves) handed out in order to the CTA free first,
-// each with a start and end and a time per 128-key step.  Constants from waves timed on 148 SMs, attention call in us, SM-wide |
-// small (requests x new tokens over cached ones, 64/8 heads of 128):
-//     32 x 64            44 |  21       32 x 300..1000       525 | 445      32 x 64 / 1024          102 | 117
-//     32 x 128           60 |  45       32 x 1024            781 | 789      32 x 256 / 1024         309 | 443
-//     32 x 256          117 |  97       16 x 2048           1199 | 1466     16 x 512 / 2048         556 | 878
-//     32 x 512          303 | 246       64 x 1..300 / 0..500  83 |  69      8 x 300 / 700            68 |  70
-// (the last two in the middle and on the right with 16/4 heads of 64 and 32/8 of 128; the least of five runs of ten calls.  The
-// median of nine on another B200: 32 x 512 326 | 263, 32 x 1024 847 | 818, 32 x 256 / 1024 328 | 440, 8 x 300 / 700 68 | 70).  The
-// line lies where both are about equal: 32 x 1024, 3 % better on the small shape there, is on the SM-wide side.  With
-// 3.3 and 3.0 us, the constants of one thread per query row, 32 x 300..1000 and 64 x 1..300 / 0..500 went to the SM-wide shape;
-// with one slope for all lengths 4 x 1407, 2 x 196..1950 and 7 x 1250..1751 went to the small one (pass, us, SM-wide | small:
-// 132 | 147, 69 | 86, 62 | 74; but 80 x 228 over 119..239 271 | 214, 12 x 210..393 over 127..212 132 | 108).
+// each with a start and end and a time per 128-key step.  Constants from waves timed on 148 SMs; attention call now, with the
+// planner's order of tiles, in us, SM-wide | small (requests x new tokens over cached ones, 64/8 heads of 128, the median of
+// seven runs of twenty calls):
+//     32 x 64            37 |  21       32 x 300..1000        381 | 418     32 x 64 / 1024          105 | 117
+//     32 x 128           59 |  44       32 x 1024             722 | 846     32 x 256 / 1024         313 | 405
+//     32 x 256          116 |  96       16 x 2048            1172 | 1467    16 x 512 / 2048         589 | 774
+//     32 x 512          252 | 247       7 x 1250..1751        317 | 393     80 x 228 / 119..239     426 | 381
+// The line lies where both are about equal; 32 x 300..1000 is on the wrong side of it.
 // Where the small shape's items take several rounds and average more than kSmallShapeSteps key steps, the SM-wide one is taken
-// whatever the estimate says, because that is too short for some of these waves by up to a third: items whose lengths differ
-// much, and the shorter steps of heads of 64.  Of 55 drawn waves that only this rule sends to the SM-wide shape the small one
-// is slower on 11, by up to a half, and faster on 44, by up to 32 % (pass, us, SM-wide | small: 69 x 14..39 over 160..3,524
-// cached tokens, 32/8 heads, 146 | 219; 51 x 25..34 over 2,234..3,626 146 | 201; 120 x 3..35 over 2,520..4,368, 16/4 of 64,
-// 153 | 201; 42 x 5 over 253..2,477, 64/8, 80 | 99; but 22 x 7..15 over 987..1,080, 40/8, 118 | 80; 32 x 4..34, 40/8, over 1,100 /
-// 1,500 / 4,096 140 | 126, 167 | 162, 430 | 406).  An estimate that tells them apart could take its place.
-// All of these figures are from before tiles were ordered by length and a launch cost 4 us less (32 x 1024 on the SM-wide shape, a
-// call at a time: 774 us before, 650 since).  With both, over 170 drawn waves the choice loses 0.6 % in the geometric mean
-// against the better shape of each wave; a fixed cost of 6 us for the SM-wide shape and no kSmallShapeSteps would lose 0.3 %: not
-// enough to move plans for.
+// whatever the estimate says, because that is too short for some of these waves by up to two fifths: items whose lengths differ
+// much, and the shorter steps of heads of 64 (69 x 14..39 over 160..3,524, 32/8 heads, 133 | 191; 120 x 3..35 over 2,520..4,368,
+// 16/4 of 64, 155 | 208; 51 x 25..34 over 2,234..3,626, 32/8, 137 | 148; 42 x 5 over 253..2,477 60 | 70; but 32 x 4..34 over
+// 1,100, 40/8, 98 | 81, over 4,096 261 | 265).  An estimate that tells them apart could take its place: over 170 drawn waves the
+// choice loses 0.6 % in the geometric mean against the better shape of each wave, and a fixed cost of 6 us for the SM-wide
+// shape without kSmallShapeSteps would lose 0.3 %, not enough to move plans for.
 constexpr int64_t kSmallShapeSteps = 8;
 struct StepCount {
     int64_t sum = 0;
